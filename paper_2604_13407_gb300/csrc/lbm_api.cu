@@ -179,6 +179,12 @@ static void fill_constants(lbm_ctx *c)
     k.k2 = p.k2;
     k.G = p.G;
     const double eps = -8.0 * (p.k1 + p.k2);
+    k.q1c = 3.0 * (p.k1 + 2.0 * p.k2);
+    k.q4a = (30.0 * eps - 15.0) / 16.0;
+    k.q4b = 3.0 * eps / 8.0;
+    k.inv_G = 1.0 / p.G;
+    int g_exp;
+    k.G_pow2 = std::frexp(p.G, &g_exp) == -0.5 && std::abs(g_exp) < 500;
     k.kq1 = 3.0 * (p.k1 + 2.0 * p.k2) * p.G;
     k.kq7 = p.k1 * p.G;
     k.c1G = (30.0 * eps - 15.0) / 16.0 * p.G;

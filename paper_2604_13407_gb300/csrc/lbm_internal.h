@@ -49,6 +49,9 @@ struct KParams {
     double eos_R, eos_T;  // raw R and T (FP64 path evaluates (rho R) T like a plain formula)
     double G;
     double k1, k2;        // raw source coefficients (FP64 path)
+    double q1c, q4a, q4b;  // 3 (k1 + 2 k2), (30 eps - 15)/16, 3 eps/8 (FP64 path, evaluated on the host)
+    double inv_G;          // 1/G
+    int G_pow2;            // 1: G is +- a power of two, so that x/G = x inv_G exactly
     // source term with G folded in (|F_int|^2/(G psi^2) = G |S|^2, S = F_int/(-G psi)):
     // Q1 = kq1 |S|^2, Q2 = q2fac Q1, Q7 = kq7 (Sx^2 - Sy^2), Q8 = kq7 Sx Sy,
     // Q4 = (c1G Sx^2 - c2G Sy^2) ux, Q6 = (c1G Sy^2 - c2G Sx^2) uy
