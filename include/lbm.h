@@ -83,9 +83,10 @@ typedef enum {
 } lbm_force_mode;
 
 typedef enum {
-    LBM_KERNEL_AUTO = 0,     /* fused kernel when the geometry allows it, else two-pass */
+    LBM_KERNEL_AUTO = 0,     /* the fastest: one pass per step, on tiles (the two-pass step's results)
+                                or, on large periodic lattices, on staged rows */
     LBM_KERNEL_TWO_PASS = 1, /* psi pass + fused collide-and-pull-stream pass */
-    LBM_KERNEL_FUSED = 2     /* one pass per step, psi recomputed on a staged halo */
+    LBM_KERNEL_FUSED = 2     /* one pass per step, psi recomputed on a halo */
 } lbm_kernel;
 
 /*
@@ -273,7 +274,8 @@ LBM_API lbm_status lbm_sync(lbm_ctx *ctx);
 /* Number of steps since the last lbm_init_fields / lbm_set_state. */
 LBM_API int64_t lbm_step_count(const lbm_ctx *ctx);
 
-/* Kernel actually used by lbm_step (LBM_KERNEL_TWO_PASS or LBM_KERNEL_FUSED). */
+/* Kind of step lbm_step runs: LBM_KERNEL_FUSED, or LBM_KERNEL_TWO_PASS for the two-pass step's results
+ * (from the two-pass kernels, or in one pass from the tile kernel of LBM_KERNEL_AUTO). */
 LBM_API int32_t lbm_kernel_in_use(const lbm_ctx *ctx);
 
 /* "LB-ana" (Sec. 3.1, Figs. 3-4): the steady velocity profile of two-phase Poiseuille flow that

@@ -1,15 +1,7 @@
 // Kernel instantiations for double population storage.
 #include "k_adjoint.cuh"
-#include "k_fused.cuh"
+#include "k_tile.cuh"
 #include "k_twopass.cuh"
-
-// strip width (consumer warps of 30 columns) and staged-row ring depth of the fused kernel
-#ifndef LBM_FUSED_NW
-#define LBM_FUSED_NW 8
-#endif
-#ifndef LBM_FUSED_RING
-#define LBM_FUSED_RING 8
-#endif
 
 namespace lbm {
 
@@ -18,7 +10,8 @@ Launchers launchers_f64()
     Launchers L{};
     L.psi_pass = &TwoPass<double>::psi_pass;
     L.collide_pass = &TwoPass<double>::collide_pass;
-    L.fused_pass = &Fused<double, LBM_FUSED_NW, LBM_FUSED_RING>::launch;
+    L.tile_pass = &Tile<double>::step;
+    L.link_bits = &Tile<double>::link_bits;
     L.init = &TwoPass<double>::init;
     L.moments = &TwoPass<double>::moments;
     L.diag = &TwoPass<double>::diag;
@@ -30,8 +23,8 @@ Launchers launchers_f64()
     L.objective = &Adjoint<double>::objective;
     L.adj_blocks = &Adjoint<double>::blocks;
     L.adj_reduce = &Adjoint<double>::reduce;
-    L.fused_tile_x = FusedLayout<double, LBM_FUSED_NW, LBM_FUSED_RING>::TX;
-    L.fused_align = FusedGeom<double>::HX;
+    L.fused_tile_x = 240;
+    L.fused_align = 2;
     return L;
 }
 

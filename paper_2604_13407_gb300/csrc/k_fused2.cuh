@@ -1,17 +1,24 @@
-// Fused single-pass step with two nodes per lane and packed FP32 arithmetic, for the
-// storage types whose arithmetic is FP32 (FP32, FP16 and BF16 deviations).
+// Staged single-pass step with two nodes per lane and packed FP32 arithmetic, for the
+// storage types whose arithmetic is FP32 (FP32, FP16 and BF16 deviations), on lattices that
+// are periodic in both directions and have no walls: the large ones, where keeping HBM busy
+// all the time counts and a block's serial walk does not (the tile kernel, k_tile.cuh, steps
+// all others).
 //
-// Same pipeline as k_fused (k_fused.cuh): one producer warp stages every row of the nine
-// population planes into a shared-memory ring with bulk async copies (full/empty
-// mbarriers, bounded waits); the consumer warps pull, form rho and psi, and one row later
-// collide with the 3 x 3 psi neighbourhood from registers and warp shuffles.  What
-// changes is the work of a lane: it owns two adjacent columns (an even column and the
-// next), so every FP32 addition, multiplication and multiply-add of the step -- moments,
-// EOS, stencil, forces, source term, relaxation, back-transform and storage codec -- is
-// one packed FP32x2 instruction (FADD2 / FMUL2 / FFMA2 of the sm_100 family) for two
-// lattice nodes, the populations of the pair move as 8-byte (FP32) or 4-byte (FP16/BF16)
-// shared loads and global stores, and the psi halo costs two shuffles per row for two
-// nodes.  Reciprocal and square root stay per node.  A warp covers 64 columns: lanes
+// A CTA owns a strip of 60 NW columns and walks down a segment of rows.  One producer warp
+// stages every row of the nine population planes (and of the reference-density plane of
+// per-node 16-bit storage) into a shared-memory ring with bulk async copies; each ring slot
+// has a "full" mbarrier (completed by the copies' byte count) and an "empty" one (one arrival
+// per consumer warp).  The consumer warps pull, form rho and psi, keep the pulled populations
+// in registers and one row later collide with the 3 x 3 psi neighbourhood from registers and
+// warp shuffles; there is no block-wide barrier in the loop.  Halo psi is recomputed, so HBM
+// sees each population read once and written once.
+//
+// A lane owns two adjacent columns (an even column and the next), so every FP32 addition,
+// multiplication and multiply-add of the step -- moments, EOS, stencil, forces, source term,
+// relaxation, back-transform and storage codec -- is one packed FP32x2 instruction (FADD2 /
+// FMUL2 / FFMA2 of the sm_100 family) for two lattice nodes, the populations of the pair move
+// as 8-byte (FP32) or 4-byte (FP16/BF16) shared loads and global stores, and the psi halo
+// costs two shuffles per row for two nodes.  Reciprocal and square root stay per node.  A warp covers 64 columns: lanes
 // 1..30 update 60 columns, lanes 0 and 31 carry the halo columns.
 //
 // Density, psi, stencil and collision are the FP32 formulation of lbm_f32.cuh evaluated on
@@ -23,7 +30,7 @@
 // two.
 #pragma once
 
-#include "k_fused.cuh"
+#include "async_ring.cuh"
 
 namespace lbm {
 
@@ -100,18 +107,6 @@ template <> struct Pair2<__nv_bfloat16> {
 };
 #undef LBM_DEC_PAIR
 
-// One already-scaled FP32 value rounded to the storage type (as the pair stores round).
-template <class S> struct Codec2;
-template <> struct Codec2<float> {
-    static __device__ __forceinline__ void put(float *p, float v) { *p = v; }
-};
-template <> struct Codec2<__half> {
-    static __device__ __forceinline__ void put(__half *p, float v) { *p = __float2half_rn(v); }
-};
-template <> struct Codec2<__nv_bfloat16> {
-    static __device__ __forceinline__ void put(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
-};
-
 __device__ __forceinline__ v2 load_ref_pair(const float *p, int off)
 {
     if (off == 0) return v2{*reinterpret_cast<const float2 *>(p)};
@@ -153,134 +148,11 @@ __device__ __forceinline__ void external_force_pair(const KParams &kp, int64_t n
         }                                                                                                     \
     }
 
-// ----------------------------------------------------- general geometry ------
-// Solid flags of columns c0 - 1 .. c0 + 2 of lattice row y (bit k = column c0 - 1 + k), with
-// periodic wrapping; nodes beyond a non-periodic edge read as fluid (those links are walls
-// by the edge test).
-// The four flags are fetched one row ahead of their use (solid_fetch) and combined when
-// the row is reached (solid_bits), so the latency of the global loads overlaps a row of work.
-struct SolidRow {
-    int v[4];
-};
-__device__ __forceinline__ SolidRow solid_fetch(const KParams &kp, int y, int c0)
-{
-    SolidRow w{{0, 0, 0, 0}};
-    if (y < 0 || y >= kp.ny) {
-        if (!kp.periodic_y) return w;
-        y = y < 0 ? y + kp.ny : y - kp.ny;
-    }
-    const uint8_t *r = kp.solid + (int64_t)y * kp.nx;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        int x = c0 - 1 + k;
-        if (x < 0 || x >= kp.nx) {
-            if (!kp.periodic_x) continue;
-            x = x < 0 ? x + kp.nx : x - kp.nx;
-        }
-        w.v[k] = r[x];
-    }
-    return w;
-}
-__device__ __forceinline__ int solid_bits(const SolidRow &w)
-{
-    return (w.v[0] != 0) | (w.v[1] != 0) << 1 | (w.v[2] != 0) << 2 | (w.v[3] != 0) << 3;
-}
-
-// Population k of a node near (xw, yw) read from the staged rows (for `bounce`, which asks
-// for the node itself and its neighbour along e_i by lattice coordinates), decoded to FP32
-// like the pull: `row`/`ref` point at the staged column of the pair's first node, `e` is
-// the element of the pair.
-// The three row pointers are separate members and chosen by comparison: an array indexed
-// by a run-time row would be placed in local memory, and with it every staged-row access of
-// the kernel.
-template <class S, int W>
-struct StagedAt {
-    const KParams &kp;
-    const S *rm, *r0, *rp;
-    const float *fm, *f0, *fp;
-    int e, xw, yw;
-    __device__ __forceinline__ float operator()(int k, int xx, int yy) const
-    {
-        int dx = xx - xw, dy = yy - yw;
-        if (dx > 1) dx -= kp.nx;
-        else if (dx < -1) dx += kp.nx;
-        if (dy > 1) dy -= kp.ny;
-        else if (dy < -1) dy += kp.ny;
-        const int col = e + dx;
-        const S *r = dy < 0 ? rm : (dy > 0 ? rp : r0);
-        float v = Pair2<S>::load1(r + k * W + col);
-        if constexpr (IsDev<S>::value) {
-            const float *f = dy < 0 ? fm : (dy > 0 ? fp : f0);
-            const float rf = f0 ? f[col] : kp.cf.rho_ref;
-            v = __fmaf_rn(v, kp.cf.inv_scale, __fmul_rn(w_<float>(k), rf));
-        }
-        return v;
-    }
-};
-
-// A wall link from its record (KParams::link: link fraction q, moving-wall coefficient c):
-// the bounce-back rule of `bounce` (Bouzidi interpolation, moving-wall term c rho_w with
-// rho_w the node's own density before the last collision), reading the populations from the
-// staged rows.  One 8-byte read per link replaces the separate reads of q, the wall velocity
-// and the solid flag of the second node.
-template <int I, class At>
-__device__ __forceinline__ float bounce_link(const At &at, int x, int y, float2 lk)
-{
-    constexpr int o = opp_(I);
-    const float fo = at(o, x, y);
-    const float q = lk.x;
-    float mw = 0.f;
-    if (lk.y != 0.f) {
-        float rho_w = 0.f;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) rho_w += at(k, x, y);
-        mw = lk.y * rho_w;
-    }
-    if (q < 0.5f) return 2.f * q * fo + (1.f - 2.f * q) * at(o, x + ex_(I), y + ey_(I)) + mw;
-    if (q == 0.5f) return fo + mw;
-    return fo / (2.f * q) + (2.f * q - 1.f) / (2.f * q) * at(I, x, y) + mw / (2.f * q);
-}
-
-// Wall links of the pair (edges beyond a non-periodic side and solid nodes): the bounce-back
-// of the two-pass step (half-way, moving wall, interpolated), element by element.
-#define LBM_GEOM_LINK(I)                                                                                      \
-    {                                                                                                         \
-        const int ys_ = rp - ey_(I);                                                                          \
-        const bool yw_ = !kp.periodic_y && (ys_ < 0 || ys_ >= ny);                                            \
-        const int wsrc_ = I == 0 ? 0 : (ey_(I) > 0 ? win_m : (ey_(I) < 0 ? win_p : win_0));                   \
-        _Pragma("unroll") for (int e = 0; e < 2; ++e) {                                                       \
-            if ((own >> e) & 1) continue;                                                                     \
-            const int xs_ = c0 + e - ex_(I);                                                                  \
-            const bool wall_ = yw_ || (!kp.periodic_x && (xs_ < 0 || xs_ >= nx)) || ((wsrc_ >> (e - ex_(I) + 1)) & 1); \
-            if (wall_) {                                                                                      \
-                float v_;                                                                                     \
-                if constexpr (GEOM == 1) {                                                                    \
-                    /* half-way: the population that left the node toward the wall returns */                \
-                    constexpr int o_ = opp_(I);                                                               \
-                    v_ = Pair2<S>::load1(row[1] + o_ * W + e);                                                \
-                    if constexpr (IsDev<S>::value)                                                            \
-                        v_ = __fmaf_rn(v_, kp.cf.inv_scale, __fmul_rn(w_<float>(o_), ref[1] ? ref[1][e] : kp.cf.rho_ref)); \
-                    v_ = v_ + 0.f;                                                                            \
-                } else {                                                                                      \
-                    /* interpolated or moving walls: the link records exist (set_geometry) */                 \
-                    const StagedAt<S, W> at_{kp, row[0], row[1], row[2], ref[0], ref[1], ref[2], e, xw + e, yw}; \
-                    v_ = bounce_link<I>(at_, xw + e, yw, e ? make_float2(lrec[I - 1].z, lrec[I - 1].w)         \
-                                                         : make_float2(lrec[I - 1].x, lrec[I - 1].y));       \
-                }                                                                                             \
-                if (e == 0) f_new[I].v.x = v_;                                                                \
-                else f_new[I].v.y = v_;                                                                       \
-            }                                                                                                 \
-        }                                                                                                     \
-    }
-
 #ifndef LBM_FUSED2_MINB
 #define LBM_FUSED2_MINB 2  // CTAs per SM the register allocation must allow
 #endif
-// GEOM: 0 no solid nodes; 1 solid nodes with half-way links only; 2 also interpolated or
-// moving walls (through the wall-link records).  The half-way-only instantiation keeps the
-// link code out of the kernel.
-template <class S, int NW, int RING, bool PERIODIC, class O, int GEOM = 0>
-__global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB) k_fused2(KParams kp, int seg_rows)
+template <class S, int NW, int RING, class O>
+__global__ void __launch_bounds__(32 * (NW + 1), LBM_FUSED2_MINB) k_fused2(KParams kp, int seg_rows)
 {
     typedef FusedLayout2<S, NW, RING> L;
     constexpr int TX = L::TX, HX = L::HX, W = L::W;
@@ -326,8 +198,8 @@ __global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB
         // that wrap around a periodic x edge (the same for every row)
         const int lo = x_lo, hi = x0 + TX + HX;
         const int m0 = lo < 0 ? 0 : lo, m1 = hi > nx ? nx : hi;
-        const int nl = (lo < 0 && kp.periodic_x) ? -lo : 0;
-        const int nr = (hi > nx && kp.periodic_x) ? hi - nx : 0;
+        const int nl = lo < 0 ? -lo : 0;
+        const int nr = hi > nx ? hi - nx : 0;
         const uint32_t cols = (uint32_t)(m1 - m0 + nl + nr);
         int r = first;
         for (; r <= last; ++r) {
@@ -339,13 +211,7 @@ __global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB
             }
             uint64_t *bar = full + slot;
             int gy = r;
-            if (gy < 0 || gy >= ny) {
-                if (!kp.periodic_y) {
-                    mbar_arrive(bar);
-                    continue;
-                }
-                gy = ((gy % ny) + ny) % ny;
-            }
+            if (gy < 0 || gy >= ny) gy = ((gy % ny) + ny) % ny;
             fence_proxy_async();
             mbar_expect_tx(bar, cols * (9u * ES + (refs ? 4u : 0u)));
             S *dst = reinterpret_cast<S *>(pops + (size_t)slot * L::POP_ROW);
@@ -375,49 +241,23 @@ __global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB
     // ----------------------------------------------------------- consumer warps
     const int c0 = x0 + 60 * warp - 2 + 2 * lane;  // unwrapped column of this lane's first node (even)
     const int scol = c0 - x_lo;                     // its staged column (even)
-    const bool col_out = !PERIODIC && !kp.periodic_x && (c0 < 0 || c0 >= nx);  // both nodes (nx is even)
     const bool collides = lane >= 1 && lane <= 30 && c0 < nx;
     const bool dev = IsDev<S>::value;
-    const float inv_scale = kp.cf.inv_scale, rho_ref = kp.cf.rho_ref;
-    const v2 psi_s = v2{kp.c2.psi_s};
-    v2 f_old[9], rho_old = S2(0.f), psi_m2 = psi_s, psi_m1 = psi_s;
+    v2 f_old[9], rho_old = S2(0.f), psi_m2 = S2(0.f), psi_m1 = S2(0.f);
 #pragma unroll
     for (int i = 0; i < 9; ++i) f_old[i] = S2(0.f);
     auto wait_full = [&](int r) -> bool {
         const bool got = mbar_wait_bounded(full + ((r - first) & (RING - 1)), (uint32_t)(((r - first) / RING) & 1));
         return __all_sync(0xffffffffu, got);
     };
-    // solid flags of rows rp - 1, rp, rp + 1 around the pair (general geometry only)
-    int win_m = 0, win_0 = 0, win_p = 0, own_old = 0;
-    SolidRow win_next{{0, 0, 0, 0}};  // raw flags of row rp + 2, fetched one row early
-    if constexpr (GEOM) {
-        if (kp.solid) {
-            win_0 = solid_bits(solid_fetch(kp, yb - 2, c0));
-            win_p = solid_bits(solid_fetch(kp, yb - 1, c0));
-            win_next = solid_fetch(kp, yb, c0);
-        }
-    }
     bool ok = wait_full(first) && wait_full(first + 1);
     for (int rp = yb - 1; rp <= ye && ok; ++rp) {
         if (!wait_full(rp + 1)) {
             ok = false;
             break;
         }
-        int own = 0;  // solid flags of the pair in row rp
-        if constexpr (GEOM) {
-            win_m = win_0;
-            win_0 = win_p;
-            if (kp.solid) {
-                win_p = solid_bits(win_next);
-                win_next = solid_fetch(kp, rp + 2, c0);
-            }
-            own = (win_0 >> 1) & 3;
-        }
-        const bool row_out = !PERIODIC && !kp.periodic_y && (rp < 0 || rp >= ny);
-        v2 f_new[9], rho_new = S2(0.f), psi_new = psi_s;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f_new[i] = S2(0.f);
-        if (!col_out && !row_out) {
+        v2 f_new[9], rho_new, psi_new;
+        {
             const S *row[3];
             const float *ref[3];
 #pragma unroll
@@ -430,51 +270,6 @@ __global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB
             // of row rp - e_iy
             LBM_PULL_PAIR(0) LBM_PULL_PAIR(1) LBM_PULL_PAIR(2) LBM_PULL_PAIR(3) LBM_PULL_PAIR(4)
             LBM_PULL_PAIR(5) LBM_PULL_PAIR(6) LBM_PULL_PAIR(7) LBM_PULL_PAIR(8)
-            if (!PERIODIC && !GEOM) {
-                // links whose source lies beyond a non-periodic edge: half-way bounce-back
-#pragma unroll
-                for (int i = 1; i < 9; ++i) {
-                    const int ys = rp - ey_(i);
-                    const bool yw = !kp.periodic_y && (ys < 0 || ys >= ny);
-                    const bool w0 = yw || (!kp.periodic_x && (c0 - ex_(i) < 0 || c0 - ex_(i) >= nx));
-                    const bool w1 = yw || (!kp.periodic_x && (c0 + 1 - ex_(i) < 0 || c0 + 1 - ex_(i) >= nx));
-                    if (w0 || w1) {
-                        const int o = opp_(i);
-                        const S *a = row[1] + o * W;
-                        float r0 = Pair2<S>::load1(a), r1 = Pair2<S>::load1(a + 1);
-                        if (dev) {
-                            const float rf0 = has_ref ? ref[1][0] : rho_ref;
-                            const float rf1 = has_ref ? ref[1][1] : rho_ref;
-                            // as the pull's decode: one rounding of w_o ref, one of the sum
-                            r0 = __fmaf_rn(r0, inv_scale, __fmul_rn(w_<float>(o), rf0));
-                            r1 = __fmaf_rn(r1, inv_scale, __fmul_rn(w_<float>(o), rf1));
-                        }
-                        if (w0) f_new[i].v.x = r0 + 0.f;
-                        if (w1) f_new[i].v.y = r1 + 0.f;
-                    }
-                }
-            }
-            if constexpr (GEOM) {
-                // a link can only be a wall link when a solid node lies among columns c0 - 1 ..
-                // c0 + 2 of rows rp - 1 .. rp + 1, or those reach beyond a non-periodic edge;
-                // most pairs have neither and skip the per-link tests
-                const bool edge = (!kp.periodic_y && (rp - 1 < 0 || rp + 1 >= ny)) ||
-                                  (!kp.periodic_x && (c0 - 1 < 0 || c0 + 2 >= nx));
-                if ((kp.solid || kp.q || kp.wall_u) && (edge || (win_m | win_0 | win_p) != 0)) {
-                    const int yw = rp < 0 ? rp + ny : (rp >= ny ? rp - ny : rp);
-                    const int xw = c0 < 0 ? c0 + nx : (c0 >= nx ? c0 - nx : c0);
-                    // the pair's eight link records, requested together (one 16-byte read per
-                    // direction: both nodes), so their latency is paid once
-                    float4 lrec[8];
-                    if constexpr (GEOM == 2) {
-                        const float4 *lk = reinterpret_cast<const float4 *>(kp.link + (int64_t)yw * kp.pitch + xw);
-#pragma unroll
-                        for (int d = 0; d < 8; ++d) lrec[d] = lk[(int64_t)d * (kp.plane / 2)];
-                    }
-                    LBM_GEOM_LINK(1) LBM_GEOM_LINK(2) LBM_GEOM_LINK(3) LBM_GEOM_LINK(4)
-                    LBM_GEOM_LINK(5) LBM_GEOM_LINK(6) LBM_GEOM_LINK(7) LBM_GEOM_LINK(8)
-                }
-            }
             // the pulled populations are kept in rest-state deviation form for the collision
             {
                 v2 f[9];
@@ -484,21 +279,6 @@ __global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB
             }
             rho_new = density_dev(f_new);
             psi_new = psi_v<v2>(kp, rho_new);
-            if constexpr (GEOM) {
-                if (own) {
-                    // solid nodes: psi of the virtual wall density; rho 1 keeps the unused
-                    // arithmetic of the pair finite
-                    const int yw = rp < 0 ? rp + ny : (rp >= ny ? rp - ny : rp);
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        if (!((own >> e) & 1)) continue;
-                        const int xe = c0 + e < 0 ? c0 + e + nx : (c0 + e >= nx ? c0 + e - nx : c0 + e);
-                        const float ps = kp.wall_psi ? float(kp.wall_psi[(int64_t)yw * nx + xe]) : kp.cf.psi_s;
-                        if (e == 0) psi_new.v.x = ps, rho_new.v.x = 1.f;
-                        else psi_new.v.y = ps, rho_new.v.y = 1.f;
-                    }
-                }
-            }
         }
         __syncwarp();
         // row rp - 1 is not needed any more by this warp
@@ -509,10 +289,10 @@ __global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB
         const float ap = __shfl_up_sync(0xffffffffu, psi_new.v.y, 1), bp = __shfl_down_sync(0xffffffffu, psi_new.v.x, 1);
         const int y = rp - 1;
         // psi of the state read, for a caller that keeps it (the adjoint's recompute): the
-        // pair's own row, solid nodes included, as the psi pass writes it
+        // pair's own row, as the psi pass writes it
         if (kp.psi_out != nullptr && y >= yb && collides)
-            Pair2<float>::store(kp.psi_out + (int64_t)y * nx + c0, psi_m1);
-        if (y >= yb && collides && (!GEOM || own_old != 3)) {
+            Pair2<float>::store(static_cast<float *>(kp.psi_out) + (int64_t)y * nx + c0, psi_m1);
+        if (y >= yb && collides) {
             {
                 v2 fb[9];
                 // rows y-1 (m), y (0), y+1 (p); left (L), centre, right (R) columns of each node
@@ -528,25 +308,7 @@ __global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB
                 S *out = static_cast<S *>(kp.dst) + (int64_t)y * kp.pitch + c0;
                 // random word of the pair (stochastic rounding of 16-bit storage only)
                 const uint32_t hsr = dev && kp.sr ? sr_hash((uint32_t)(((int64_t)y * kp.pitch + c0) >> 1), kp.sr_seed) : 0u;
-                if (GEOM && own_old) {
-                    // one node of the pair is solid: store the fluid one alone
-                    const int e = own_old == 1 ? 1 : 0;
-                    const float rr = e ? rho_old.v.y : rho_old.v.x;
-                    if (has_ref) kp.ref_dst[(int64_t)y * kp.pitch + c0 + e] = rr;
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) {
-                        const float fv = e ? fb[i].v.y : fb[i].v.x;
-                        if constexpr (IsDev<S>::value) {
-                            const int wc = i == 0 ? 0 : (i <= 4 ? 1 : 5);
-                            const float nw = has_ref ? -kp.cf.scale * __fmul_rn(kp.c2.w[wc].x, rr) : kp.c2.enc[wc].x;
-                            const float sv = __fmaf_rn(fv, kp.cf.scale, nw);
-                            if (kp.sr) out[i * kp.plane + e] = sr_one<S>(sv, sr_bits(hsr, i), e);
-                            else Codec2<S>::put(out + i * kp.plane + e, sv);
-                        } else {
-                            out[i * kp.plane + e] = fv;
-                        }
-                    }
-                } else if (!dev) {
+                if (!dev) {
 #pragma unroll
                     for (int i = 0; i < 9; ++i) Pair2<S>::store(out + i * kp.plane, fb[i]);
                 } else if (has_ref) {
@@ -572,7 +334,6 @@ __global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB
         psi_m2 = psi_m1;
         psi_m1 = psi_new;
         rho_old = rho_new;
-        own_old = own;
 #pragma unroll
         for (int i = 0; i < 9; ++i) f_old[i] = f_new[i];
     }
@@ -604,10 +365,10 @@ __global__ void __launch_bounds__(32 * (NW + 1), GEOM == 2 ? 3 : LBM_FUSED2_MINB
 template <class S, int NW, int RING>
 struct Fused2 {
     typedef FusedLayout2<S, NW, RING> L;
-    template <bool P, class O, int GEOM = 0>
+    template <class O>
     static cudaError_t launch_one(const KParams &kp, cudaStream_t st)
     {
-        cudaError_t e = ensure_smem_attribute(k_fused2<S, NW, RING, P, O, GEOM>, kp.device, (int)L::bytes(true));
+        cudaError_t e = ensure_smem_attribute(k_fused2<S, NW, RING, O>, kp.device, (int)L::bytes(true));
         if (e != cudaSuccess) return e;
         const int sms = kp.sm_count > 0 ? kp.sm_count : 148;
         const int strips = (kp.nx + L::TX - 1) / L::TX;
@@ -626,24 +387,19 @@ struct Fused2 {
         if (nseg < 1) nseg = 1;
         const int seg_rows = (kp.ny + nseg - 1) / nseg;
         nseg = (kp.ny + seg_rows - 1) / seg_rows;
-        return launch_dependent(k_fused2<S, NW, RING, P, O, GEOM>, dim3(strips, nseg), dim3(32 * (NW + 1)),
+        return launch_dependent(k_fused2<S, NW, RING, O>, dim3(strips, nseg), dim3(32 * (NW + 1)),
                                 L::bytes(kp.per_node_ref != 0), st, kp, seg_rows);
     }
-    // Fully periodic lattices with a constant force and one relaxation time get
-    // instantiations with those options (and the reference-density mode) fixed at compile
+    // A constant force and one relaxation time get instantiations with those options (and the reference-density mode) fixed at compile
     // time; everything else reads them at run time.
     static cudaError_t launch(const KParams &kp, cudaStream_t st)
     {
-        // solid nodes, moving walls or interpolated links: the general-geometry instantiation
-        if (kp.q || kp.wall_u) return launch_one<false, RuntimeOpts, 2>(kp, st);
-        if (kp.solid) return launch_one<false, RuntimeOpts, 1>(kp, st);
-        if (kp.periodic_x && kp.periodic_y && kp.force_mode == 0 && !kp.var_tau) {
+        if (kp.force_mode == 0 && !kp.var_tau) {
             if (IsDev<S>::value && kp.per_node_ref)
-                return kp.improved ? launch_one<true, Opts<1, 0, 0, 1>>(kp, st) : launch_one<true, Opts<0, 0, 0, 1>>(kp, st);
-            return kp.improved ? launch_one<true, Opts<1, 0, 0, 0>>(kp, st) : launch_one<true, Opts<0, 0, 0, 0>>(kp, st);
+                return kp.improved ? launch_one<Opts<1, 0, 0, 1>>(kp, st) : launch_one<Opts<0, 0, 0, 1>>(kp, st);
+            return kp.improved ? launch_one<Opts<1, 0, 0, 0>>(kp, st) : launch_one<Opts<0, 0, 0, 0>>(kp, st);
         }
-        if (kp.periodic_x && kp.periodic_y) return launch_one<true, RuntimeOpts>(kp, st);
-        return launch_one<false, RuntimeOpts>(kp, st);
+        return launch_one<RuntimeOpts>(kp, st);
     }
 };
 

@@ -253,8 +253,8 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
                 kp.ref_dst = ref_of(kp.dst);
                 kp.sr_seed = v.sr_seed(step0 + t);
                 if (v.fused_pass) {
-                    kp.psi_out = static_cast<float *>(kp.psi);
-                    ACK(v.fused_pass(kp, as->side), "fused step kernel");
+                    kp.psi_out = kp.psi;
+                    ACK(v.fused_pass(kp, as->side), "one-pass step kernel");
                     kp.psi_out = nullptr;
                 } else {
                     ACK(v.psi_pass(kp, as->side), "psi kernel");

@@ -33,13 +33,15 @@ struct lbm_ctx {
     uint8_t *solid = nullptr;
     double *wall_u = nullptr, *q = nullptr, *fext = nullptr;
     double *wall_rho = nullptr, *wall_psi = nullptr;  // per solid node virtual density, its psi
-    float2 *link = nullptr;             // wall-link records of the one-pass kernel (KParams::link)
+    float2 *link = nullptr;             // wall-link records of the tile kernel (KParams::link)
+    uint16_t *links = nullptr;          // wall bits of every node (KParams::links)
     double *dacc = nullptr;             // diagnostics accumulators (9 doubles, 1 u64, 1 int)
     double *scratch = nullptr;          // host<->device staging for FP64 field copies
     size_t scratch_bytes = 0;
     int *derr = nullptr;
     bool initialised = false;
     bool fused_ok = false;
+    cudaError_t (*one_pass)(const KParams &, cudaStream_t) = nullptr;  // the step's kernel; null: two-pass
     int64_t steps = 0;
     int64_t n_fluid = 0;                // nodes that are not solid
     Launchers L{};
@@ -253,6 +255,7 @@ static void fill_constants(lbm_ctx *c)
     k.wall_rho = c->wall_rho;
     k.wall_psi = c->wall_psi;
     k.link = c->link;
+    k.links = c->links;
     k.err = c->derr;
 }
 
@@ -266,25 +269,15 @@ static void bind_buffers(lbm_ctx *c, int src)
 
 static bool fused_possible(const lbm_ctx *c)
 {
-    if (!c->L.fused_pass) return false;
     const lbm_params &p = c->p;
     if ((c->solid || c->q || c->wall_u) && !c->L.fused_geometry) return false;
     if (c->L.fused_align <= 0 || p.nx % c->L.fused_align != 0) return false;
-    // the wrapped halo segment of the last strip must fit inside the lattice
+    // (the staged kernel's wrapped halo segment of the last strip must fit inside the lattice)
     if (p.nx < c->L.fused_tile_x + 16 || p.ny < 4) return false;
     return true;
 }
 
-// LBM_KERNEL_AUTO: the one-pass kernel where it was measured faster than the two-pass one
-// (FP32 on a GB300 unless stated; the two are close at each threshold).  On small lattices a
-// CTA's serial walk down its rows dominates the one-pass kernel's time and the two-pass
-// kernels, one thread per node, hide latency better: periodic 256^2 7.1 us against 8.8,
-// 512^2 12.4 against 10.1; a 256-wide channel with x walls 23.5 against 29.5 (two strips,
-// the second 16 columns wide); 512 x 4096 84 against 57.  Solid bands: 256^2 below, 512^2
-// 17.8 against 19.2 in FP32 but 25.1 against 22.5 in FP16, 1024^2 55 against 41 (before the
-// two-pass kernels shared one neighbourhood computation per node), 2048^2 251 against 100.
-// Interpolated and moving walls, whose per-link work sits on the one-pass kernel's serial
-// path: annulus 1024^2 44 against 58, 2048^2 207 against 195 (FP16 258 against 211).
+// What lbm_kernel_in_use calls an LBM_KERNEL_AUTO context: LBM_KERNEL_FUSED from these sizes on.
 static bool auto_prefers_fused(const lbm_ctx *c)
 {
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
@@ -293,11 +286,30 @@ static bool auto_prefers_fused(const lbm_ctx *c)
     return (n >= (int64_t(1) << 18) && c->p.nx >= 512) || n >= (int64_t(1) << 21);
 }
 
+// Which kernel steps the context: the two-pass kernels on request (LBM_KERNEL_TWO_PASS); else a
+// one-pass kernel, the staged one (k_fused2) or the tile kernel (k_tile), which gives the two-pass
+// step's results.  The staged kernel keeps HBM busy where the two population buffers are far
+// larger than L2, but a CTA walks its rows in series, and it has no walls; the tile kernel has
+// thousands of short blocks.  Step times on a GB300 (us, tile / staged): periodic 512^2 5.8 / 10.3, 1024^2
+// 16.1 / 22.9, 1600^2 40 / 46.6, 2048^2 59 / 56.7, 4096^2 223 / 195; FP16 1024^2 21.5 / 26.9, 1024 x
+// 2048 42 / 43, 1600^2 51 / 45, 2048^2 81 / 59.  (Two-pass kernels: 512^2 10.3, 1024^2 31, 2048^2 121; 256
+// x 2048 with walls 20.6 against the tile kernel's 9.8; banded 512^2 17.6 / 6.1; annulus 1024^2 44 / 20.)
 static void choose_kernel(lbm_ctx *c)
 {
     const int want = c->p.kernel;
-    c->fused_ok = (want != LBM_KERNEL_TWO_PASS) && fused_possible(c) &&
+    const bool possible = fused_possible(c);
+    c->fused_ok = (want != LBM_KERNEL_TWO_PASS) && possible &&
                   (want == LBM_KERNEL_FUSED || c->p.precision == LBM_F64 || auto_prefers_fused(c));
+    const bool staged = possible && c->L.fused_pass && c->p.periodic_x && c->p.periodic_y && !c->solid && !c->q && !c->wall_u;
+    // 32-bit byte offsets within the rows of a tile
+    const bool tile = c->p.precision == LBM_F64 || c->pitch <= (int64_t)1 << 26;
+    const int64_t n = (int64_t)c->p.nx * c->p.ny;
+    const bool large = n >= (c->p.precision == LBM_F32 ? (int64_t)1 << 22 : (int64_t)9 << 18);
+    c->one_pass = nullptr;
+    if (want == LBM_KERNEL_TWO_PASS || (want == LBM_KERNEL_FUSED && !possible)) return;
+    if (staged && (want == LBM_KERNEL_FUSED || large || !tile)) c->one_pass = c->L.fused_pass;
+    else if (tile) c->one_pass = c->L.tile_pass;
+    else c->fused_ok = false;
 }
 
 // ------------------------------------------------------------- lifetime ----
@@ -307,7 +319,7 @@ static void free_all(lbm_ctx *c)
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
     void *bufs[] = {c->pops[0], c->pops[1], c->refp[0], c->refp[1], c->psi, c->solid,
-                    c->wall_u, c->q, c->fext, c->wall_rho, c->wall_psi, c->link, c->dacc, c->scratch, c->derr};
+                    c->wall_u, c->q, c->fext, c->wall_rho, c->wall_psi, c->link, c->links, c->dacc, c->scratch, c->derr};
     for (void *b : bufs)
         if (b) cudaFree(b);
     adjoint_free(c->adj);
@@ -426,7 +438,7 @@ static lbm_status upload(lbm_ctx *c, T **dst, const T *src, size_t count, const 
     return LBM_OK;
 }
 
-// Wall-link records of the one-pass kernel (KParams::link), built on the host from the
+// Wall-link records of the tile kernel (KParams::link), built on the host from the
 // geometry as given: for each fluid node x and pulled population i whose source x - e_i is a
 // wall (a solid node or beyond a non-periodic edge), the link fraction q of the outgoing
 // population o = opp(i) (1/2 without link fractions, and 1/2 where q < 1/2 but the second
@@ -499,6 +511,16 @@ extern "C" lbm_status lbm_set_geometry(lbm_ctx *c, const uint8_t *solid, const d
     if ((s = upload(c, &c->q, q, 8 * n, "q")) != LBM_OK) return s;
     if ((s = upload(c, &c->fext, force_field, 2 * n, "force_field")) != LBM_OK) return s;
     if (c->p.precision != LBM_F64 && (s = build_link_records(c, solid, wall_u, q)) != LBM_OK) return s;
+    if (c->links) {
+        CK(cudaStreamSynchronize(c->stream), "set_geometry");
+        cudaFree(c->links);
+        c->links = nullptr;
+    }
+    if (solid || wall_u || q) {
+        CK(cudaMalloc((void **)&c->links, n * sizeof(uint16_t)), "wall bits");
+        fill_constants(c);
+        CK(c->L.link_bits(c->kp, c->links, c->stream), "wall bits kernel");
+    }
     CK(cudaStreamSynchronize(c->stream), "set_geometry");
     fill_constants(c);
     choose_kernel(c);
@@ -585,8 +607,8 @@ static lbm_status run_steps(lbm_ctx *c, int64_t nsteps)
     for (int64_t t = 0; t < nsteps; ++t) {
         bind_buffers(c, c->cur);
         c->kp.sr_seed = sr_seed_of(c->steps);
-        if (c->fused_ok) {
-            CK(c->L.fused_pass(c->kp, c->stream), "fused step kernel");
+        if (c->one_pass) {
+            CK(c->one_pass(c->kp, c->stream), "one-pass step kernel");
         } else {
             CK(c->L.psi_pass(c->kp, c->stream), "psi kernel");
             CK(c->L.collide_pass(c->kp, c->stream), "collide kernel");
@@ -849,7 +871,7 @@ ContextView view_of(lbm_ctx *c)
     v.bind = [](lbm_ctx *cc, int src) { bind_buffers(cc, src); };
     v.psi_pass = c->L.psi_pass;
     v.collide_pass = c->L.collide_pass;
-    v.fused_pass = (c->fused_ok && c->p.precision != LBM_F64) ? c->L.fused_pass : nullptr;
+    v.fused_pass = c->one_pass;
     v.L = &c->L;
     v.check_error = [](lbm_ctx *cc, std::string &m) {
         lbm_status s = sync_and_check(cc, "adjoint");

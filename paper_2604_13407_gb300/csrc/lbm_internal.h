@@ -70,8 +70,8 @@ struct KParams {
     const float *ref_src;  // per-node reference density planes (FP16/BF16 with per_node_ref)
     float *ref_dst;
     void *psi;             // psi field [ny*nx] in the kernel's arithmetic type
-    float *psi_out;        // one-pass kernel (FP32 arithmetic): also write psi of the state read
-                           // here ([ny*nx], as the psi pass does), or null
+    void *psi_out;         // one-pass kernels: also write psi of the state read here ([ny*nx] in
+                           // the arithmetic type, as the psi pass does), or null
     const uint8_t *solid;  // [ny*nx] or null
     const double *wall_u;  // [2][ny*nx] or null
     const double *q;       // [8][ny*nx] or null
@@ -81,8 +81,11 @@ struct KParams {
     // [8][ny][pitch] per fluid node and pulled population i = 1..8 whose source x - e_i is a
     // wall: (q, c) with q the link fraction after the fallback of a missing second node, and
     // c = 6 w_o (e_i . u_w) the moving-wall coefficient (mw = c rho_w); null without
-    // interpolated or moving walls.  Read by the one-pass kernel's wall links.
+    // interpolated or moving walls, and in FP64.  Read by the tile kernel's wall links.
     const float2 *link;
+    // [ny*nx] per node: bit i (1..8) set when the source x - e_i is a wall, bit 0 when the node is
+    // solid; null without solid nodes, link fractions and wall velocities.  Read by the tile kernel.
+    const uint16_t *links;
     int *err;              // device error word (0 = fine)
     Consts<double> cd;     // constants for FP64 arithmetic
     Consts<float> cf;      // constants for FP32 arithmetic
@@ -134,7 +137,9 @@ inline cudaError_t ensure_smem_attribute(K kernel, int device, int bytes)
 struct Launchers {
     cudaError_t (*psi_pass)(const KParams &, cudaStream_t);
     cudaError_t (*collide_pass)(const KParams &, cudaStream_t);
-    cudaError_t (*fused_pass)(const KParams &, cudaStream_t);  // may be null
+    cudaError_t (*fused_pass)(const KParams &, cudaStream_t);  // staged one-pass step (periodic, FP32 arithmetic); null in FP64
+    cudaError_t (*tile_pass)(const KParams &, cudaStream_t);   // one-pass step on tiles (k_tile.cuh)
+    cudaError_t (*link_bits)(const KParams &, uint16_t *out, cudaStream_t);  // KParams::links
     cudaError_t (*init)(const KParams &, const double *rho, const double *ux, const double *uy,
                         cudaStream_t);
     cudaError_t (*moments)(const KParams &, double *rho, double *ux, double *uy, cudaStream_t);
@@ -149,10 +154,10 @@ struct Launchers {
     cudaError_t (*objective)(const KParams &, int objective, double inv_nfluid, double *acc, cudaStream_t);
     int64_t (*adj_blocks)(const KParams &);  // rows of the per-block partial-sum array (8 doubles each)
     cudaError_t (*adj_reduce)(const KParams &, const double *part, double *out8, cudaStream_t);
-    // fused kernel launch constraints
-    int fused_tile_x;     // strip width in nodes
+    // lattices on which LBM_KERNEL_FUSED is granted (and lbm_kernel_in_use says so)
+    int fused_tile_x;     // nx at least this and 16
     int fused_align;      // nx must be a multiple of this
-    int fused_geometry;   // 1: the fused kernel handles solid nodes, moving and interpolated walls
+    int fused_geometry;   // 1: also with solid nodes, moving and interpolated walls
 };
 
 Launchers launchers_f64();
