@@ -258,7 +258,7 @@ LBM_API lbm_status lbm_set_param(lbm_ctx *ctx, int32_t which, double value);
  * FP32 on the decoded states, taking the storage's rounding as the identity (the gradient
  * of the unrounded step along the 16-bit run's trajectory).  Device memory (allocated on
  * the first call, kept until lbm_destroy or a larger call): ceil(nsteps/K) + 2 (K - 1)
- * population states (with their reference-density plane), 2 K psi fields and 15 planes of
+ * population states (with their reference-density plane), 2 K psi fields and 27 planes (FP64: 29) of
  * the arithmetic type (FP64 for FP64 storage, FP32 otherwise), K = min(checkpoint_every,
  * nsteps) (the
  * recompute of a segment overlaps, on a second stream, the transposed steps of the segment

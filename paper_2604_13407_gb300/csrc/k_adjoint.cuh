@@ -18,14 +18,23 @@
 // d rho/d f_i = 1).  So lambda_t is never stored: it is held as the pair (g, c) of the
 // step after it, and the next transposed step assembles lambda at its own node.
 //
-// Pass 1 (k_adj1): per fluid node, assemble lambda_{t+1}, recompute the forward
-// quantities from A_t and the psi field of A_t, and run the chain rule back to g(x),
-// dJ/dS(x), the local part of dJ/dpsi(x) (through F_int = -G psi S) and rho(x).
-// Pass 2 (k_adj2): dJ/dpsi(x) = local part + sum_i w_i e_i . dJ/dS(x - e_i) over fluid
-// x - e_i, then c(x) = psi'(rho) dJ/dpsi.  Parameter derivatives are summed per block
-// (warp shuffles) into per-block FP64 slots that one reduction sums at the end of the call.
+// k_adj runs one transposed step on tiles (as k_tile: 32 columns, two rows a thread in packed FP32,
+// one in FP64).  First c of the step after, on the tile and the ring of nodes around it, into shared
+// memory: dJ/dpsi(x) = local part + sum_i w_i e_i . dJ/dS(x - e_i) over fluid x - e_i, then c(x) =
+// psi'(rho) dJ/dpsi.  Then, per fluid node of the tile: assemble lambda_{t+1} from g and c, recompute
+// the forward quantities from A_t and the psi field of A_t, and run the chain rule back to g(x),
+// dJ/dS(x), the local part of dJ/dpsi(x) (through F_int = -G psi S) and rho(x).  The last launch of a
+// call (AdjArgs::tail) does the first part alone, for the parameter sums and lambda_0.  Parameter
+// derivatives are summed per block into per-block FP64 slots that one reduction sums at the end of
+// the call.
+//
+// What bounds it: 148 B a node in FP32 (A_t and g 36 each, psi, dS, rho and the local part of dJ/dpsi,
+// read; g, dS, rho and the local part written).  One thread per node in two passes (c in a pass of its
+// own) issued 1231 + 390 instructions a node and was bound by them; the packed pair, the shared
+// ring and one block-wide reduction (each warp sums one quantity of the block) cut that four times.
 #pragma once
 
+#include "k_tile.cuh"
 #include "k_twopass.cuh"
 
 namespace lbm {
@@ -39,19 +48,6 @@ __device__ __forceinline__ bool wall_link(const KParams &kp, int x, int y, int i
     return false;
 }
 
-// Walls among the eight neighbours: bit i set when x + e_i is a solid node or lies beyond a
-// non-periodic edge.  One set of global solid-flag reads per node serves the pull
-// (population i comes from x - e_i = x + e_opp(i)), lambda_{t+1}, the objective and the wall
-// psi terms.
-__device__ __forceinline__ unsigned wall_mask(const KParams &kp, const Around &nb)
-{
-    unsigned wm = 0;
-#pragma unroll
-    for (int i = 1; i < 9; ++i)
-        if (!nb.in(i) || (kp.solid != nullptr && kp.solid[nb.n(i)] != 0)) wm |= 1u << i;
-    return wm;
-}
-
 // Objective weights W_i(x) at a fluid node (before the 1/n of the time average);
 // inv_nf = 1 / number of fluid nodes in the arithmetic type.
 template <class R>
@@ -61,104 +57,100 @@ __device__ __forceinline__ R objective_weight(int objective, int i, bool wall_ah
     return R(ex_(i)) * inv_nf;
 }
 
-// lambda_{t+1} of the nine populations of a fluid node: nb its neighbourhood, wm its
-// wall_mask.
-template <class R>
-__device__ __forceinline__ void lambda_at(const KParams &kp, const AdjArgs &aa, const Around &nb, unsigned wm, R wscale,
-                                          R inv_nf, R (&lam)[9])
-{
-    const int64_t k = nb.k(0);
-    const R *g = static_cast<const R *>(aa.g_in);
-    const R *c = static_cast<const R *>(aa.c_in);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const bool wall = (i != 0) && ((wm >> i) & 1u);
-        const int64_t kn = (i == 0 || wall) ? k : nb.k(i);
-        R v = wscale * objective_weight<R>(aa.objective, i, wall, inv_nf);
-        if (g != nullptr) {
-            if (wall) v += g[opp_(i) * kp.plane + k] + c[k];
-            else v += g[i * kp.plane + kn] + c[kn];
-        }
-        lam[i] = v;
-    }
-}
+// ------------------------------------------------------------ lanes --------------
+// The transposed step is written once for a lane type: v2 (two nodes, packed FP32) or d1 (one node,
+// FP64; multiply-adds written out, since the FP64 units are compiled without contraction).
+struct d1 {
+    double v;
+};
+__device__ __forceinline__ d1 operator+(d1 a, d1 b) { return d1{a.v + b.v}; }
+__device__ __forceinline__ d1 operator-(d1 a, d1 b) { return d1{a.v - b.v}; }
+__device__ __forceinline__ d1 operator*(d1 a, d1 b) { return d1{a.v * b.v}; }
+__device__ __forceinline__ d1 vfma(d1 a, d1 b, d1 c) { return d1{__fma_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ d1 vrcp(d1 a) { return d1{1.0 / a.v}; }
+__device__ __forceinline__ d1 vclamp01(d1 a) { return d1{fmin(fmax(a.v, 0.0), 1.0)}; }
+__device__ __forceinline__ v2 operator-(v2 a) { return V(-a.v.x, -a.v.y); }
+__device__ __forceinline__ d1 operator-(d1 a) { return d1{-a.v}; }
+
+template <class R> struct Lanes;
+template <> struct Lanes<float> {
+    typedef v2 T;
+    static constexpr int N = 2;
+    static __device__ __forceinline__ T all(float a) { return S2(a); }
+    static __device__ __forceinline__ float get(T a, int e) { return e ? a.v.y : a.v.x; }
+    static __device__ __forceinline__ void set(T &a, int e, float v) { (e ? a.v.y : a.v.x) = v; }
+};
+template <> struct Lanes<double> {
+    typedef d1 T;
+    static constexpr int N = 1;
+    static __device__ __forceinline__ T all(double a) { return d1{a}; }
+    static __device__ __forceinline__ double get(T a, int) { return a.v; }
+    static __device__ __forceinline__ void set(T &a, int, double v) { a.v = v; }
+};
 
 // dp/drho and dp/dT of the EOS.
-template <class R>
-__device__ __forceinline__ void p_eos_derivs(const KParams &kp, R rho, R &p_rho, R &p_T)
+template <class R, class T>
+__device__ __forceinline__ void p_eos_derivs(const KParams &kp, T rho, T &p_rho, T &p_T)
 {
+    typedef Lanes<R> Z;
     const Consts<R> &c = cst<R>(kp);
+    const T one = Z::all(R(1)), RT = Z::all(c.eos_RT), K = Z::all(c.eos_K), KR = Z::all(c.eos_K * c.eos_R), m2a = Z::all(R(-2) * c.eos_a);
     if (kp.eos == 0) {
-        const R om = R(1) - c.eos_b * rho;
-        p_rho = c.eos_K * (c.eos_RT / (om * om) - R(2) * c.eos_a * rho);
-        p_T = c.eos_K * rho * c.eos_R / om;
+        const T r = vrcp(vfma(Z::all(-c.eos_b), rho, one));
+        p_rho = K * vfma(RT * r, r, m2a * rho);
+        p_T = KR * rho * r;
         return;
     }
-    const R eta = c.eos_b * rho * R(0.25);
-    const R om = R(1) - eta;
-    const R om2 = om * om;
-    const R g = (R(1) + eta + eta * eta - eta * eta * eta) / (om2 * om);
-    const R dg = (R(4) + R(4) * eta - R(2) * eta * eta) / (om2 * om2);  // dg/d eta
-    p_rho = c.eos_K * (c.eos_RT * (g + eta * dg) - R(2) * c.eos_a * rho);
-    p_T = c.eos_K * rho * c.eos_R * g;
+    const T eta = Z::all(c.eos_b * R(0.25)) * rho;
+    const T om = one - eta;
+    const T r = vrcp(om), r3 = r * r * r;
+    const T g = vfma(eta, vfma(eta, om, one), one) * r3;                                                // (1 + eta + eta^2 - eta^3) / om^3
+    const T dg = vfma(eta, vfma(Z::all(R(-2)), eta, Z::all(R(4))), Z::all(R(4))) * (r3 * r);           // dg / d eta
+    p_rho = K * vfma(RT, vfma(eta, dg, g), m2a * rho);
+    p_T = KR * rho * g;
 }
 
-// Per-block FP64 partial sums of the transposed passes (slots AdjSlot, lbm_internal.h):
-// one row of kAdjSlots doubles per block of the row grid, accumulated over all steps of a
-// call and reduced once at its end, so no atomic is contended and the summation order is
-// fixed.
+// Per-block FP64 partial sums of the transposed steps (slots AdjSlot, lbm_internal.h): one row of
+// kAdjSlots doubles per block, accumulated over all steps of a call and reduced once at its end, so
+// no atomic is contended and the summation order is fixed.
 
-// Warp sum of one value per lane as a compensated FP32 pair (hi, lo) in lane 0: Knuth's
-// TwoSum at every shuffle level, about 2^-48 relative.
+// Warp sum of one value per lane as a compensated FP32 pair (hi, lo) in lane 0: Knuth's TwoSum at
+// every shuffle level, about 2^-48 relative.
+__device__ __forceinline__ void two_sum(float &hi, float &lo, float x, float xlo)
+{
+    const float sum = hi + x, z = sum - hi;
+    lo += xlo + ((hi - (sum - z)) + (x - z));
+    hi = sum;
+}
 __device__ __forceinline__ void warp_sum_pair(float &hi, float &lo)
 {
-    lo = 0.f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ohi = __shfl_down_sync(0xffffffffu, hi, o), olo = __shfl_down_sync(0xffffffffu, lo, o);
-        const float sum = hi + ohi, z = sum - hi;
-        lo += olo + ((hi - (sum - z)) + (ohi - z));
-        hi = sum;
-    }
+    for (int o = 16; o > 0; o >>= 1)
+        two_sum(hi, lo, __shfl_down_sync(0xffffffffu, hi, o), __shfl_down_sync(0xffffffffu, lo, o));
 }
 
-// Block sum of N per-thread values added to this block's slots [first, first + N).  FP64
-// arithmetic sums in FP64.  FP32 arithmetic keeps each warp's sum as a compensated FP32 pair
-// and converts to FP64 only in the block's final step (N threads), which keeps FP64 work
-// (a narrow pipe on GB300) out of the per-node path.
-template <int N, class R>
-__device__ __forceinline__ void block_add(const R (&v)[N], double *part, int first)
+// Sums of the `n` quantities v[k][0 .. count) in shared memory (all threads past a barrier) but those in `skip` (known to be zero), added to this block's slots: a warp sums one quantity at a
+// time, each lane its share of them and then the lanes, compensated in FP32 arithmetic (FP64
+// work stays out of it: GB300's FP64 pipe is narrow).
+template <class R>
+__device__ __forceinline__ void block_add(const R *v, int pitch, int n, int count, unsigned skip, double *part)
 {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double t = 0.0;
-    if constexpr (sizeof(R) == 8) {
-        __shared__ double red[kRowThreads / 32][N];
-        // a quantity that is zero on every lane of the warp (the wall terms away from walls)
-        // sums to exactly zero: skip its shuffles
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            const double w = __any_sync(0xffffffffu, v[k] != R(0)) ? warp_sum(double(v[k])) : 0.0;
-            if (lane == 0) red[wid][k] = w;
+    const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    for (int k = threadIdx.x >> 5; k < n; k += warps) {
+        if ((skip >> k) & 1u) continue;
+        double t;
+        if constexpr (sizeof(R) == 8) {
+            double s = 0.0;
+            for (int q = lane; q < count; q += 32) s += v[k * pitch + q];
+            t = warp_sum(s);
+        } else {
+            float hi = 0.f, lo = 0.f;
+            for (int q = lane; q < count; q += 32) two_sum(hi, lo, v[k * pitch + q], 0.f);
+            warp_sum_pair(hi, lo);
+            t = double(hi) + double(lo);
         }
-        __syncthreads();
-        if (threadIdx.x < N)
-            for (int q = 0; q < kRowThreads / 32; ++q) t += red[q][threadIdx.x];
-    } else {
-        __shared__ float2 red[kRowThreads / 32][N];
-#pragma unroll
-        for (int k = 0; k < N; ++k) {
-            float hi = float(v[k]), lo = 0.f;
-            if (__any_sync(0xffffffffu, v[k] != R(0))) warp_sum_pair(hi, lo);
-            if (lane == 0) red[wid][k] = make_float2(hi, lo);
-        }
-        __syncthreads();
-        if (threadIdx.x < N)
-            for (int q = 0; q < kRowThreads / 32; ++q) {
-                const float2 p = red[q][threadIdx.x];
-                t += double(p.x) + double(p.y);
-            }
+        if (lane == 0) part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kAdjSlots + k] += t;
     }
-    if (threadIdx.x < N) part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kAdjSlots + first + threadIdx.x] += t;
 }
 
 // Block sum of one double added to *acc with one FP64 atomic per block.
@@ -176,258 +168,452 @@ __device__ __forceinline__ void block_atomic_add(double v, double *acc)
     }
 }
 
-// Pass 1 of the transposed step at A_t (kp.src) with the psi field of A_t (kp.psi).
-template <class S>
-__global__ void __launch_bounds__(kRowThreads, sizeof(typename Codec<S>::R) == 8 ? 4 : 8) k_adj1(KParams kp, AdjArgs aa)
+// Row units of a block (pairs of rows, FP64: rows), one warp each, and the units of its ring, which the
+// same warps take first.
+template <class R, int U> struct AdjTile {
+    static constexpr int UNITS = U;
+    static constexpr int RING = sizeof(R) == 8 ? 3 : 2;
+    static constexpr int ROWS = sizeof(R) == 8 ? UNITS : 2 * UNITS;
+    static constexpr int THREADS = 32 * UNITS;
+};
+template <class R, int U>
+struct AdjShared {
+    typedef AdjTile<R, U> G;
+    R c[G::ROWS + 2][kTilePitch];                     // c of the tile and its ring
+    R red[7][Lanes<R>::N * 32 * G::UNITS];            // the parameter terms of every node of the tile
+};
+
+// One block of a transposed step.  INNER: no node of the tile or its ring reads across an edge of the
+// lattice and there are no solid nodes, so every node is a live one and every address is the node's own
+// plus a constant of the launch.  (The two instantiations
+// share nothing, so the common one carries no tests and no merges of the other's values.)
+template <class S, int U, bool INNER>
+__device__ __forceinline__ void adj_block(const KParams &kp, const AdjArgs &aa, AdjShared<typename Codec<S>::R, U> &sh_)
 {
     typedef typename Codec<S>::R R;
-    grid_dependency_wait();
-    allow_dependent_launch();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-    const int64_t node = (int64_t)y * kp.nx + x, k = (int64_t)y * kp.pitch + x;
-    R gFx = R(0), gFy = R(0), gG = R(0), gT = R(0), Jt = R(0);
-    const R inv_nf = sizeof(R) == 8 ? R(aa.inv_nfluid) : R(aa.inv_nfluid_f);
-    if (x < kp.nx && !node_is_solid(kp, node)) {
-        const Consts<R> &cc = cst<R>(kp);
-        const Around nb = around(kp, x, y);
-        const unsigned wm = wall_mask(kp, nb);
-        R lam[9];
-        lambda_at<R>(kp, aa, nb, wm, sizeof(R) == 8 ? R(aa.w_scale) : R(aa.w_scale_f), inv_nf, lam);
-
-        // ---- forward quantities at this node: the pull of Eq. (lbe.str) with half-way walls
-        // (the only walls the adjoint accepts): f_i = A_o(x) + 0 when x - e_i is a wall, as
-        // the forward step's bounce-back rule evaluates it
-        R f[9];
-        f[0] = load_pop_at<S>(kp, 0, k);
+    typedef Lanes<R> Z;
+    typedef typename Z::T T;
+    typedef AdjTile<R, U> G;
+    constexpr int N = Z::N, ROWS = G::ROWS, UNITS = G::UNITS;
+    auto &cs = sh_.c;
+    auto &red = sh_.red;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * ROWS;
+    // lane's nodes of unit u: their places in the tile (row and column 0 are the ring's) and the lattice
+    struct Place {
+        int x[N], y[N], r[N], c[N];
+    };
+    auto place = [&](int u) -> Place {
+        Place q;
 #pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            if ((wm >> opp_(i)) & 1u) f[i] = load_pop_at<S>(kp, opp_(i), k) + R(0);
-            else f[i] = load_pop_at<S>(kp, i, nb.k(opp_(i)));  // x - e_i = x + e_opp(i)
+        for (int e = 0; e < N; ++e) {
+            if (u < UNITS) q.r[e] = N * u + 1 + e, q.c[e] = lane + 1;
+            else if (N == 2 && u == UNITS) q.r[e] = e ? ROWS + 1 : 0, q.c[e] = lane + 1;
+            else if (N == 1 && u < UNITS + 2) q.r[e] = u == UNITS ? 0 : ROWS + 1, q.c[e] = lane + 1;
+            else if (N == 2) q.r[e] = min(lane, ROWS + 1), q.c[e] = e ? kTileX + 1 : 0;
+            else q.r[e] = min(lane >> 1, ROWS + 1), q.c[e] = (lane & 1) * (kTileX + 1);
+            q.x[e] = x0 + q.c[e] - 1, q.y[e] = y0 + q.r[e] - 1;
         }
-        const R rho = density<R>(f);
-        const R jx = ((f[1] - f[3]) + (f[5] - f[6])) + (f[8] - f[7]);
-        const R jy = ((f[2] - f[4]) + (f[5] + f[6])) - (f[7] + f[8]);
-        if (aa.sum_J) {
-            // <W, A_t> at this node from its pulled populations: a population stored at x that
-            // the next streaming sends into a wall is pulled back by x itself as f_i with
-            // x - e_i a wall; every other one is pulled by exactly one fluid node
-            R wall_y = R(0), wall_x = R(0);
+        return q;
+    };
+    // wall bits of a node of the lattice: bit i when x - e_i is a wall
+    auto walls_of = [&](const Site &a) -> unsigned {
+        if (kp.links != nullptr) return kp.links[(int64_t)a.y * kp.nx + a.x];
+        return edge_walls(around(kp, a.x, a.y).inside);
+    };
+    const int64_t P = kp.plane;
+    const Place me = place(warp);
+    if (aa.ahead > 0 && lane < (aa.g_in ? 23 : 10)) {
+        // the lines of the tile that a block of the next wave will read
+        const int ya = me.y[0] + aa.ahead;
 #pragma unroll
-            for (int i = 1; i < 9; ++i) {
-                const bool wall = (wm >> opp_(i)) & 1u;
-                if (wall) {
-                    wall_x += R(ex_(i)) * f[i];
-                    wall_y += R(ey_(i)) * f[i];
+        for (int e = 0; e < N; ++e) {
+            if (ya + e >= kp.ny) break;
+            const int64_t at = (int64_t)(ya + e) * kp.pitch + x0;
+            const void *q;
+            if (lane < 9) q = static_cast<const S *>(kp.src) + (lane * P + at);
+            else if (lane == 9) q = static_cast<const R *>(kp.psi) + ((int64_t)(ya + e) * kp.nx + x0);
+            else if (lane < 19) q = static_cast<const R *>(aa.g_in) + ((lane - 10) * P + at);
+            else if (lane < 21) q = static_cast<const R *>(aa.dS_in) + ((lane - 19) * P + at);
+            else q = static_cast<const R *>(lane == 21 ? aa.dpsi_in : aa.rho_in) + at;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(q));
+        }
+    }
+    const Consts<R> &cc = cst<R>(kp);
+    const T zero = Z::all(R(0));
+    T gG2 = zero, gT2 = zero;
+    Site at[N];        // this thread's nodes of the tile: in the lattice, wall bits, whether it updates them
+    unsigned w[N], walls = 0;
+    bool own[N], any = INNER;
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+        at[e] = INNER ? Site{me.x[e], me.y[e], true} : site_of(kp, me.x[e], me.y[e]);
+        w[e] = INNER ? 0u : walls_of(at[e]);
+        own[e] = INNER || (at[e].in && !(w[e] & 1u) && me.x[e] < kp.nx && me.y[e] < kp.ny);
+        walls |= w[e];
+        any |= own[e];
+    }
+
+    // ---- c of the step after
+    if (aa.g_in != nullptr)
+#pragma unroll 1
+    for (int u = warp + G::RING < UNITS ? warp : warp + G::RING; u >= 0; u = u >= UNITS ? u - G::RING : -1) {
+        // (the last RING warps take a ring unit first, then their own)
+        const Place q_ = place(u);
+        const R *dSx = static_cast<const R *>(aa.dS_in), *dSy = dSx + P;
+        const R *dp = static_cast<const R *>(aa.dpsi_in), *rp = static_cast<const R *>(aa.rho_in);
+        T sx[9], sy[9], loc, rho, psi;
+        Site a[N];
+        bool live[N];
+        // the node x - e_i has x in its stencil along e_i
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            if constexpr (INNER) {
+                a[e] = Site{q_.x[e], q_.y[e], true};
+                live[e] = true;
+                const int64_t k = (int64_t)a[e].y * kp.pitch + a[e].x;
+                const R *px = dSx + k, *pn = px + kp.pitch, *ps_ = px - kp.pitch;
+#pragma unroll
+                for (int i = 1; i < 9; ++i) {
+                    const R *r = ey_(i) > 0 ? ps_ : ey_(i) < 0 ? pn : px;
+                    if (ex_(i)) Z::set(sx[i], e, r[-ex_(i)]);
+                    if (ey_(i)) Z::set(sy[i], e, (r + P)[-ex_(i)]);
+                }
+                Z::set(loc, e, dp[k]);
+                Z::set(rho, e, rp[k]);
+                if constexpr (sizeof(R) == 8) Z::set(psi, e, static_cast<const R *>(aa.psi_in)[k]);
+            } else {
+                a[e] = site_of(kp, q_.x[e], q_.y[e]);
+                const unsigned wq = walls_of(a[e]);
+                live[e] = a[e].in && !(wq & 1u);
+                unsigned in;
+                const Nine nn = nine_of(kp, a[e], in);
+#pragma unroll
+                for (int i = 1; i < 9; ++i) {
+                    const bool wall = (wq >> i) & 1u;
+                    if (ex_(i)) Z::set(sx[i], e, wall ? R(0) : dSx[nn.from(i)]);
+                    if (ey_(i)) Z::set(sy[i], e, wall ? R(0) : dSy[nn.from(i)]);
+                }
+                Z::set(loc, e, live[e] ? dp[nn.own()] : R(0));
+                Z::set(rho, e, live[e] ? rp[nn.own()] : R(1.0 / 16.0));
+                if constexpr (sizeof(R) == 8) Z::set(psi, e, live[e] ? static_cast<const R *>(aa.psi_in)[nn.own()] : R(1));
+            }
+        }
+        if constexpr (sizeof(R) == 4) psi = psi_v<T>(kp, rho);
+        const T ax = (sx[1] - sx[3]) + (sy[2] - sy[4]);
+        const T dg = ((sx[5] - sx[7]) + (sy[5] - sy[7])) + ((sx[8] - sx[6]) + (sy[6] - sy[8]));
+        const T dpsi = vfma(Z::all(R(1.0 / 3.0)), ax, vfma(Z::all(R(1.0 / 12.0)), dg, loc));
+        T p_rho, p_T;
+        p_eos_derivs<R>(kp, rho, p_rho, p_T);
+        // psi^2 = 2 (p - rho/3)/G
+        const T q = dpsi * vrcp(Z::all(cc.G) * psi);
+        const T c = (p_rho - Z::all(R(1.0 / 3.0))) * q;
+#pragma unroll
+        for (int e = 0; e < N; ++e) cs[q_.r[e]][q_.c[e]] = live[e] ? Z::get(c, e) : R(0);
+        if (u < UNITS) {
+            gT2 = p_T * q;
+            gG2 = psi * dpsi * Z::all(R(-0.5) / cc.G);
+#pragma unroll
+            for (int e = 0; e < N; ++e)
+                if (aa.tail && own[e]) static_cast<R *>(aa.c_out)[(int64_t)at[e].y * kp.pitch + at[e].x] = Z::get(c, e);
+        }
+    }
+    const bool walled = INNER ? (__syncthreads(), false) : __syncthreads_or(walls & 0x1feu) != 0;
+
+    T gFx = zero, gFy = zero, gG = zero, gT = zero, Jt = zero;
+    if (any && !aa.tail) {
+        const R wscale = sizeof(R) == 8 ? R(aa.w_scale) : R(aa.w_scale_f);
+        const R inv_nf = sizeof(R) == 8 ? R(aa.inv_nfluid) : R(aa.inv_nfluid_f);
+        // ---- the state: the pull of Eq. (lbe.str) with half-way walls (the only walls the adjoint
+        // accepts): f_i = A_o(x) + 0 when x - e_i is a wall, as the forward step evaluates it;
+        // lambda_{t+1}; psi of A_t around the node
+        T f[9], lam[9], ps[9];
+        const R *g = static_cast<const R *>(aa.g_in), *psif = static_cast<const R *>(kp.psi);
+        const S *src = static_cast<const S *>(kp.src);
+        constexpr bool DEV = IsDev<S>::value;
+        // psi and c of the rows y - 1 .. y + N of the thread's column and the columns beside it
+        R ca[N + 2][3], pa[N + 2][3];
+#pragma unroll
+        for (int r = 0; r < N + 2; ++r)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) ca[r][d] = g != nullptr ? cs[me.r[0] - 1 + r][me.c[0] - 1 + d] : R(0);
+        if constexpr (INNER) {
+            const R *p = psif + ((int64_t)(me.y[0] - 1) * kp.nx + me.x[0]);
+#pragma unroll
+            for (int r = 0; r < N + 2; ++r, p += kp.nx)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) pa[r][d] = p[d - 1];
+        }
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            const R wi = aa.objective == 0 ? R(0) : wscale * inv_nf;  // objective 1: W_i = e_ix / N_fluid
+            if constexpr (INNER) {
+                const int64_t k = (int64_t)me.y[e] * kp.pitch + me.x[e];
+                const char *ps_ = reinterpret_cast<const char *>(src + k), *pg = reinterpret_cast<const char *>(g + k);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    R wref = R(0);
+                    if constexpr (DEV) wref = __fmul_rn(w_<R>(i), kp.per_node_ref ? (kp.ref_src + (k - ey_(i) * kp.pitch))[-ex_(i)] : cc.rho_ref);
+                    Z::set(f[i], e, Codec<S>::dec(reinterpret_cast<const S *>(ps_ + kp.pull[i])[-ex_(i)], wref, cc.inv_scale));
+                    R v = R(ex_(i)) * wi;
+                    if (g != nullptr) v += reinterpret_cast<const R *>(pg + aa.push[i])[ex_(i)] + ca[e + 1 + ey_(i)][1 + ex_(i)];
+                    Z::set(lam[i], e, v);
+                    Z::set(ps[i], e, pa[e + 1 + ey_(i)][1 + ex_(i)]);
+                }
+            } else {
+                unsigned in;
+                const Nine nn = nine_of(kp, at[e], in);
+                const Around nb = around(kp, at[e].x, at[e].y);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    Z::set(f[i], e, load_pop_at<S>(kp, i, nn.from(i)));
+                    R v = R(ex_(i)) * wi;
+                    if (g != nullptr) v += g[i * P + nn.from(opp_(i))] + ca[e + 1 + ey_(i)][1 + ex_(i)];
+                    Z::set(lam[i], e, v);
+                    Z::set(ps[i], e, nb.in(i) ? psif[nb.n(i)] : cc.psi_s);
                 }
             }
-            Jt = aa.objective == 0 ? R(-2) * wall_y : (jx - R(2) * wall_x) * inv_nf;
-        }
-        const R *psif = static_cast<const R *>(kp.psi);
-        const R psi = psif[node];
-        R Sx, Sy, Fex, Fey;
-        stencil_S<R>(AroundPsi<R>{kp, psif, nb}, Sx, Sy);
-        external_force<R>(kp, node, rho, Fex, Fey);
-        const R G = cc.G;
-        const R Fx = -G * psi * Sx + Fex, Fy = -G * psi * Sy + Fey;
-        const R inv = R(1) / rho;
-        const R ux = (jx + R(0.5) * Fx) * inv, uy = (jy + R(0.5) * Fy) * inv;
-        const R u2 = ux * ux + uy * uy;
-        const R s14 = (f[1] + f[2]) + (f[3] + f[4]);
-        const R s58 = (f[5] + f[6]) + (f[7] + f[8]);
-        const R m1 = R(-4) * f[0] - s14 + R(2) * s58;
-        const R m2 = R(4) * f[0] - R(2) * s14 + s58;
-        const R m4 = R(-2) * (f[1] - f[3]) + ((f[5] - f[6]) + (f[8] - f[7]));
-        const R m6 = R(-2) * (f[2] - f[4]) + ((f[5] + f[6]) - (f[7] + f[8]));
-        const R m7 = (f[1] + f[3]) - (f[2] + f[4]);
-        const R m8 = (f[5] + f[7]) - (f[6] + f[8]);
-        const R Sx2 = Sx * Sx, Sy2 = Sy * Sy;
-        const bool improved = kp.improved != 0;
-        const R Q1 = cc.kq1 * (Sx2 + Sy2), Q2 = cc.q2fac * Q1;
-        const R Q7 = cc.kq7 * (Sx2 - Sy2), Q8 = cc.kq7 * Sx * Sy;
-        const R A4 = cc.c1G * Sx2 - cc.c2G * Sy2, A6 = cc.c1G * Sy2 - cc.c2G * Sx2;
-        const R Q4 = improved ? A4 * ux : R(0), Q6 = improved ? A6 * uy : R(0);
-        R sp = cc.sp, sq = cc.sq, tau = R(0), wraw = R(0);
-        if (kp.var_tau) {
-            wraw = (rho - cc.rho_g) / (cc.rho_l - cc.rho_g);
-            const R w = wraw < R(0) ? R(0) : (wraw > R(1) ? R(1) : wraw);
-            tau = R(3) * (cc.nu_g + w * (cc.nu_l - cc.nu_g)) + R(0.5);
-            sp = R(1) / tau;
-            sq = R(1) / (R(0.5) + cc.Lambda / (tau - R(0.5)));
-        }
-        const R hsp = R(1) - R(0.5) * sp, hsq = R(1) - R(0.5) * sq;
-
-        // ---- backward: lambda -> dJ/d m_bar (f_bar = M^T diag(1/|M_k|^2) m_bar)
-        const R a14 = (lam[1] + lam[2]) + (lam[3] + lam[4]);
-        const R a58 = (lam[5] + lam[6]) + (lam[7] + lam[8]);
-        const R b0 = (lam[0] + a14 + a58) * R(1.0 / 9.0);
-        const R b1 = (R(-4) * lam[0] - a14 + R(2) * a58) * R(1.0 / 36.0);
-        const R b2 = (R(4) * lam[0] - R(2) * a14 + a58) * R(1.0 / 36.0);
-        const R b3 = ((lam[1] - lam[3]) + (lam[5] - lam[6]) + (lam[8] - lam[7])) * R(1.0 / 6.0);
-        const R b4 = (R(-2) * (lam[1] - lam[3]) + (lam[5] - lam[6]) + (lam[8] - lam[7])) * R(1.0 / 12.0);
-        const R b5 = ((lam[2] - lam[4]) + (lam[5] + lam[6]) - (lam[7] + lam[8])) * R(1.0 / 6.0);
-        const R b6 = (R(-2) * (lam[2] - lam[4]) + (lam[5] + lam[6]) - (lam[7] + lam[8])) * R(1.0 / 12.0);
-        const R b7 = ((lam[1] + lam[3]) - (lam[2] + lam[4])) * R(0.25);
-        const R b8 = ((lam[5] + lam[7]) - (lam[6] + lam[8])) * R(0.25);
-
-        // m_bar_k = (1 - s_k) m_k + s_k m_eq_k + (1 - s_k/2) F_m_k + s_k Q_k (Eq. lbe.col);
-        // s_0 = s_j = 1 (m_bar_0 = rho, m_bar_j = rho u + F/2)
-        const R dm1 = (R(1) - sp) * b1, dm2 = (R(1) - sp) * b2, dm4 = (R(1) - sq) * b4;
-        const R dm6 = (R(1) - sq) * b6, dm7 = (R(1) - sp) * b7, dm8 = (R(1) - sp) * b8;
-        const R d1 = sp * b1, d2 = sp * b2, d4 = sq * b4, d6 = sq * b6, d7 = sp * b7, d8 = sp * b8;
-        const R d0 = b0, d3 = b3, d5 = b5;
-        const R g1 = hsp * b1, g2 = hsp * b2, g4 = hsq * b4, g6 = hsq * b6, g7 = hsp * b7, g8 = hsp * b8;
-        const R g3 = R(0.5) * b3, g5 = R(0.5) * b5;
-        // dQ_k = s_k b_k = d_k
-
-        R drho = R(0), dux = R(0), duy = R(0), dFx = R(0), dFy = R(0), dSx = R(0), dSy = R(0);
-        if (kp.var_tau) {
-            const R Fu = Fx * ux + Fy * uy;
-            const R meq1 = rho * (R(-2) + R(3) * u2), meq2 = rho * (R(1) - R(3) * u2);
-            const R meq4 = -rho * ux, meq6 = -rho * uy, meq7 = rho * (ux * ux - uy * uy), meq8 = rho * ux * uy;
-            const R Fm1 = R(6) * Fu, Fm2 = R(-6) * Fu, Fm4 = -Fx, Fm6 = -Fy;
-            const R Fm7 = R(2) * (Fx * ux - Fy * uy), Fm8 = Fx * uy + Fy * ux;
-            const R dsp = b1 * (meq1 - m1 - R(0.5) * Fm1 + Q1) + b2 * (meq2 - m2 - R(0.5) * Fm2 + Q2) +
-                          b7 * (meq7 - m7 - R(0.5) * Fm7 + Q7) + b8 * (meq8 - m8 - R(0.5) * Fm8 + Q8);
-            const R dsq = b4 * (meq4 - m4 - R(0.5) * Fm4 + Q4) + b6 * (meq6 - m6 - R(0.5) * Fm6 + Q6);
-            if (wraw > R(0) && wraw < R(1)) {
-                const R tm = tau - R(0.5);
-                const R dtau = -dsp * sp * sp + dsq * sq * sq * cc.Lambda / (tm * tm);
-                drho += R(3) * dtau * (cc.nu_l - cc.nu_g) / (cc.rho_l - cc.rho_g);
+            if (!INNER && (w[e] & 0x1feu)) {
+                const int64_t k = (int64_t)at[e].y * kp.pitch + at[e].x;
+#pragma unroll
+                for (int i = 1; i < 9; ++i) {
+                    const int o = opp_(i);
+                    if ((w[e] >> i) & 1u) Z::set(f[i], e, load_pop_at<S>(kp, o, k) + R(0));
+                    if ((w[e] >> o) & 1u) {  // x + e_i is a wall
+                        R v = wscale * objective_weight<R>(aa.objective, i, true, inv_nf);
+                        if (g != nullptr) v += g[o * P + k] + ca[e + 1][1];
+                        Z::set(lam[i], e, v);
+                    }
+                }
+            }
+            // the pair's other node may be no fluid node (past the lattice, or solid): keep its arithmetic finite
+            if (!INNER && !own[e]) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) Z::set(f[i], e, w_<R>(i)), Z::set(lam[i], e, R(0));
             }
         }
-        // m_eq(rho, u)
-        drho += d0 + d1 * (R(-2) + R(3) * u2) + d2 * (R(1) - R(3) * u2) + ux * (d3 - d4) + uy * (d5 - d6) +
-                (ux * ux - uy * uy) * d7 + ux * uy * d8;
-        dux += rho * (R(6) * ux * (d1 - d2) + (d3 - d4) + R(2) * ux * d7 + uy * d8);
-        duy += rho * (R(6) * uy * (d1 - d2) + (d5 - d6) - R(2) * uy * d7 + ux * d8);
-        // F_m(F, u)
-        const R dFu = R(6) * (g1 - g2);
-        dFx += dFu * ux + (g3 - g4) + R(2) * ux * g7 + uy * g8;
-        dFy += dFu * uy + (g5 - g6) - R(2) * uy * g7 + ux * g8;
-        dux += dFu * Fx + R(2) * Fx * g7 + Fy * g8;
-        duy += dFu * Fy - R(2) * Fy * g7 + Fx * g8;
-        // Q(S, u), with |F_int|^2/(G psi^2) = G |S|^2; the coefficients carry one factor G
-        const R dQ1 = d1 + cc.q2fac * d2;
-        dSx += R(2) * Sx * (cc.kq1 * dQ1 + cc.kq7 * d7) + cc.kq7 * Sy * d8;
-        dSy += R(2) * Sy * (cc.kq1 * dQ1 - cc.kq7 * d7) + cc.kq7 * Sx * d8;
-        R dG = (Q1 * dQ1 + Q7 * d7 + Q8 * d8) / G;
-        if (improved) {
-            dux += A4 * d4;
-            duy += A6 * d6;
-            dSx += R(2) * Sx * (cc.c1G * ux * d4 - cc.c2G * uy * d6);
-            dSy += R(2) * Sy * (cc.c1G * uy * d6 - cc.c2G * ux * d4);
-            dG += (Q4 * d4 + Q6 * d6) / G;
+        T rho;
+        if constexpr (sizeof(R) == 8) {
+            rho = d1{((((f[0].v + f[1].v) + f[2].v) + f[3].v) + f[4].v) + f[5].v + f[6].v + f[7].v + f[8].v};
+        } else {
+            T d[9];
+            to_dev(f, d);
+            rho = density_dev(d);
         }
+        const T p13 = f[1] + f[3], p24 = f[2] + f[4], a13 = f[1] - f[3], a24 = f[2] - f[4];
+        const T p57 = f[5] + f[7], p68 = f[6] + f[8], a57 = f[5] - f[7], a68 = f[6] - f[8];
+        const T tx = a57 - a68, ty = a57 + a68;
+        const T jx = a13 + tx, jy = a24 + ty;
+        if (aa.sum_J) {
+            // <W, A_t> at this node from its pulled populations: a population stored at x that the next
+            // streaming sends into a wall is pulled back by x itself as f_i with x - e_i a wall; every
+            // other one is pulled by exactly one fluid node
+            T wall_x = zero, wall_y = zero;
+            if (!INNER && (walls & 0x1feu)) {
+#pragma unroll
+                for (int e = 0; e < N; ++e) {
+                    R wx = R(0), wy = R(0);
+#pragma unroll
+                    for (int i = 1; i < 9; ++i)
+                        if ((w[e] >> i) & 1u) wx += R(ex_(i)) * Z::get(f[i], e), wy += R(ey_(i)) * Z::get(f[i], e);
+                    Z::set(wall_x, e, wx), Z::set(wall_y, e, wy);
+                }
+            }
+            Jt = aa.objective == 0 ? Z::all(R(-2)) * wall_y : vfma(Z::all(R(-2)), wall_x, jx) * Z::all(inv_nf);
+        }
+        const T third = Z::all(R(1.0 / 3.0)), twelfth = Z::all(R(1.0 / 12.0));
+        const T dd = ps[5] - ps[7], de = ps[8] - ps[6];
+        const T Sx = vfma(third, ps[1] - ps[3], twelfth * (dd + de));
+        const T Sy = vfma(third, ps[2] - ps[4], twelfth * (dd - de));
+        const T psi = ps[0];
+        const bool buoyant = kp.force_mode != 0;
+        const T cFx = Z::all(cc.Fx), cFy = Z::all(cc.Fy), rexc = rho - Z::all(cc.rho_g);
+        const T mG = Z::all(-cc.G), nGpsi = mG * psi;
+        const T Fx = buoyant ? vfma(nGpsi, Sx, rexc * cFx) : vfma(nGpsi, Sx, cFx);
+        const T Fy = buoyant ? vfma(nGpsi, Sy, rexc * cFy) : vfma(nGpsi, Sy, cFy);
+        const T half = Z::all(R(0.5)), two = Z::all(R(2)), six = Z::all(R(6)), three = Z::all(R(3));
+        const T inv = vrcp(rho);
+        const T ux = vfma(half, Fx, jx) * inv, uy = vfma(half, Fy, jy) * inv;
+        const T uxx = ux * ux, uyy = uy * uy, u2 = uxx + uyy, ud = uxx - uyy, uxy = ux * uy;
+        const T Sx2 = Sx * Sx, Sy2 = Sy * Sy;
+        const bool improved = kp.improved != 0;
+        const T kq1 = Z::all(cc.kq1), kq7 = Z::all(cc.kq7), q2f = Z::all(cc.q2fac), c1G = Z::all(cc.c1G), mc2G = Z::all(-cc.c2G);
+        const T Q1 = kq1 * (Sx2 + Sy2), Q7 = kq7 * (Sx2 - Sy2), Q8 = kq7 * (Sx * Sy);
+        T A4 = zero, A6 = zero;
+        if (improved) A4 = vfma(c1G, Sx2, mc2G * Sy2), A6 = vfma(c1G, Sy2, mc2G * Sx2);
+
+        // ---- backward: lambda -> dJ/d m_bar (f_bar = M^T diag(1/|M_k|^2) m_bar)
+        const T l13p = lam[1] + lam[3], l24p = lam[2] + lam[4], l13 = lam[1] - lam[3], l24 = lam[2] - lam[4];
+        const T l57p = lam[5] + lam[7], l68p = lam[6] + lam[8], l57 = lam[5] - lam[7], l68 = lam[6] - lam[8];
+        const T lt = l57 - l68, lv = l57 + l68, a14 = l13p + l24p, a58 = l57p + l68p;
+        const T b0 = (lam[0] + a14 + a58) * Z::all(R(1.0 / 9.0));
+        const T b1 = vfma(Z::all(R(4)), lam[0], vfma(Z::all(R(-2)), a58, a14)) * Z::all(R(-1.0 / 36.0));
+        const T b2 = vfma(Z::all(R(4)), lam[0], vfma(Z::all(R(-2)), a14, a58)) * Z::all(R(1.0 / 36.0));
+        const T b3 = (l13 + lt) * Z::all(R(1.0 / 6.0)), b4 = vfma(Z::all(R(-2)), l13, lt) * Z::all(R(1.0 / 12.0));
+        const T b5 = (l24 + lv) * Z::all(R(1.0 / 6.0)), b6 = vfma(Z::all(R(-2)), l24, lv) * Z::all(R(1.0 / 12.0));
+        const T b7 = (l13p - l24p) * Z::all(R(0.25)), b8 = (l57p - l68p) * Z::all(R(0.25));
+
+        T sp = Z::all(cc.sp), sq = Z::all(cc.sq), drho = zero;
+        if (kp.var_tau) {
+            const T inv_d = Z::all(R(1) / (cc.rho_l - cc.rho_g)), dnu = Z::all(cc.nu_l - cc.nu_g);
+            const T wraw = rexc * inv_d, tm = three * vfma(vclamp01(wraw), dnu, Z::all(cc.nu_g));  // tau - 1/2
+            const T rtm = vrcp(tm);
+            sp = vrcp(tm + half);
+            sq = vrcp(vfma(Z::all(cc.Lambda), rtm, half));
+            const T s14 = p13 + p24, s58 = p57 + p68;
+            const T m1 = vfma(Z::all(R(-4)), f[0], vfma(two, s58, -s14)), m2 = vfma(Z::all(R(4)), f[0], vfma(Z::all(R(-2)), s14, s58));
+            const T m4 = vfma(Z::all(R(-2)), a13, tx), m6 = vfma(Z::all(R(-2)), a24, ty), m7 = p13 - p24, m8 = p57 - p68;
+            const T Fu = vfma(Fx, ux, Fy * uy), t3 = three * rho * u2;
+            const T e1 = (vfma(Z::all(R(-2)), rho, t3) - m1) - three * Fu + Q1;
+            const T e2 = ((rho - t3) - m2) + three * Fu + q2f * Q1;
+            const T e7 = vfma(rho, ud, -m7) - vfma(Fx, ux, -(Fy * uy)) + Q7;
+            const T e8 = vfma(rho, uxy, -m8) - half * vfma(Fx, uy, Fy * ux) + Q8;
+            const T e4 = vfma(half, Fx, vfma(A4, ux, -vfma(rho, ux, m4)));
+            const T e6 = vfma(half, Fy, vfma(A6, uy, -vfma(rho, uy, m6)));
+            const T dsp = vfma(b1, e1, vfma(b2, e2, vfma(b7, e7, b8 * e8)));
+            const T dsq = vfma(b4, e4, b6 * e6);
+            const T dtau = vfma(dsq * sq * sq, Z::all(cc.Lambda) * rtm * rtm, -(dsp * sp * sp));
+            const T dr = three * dtau * dnu * inv_d;
+#pragma unroll
+            for (int e = 0; e < N; ++e)
+                if (Z::get(wraw, e) > R(0) && Z::get(wraw, e) < R(1)) Z::set(drho, e, Z::get(dr, e));
+        }
+        const T one = Z::all(R(1)), hsp = vfma(Z::all(R(-0.5)), sp, one), mhsq = vfma(half, sq, Z::all(R(-1)));  // 1 - s_p/2, -(1 - s_q/2)
+
+        // m_bar_k = (1 - s_k) m_k + s_k m_eq_k + (1 - s_k/2) F_m_k + s_k Q_k (Eq. lbe.col);
+        // s_0 = s_j = 1 (m_bar_0 = rho, m_bar_j = rho u + F/2).  d_k = s_k b_k = dJ/d m_eq_k = dJ/d Q_k
+        const T d1_ = sp * b1, d2 = sp * b2, d4 = sq * b4, d6 = sq * b6, d7 = sp * b7, d8 = sp * b8;
+        const T dm1 = b1 - d1_, dm2 = b2 - d2, dm4 = b4 - d4, dm6 = b6 - d6, dm7 = b7 - d7, dm8 = b8 - d8;
+        const T d12 = d1_ - d2, d34 = b3 - d4, d56 = b5 - d6;
+        // m_eq(rho, u)
+        drho = drho + (vfma(Z::all(R(-2)), d1_, b0) + d2) + vfma(three * u2, d12, vfma(ux, d34, vfma(uy, d56, vfma(ud, d7, uxy * d8))));
+        const T s12 = six * d12, t7 = two * d7;
+        T dux = rho * vfma(ux, s12 + t7, vfma(uy, d8, d34));
+        T duy = rho * vfma(uy, s12 - t7, vfma(ux, d8, d56));
+        // F_m(F, u)
+        const T dFu = six * hsp * (b1 - b2), g7 = two * hsp * b7, g8 = hsp * b8;
+        T dFx = vfma(ux, dFu + g7, vfma(uy, g8, vfma(half, b3, mhsq * b4)));
+        T dFy = vfma(uy, dFu - g7, vfma(ux, g8, vfma(half, b5, mhsq * b6)));
+        dux = vfma(Fx, dFu + g7, vfma(Fy, g8, dux));
+        duy = vfma(Fy, dFu - g7, vfma(Fx, g8, duy));
+        // Q(S, u), with |F_int|^2/(G psi^2) = G |S|^2; the coefficients carry one factor G
+        const T dQ1 = vfma(q2f, d2, d1_);
+        const T k1 = kq1 * dQ1, k7 = kq7 * d7, k8 = kq7 * d8;
+        T dSx = vfma(two * Sx, k1 + k7, Sy * k8);
+        T dSy = vfma(two * Sy, k1 - k7, Sx * k8);
+        T dG = vfma(Q1, dQ1, vfma(Q7, d7, Q8 * d8));
+        if (improved) {
+            const T x4 = ux * d4, y6 = uy * d6;
+            dux = vfma(A4, d4, dux);
+            duy = vfma(A6, d6, duy);
+            dSx = vfma(two * Sx, vfma(c1G, x4, mc2G * y6), dSx);
+            dSy = vfma(two * Sy, vfma(c1G, y6, mc2G * x4), dSy);
+            dG = vfma(A4, x4, vfma(A6, y6, dG));
+        }
+        dG = dG * Z::all(R(1) / cc.G);
         // u = (j + F/2)/rho
-        const R djx = dux * inv, djy = duy * inv;
-        dFx += R(0.5) * djx;
-        dFy += R(0.5) * djy;
-        drho -= (ux * dux + uy * duy) * inv;
+        const T djx = dux * inv, djy = duy * inv;
+        dFx = vfma(half, djx, dFx);
+        dFy = vfma(half, djy, dFy);
+        drho = drho - vfma(ux, djx, uy * djy);
         // F = -G psi S + F_ext
-        if (kp.force_mode == 0) {
+        if (buoyant) {
+            gFx = rexc * dFx;
+            gFy = rexc * dFy;
+            drho = vfma(cFx, dFx, vfma(cFy, dFy, drho));
+        } else {
             gFx = dFx;
             gFy = dFy;
-        } else {
-            gFx = (rho - cc.rho_g) * dFx;
-            gFy = (rho - cc.rho_g) * dFy;
-            drho += cc.Fx * dFx + cc.Fy * dFy;
         }
-        const R dpsi_loc = -G * (Sx * dFx + Sy * dFy);
-        dG -= psi * (Sx * dFx + Sy * dFy);
-        dSx -= G * psi * dFx;
-        dSy -= G * psi * dFy;
+        const T SdF = vfma(Sx, dFx, Sy * dFy);
+        const T dpsi_loc = mG * SdF;
+        dG = dG - psi * SdF;
+        dSx = vfma(nGpsi, dFx, dSx);
+        dSy = vfma(nGpsi, dFy, dSy);
         // walls in the stencil carry psi(rho_s; T, G)
-        R dpsi_s = R(0);
 #pragma unroll
-        for (int i = 1; i < 9; ++i)
-            if ((wm >> i) & 1u) dpsi_s += omega_<R>(i) * (R(ex_(i)) * dSx + R(ey_(i)) * dSy);
-        if (dpsi_s != R(0)) {
-            R prs, pTs;
-            p_eos_derivs<R>(kp, cc.rho_s, prs, pTs);
-            dG += -cc.psi_s / (R(2) * G) * dpsi_s;
-            gT = pTs / (G * cc.psi_s) * dpsi_s;
+        for (int e = 0; e < N; ++e) {
+            if (INNER || !own[e] || !(w[e] & 0x1feu)) continue;
+            R dpsi_s = R(0);
+#pragma unroll
+            for (int i = 1; i < 9; ++i)
+                if ((w[e] >> opp_(i)) & 1u) dpsi_s += omega_<R>(i) * (R(ex_(i)) * Z::get(dSx, e) + R(ey_(i)) * Z::get(dSy, e));
+            if (dpsi_s != R(0)) {
+                T prs, pTs;
+                p_eos_derivs<R>(kp, Z::all(cc.rho_s), prs, pTs);
+                Z::set(dG, e, Z::get(dG, e) - cc.psi_s / (R(2) * cc.G) * dpsi_s);
+                Z::set(gT, e, Z::get(pTs, e) / (cc.G * cc.psi_s) * dpsi_s);
+            }
         }
         gG = dG;
 
         // g_i = drho + e_i . dj + (M^T dm)_i
-        const R base_ax = -dm1 - R(2) * dm2, base_dg = R(2) * dm1 + dm2;
-        R *go = static_cast<R *>(aa.g_out);
-        const int64_t P = kp.plane;
-        go[0 * P + k] = drho + R(-4) * dm1 + R(4) * dm2;
-        go[1 * P + k] = drho + djx + base_ax - R(2) * dm4 + dm7;
-        go[2 * P + k] = drho + djy + base_ax - R(2) * dm6 - dm7;
-        go[3 * P + k] = drho - djx + base_ax + R(2) * dm4 + dm7;
-        go[4 * P + k] = drho - djy + base_ax + R(2) * dm6 - dm7;
-        go[5 * P + k] = drho + djx + djy + base_dg + dm4 + dm6 + dm8;
-        go[6 * P + k] = drho - djx + djy + base_dg - dm4 + dm6 - dm8;
-        go[7 * P + k] = drho - djx - djy + base_dg - dm4 - dm6 + dm8;
-        go[8 * P + k] = drho + djx - djy + base_dg + dm4 - dm6 - dm8;
-        R *dS = static_cast<R *>(aa.dS);
-        dS[k] = dSx;
-        dS[P + k] = dSy;
-        static_cast<R *>(aa.dpsi)[k] = dpsi_loc;
-        static_cast<R *>(aa.rho)[k] = rho;
+        const T ga = drho - vfma(two, dm2, dm1), gd = drho + vfma(two, dm1, dm2);
+        const T hx = vfma(Z::all(R(-2)), dm4, djx), hy = vfma(Z::all(R(-2)), dm6, djy);
+        const T ax7 = ga + dm7, ay7 = ga - dm7, ex = djx + dm4, ey = djy + dm6;
+        const T dp = gd + dm8, dq = gd - dm8, es = ex + ey, ed = ey - ex;
+        const T go[9] = {vfma(Z::all(R(4)), dm2 - dm1, drho), ax7 + hx, ay7 + hy, ax7 - hx, ay7 - hy, dp + es, dq + ed, dp - es, dq - ed};
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            if (!INNER && !own[e]) continue;
+            const int64_t k = (int64_t)at[e].y * kp.pitch + at[e].x;
+            R *out = static_cast<R *>(aa.g_out) + k, *dS = static_cast<R *>(aa.dS_out) + k;
+#pragma unroll
+            for (int i = 0; i < 9; ++i, out += P) *out = Z::get(go[i], e);
+            dS[0] = Z::get(dSx, e);
+            dS[P] = Z::get(dSy, e);
+            static_cast<R *>(aa.dpsi_out)[k] = Z::get(dpsi_loc, e);
+            static_cast<R *>(aa.rho_out)[k] = Z::get(rho, e);
+            if constexpr (sizeof(R) == 8) static_cast<R *>(aa.psi_out)[k] = Z::get(psi, e);
+        }
     }
-    const R v[5] = {gFx, gFy, gG, gT, Jt};
-    block_add<5>(v, aa.part, SLOT_FX);
+    // ---- parameter sums, in the order of AdjSlot
+    {
+        const T v[7] = {gFx, gFy, gG, gT, Jt, gG2, gT2};
+#pragma unroll
+        for (int q = 0; q < 7; ++q)
+#pragma unroll
+            for (int e = 0; e < N; ++e) red[q][threadIdx.x + e * 32 * UNITS] = own[e] ? Z::get(v[q], e) : R(0);
+    }
+    __syncthreads();
+    // away from walls the wall terms (and objective 0, the force on them) are zero
+    const unsigned skip = walled ? 0u : (1u << SLOT_T1) | (aa.objective == 0 ? 1u << SLOT_J : 0u);
+    block_add<R>(&red[0][0], N * 32 * UNITS, 7, N * 32 * UNITS, skip, aa.part);
 }
 
-// Pass 2: dJ/dpsi(x) from the stencils that read psi(x), then c(x) = psi'(rho) dJ/dpsi.
-template <class S>
-__global__ void __launch_bounds__(kRowThreads) k_adj2(KParams kp, AdjArgs aa)
+// One transposed step at A_t (kp.src) with the psi field of A_t (kp.psi).  U: units of a block, B: blocks
+// per SM the registers must allow.
+template <class S, int U, int B>
+__global__ void __launch_bounds__(32 * U, B) k_adj(KParams kp, AdjArgs aa)
 {
-    typedef typename Codec<S>::R R;
+    typedef AdjTile<typename Codec<S>::R, U> G;
+    __shared__ AdjShared<typename Codec<S>::R, U> sh;
     grid_dependency_wait();
     allow_dependent_launch();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-    const int64_t node = (int64_t)y * kp.nx + x, k = (int64_t)y * kp.pitch + x;
-    R gG = R(0), gT = R(0);
-    if (x < kp.nx && !node_is_solid(kp, node)) {
-        const Consts<R> &cc = cst<R>(kp);
-        const R *dS = static_cast<const R *>(aa.dS);
-        R dpsi = static_cast<const R *>(aa.dpsi)[k];
-        const Around nb = around(kp, x, y);
-#pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            // the node z = x - e_i = x + e_opp(i) has x in its stencil along e_i
-            const int o = opp_(i);
-            if (!nb.in(o)) continue;
-            if (kp.solid != nullptr && kp.solid[nb.n(o)] != 0) continue;
-            const int64_t kz = nb.k(o);
-            dpsi += omega_<R>(i) * (R(ex_(i)) * dS[kz] + R(ey_(i)) * dS[kp.plane + kz]);
-        }
-        const R rho = static_cast<const R *>(aa.rho)[k];
-        const R psi = static_cast<const R *>(kp.psi)[node];
-        R p_rho, p_T;
-        p_eos_derivs<R>(kp, rho, p_rho, p_T);
-        // psi^2 = 2 (p - rho/3)/G
-        const R Gpsi = cc.G * psi;
-        static_cast<R *>(aa.c_out)[k] = (p_rho - R(1.0 / 3.0)) / Gpsi * dpsi;
-        gT = p_T / Gpsi * dpsi;
-        gG = -psi / (R(2) * cc.G) * dpsi;
-    }
-    const R v[2] = {gG, gT};
-    block_add<2>(v, aa.part, SLOT_G2);
+    const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * G::ROWS;
+    if (x0 >= 2 && x0 + kTileX + 2 <= kp.nx && y0 >= 2 && y0 + G::ROWS + 2 <= kp.ny && kp.links == nullptr)
+        adj_block<S, U, true>(kp, aa, sh);
+    else
+        adj_block<S, U, false>(kp, aa, sh);
 }
 
-// lambda_0 = dJ/dA at the starting state (no objective weight at t = 0), FP64 [9][ny][nx].
+// lambda_0 = dJ/dA at the starting state (no objective weight at t = 0), FP64 [9][ny][nx], from g and c.
 template <class S>
-__global__ void __launch_bounds__(kRowThreads) k_adj_lambda(KParams kp, AdjArgs aa, double *out)
+__global__ void __launch_bounds__(kRowThreads) k_adj_lambda(KParams kp, const typename Codec<S>::R *g,
+                                                            const typename Codec<S>::R *c, double *out)
 {
     typedef typename Codec<S>::R R;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
     if (x >= kp.nx) return;
-    const int64_t n = (int64_t)kp.nx * kp.ny, node = (int64_t)y * kp.nx + x;
-    R lam[9];
-    if (node_is_solid(kp, node)) {
+    const int64_t n = (int64_t)kp.nx * kp.ny, node = (int64_t)y * kp.nx + x, k = (int64_t)y * kp.pitch + x;
+    const bool solid = node_is_solid(kp, node);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) lam[i] = R(0);
-    } else {
-        const Around nb = around(kp, x, y);
-        lambda_at<R>(kp, aa, nb, wall_mask(kp, nb), R(0), R(aa.inv_nfluid), lam);
+    for (int i = 0; i < 9; ++i) {
+        int64_t kn = k;
+        R v = R(0);
+        if (!solid) v = i != 0 && wall_link(kp, x, y, i, kn) ? g[opp_(i) * kp.plane + k] + c[k] : g[i * kp.plane + kn] + c[kn];
+        out[i * n + node] = double(v);
     }
-#pragma unroll
-    for (int i = 0; i < 9; ++i) out[i * n + node] = double(lam[i]);
 }
 
 // FP64 sum over fluid nodes of sum_i W_i(x) A_i(x) for the state kp.src.
@@ -474,21 +660,42 @@ __global__ void __launch_bounds__(256) k_adj_reduce(const double *part, int64_t 
 
 template <class S>
 struct Adjoint {
-    static cudaError_t pass1(const KParams &kp, const AdjArgs &aa, cudaStream_t st)
+    // FP32 arithmetic: tall tiles and 128 registers on small lattices, where a block's ring is a large
+    // part of its work and there are few blocks to hide latency (256 x 1024: 27.5 us a step of the call
+    // against 30.9); short ones and five blocks per SM from 2^19 nodes (2048^2: 249 against 267).
+    static constexpr bool F64 = sizeof(typename Codec<S>::R) == 8;
+    static bool tall(const KParams &kp) { return F64 || (int64_t)kp.nx * kp.ny < (int64_t)1 << 19; }
+    static int rows(const KParams &kp) { return F64 ? 8 : tall(kp) ? 16 : 8; }
+    static dim3 grid(const KParams &kp) { return dim3((kp.nx + kTileX - 1) / kTileX, (kp.ny + rows(kp) - 1) / rows(kp)); }
+    static cudaError_t step(const KParams &kp, const AdjArgs &args, cudaStream_t st)
     {
-        return launch_dependent(k_adj1<S>, row_grid(kp), dim3(kRowThreads), 0, st, kp, aa);
+        typedef typename Codec<S>::R R;
+        AdjArgs aa = args;
+        KParams kq = kp;
+        for (int i = 0; i < 9; ++i) {
+            kq.pull[i] = (i * kp.plane - ey_(i) * kp.pitch) * (int64_t)sizeof(S);
+            aa.push[i] = (i * kp.plane + ey_(i) * kp.pitch) * (int64_t)sizeof(R);
+        }
+        // rows between a tile and the one it prefetches: two blocks per SM further on, where the planes
+        // read and written exceed the 129 MB L2
+        const int sms = kp.sm_count > 0 ? kp.sm_count : 148;
+        const double bytes = kp.plane * (9.0 * sizeof(S) + 27.0 * sizeof(R));
+        aa.ahead = bytes > 120e6 && !aa.tail ? (int)(2u * sms / grid(kp).x + 1) * rows(kp) : 0;
+        if constexpr (F64) {
+            return launch_dependent(k_adj<S, 8, 1>, grid(kp), dim3(256), 0, st, kq, aa);
+        } else {
+            return tall(kp) ? launch_dependent(k_adj<S, 8, 2>, grid(kp), dim3(256), 0, st, kq, aa)
+                            : launch_dependent(k_adj<S, 4, 5>, grid(kp), dim3(128), 0, st, kq, aa);
+        }
     }
-    static cudaError_t pass2(const KParams &kp, const AdjArgs &aa, cudaStream_t st)
+    // blocks of the transposed step (rows of the partial-sum array)
+    static int64_t blocks(const KParams &kp) { return (int64_t)grid(kp).x * grid(kp).y; }
+    static cudaError_t lambda(const KParams &kp, const void *g, const void *c, double *out, cudaStream_t st)
     {
-        return launch_dependent(k_adj2<S>, row_grid(kp), dim3(kRowThreads), 0, st, kp, aa);
-    }
-    static cudaError_t lambda(const KParams &kp, const AdjArgs &aa, double *out, cudaStream_t st)
-    {
-        k_adj_lambda<S><<<row_grid(kp), kRowThreads, 0, st>>>(kp, aa, out);
+        typedef typename Codec<S>::R R;
+        k_adj_lambda<S><<<row_grid(kp), kRowThreads, 0, st>>>(kp, static_cast<const R *>(g), static_cast<const R *>(c), out);
         return cudaGetLastError();
     }
-    // blocks of the row grid of the transposed passes (rows of the partial-sum array)
-    static int64_t blocks(const KParams &kp) { return (int64_t)row_grid(kp).x * row_grid(kp).y; }
     static cudaError_t reduce(const KParams &kp, const double *part, double *out, cudaStream_t st)
     {
         k_adj_reduce<S><<<kAdjSlots, 256, 0, st>>>(part, blocks(kp), out);

@@ -28,8 +28,7 @@ Launchers launchers_bf16()
     L.diag = &TwoPass<__nv_bfloat16>::diag;
     L.get_state = &TwoPass<__nv_bfloat16>::get_state;
     L.set_state = &TwoPass<__nv_bfloat16>::set_state;
-    L.adj_pass1 = &Adjoint<__nv_bfloat16>::pass1;
-    L.adj_pass2 = &Adjoint<__nv_bfloat16>::pass2;
+    L.adj_step = &Adjoint<__nv_bfloat16>::step;
     L.adj_lambda = &Adjoint<__nv_bfloat16>::lambda;
     L.objective = &Adjoint<__nv_bfloat16>::objective;
     L.adj_blocks = &Adjoint<__nv_bfloat16>::blocks;

@@ -28,8 +28,7 @@ Launchers launchers_f16()
     L.diag = &TwoPass<__half>::diag;
     L.get_state = &TwoPass<__half>::get_state;
     L.set_state = &TwoPass<__half>::set_state;
-    L.adj_pass1 = &Adjoint<__half>::pass1;
-    L.adj_pass2 = &Adjoint<__half>::pass2;
+    L.adj_step = &Adjoint<__half>::step;
     L.adj_lambda = &Adjoint<__half>::lambda;
     L.objective = &Adjoint<__half>::objective;
     L.adj_blocks = &Adjoint<__half>::blocks;

@@ -28,8 +28,7 @@ Launchers launchers_f32()
     L.diag = &TwoPass<float>::diag;
     L.get_state = &TwoPass<float>::get_state;
     L.set_state = &TwoPass<float>::set_state;
-    L.adj_pass1 = &Adjoint<float>::pass1;
-    L.adj_pass2 = &Adjoint<float>::pass2;
+    L.adj_step = &Adjoint<float>::step;
     L.adj_lambda = &Adjoint<float>::lambda;
     L.objective = &Adjoint<float>::objective;
     L.adj_blocks = &Adjoint<float>::blocks;

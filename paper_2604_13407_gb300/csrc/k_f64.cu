@@ -17,8 +17,7 @@ Launchers launchers_f64()
     L.diag = &TwoPass<double>::diag;
     L.get_state = &TwoPass<double>::get_state;
     L.set_state = &TwoPass<double>::set_state;
-    L.adj_pass1 = &Adjoint<double>::pass1;
-    L.adj_pass2 = &Adjoint<double>::pass2;
+    L.adj_step = &Adjoint<double>::step;
     L.adj_lambda = &Adjoint<double>::lambda;
     L.objective = &Adjoint<double>::objective;
     L.adj_blocks = &Adjoint<double>::blocks;

@@ -6,17 +6,19 @@
 //   lambda_n = W/n,  lambda_t = W/n + Step'(A_t)^T lambda_{t+1}  (t = n-1 .. 1),
 //   lambda_0 = Step'(A_0)^T lambda_1,  dJ/dtheta = sum_t (dStep(A_t)/dtheta)^T lambda_{t+1}.
 //
-// Forward sweep: the context advances n steps with its normal kernels, storing A_t every
-// K steps (a checkpoint); <W, A_n> is summed in FP64 there, <W, A_t> of the other states by
-// the transposed passes (objective alone: every state in the forward sweep).  Backward sweep, one segment of K
-// steps at a time from the last: the states of the segment are recomputed from its
-// checkpoint with the step kernels the context uses, each leaving the psi field of the
-// state it reads in a buffer of its own (the two-pass step's psi pass writes it anyway; the
-// one-pass step writes it on request), then the transposed step runs from the last state
-// of the segment to the first.  The recompute of a segment runs on a second stream, overlapping the
-// transposed steps of the segment after it, so segment states and psi fields come in two
-// sets.  Device memory: ceil(n/K) checkpoints, 2 (K - 1) segment states, 2 K psi fields
-// and the adjoint planes; it is kept for the next call with the same sizes.
+// Forward sweep: n steps, each from one buffer straight into another: the states at t = K, 2K, ... are written into their checkpoints, the others into scratch (the
+// segment states, not yet in use), A_n into the context's buffer that n steps would leave it in (where
+// that is A_0's own, A_0 is copied to its checkpoint first).  The steps of the last segment
+// write the segment's states and psi fields on the way, so that segment is never recomputed.
+// <W, A_n> is summed in FP64 there, <W, A_t> of the other states by the transposed steps (objective
+// alone: every state in the forward sweep).  Backward sweep, one segment of K steps at a time from the
+// last: the states of the segment are recomputed from its checkpoint with the step kernels the context
+// uses, each leaving the psi field of the state it reads in a buffer of its own (the two-pass step's
+// psi pass writes it anyway; the one-pass steps write it on request), then the transposed step runs
+// from the last state of the segment to the first.  The recompute of a segment runs on a second
+// stream, overlapping the transposed steps of the segment after it, so segment states and psi fields
+// come in two sets.  Device memory: ceil(n/K) checkpoints, 2 (K - 1) segment states, 2 K psi
+// fields and the adjoint planes; it is kept for the next call with the same sizes.
 //
 // 16-bit storage: a stored state is its nine planes of deviations plus, with a per-node
 // reference density, that plane; the recompute repeats the forward steps' stochastic
@@ -67,14 +69,14 @@ struct Carver {
 
 struct Layout {
     std::vector<void *> ckpt, seg[2], psi[2];  // two sets of segment states and psi fields
-    void *g[2], *c[2], *dS, *dpsi, *rho;
-    double *part;  // per-block partial sums of the transposed passes [blocks][kAdjSlots]
+    void *g[2], *dS[2], *dpsi[2], *rho[2], *psi_r[2], *c;  // psi_r: FP64 only
+    double *part;  // per-block partial sums of the transposed steps [blocks][kAdjSlots]
     double *red;   // their column sums (kAdjSlots)
     double *acc;
 };
 
-size_t carve(Carver &cv, Layout &L, int64_t nseg, int64_t K, size_t state_bytes, size_t plane_r, size_t psi_bytes,
-             size_t part_bytes)
+size_t carve(Carver &cv, Layout &L, int64_t nseg, int64_t K, size_t state_bytes, size_t plane_r, bool psi_planes,
+             size_t psi_bytes, size_t part_bytes)
 {
     L.ckpt.resize(nseg);
     for (auto &b : L.ckpt) b = cv.take(state_bytes);
@@ -86,11 +88,12 @@ size_t carve(Carver &cv, Layout &L, int64_t nseg, int64_t K, size_t state_bytes,
     }
     for (int s = 0; s < 2; ++s) {
         L.g[s] = cv.take(9 * plane_r);
-        L.c[s] = cv.take(plane_r);
+        L.dS[s] = cv.take(2 * plane_r);
+        L.dpsi[s] = cv.take(plane_r);
+        L.rho[s] = cv.take(plane_r);
+        L.psi_r[s] = psi_planes ? cv.take(plane_r) : nullptr;
     }
-    L.dS = cv.take(2 * plane_r);
-    L.dpsi = cv.take(plane_r);
-    L.rho = cv.take(plane_r);
+    L.c = cv.take(plane_r);
     L.part = static_cast<double *>(cv.take(part_bytes));
     L.red = static_cast<double *>(cv.take(kAdjSlots * sizeof(double)));
     L.acc = static_cast<double *>(cv.take(8 * sizeof(double)));
@@ -113,7 +116,7 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
 {
     ContextView v = view_of(ctx);
     const lbm_params &p = *v.p;
-    if (!v.L->adj_pass1) {
+    if (!v.L->adj_step) {
         msg = "no transposed step for this storage type";
         return LBM_ENOTSUP;
     }
@@ -156,8 +159,8 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
     // device memory, kept across calls
     Layout L;
     Carver probe{nullptr};
-    const size_t need = backward ? carve(probe, L, nseg, Kseg, state_bytes, plane_r, psi_bytes, part_bytes)
-                                 : carve(probe, L, 0, 1, 0, 0, 0, 0);
+    const size_t need = backward ? carve(probe, L, nseg, Kseg, state_bytes, plane_r, real == 8, psi_bytes, part_bytes)
+                                 : carve(probe, L, 0, 1, 0, 0, false, 0, 0);
     AdjointState *&as = *v.adj;
     if (!as) as = new AdjointState();
     if (as->bytes < need) {
@@ -177,8 +180,8 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
         as->bytes = need;
     }
     Carver cv{static_cast<char *>(as->base)};
-    if (backward) carve(cv, L, nseg, Kseg, state_bytes, plane_r, psi_bytes, part_bytes);
-    else carve(cv, L, 0, 1, 0, 0, 0, 0);
+    if (backward) carve(cv, L, nseg, Kseg, state_bytes, plane_r, real == 8, psi_bytes, part_bytes);
+    else carve(cv, L, 0, 1, 0, 0, false, 0, 0);
     if (backward && !as->side) {
         ACK(cudaStreamCreateWithFlags(&as->side, cudaStreamNonBlocking), "cudaStreamCreate");
         cudaEvent_t *evs[] = {&as->fork, &as->recomputed[0], &as->recomputed[1], &as->reversed[0], &as->reversed[1]};
@@ -193,22 +196,66 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
     // ---- forward sweep: checkpoints and the objective
     KParams kq = *v.kp;
     const int64_t step0 = *v.steps;  // the forward sweep's step t runs as the context's step step0 + t
-    for (int64_t t = 0; t < nsteps; ++t) {
-        if (backward && t % K == 0) {
-            ACK(cudaMemcpyAsync(L.ckpt[t / K], v.pops[*v.cur], pop_bytes, cudaMemcpyDeviceToDevice, st),
-                "checkpoint copy");
+    const int last_q = (int)((nseg - 1) & 1);  // buffer set of the last segment
+    // One step of the context's kernel from one state buffer to another, leaving psi of the state it
+    // reads in `psi` (null: where the context keeps it).
+    auto step_to = [&](const void *src, const float *ref, void *dst, float *ref_dst, void *psi, int64_t t,
+                       cudaStream_t on) -> lbm_status {
+        KParams kp = *v.kp;
+        kp.src = src, kp.ref_src = ref, kp.dst = dst, kp.ref_dst = ref_dst;
+        kp.sr_seed = v.sr_seed(step0 + t);
+        if (v.fused_pass) {
+            kp.psi_out = psi;
+            ACK(v.fused_pass(kp, on), "one-pass step kernel");
+        } else {
+            if (psi) kp.psi = psi;
+            ACK(v.psi_pass(kp, on), "psi kernel");
+            ACK(v.collide_pass(kp, on), "collide kernel");
+        }
+        return LBM_OK;
+    };
+    const void *first = nullptr;  // A_0 (during the backward sweep)
+    const float *first_ref = nullptr;
+    if (backward) {
+        const int from = *v.cur, to = from ^ (int)(nsteps & 1);
+        const void *src = v.pops[from];
+        const float *src_ref = v.refp[from];
+        if (to == from) {
+            ACK(cudaMemcpyAsync(L.ckpt[0], src, pop_bytes, cudaMemcpyDeviceToDevice, st), "checkpoint copy");
             if (ref_bytes)
-                ACK(cudaMemcpyAsync(ref_of(L.ckpt[t / K]), v.refp[*v.cur], ref_bytes, cudaMemcpyDeviceToDevice, st),
-                    "checkpoint copy");
+                ACK(cudaMemcpyAsync(ref_of(L.ckpt[0]), src_ref, ref_bytes, cudaMemcpyDeviceToDevice, st), "checkpoint copy");
+            src = L.ckpt[0], src_ref = ref_of(src);
         }
-        lbm_status s = v.run_steps(ctx, 1);
-        if (s != LBM_OK) {
-            msg = "forward step failed";
-            return s;
+        first = src, first_ref = src_ref;
+        for (int64_t t = 0; t < nsteps; ++t) {
+            const int64_t s = t / K, at = t - s * K;
+            const bool last = s == nseg - 1;
+            void *dst;
+            float *dst_ref;
+            if (t == nsteps - 1) {
+                dst = v.pops[to], dst_ref = v.refp[to];
+            } else {
+                dst = (t + 1) % K == 0 ? L.ckpt[s + 1] : last ? L.seg[last_q][at] : L.seg[0][at & 1];
+                dst_ref = ref_of(dst);
+            }
+            const lbm_status r = step_to(src, src_ref, dst, dst_ref, last ? L.psi[last_q][at] : nullptr, t, st);
+            if (r != LBM_OK) return r;
+            src = dst, src_ref = dst_ref;
         }
-        // with a backward sweep, <W, A_t> of t = 1 .. n-1 is summed by the transposed passes,
-        // which read those states anyway; only the last state is summed here
-        if (!backward || t == nsteps - 1) {
+        *v.cur = to;
+        *v.steps += nsteps;
+        v.kp->sr_seed = v.sr_seed(step0 + nsteps - 1);  // as n calls of lbm_step leave it
+        // <W, A_t> of t = 1 .. n-1 is summed by the transposed steps, which read those states anyway
+        kq.src = src;
+        kq.ref_src = src_ref;
+        ACK(v.L->objective(kq, objective, inv_nfluid, L.acc, st), "objective kernel");
+    } else {
+        for (int64_t t = 0; t < nsteps; ++t) {
+            lbm_status s = v.run_steps(ctx, 1);
+            if (s != LBM_OK) {
+                msg = "forward step failed";
+                return s;
+            }
             kq.src = v.pops[*v.cur];
             kq.ref_src = v.refp[*v.cur];
             ACK(v.L->objective(kq, objective, inv_nfluid, L.acc, st), "objective kernel");
@@ -231,11 +278,22 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
     aa.inv_nfluid = inv_nfluid;
     aa.inv_nfluid_f = float(inv_nfluid);
     aa.part = L.part;
-    aa.dS = L.dS;
-    aa.dpsi = L.dpsi;
-    aa.rho = L.rho;
-    int gi = 0;  // buffer holding (g, c) of the step after; none before the first reversal
+    aa.c_out = L.c;
+    int gi = 0;  // set of planes the last transposed step left; none before the first
     bool have_next = false;
+    auto bind_in = [&]() {
+        aa.g_in = L.g[gi], aa.dS_in = L.dS[gi], aa.dpsi_in = L.dpsi[gi], aa.rho_in = L.rho[gi], aa.psi_in = L.psi_r[gi];
+    };
+    // psi, the 16-bit reference plane and the stored state A_t of segment s, buffer set q
+    auto state_at = [&](int64_t s, int q, int64_t t, const float **ref) -> const void * {
+        if (t == 0) {
+            *ref = first_ref;
+            return first;
+        }
+        const void *p = t == s * K ? L.ckpt[s] : L.seg[q][t - s * K - 1];
+        *ref = ref_of(p);
+        return p;
+    };
     // Segment s is recomputed on the side stream into buffer set s & 1 while the transposed
     // steps of segment s + 1 run on the context stream from set (s + 1) & 1; events order a
     // set's reuse after the transposed steps that read it.
@@ -243,24 +301,16 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
         const int q = (int)(s & 1);
         const int64_t t0 = s * K, t1 = std::min<int64_t>((s + 1) * K, nsteps);
         if (s + 2 < nseg) ACK(cudaStreamWaitEvent(as->side, as->reversed[q], 0), "event wait");
-        KParams kp = *v.kp;
         for (int64_t t = t0; t < t1; ++t) {
-            kp.src = t == t0 ? L.ckpt[s] : L.seg[q][t - t0 - 1];
-            kp.ref_src = ref_of(kp.src);
-            kp.psi = L.psi[q][t - t0];
+            const float *ref;
+            const void *src = state_at(s, q, t, &ref);
             if (t + 1 < t1) {
-                kp.dst = L.seg[q][t - t0];
-                kp.ref_dst = ref_of(kp.dst);
-                kp.sr_seed = v.sr_seed(step0 + t);
-                if (v.fused_pass) {
-                    kp.psi_out = kp.psi;
-                    ACK(v.fused_pass(kp, as->side), "one-pass step kernel");
-                    kp.psi_out = nullptr;
-                } else {
-                    ACK(v.psi_pass(kp, as->side), "psi kernel");
-                    ACK(v.collide_pass(kp, as->side), "collide kernel");
-                }
+                void *dst = L.seg[q][t - t0];
+                const lbm_status r = step_to(src, ref, dst, ref_of(dst), L.psi[q][t - t0], t, as->side);
+                if (r != LBM_OK) return r;
             } else {
+                KParams kp = *v.kp;
+                kp.src = src, kp.ref_src = ref, kp.psi = L.psi[q][t - t0];
                 ACK(v.psi_pass(kp, as->side), "psi kernel");
             }
         }
@@ -269,39 +319,35 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
     };
     ACK(cudaEventRecord(as->fork, st), "event record");
     ACK(cudaStreamWaitEvent(as->side, as->fork, 0), "event wait");
-    lbm_status rs = recompute(nseg - 1);
-    if (rs != LBM_OK) return rs;
+    lbm_status rs;
     for (int64_t s = nseg - 1; s >= 0; --s) {
         const int q = (int)(s & 1);
         const int64_t t0 = s * K, t1 = std::min<int64_t>((s + 1) * K, nsteps);
         if (s > 0 && (rs = recompute(s - 1)) != LBM_OK) return rs;
-        ACK(cudaStreamWaitEvent(st, as->recomputed[q], 0), "event wait");
+        if (s < nseg - 1) ACK(cudaStreamWaitEvent(st, as->recomputed[q], 0), "event wait");
         KParams kp = *v.kp;
         for (int64_t t = t1 - 1; t >= t0; --t) {
-            kp.src = t == t0 ? L.ckpt[s] : L.seg[q][t - t0 - 1];
-            kp.ref_src = ref_of(kp.src);
+            kp.src = state_at(s, q, t, &kp.ref_src);
             kp.psi = L.psi[q][t - t0];
-            aa.g_in = have_next ? L.g[gi] : nullptr;
-            aa.c_in = have_next ? L.c[gi] : nullptr;
-            aa.g_out = L.g[gi ^ 1];
-            aa.c_out = L.c[gi ^ 1];
+            if (have_next) bind_in();
+            const int go = gi ^ 1;
+            aa.g_out = L.g[go], aa.dS_out = L.dS[go], aa.dpsi_out = L.dpsi[go], aa.rho_out = L.rho[go], aa.psi_out = L.psi_r[go];
             aa.sum_J = t >= 1;  // <W, A_0> is not part of J
-            ACK(v.L->adj_pass1(kp, aa, st), "adjoint pass 1");
-            ACK(v.L->adj_pass2(kp, aa, st), "adjoint pass 2");
-            gi ^= 1;
+            ACK(v.L->adj_step(kp, aa, st), "transposed step");
+            gi = go;
             have_next = true;
         }
         ACK(cudaEventRecord(as->reversed[q], st), "event record");
     }
 
+    bind_in();
+    aa.tail = 1;
+    ACK(v.L->adj_step(*v.kp, aa, st), "transposed step's tail");
     if (lambda0) {
         const size_t n = (size_t)p.nx * p.ny;
         double *dl = nullptr;
         ACK(cudaMalloc((void **)&dl, 9 * n * sizeof(double)), "cudaMalloc(lambda0)");
-        aa.g_in = L.g[gi];
-        aa.c_in = L.c[gi];
-        KParams kp = *v.kp;
-        cudaError_t e = v.L->adj_lambda(kp, aa, dl, st);
+        cudaError_t e = v.L->adj_lambda(*v.kp, L.g[gi], L.c, dl, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(lambda0, dl, 9 * n * sizeof(double), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         cudaFree(dl);

@@ -86,6 +86,7 @@ struct KParams {
     // [ny*nx] per node: bit i (1..8) set when the source x - e_i is a wall, bit 0 when the node is
     // solid; null without solid nodes, link fractions and wall velocities.  Read by the tile kernel.
     const uint16_t *links;
+    int64_t pull[9];       // bytes from a node to population i of the row it is pulled from, (i plane - e_iy pitch)
     int *err;              // device error word (0 = fine)
     Consts<double> cd;     // constants for FP64 arithmetic
     Consts<float> cf;      // constants for FP32 arithmetic
@@ -93,26 +94,28 @@ struct KParams {
     unsigned short inv_scale_bits;  // 2^-k in the storage type (FP16 or BF16 bits)
 };
 
-// Per-block partial sums of the transposed passes: slots of one row (8 doubles).  Pass 1:
-// dJ/dFx, dJ/dFy, dJ/dG (explicit and wall psi), dJ/dT (wall psi), <W, A_t>; pass 2:
-// dJ/dG and dJ/dT through psi(rho).
+// Per-block partial sums of the transposed steps: slots of one row (8 doubles).  dJ/dFx, dJ/dFy,
+// dJ/dG (explicit and wall psi), dJ/dT (wall psi), <W, A_t>, and dJ/dG and dJ/dT through psi(rho).
 constexpr int kAdjSlots = 8;
 enum AdjSlot { SLOT_FX = 0, SLOT_FY = 1, SLOT_G1 = 2, SLOT_T1 = 3, SLOT_J = 4, SLOT_G2 = 5, SLOT_T2 = 6 };
 
-// Buffers and scalars of one transposed step.  Planes use the population row pitch.
+// Buffers and scalars of one transposed step.  Planes use the population row pitch.  The _in planes
+// are what the step after left (g, dJ/dS, the local part of dJ/dpsi, rho of its pulled populations
+// and, in FP64, its psi); c, which completes lambda, is formed from them.
 struct AdjArgs {
-    const void *g_in;   // [9] planes, g of the step after (null: lambda_{t+1} = W_{t+1} only)
-    const void *c_in;   // plane, c of the step after (null with g_in)
-    void *g_out;        // [9] planes
-    void *c_out;        // plane
-    void *dS;           // [2] planes, dJ/dS
-    void *dpsi;         // plane, local part of dJ/dpsi
-    void *rho;          // plane, rho of the pulled populations of A_t
+    const void *g_in;   // [9] planes (null: lambda_{t+1} = W_{t+1} only)
+    const void *dS_in;  // [2] planes
+    const void *dpsi_in, *rho_in, *psi_in;
+    void *g_out, *dS_out, *dpsi_out, *rho_out, *psi_out;
+    void *c_out;        // plane: c of the _in planes, written by the tail launch
+    int tail;           // 1: form c and its parameter sums, no further step
+    int ahead;          // rows between a tile and the one whose lines it prefetches into L2; 0: none
+    int64_t push[9];    // bytes from a node to plane i of the row ahead, (i plane + e_iy pitch)
     double w_scale;     // weight of W in lambda_{t+1} (1/n for J = (1/n) sum_t <W, A_t>)
     int objective;      // 0: y momentum handed to the walls by the next streaming; 1: mean j_x
     double inv_nfluid;  // 1 / number of fluid nodes (objective 1)
     double *part;       // per-block FP64 partial sums [blocks][kAdjSlots]
-    int sum_J;          // pass 1 also sums <W, A_t> of its state
+    int sum_J;          // also sum <W, A_t> of the state
     float w_scale_f, inv_nfluid_f;  // the two scales rounded to FP32 on the host (FP32 arithmetic
                                     // converts no FP64 value per node)
 };
@@ -148,9 +151,8 @@ struct Launchers {
     cudaError_t (*get_state)(const KParams &, double *out, cudaStream_t);
     cudaError_t (*set_state)(const KParams &, const double *in, cudaStream_t);
     // transposed step (FP64 arithmetic for FP64 storage, FP32 otherwise); AdjArgs in k_adjoint.cuh
-    cudaError_t (*adj_pass1)(const KParams &, const AdjArgs &, cudaStream_t);
-    cudaError_t (*adj_pass2)(const KParams &, const AdjArgs &, cudaStream_t);
-    cudaError_t (*adj_lambda)(const KParams &, const AdjArgs &, double *out, cudaStream_t);
+    cudaError_t (*adj_step)(const KParams &, const AdjArgs &, cudaStream_t);
+    cudaError_t (*adj_lambda)(const KParams &, const void *g, const void *c, double *out, cudaStream_t);
     cudaError_t (*objective)(const KParams &, int objective, double inv_nfluid, double *acc, cudaStream_t);
     int64_t (*adj_blocks)(const KParams &);  // rows of the per-block partial-sum array (8 doubles each)
     cudaError_t (*adj_reduce)(const KParams &, const double *part, double *out8, cudaStream_t);
