@@ -15,6 +15,12 @@
 // A tile of n pairs (rows) has n warps for them; one more warp pulls the rows above and below the
 // tile and one the columns beside it (FP64: two and one), for psi only.  The tile's height is
 // chosen per launch (tile_height) so that the last wave of blocks is nearly full.
+//
+// What bounds it (FP32): small lattices the latency of one block's chain, mid-size ones instruction
+// issue (578 a pair of rows and 32 columns, ring included; the two-pass kernels 1840), from 2048^2 on HBM:
+// 4096^2 193 us, 94 % of the measured copy rate at 72 B a node. Four pairs and five blocks per SM (64
+// registers) against two blocks of eight pairs: 512 x 4096 46 -> 36 us; the L2 prefetch 70 -> 59 at 2048^2;
+// the instantiation without edge tests (INNER) 59 -> 52, FP16 81 -> 67.
 #pragma once
 
 #include "lbm_device.cuh"
@@ -94,15 +100,27 @@ static __global__ void __launch_bounds__(128) k_link_bits(KParams kp, uint16_t *
     out[nb.n(0)] = (uint16_t)w;
 }
 
+// A stored population as FP32: converted and multiplied in one mixed-precision instruction (exact
+// product, one rounding of the sum: Codec's value).
 template <class S> struct Raw;
 template <> struct Raw<float> {
-    static __device__ __forceinline__ float f(float v, float, float) { return v; }
+    static __device__ __forceinline__ float f(float v, float, const KParams &) { return v; }
 };
 template <> struct Raw<__half> {
-    static __device__ __forceinline__ float f(__half v, float wref, float inv) { return __fmaf_rn(__half2float(v), inv, wref); }
+    static __device__ __forceinline__ float f(__half v, float wref, const KParams &kp)
+    {
+        float x;
+        asm("fma.rn.f32.f16 %0, %1, %2, %3;" : "=f"(x) : "h"(__half_as_ushort(v)), "h"(kp.inv_scale_bits), "f"(wref));
+        return x;
+    }
 };
 template <> struct Raw<__nv_bfloat16> {
-    static __device__ __forceinline__ float f(__nv_bfloat16 v, float wref, float inv) { return __fmaf_rn(__bfloat162float(v), inv, wref); }
+    static __device__ __forceinline__ float f(__nv_bfloat16 v, float wref, const KParams &kp)
+    {
+        float x;
+        asm("fma.rn.f32.bf16 %0, %1, %2, %3;" : "=f"(x) : "h"(__bfloat16_as_ushort(v)), "h"(kp.inv_scale_bits), "f"(wref));
+        return x;
+    }
 };
 
 // Offsets (elements; a plane of a lattice of 2^31 nodes still fits 32 bits) of the 3 x 3 neighbourhood
@@ -124,22 +142,13 @@ __device__ __forceinline__ Nine nine_of(const KParams &kp, const Site &s, unsign
     inside = a.inside;
     return n;
 }
-// Element at a byte offset of 32 bits from a base that is the same for all threads.
-template <class T>
-__device__ __forceinline__ T &at_bytes(T *base, uint32_t bytes)
-{
-    typedef typename std::conditional<std::is_const<T>::value, const char, char>::type B;
-    return *reinterpret_cast<T *>(reinterpret_cast<B *>(base) + bytes);
-}
-
-// GEOM: 0 no solid nodes; 1 solid nodes with half-way links; 2 also interpolated or moving walls.
-template <class S, int GEOM, class O>
-__global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, int ahead)
+// One block of a step.  GEOM: 0 no solid nodes; 1 solid nodes with half-way links; 2 also interpolated
+// or moving walls.  INNER: the tile lies inside the lattice and no node of it or its ring pulls across
+// an edge, so every address is the node's own plus a constant of the launch (KParams::pull).
+template <class S, int GEOM, class O, bool INNER>
+__device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float (&sm)[2 * kTilePairs + 2][kTilePitch])
 {
     constexpr bool DEV = IsDev<S>::value;
-    __shared__ float sm[2 * kTilePairs + 2][kTilePitch];
-    grid_dependency_wait();
-    allow_dependent_launch();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int np = (blockDim.x >> 5) - 2, rows = 2 * np;  // pairs and rows of this launch's tiles
     const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * rows;
@@ -157,109 +166,113 @@ __global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, 
         ax = x0 - 1, bx = x0 + kTileX, ay = by = y0 + r - 1;
         ra = rb = r, ca = 0, cb = kTileX + 1;
     }
-    // no node of the tile or its ring pulls across an edge of the lattice
-    const bool inner = x0 >= 2 && x0 + kTileX + 2 <= kp.nx && y0 >= 2 && y0 + rows + 2 <= kp.ny;
-    Site a{ax, ay, true}, b{bx, by, true};
-    if (!inner) a = site_of(kp, ax, ay), b = site_of(kp, bx, by);
-    const uint32_t node_a = (uint32_t)a.y * (uint32_t)kp.nx + a.x, node_b = (uint32_t)b.y * (uint32_t)kp.nx + b.x;
-    const uint32_t ka = (uint32_t)a.y * (uint32_t)kp.pitch + a.x, kb = (uint32_t)b.y * (uint32_t)kp.pitch + b.x;
-    // the same from the first row of the tile (y0 - 1 counts from -1), small at any lattice size
-    const uint32_t ta = (uint32_t)(ay - y0 + 1) * (uint32_t)kp.pitch + ax, tb = (uint32_t)(by - y0 + 1) * (uint32_t)kp.pitch + bx;
-    const int64_t row0 = (int64_t)(y0 - 1) * kp.pitch;
-    unsigned wa = 0, wb = 0;  // wall bits
-    if (GEOM) wa = kp.links[node_a], wb = kp.links[node_b];
-
     if (ahead > 0 && warp < np && lane < 18) {
-        // the lines of the tile that a block of the next wave will pull
+        // the lines of the tile that a block of the next wave will pull (row y, columns x0 .. x0 + 31)
         const int i = lane < 9 ? lane : lane - 9, y = ay + (lane < 9 ? 0 : 1) + ahead;
-        if (y < kp.ny) {  // columns x0 .. x0 + 31 of row y: x0 < nx, so the address is inside the plane
+        if (y < kp.ny) {
             const S *p = static_cast<const S *>(kp.src) + (i * kp.plane + (int64_t)y * kp.pitch + x0);
             asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
         }
     }
+    Site a{ax, ay, true}, b{bx, by, true};
+    if constexpr (!INNER) a = site_of(kp, ax, ay), b = site_of(kp, bx, by);
+    const uint32_t node_a = (uint32_t)a.y * (uint32_t)kp.nx + a.x, node_b = (uint32_t)b.y * (uint32_t)kp.nx + b.x;
+    const uint32_t ka = (uint32_t)a.y * (uint32_t)kp.pitch + a.x, kb = (uint32_t)b.y * (uint32_t)kp.pitch + b.x;
+    unsigned wa = 0, wb = 0;  // wall bits
+    if (GEOM) wa = kp.links[node_a], wb = kp.links[node_b];
 
     // pull, Eq. (lbe.str)
+    const S *src = static_cast<const S *>(kp.src);
     v2x f[9];
-    {
-        const S *src = static_cast<const S *>(kp.src);
-        S va[9], vb[9];
-        float refa[9], refb[9];
-        if (inner) {
-            // every source is the node's own offset plus a constant of the launch
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const int64_t shift = row0 - (int64_t)ey_(i) * kp.pitch - ex_(i);
-                const S *p = src + (i * kp.plane + shift);
-                va[i] = at_bytes(p, ta * (uint32_t)sizeof(S)), vb[i] = at_bytes(p, tb * (uint32_t)sizeof(S));
-                if (has_ref) refa[i] = at_bytes(kp.ref_src + shift, ta * 4u), refb[i] = at_bytes(kp.ref_src + shift, tb * 4u);
-            }
-        } else {
-            unsigned ia, ib;
-            const Nine na = nine_of(kp, a, ia), nb = nine_of(kp, b, ib);
-            if (GEOM == 0) wa = edge_walls(ia), wb = edge_walls(ib);
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const S *p = src + i * kp.plane;
-                va[i] = p[na.from(i)], vb[i] = p[nb.from(i)];
-                if (has_ref) refa[i] = kp.ref_src[na.from(i)], refb[i] = kp.ref_src[nb.from(i)];
-            }
-        }
+    S va[9], vb[9];
+    float refa[9], refb[9];
+    if constexpr (INNER) {
+        const char *pa = reinterpret_cast<const char *>(src + ka), *pb = reinterpret_cast<const char *>(src + kb);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            float wra = 0.f, wrb = 0.f;
-            if (DEV) {
-                wra = __fmul_rn(w_<float>(i), has_ref ? refa[i] : kp.cf.rho_ref);
-                wrb = __fmul_rn(w_<float>(i), has_ref ? refb[i] : kp.cf.rho_ref);
-            }
-            f[i] = X2(Raw<S>::f(va[i], wra, kp.cf.inv_scale), Raw<S>::f(vb[i], wrb, kp.cf.inv_scale));
+            va[i] = reinterpret_cast<const S *>(pa + kp.pull[i])[-ex_(i)];
+            vb[i] = reinterpret_cast<const S *>(pb + kp.pull[i])[-ex_(i)];
         }
-        if ((wa | wb) & 0x1feu) {
-            // wall links: the population that left the node toward the wall comes back
+        if (has_ref) {
+            const float *qa = kp.ref_src + ka, *qb = kp.ref_src + kb;
+            const int64_t P = kp.pitch;
+            if (warp < np) {  // rows y and y + 1: twelve references for both nodes
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const unsigned w = e ? wb : wa;
-                if (!(w & 0x1feu) || (w & 1u)) continue;
-                const uint32_t k = e ? kb : ka;
-                auto own = [&](int i) -> float {
-                    float wr = 0.f;
-                    if (DEV) wr = __fmul_rn(w_<float>(i), has_ref ? (e ? refb[0] : refa[0]) : kp.cf.rho_ref);
-                    return Raw<S>::f((src + i * kp.plane)[k], wr, kp.cf.inv_scale);
-                };
-                float rho_w = 0.f;
-                bool summed = false;
-#pragma unroll
-                for (int i = 1; i < 9; ++i) {
-                    if (!((w >> i) & 1u)) continue;
-                    const int o = opp_(i);
-                    const float fo = own(o);
-                    float g = fo + 0.f;
-                    if constexpr (GEOM == 2) {
-                        // interpolated or moving wall: link fraction and moving-wall coefficient
-                        const float2 lk = kp.link[(int64_t)(i - 1) * kp.plane + k];
-                        float mw = 0.f;
-                        if (lk.y != 0.f) {
-                            if (!summed) {
-#pragma unroll
-                                for (int n = 0; n < 9; ++n) rho_w += own(n);
-                                summed = true;
-                            }
-                            mw = lk.y * rho_w;
-                        }
-                        const float q = lk.x;
-                        if (q < 0.5f) {
-                            // fbar_o of the second node x + e_i (fluid: the record's q is 1/2 otherwise),
-                            // which is what the pull of population o brought here
-                            const float f2 = e ? f[o].v.y : f[o].v.x;
-                            g = 2.f * q * fo + (1.f - 2.f * q) * f2 + mw;
-                        } else if (q == 0.5f) {
-                            g = fo + mw;
-                        } else {
-                            g = fo / (2.f * q) + (2.f * q - 1.f) / (2.f * q) * own(i) + mw / (2.f * q);
-                        }
-                    }
-                    if (e) f[i].v.y = g;
-                    else f[i].v.x = g;
+                for (int d = -1; d <= 1; ++d) {
+                    const int up = d < 0 ? 5 : d > 0 ? 6 : 2, in = d < 0 ? 1 : d > 0 ? 3 : 0, dn = d < 0 ? 8 : d > 0 ? 7 : 4;
+                    refa[up] = (qa - P)[d];
+                    refa[in] = refb[up] = qa[d];
+                    refa[dn] = refb[in] = qb[d];
+                    refb[dn] = (qb + P)[d];
                 }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) refa[i] = (qa - ey_(i) * P)[-ex_(i)], refb[i] = (qb - ey_(i) * P)[-ex_(i)];
+            }
+        }
+    } else {
+        unsigned ia, ib;
+        const Nine na = nine_of(kp, a, ia), nb = nine_of(kp, b, ib);
+        if (GEOM == 0) wa = edge_walls(ia), wb = edge_walls(ib);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const S *p = src + i * kp.plane;
+            va[i] = p[na.from(i)], vb[i] = p[nb.from(i)];
+            if (has_ref) refa[i] = kp.ref_src[na.from(i)], refb[i] = kp.ref_src[nb.from(i)];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        v2x wr = X2(0.f, 0.f);
+        if (DEV) wr = has_ref ? v2x{kp.c2.w[i]} * X2(refa[i], refb[i]) : v2x{kp.c2.dec[i]};
+        f[i] = X2(Raw<S>::f(va[i], wr.v.x, kp), Raw<S>::f(vb[i], wr.v.y, kp));
+    }
+    if ((!INNER || GEOM) && ((wa | wb) & 0x1feu)) {
+        // wall links: the population that left the node toward the wall comes back
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const unsigned w = e ? wb : wa;
+            if (!(w & 0x1feu) || (w & 1u)) continue;
+            const uint32_t k = e ? kb : ka;
+            auto own = [&](int i) -> float {
+                float wr = 0.f;
+                if (DEV) wr = __fmul_rn(w_<float>(i), has_ref ? (e ? refb[0] : refa[0]) : kp.cf.rho_ref);
+                return Raw<S>::f((src + i * kp.plane)[k], wr, kp);
+            };
+            float rho_w = 0.f;
+            bool summed = false;
+#pragma unroll
+            for (int i = 1; i < 9; ++i) {
+                if (!((w >> i) & 1u)) continue;
+                const int o = opp_(i);
+                const float fo = own(o);
+                float g = fo + 0.f;
+                if constexpr (GEOM == 2) {
+                    // interpolated or moving wall: link fraction and moving-wall coefficient
+                    const float2 lk = kp.link[(int64_t)(i - 1) * kp.plane + k];
+                    float mw = 0.f;
+                    if (lk.y != 0.f) {
+                        if (!summed) {
+#pragma unroll
+                            for (int n = 0; n < 9; ++n) rho_w += own(n);
+                            summed = true;
+                        }
+                        mw = lk.y * rho_w;
+                    }
+                    const float q = lk.x;
+                    if (q < 0.5f) {
+                        // fbar_o of the second node x + e_i (fluid: the record's q is 1/2 otherwise), which
+                        // is what the pull of population o brought here
+                        const float f2 = e ? f[o].v.y : f[o].v.x;
+                        g = 2.f * q * fo + (1.f - 2.f * q) * f2 + mw;
+                    } else if (q == 0.5f) {
+                        g = fo + mw;
+                    } else {
+                        g = fo / (2.f * q) + (2.f * q - 1.f) / (2.f * q) * own(i) + mw / (2.f * q);
+                    }
+                }
+                if (e) f[i].v.y = g;
+                else f[i].v.x = g;
             }
         }
     }
@@ -271,13 +284,13 @@ __global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, 
         if (wa & 1u) psi.v.x = kp.wall_psi ? float(kp.wall_psi[node_a]) : kp.cf.psi_s, rho.v.x = 1.f;
         if (wb & 1u) psi.v.y = kp.wall_psi ? float(kp.wall_psi[node_b]) : kp.cf.psi_s, rho.v.y = 1.f;
     }
-    if (!a.in) psi.v.x = kp.cf.psi_s;
-    if (!b.in) psi.v.y = kp.cf.psi_s;
+    if (!INNER && !a.in) psi.v.x = kp.cf.psi_s;
+    if (!INNER && !b.in) psi.v.y = kp.cf.psi_s;
     sm[ra][ca] = psi.v.x;
     sm[rb][cb] = psi.v.y;
     __syncthreads();
     if (warp >= np) return;
-    const bool la = ax < kp.nx && ay < kp.ny, lb = ax < kp.nx && by < kp.ny;
+    const bool la = INNER || (ax < kp.nx && ay < kp.ny), lb = INNER || (ax < kp.nx && by < kp.ny);
     if (!la) return;
     if (kp.psi_out != nullptr) {
         float *out = static_cast<float *>(kp.psi_out);
@@ -313,13 +326,12 @@ __global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, 
     collide_v<v2x, O>(kp, d, rho, psi, Sx, Sy, Fex, Fey, fb, ux, uy);
 
     // encode and store
-    S *dst = static_cast<S *>(kp.dst);
+    S *da = static_cast<S *>(kp.dst) + ka, *db = static_cast<S *>(kp.dst) + kb;
     if constexpr (!DEV) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            S *p = dst + (i * kp.plane + row0);
-            if (sa) at_bytes(p, ta * 4u) = fb[i].v.x;
-            if (sb) at_bytes(p, tb * 4u) = fb[i].v.y;
+        for (int i = 0; i < 9; ++i, da += kp.plane, db += kp.plane) {
+            if (sa) *da = fb[i].v.x;
+            if (sb) *db = fb[i].v.y;
         }
     } else {
         if (has_ref) {
@@ -331,9 +343,8 @@ __global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, 
         // both columns are the same, so one conversion rounds the two rows
         const unsigned pick = (ka & 1u) ? 0x7632u : 0x5410u;
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const float w = w_<float>(i);
-            const v2x wr = has_ref ? X2(__fmul_rn(w, rho.v.x), __fmul_rn(w, rho.v.y)) : v2x{kp.c2.dec[i]};
+        for (int i = 0; i < 9; ++i, da += kp.plane, db += kp.plane) {
+            const v2x wr = has_ref ? v2x{kp.c2.w[i]} * rho : v2x{kp.c2.dec[i]};
             const v2x s = (fb[i] - wr) * v2x{kp.c2.scale};
             uint32_t h;
             if (kp.sr) {
@@ -343,11 +354,21 @@ __global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, 
                 h = (uint32_t)*reinterpret_cast<const unsigned short *>(&lo) |
                     (uint32_t)*reinterpret_cast<const unsigned short *>(&hi) << 16;
             }
-            S *p = dst + (i * kp.plane + row0);
-            if (sa) at_bytes(p, ta * 2u) = SRound<S>::from_bits((unsigned short)(h & 0xffffu));
-            if (sb) at_bytes(p, tb * 2u) = SRound<S>::from_bits((unsigned short)(h >> 16));
+            if (sa) *da = SRound<S>::from_bits((unsigned short)(h & 0xffffu));
+            if (sb) *db = SRound<S>::from_bits((unsigned short)(h >> 16));
         }
     }
+}
+
+template <class S, int GEOM, class O>
+__global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, int ahead)
+{
+    __shared__ float sm[2 * kTilePairs + 2][kTilePitch];
+    grid_dependency_wait();
+    allow_dependent_launch();
+    const int rows = 2 * ((blockDim.x >> 5) - 2), x0 = blockIdx.x * kTileX, y0 = blockIdx.y * rows;
+    if (x0 >= 2 && x0 + kTileX + 2 <= kp.nx && y0 >= 2 && y0 + rows + 2 <= kp.ny) tile2_block<S, GEOM, O, true>(kp, ahead, sm);
+    else tile2_block<S, GEOM, O, false>(kp, ahead, sm);
 }
 
 // FP64: one node per thread.  Warps 0 .. n-1 own the tile's rows, two more the rows above and below
@@ -436,9 +457,11 @@ struct Tile {
             // two population buffers exceed the 129 MB L2 (below that the lines are in L2 anyway)
             const int sms = kp.sm_count > 0 ? kp.sm_count : 148;
             const int ahead = 2.0 * 9.0 * kp.plane * sizeof(S) > 120e6 ? (int)(3u * sms / grid.x + 1) * 2 * h : 0;
-            if (kp.q || kp.wall_u) return launch_dependent(k_tile2<S, 2, RuntimeOpts>, grid, block, 0, st, kp, ahead);
-            if (kp.solid) return launch_dependent(k_tile2<S, 1, RuntimeOpts>, grid, block, 0, st, kp, ahead);
-            return launch_dependent(k_tile2<S, 0, RuntimeOpts>, grid, block, 0, st, kp, ahead);
+            KParams kq = kp;
+            for (int i = 0; i < 9; ++i) kq.pull[i] = (i * kp.plane - ey_(i) * kp.pitch) * (int64_t)sizeof(S);
+            if (kp.q || kp.wall_u) return launch_dependent(k_tile2<S, 2, RuntimeOpts>, grid, block, 0, st, kq, ahead);
+            if (kp.solid) return launch_dependent(k_tile2<S, 1, RuntimeOpts>, grid, block, 0, st, kq, ahead);
+            return launch_dependent(k_tile2<S, 0, RuntimeOpts>, grid, block, 0, st, kq, ahead);
         }
     }
 };

@@ -288,12 +288,13 @@ static bool auto_prefers_fused(const lbm_ctx *c)
 
 // Which kernel steps the context: the two-pass kernels on request (LBM_KERNEL_TWO_PASS); else a
 // one-pass kernel, the staged one (k_fused2) or the tile kernel (k_tile), which gives the two-pass
-// step's results.  The staged kernel keeps HBM busy where the two population buffers are far
-// larger than L2, but a CTA walks its rows in series, and it has no walls; the tile kernel has
-// thousands of short blocks.  Step times on a GB300 (us, tile / staged): periodic 512^2 5.8 / 10.3, 1024^2
-// 16.1 / 22.9, 1600^2 40 / 46.6, 2048^2 59 / 56.7, 4096^2 223 / 195; FP16 1024^2 21.5 / 26.9, 1024 x
-// 2048 42 / 43, 1600^2 51 / 45, 2048^2 81 / 59.  (Two-pass kernels: 512^2 10.3, 1024^2 31, 2048^2 121; 256
-// x 2048 with walls 20.6 against the tile kernel's 9.8; banded 512^2 17.6 / 6.1; annulus 1024^2 44 / 20.)
+// step's results.  The staged kernel reads each row once where the tile kernel re-reads its tiles'
+// rings from L2, but a CTA walks its rows in series, and it has no walls; the tile kernel has thousands
+// of short blocks.  Step times on a GB300 (us, tile / staged): FP32 periodic 512^2 5.4 / 10.3, 1024^2
+// 14.4 / 22.9, 2048^2 52 / 56.7, 4096^2 193 / 195, 8192^2 788 / 745; FP16, whose ring costs instructions
+// and not bytes, 1024^2 18.5 / 26.9, 1024 x 2048 35 / 43, 2048^2 67 / 59, 4096^2 249 / 194.  (Two-pass
+// kernels, FP32: 512^2 10.3, 1024^2 31, 2048^2 121; 256 x 2048 with walls 20.6 against the tile kernel's
+// 9.2; banded 512^2 17.6 / 5.9; annulus 1024^2 44 / 20.)
 static void choose_kernel(lbm_ctx *c)
 {
     const int want = c->p.kernel;
@@ -301,10 +302,9 @@ static void choose_kernel(lbm_ctx *c)
     c->fused_ok = (want != LBM_KERNEL_TWO_PASS) && possible &&
                   (want == LBM_KERNEL_FUSED || c->p.precision == LBM_F64 || auto_prefers_fused(c));
     const bool staged = possible && c->L.fused_pass && c->p.periodic_x && c->p.periodic_y && !c->solid && !c->q && !c->wall_u;
-    // 32-bit byte offsets within the rows of a tile
-    const bool tile = c->p.precision == LBM_F64 || c->pitch <= (int64_t)1 << 26;
+    const bool tile = c->L.tile_pass != nullptr;
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
-    const bool large = n >= (c->p.precision == LBM_F32 ? (int64_t)1 << 22 : (int64_t)9 << 18);
+    const bool large = n >= (c->p.precision == LBM_F32 ? (int64_t)1 << 25 : (int64_t)3 << 20);
     c->one_pass = nullptr;
     if (want == LBM_KERNEL_TWO_PASS || (want == LBM_KERNEL_FUSED && !possible)) return;
     if (staged && (want == LBM_KERNEL_FUSED || large || !tile)) c->one_pass = c->L.fused_pass;
