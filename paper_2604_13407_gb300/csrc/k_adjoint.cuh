@@ -110,49 +110,6 @@ __device__ __forceinline__ void p_eos_derivs(const KParams &kp, T rho, T &p_rho,
     p_T = KR * rho * g;
 }
 
-// Per-block FP64 partial sums of the transposed steps (slots AdjSlot, lbm_internal.h): one row of
-// kAdjSlots doubles per block, accumulated over all steps of a call and reduced once at its end, so
-// no atomic is contended and the summation order is fixed.
-
-// Warp sum of one value per lane as a compensated FP32 pair (hi, lo) in lane 0: Knuth's TwoSum at
-// every shuffle level, about 2^-48 relative.
-__device__ __forceinline__ void two_sum(float &hi, float &lo, float x, float xlo)
-{
-    const float sum = hi + x, z = sum - hi;
-    lo += xlo + ((hi - (sum - z)) + (x - z));
-    hi = sum;
-}
-__device__ __forceinline__ void warp_sum_pair(float &hi, float &lo)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        two_sum(hi, lo, __shfl_down_sync(0xffffffffu, hi, o), __shfl_down_sync(0xffffffffu, lo, o));
-}
-
-// Sums of the `n` quantities v[k][0 .. count) in shared memory (all threads past a barrier) but those in `skip` (known to be zero), added to this block's slots: a warp sums one quantity at a
-// time, each lane its share of them and then the lanes, compensated in FP32 arithmetic (FP64
-// work stays out of it: GB300's FP64 pipe is narrow).
-template <class R>
-__device__ __forceinline__ void block_add(const R *v, int pitch, int n, int count, unsigned skip, double *part)
-{
-    const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
-    for (int k = threadIdx.x >> 5; k < n; k += warps) {
-        if ((skip >> k) & 1u) continue;
-        double t;
-        if constexpr (sizeof(R) == 8) {
-            double s = 0.0;
-            for (int q = lane; q < count; q += 32) s += v[k * pitch + q];
-            t = warp_sum(s);
-        } else {
-            float hi = 0.f, lo = 0.f;
-            for (int q = lane; q < count; q += 32) two_sum(hi, lo, v[k * pitch + q], 0.f);
-            warp_sum_pair(hi, lo);
-            t = double(hi) + double(lo);
-        }
-        if (lane == 0) part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kAdjSlots + k] += t;
-    }
-}
-
 // Block sum of one double added to *acc with one FP64 atomic per block.
 __device__ __forceinline__ void block_atomic_add(double v, double *acc)
 {
@@ -567,7 +524,8 @@ __device__ __forceinline__ void adj_block(const KParams &kp, const AdjArgs &aa, 
             if constexpr (sizeof(R) == 8) static_cast<R *>(aa.psi_out)[k] = Z::get(psi, e);
         }
     }
-    // ---- parameter sums, in the order of AdjSlot
+    // ---- parameter sums, in the order of AdjSlot: one row of FP64 partial sums per block, accumulated over
+    // all steps of a call and reduced once at its end (no contended atomics, a fixed order)
     {
         const T v[7] = {gFx, gFy, gG, gT, Jt, gG2, gT2};
 #pragma unroll
@@ -578,7 +536,8 @@ __device__ __forceinline__ void adj_block(const KParams &kp, const AdjArgs &aa, 
     __syncthreads();
     // away from walls the wall terms (and objective 0, the force on them) are zero
     const unsigned skip = walled ? 0u : (1u << SLOT_T1) | (aa.objective == 0 ? 1u << SLOT_J : 0u);
-    block_add<R>(&red[0][0], N * 32 * UNITS, 7, N * 32 * UNITS, skip, aa.part);
+    block_add<R>(&red[0][0], N * 32 * UNITS, 7, N * 32 * UNITS, UNITS, skip,
+                 [&](int q, double t) { aa.part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kAdjSlots + q] += t; });
 }
 
 // One transposed step at A_t (kp.src) with the psi field of A_t (kp.psi).  U: units of a block, B: blocks

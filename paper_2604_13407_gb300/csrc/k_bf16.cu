@@ -24,8 +24,9 @@ Launchers launchers_bf16()
     L.tile_pass = &Tile<__nv_bfloat16>::step;
     L.link_bits = &Tile<__nv_bfloat16>::link_bits;
     L.init = &TwoPass<__nv_bfloat16>::init;
-    L.moments = &TwoPass<__nv_bfloat16>::moments;
-    L.diag = &TwoPass<__nv_bfloat16>::diag;
+    L.moments = &Tile<__nv_bfloat16>::moments;
+    L.diag = &Tile<__nv_bfloat16>::diag;
+    L.diag_rows = &Tile<__nv_bfloat16>::diag_rows;
     L.get_state = &TwoPass<__nv_bfloat16>::get_state;
     L.set_state = &TwoPass<__nv_bfloat16>::set_state;
     L.adj_step = &Adjoint<__nv_bfloat16>::step;

@@ -24,8 +24,9 @@ Launchers launchers_f16()
     L.tile_pass = &Tile<__half>::step;
     L.link_bits = &Tile<__half>::link_bits;
     L.init = &TwoPass<__half>::init;
-    L.moments = &TwoPass<__half>::moments;
-    L.diag = &TwoPass<__half>::diag;
+    L.moments = &Tile<__half>::moments;
+    L.diag = &Tile<__half>::diag;
+    L.diag_rows = &Tile<__half>::diag_rows;
     L.get_state = &TwoPass<__half>::get_state;
     L.set_state = &TwoPass<__half>::set_state;
     L.adj_step = &Adjoint<__half>::step;

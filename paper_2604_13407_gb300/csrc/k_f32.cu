@@ -24,8 +24,9 @@ Launchers launchers_f32()
     L.tile_pass = &Tile<float>::step;
     L.link_bits = &Tile<float>::link_bits;
     L.init = &TwoPass<float>::init;
-    L.moments = &TwoPass<float>::moments;
-    L.diag = &TwoPass<float>::diag;
+    L.moments = &Tile<float>::moments;
+    L.diag = &Tile<float>::diag;
+    L.diag_rows = &Tile<float>::diag_rows;
     L.get_state = &TwoPass<float>::get_state;
     L.set_state = &TwoPass<float>::set_state;
     L.adj_step = &Adjoint<float>::step;

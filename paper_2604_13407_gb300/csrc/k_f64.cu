@@ -13,8 +13,9 @@ Launchers launchers_f64()
     L.tile_pass = &Tile<double>::step;
     L.link_bits = &Tile<double>::link_bits;
     L.init = &TwoPass<double>::init;
-    L.moments = &TwoPass<double>::moments;
-    L.diag = &TwoPass<double>::diag;
+    L.moments = &Tile<double>::moments;
+    L.diag = &Tile<double>::diag;
+    L.diag_rows = &Tile<double>::diag_rows;
     L.get_state = &TwoPass<double>::get_state;
     L.set_state = &TwoPass<double>::set_state;
     L.adj_step = &Adjoint<double>::step;

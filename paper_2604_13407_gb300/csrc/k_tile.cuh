@@ -21,6 +21,11 @@
 // 4096^2 193 us, 94 % of the measured copy rate at 72 B a node. Four pairs and five blocks per SM (64
 // registers) against two blocks of eight pairs: 512 x 4096 46 -> 36 us; the L2 prefetch 70 -> 59 at 2048^2;
 // the instantiation without edge tests (INNER) 59 -> 52, FP16 81 -> 67.
+//
+// lbm_get_moments and lbm_get_diagnostics run the same tiles (k_read2, k_read1): one launch where a psi
+// pass and a node pass read the populations twice (8192^2 moments 2.04 -> 0.71 ms, bound by its 60 B a
+// node), and block sums into rows that one reduction adds where every block put ten atomics on the
+// same addresses (256 x 2048 diagnostics 123 -> 23 us).
 #pragma once
 
 #include "lbm_device.cuh"
@@ -45,6 +50,54 @@ __device__ __forceinline__ v2x vsqrt(v2x a) { return X2(sqrt32(a.v.x), sqrt32(a.
 __device__ __forceinline__ v2x vclamp01(v2x a) { return X2(fminf(fmaxf(a.v.x, 0.f), 1.f), fminf(fmaxf(a.v.y, 0.f), 1.f)); }
 template <> __device__ __forceinline__ v2x ks<v2x>(float a) { return X2(a, a); }
 template <> __device__ __forceinline__ v2x kc<v2x>(const float2 &c) { return v2x{c}; }
+
+// ------------------------------------------------------------- block sums --------
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Warp sum of one value per lane as a compensated FP32 pair (hi, lo) in lane 0: Knuth's TwoSum at
+// every shuffle level, about 2^-48 relative.
+__device__ __forceinline__ void two_sum(float &hi, float &lo, float x, float xlo)
+{
+    const float sum = hi + x, z = sum - hi;
+    lo += xlo + ((hi - (sum - z)) + (x - z));
+    hi = sum;
+}
+__device__ __forceinline__ void warp_sum_pair(float &hi, float &lo)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        two_sum(hi, lo, __shfl_down_sync(0xffffffffu, hi, o), __shfl_down_sync(0xffffffffu, lo, o));
+}
+
+// Sums of the `n` quantities v[k][0 .. count) in shared memory (all threads past a barrier) but those
+// in `skip` (known to be zero), handed to put(k, sum) by one lane: a warp of `warps` sums one quantity at
+// a time, each lane its share and then the lanes, compensated in FP32 arithmetic (FP64 work stays out
+// of it: GB300's FP64 pipe is narrow).
+template <class R, class Put>
+__device__ __forceinline__ void block_add(const R *v, int pitch, int n, int count, int warps, unsigned skip, const Put &put)
+{
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < n; k += warps) {
+        if ((skip >> k) & 1u) continue;
+        double t;
+        if constexpr (sizeof(R) == 8) {
+            double s = 0.0;
+            for (int q = lane; q < count; q += 32) s += v[k * pitch + q];
+            t = warp_sum(s);
+        } else {
+            float hi = 0.f, lo = 0.f;
+            for (int q = lane; q < count; q += 32) two_sum(hi, lo, v[k * pitch + q], 0.f);
+            warp_sum_pair(hi, lo);
+            t = double(hi) + double(lo);
+        }
+        if (lane == 0) put(k, t);
+    }
+}
 
 // ------------------------------------------------------------------ tiles --------
 constexpr int kTileX = 32;        // columns of a tile
@@ -142,12 +195,39 @@ __device__ __forceinline__ Nine nine_of(const KParams &kp, const Site &s, unsign
     inside = a.inside;
     return n;
 }
-// One block of a step.  GEOM: 0 no solid nodes; 1 solid nodes with half-way links; 2 also interpolated
-// or moving walls.  INNER: the tile lies inside the lattice and no node of it or its ring pulls across
-// an edge, so every address is the node's own plus a constant of the launch (KParams::pull).
-template <class S, int GEOM, class O, bool INNER>
-__device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float (&sm)[2 * kTilePairs + 2][kTilePitch])
+// What a tile's kernel leaves: the next state; rho and u of the state read (lbm_get_moments); or the
+// block's sums for lbm_get_diagnostics, one row of kDiagSlots doubles (kDiagSums sums, the largest |u|,
+// the number of nodes whose density or velocity is not finite).
+enum TileMode { TILE_STEP = 0, TILE_MOMENTS = 1, TILE_DIAG = 2 };
+constexpr int kDiagSums = 9, kDiagSlots = 11;
+struct TileOut {
+    double *rho, *ux, *uy;  // [ny*nx], each may be null
+    double *part;           // [blocks][kDiagSlots]
+};
+
+// A float as a double without the conversion instruction, which runs on the narrow FP64 pipe.
+__device__ __forceinline__ double widen(float x)
 {
+    const unsigned b = __float_as_uint(x), e = b & 0x7f800000u;
+    if (e - 0x00800000u >= 0x7f000000u) return double(x);  // zero, subnormal, infinite or NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// One block of a step.  GEOM: 0 no solid nodes; 1 solid nodes with half-way links; 2 also interpolated
+// or moving walls; 3 any of these, told apart at run time.  INNER: the tile lies inside the lattice and no node of it or its ring pulls across
+// an edge, so every address is the node's own plus a constant of the launch (KParams::pull).
+struct Tile2Shared {
+    float psi[2 * kTilePairs + 2][kTilePitch];
+};
+struct Tile2SharedDiag : Tile2Shared {
+    float v[kDiagSums][64 * kTilePairs];
+    float umax[kTilePairs];
+    int bad[kTilePairs];
+};
+template <class S, int GEOM, class O, int MODE, bool INNER, class Shared>
+__device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const TileOut &out, Shared &sh)
+{
+    auto &sm = sh.psi;
     constexpr bool DEV = IsDev<S>::value;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int np = (blockDim.x >> 5) - 2, rows = 2 * np;  // pairs and rows of this launch's tiles
@@ -179,7 +259,8 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float 
     const uint32_t node_a = (uint32_t)a.y * (uint32_t)kp.nx + a.x, node_b = (uint32_t)b.y * (uint32_t)kp.nx + b.x;
     const uint32_t ka = (uint32_t)a.y * (uint32_t)kp.pitch + a.x, kb = (uint32_t)b.y * (uint32_t)kp.pitch + b.x;
     unsigned wa = 0, wb = 0;  // wall bits
-    if (GEOM) wa = kp.links[node_a], wb = kp.links[node_b];
+    const bool masked = GEOM == 3 ? kp.links != nullptr : GEOM != 0;
+    if (masked) wa = kp.links[node_a], wb = kp.links[node_b];
 
     // pull, Eq. (lbe.str)
     const S *src = static_cast<const S *>(kp.src);
@@ -213,7 +294,7 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float 
     } else {
         unsigned ia, ib;
         const Nine na = nine_of(kp, a, ia), nb = nine_of(kp, b, ib);
-        if (GEOM == 0) wa = edge_walls(ia), wb = edge_walls(ib);
+        if (!masked) wa = edge_walls(ia), wb = edge_walls(ib);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             const S *p = src + i * kp.plane;
@@ -227,6 +308,7 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float 
         if (DEV) wr = has_ref ? v2x{kp.c2.w[i]} * X2(refa[i], refb[i]) : v2x{kp.c2.dec[i]};
         f[i] = X2(Raw<S>::f(va[i], wr.v.x, kp), Raw<S>::f(vb[i], wr.v.y, kp));
     }
+    v2x momx = X2(0.f, 0.f), momy = momx;  // momentum handed to the walls (diagnostics)
     if ((!INNER || GEOM) && ((wa | wb) & 0x1feu)) {
         // wall links: the population that left the node toward the wall comes back
 #pragma unroll
@@ -247,7 +329,7 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float 
                 const int o = opp_(i);
                 const float fo = own(o);
                 float g = fo + 0.f;
-                if constexpr (GEOM == 2) {
+                if constexpr (GEOM >= 2) if (GEOM == 2 || kp.link != nullptr) {
                     // interpolated or moving wall: link fraction and moving-wall coefficient
                     const float2 lk = kp.link[(int64_t)(i - 1) * kp.plane + k];
                     float mw = 0.f;
@@ -273,6 +355,10 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float 
                 }
                 if (e) f[i].v.y = g;
                 else f[i].v.x = g;
+                if constexpr (MODE == TILE_DIAG) {
+                    float &mx = e ? momx.v.y : momx.v.x, &my = e ? momy.v.y : momy.v.x;
+                    mx += -float(ex_(i)) * (fo + g), my += -float(ey_(i)) * (fo + g);
+                }
             }
         }
     }
@@ -289,19 +375,22 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float 
     sm[ra][ca] = psi.v.x;
     sm[rb][cb] = psi.v.y;
     __syncthreads();
-    if (warp >= np) return;
+    if constexpr (MODE != TILE_DIAG)
+        if (warp >= np) return;
     const bool la = INNER || (ax < kp.nx && ay < kp.ny), lb = INNER || (ax < kp.nx && by < kp.ny);
-    if (!la) return;
-    if (kp.psi_out != nullptr) {
+    if constexpr (MODE != TILE_DIAG)
+        if (!la) return;
+    if (MODE == TILE_STEP && kp.psi_out != nullptr) {
         float *out = static_cast<float *>(kp.psi_out);
         out[node_a] = psi.v.x;
         if (lb) out[node_b] = psi.v.y;
     }
-    const bool sa = !(GEOM && (wa & 1u)), sb = lb && !(GEOM && (wb & 1u));
-    if (!sa && !sb) return;
+    const bool sa = la && !(GEOM && (wa & 1u)), sb = lb && !(GEOM && (wb & 1u));
+    if constexpr (MODE == TILE_STEP)
+        if (!sa && !sb) return;
 
     // S of Eq. (fint) from the four psi rows around the pair
-    const float *q = &sm[2 * warp][lane];
+    const float *q = &sm[MODE == TILE_DIAG ? min(2 * warp, 2 * kTilePairs - 2) : 2 * warp][lane];
     float c[4][3];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
@@ -324,6 +413,58 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float 
         Fex = Fey = X2(0.f, 0.f);
     }
     collide_v<v2x, O>(kp, d, rho, psi, Sx, Sy, Fex, Fey, fb, ux, uy);
+
+    if constexpr (MODE == TILE_MOMENTS) {
+        // solid nodes report their virtual density at rest
+        auto put = [&](bool fluid, uint32_t n, float r, float u, float v) {
+            if (out.rho) out.rho[n] = fluid ? widen(r) : (kp.wall_rho ? kp.wall_rho[n] : kp.rho_s);
+            if (out.ux) out.ux[n] = fluid ? widen(u) : 0.0;
+            if (out.uy) out.uy[n] = fluid ? widen(v) : 0.0;
+        };
+        put(sa, node_a, rho.v.x, ux.v.x, uy.v.x);
+        if (lb) put(sb, node_b, rho.v.y, ux.v.y, uy.v.y);
+        return;
+    }
+    if constexpr (MODE == TILE_DIAG) {
+        const v2x jx = ((f[1] - f[3]) + (f[5] - f[6])) + (f[8] - f[7]), jy = ((f[2] - f[4]) + (f[5] + f[6])) - (f[7] + f[8]);
+        const v2x nGpsi = v2x{kp.c2.m_G} * psi, Fx = vfma(nGpsi, Sx, Fex), Fy = vfma(nGpsi, Sy, Fey);
+        const float half_lg = float(0.5 * (kp.rho_l + kp.rho_g));
+        float um = 0.f;
+        int bad = 0;
+        if (warp < np) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                auto get = [&](v2x a) { return e ? a.v.y : a.v.x; };
+                const bool on = e ? sb : sa;
+                const float r = get(rho), u = get(ux), v = get(uy);
+                const bool liquid = on && r > half_lg;
+                const float t[kDiagSums] = {r, get(jx), get(jy), get(Fx), get(Fy), get(momx), get(momy), r * v, r};
+#pragma unroll
+                for (int k = 0; k < kDiagSums; ++k) sh.v[k][threadIdx.x + 32 * kTilePairs * e] = (k < 7 ? on : liquid) ? t[k] : 0.f;
+                if (on) {
+                    const float w = sqrtf(u * u + v * v);
+                    um = fmaxf(um, w);
+                    if (!isfinite(r) || !isfinite(w)) bad += 1;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                um = fmaxf(um, __shfl_down_sync(0xffffffffu, um, o));
+                bad += __shfl_down_sync(0xffffffffu, bad, o);
+            }
+            if (lane == 0) sh.umax[warp] = um, sh.bad[warp] = bad;
+        }
+        __syncthreads();
+        double *row = out.part + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kDiagSlots;
+        block_add<float>(&sh.v[0][0], 64 * kTilePairs, kDiagSums, 64 * kTilePairs, kTilePairs + 2, 0u,
+                         [&](int k, double t) { row[k] = t; });
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < kTilePairs; ++w) um = fmaxf(um, sh.umax[w]), bad += sh.bad[w];
+            row[kDiagSums] = double(um);
+            row[kDiagSums + 1] = double(bad);
+        }
+        return;
+    }
 
     // encode and store
     S *da = static_cast<S *>(kp.dst) + ka, *db = static_cast<S *>(kp.dst) + kb;
@@ -360,15 +501,54 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, float 
     }
 }
 
+__device__ __forceinline__ bool tile_inner(const KParams &kp, int rows)
+{
+    const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * rows;
+    return x0 >= 2 && x0 + kTileX + 2 <= kp.nx && y0 >= 2 && y0 + rows + 2 <= kp.ny;
+}
 template <class S, int GEOM, class O>
 __global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, int ahead)
 {
-    __shared__ float sm[2 * kTilePairs + 2][kTilePitch];
+    __shared__ Tile2Shared sh;
     grid_dependency_wait();
     allow_dependent_launch();
-    const int rows = 2 * ((blockDim.x >> 5) - 2), x0 = blockIdx.x * kTileX, y0 = blockIdx.y * rows;
-    if (x0 >= 2 && x0 + kTileX + 2 <= kp.nx && y0 >= 2 && y0 + rows + 2 <= kp.ny) tile2_block<S, GEOM, O, true>(kp, ahead, sm);
-    else tile2_block<S, GEOM, O, false>(kp, ahead, sm);
+    const TileOut none{};
+    if (tile_inner(kp, 2 * ((blockDim.x >> 5) - 2))) tile2_block<S, GEOM, O, TILE_STEP, true>(kp, ahead, none, sh);
+    else tile2_block<S, GEOM, O, TILE_STEP, false>(kp, ahead, none, sh);
+}
+// The readings of a state, on tiles of kTilePairs pairs (the whole block's sums want a full one).
+template <class S, int MODE>
+__global__ void __launch_bounds__(32 * (kTilePairs + 2), MODE == TILE_MOMENTS ? 5 : 4) k_read2(KParams kp, int ahead, TileOut out)
+{
+    __shared__ typename std::conditional<MODE == TILE_DIAG, Tile2SharedDiag, Tile2Shared>::type sh;
+    if (tile_inner(kp, 2 * kTilePairs)) tile2_block<S, 3, RuntimeOpts, MODE, true>(kp, ahead, out, sh);
+    else tile2_block<S, 3, RuntimeOpts, MODE, false>(kp, ahead, out, sh);
+}
+
+// Column sums of the blocks' rows (kDiagSlots columns; the largest |u| by maximum), one block per column
+// in a fixed order.
+template <class S>
+__global__ void __launch_bounds__(256) k_diag_reduce(const double *part, int64_t blocks, double *out)
+{
+    __shared__ double red[8];
+    const int k = blockIdx.x;
+    const bool top = k == kDiagSums;
+    double s = 0.0;
+    for (int64_t b = threadIdx.x; b < blocks; b += blockDim.x) {
+        const double x = part[b * kDiagSlots + k];
+        s = top ? fmax(s, x) : s + x;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double x = __shfl_down_sync(0xffffffffu, s, o);
+        s = top ? fmax(s, x) : s + x;
+    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < 8; ++q) s = top ? fmax(s, red[q]) : s + red[q];
+        out[k] = s;
+    }
 }
 
 // FP64: one node per thread.  Warps 0 .. n-1 own the tile's rows, two more the rows above and below
@@ -378,12 +558,18 @@ struct PlaneAt {
     __device__ __forceinline__ double operator()(int k, int x, int y) const { return load_pop<double>(kp, k, x, y); }
     __device__ __forceinline__ double at_k(int k, int64_t kk) const { return load_pop_at<double>(kp, k, kk); }
 };
-template <int GEOM>
-__global__ void __launch_bounds__(32 * (kTileRows + 3), 2) k_tile1(KParams kp)
+struct Tile1Shared {
+    double psi[kTileRows + 2][kTilePitch];
+};
+struct Tile1SharedDiag : Tile1Shared {
+    double v[kDiagSums][32 * kTileRows];
+    double umax[kTileRows];
+    int bad[kTileRows];
+};
+template <int MODE, class Shared>
+__device__ __forceinline__ void tile1_block(const KParams &kp, const TileOut &out, Shared &sh)
 {
-    __shared__ double sm[kTileRows + 2][kTilePitch];
-    grid_dependency_wait();
-    allow_dependent_launch();
+    auto &sm = sh.psi;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rows = (blockDim.x >> 5) - 3;
     const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * rows;
@@ -397,28 +583,102 @@ __global__ void __launch_bounds__(32 * (kTileRows + 3), 2) k_tile1(KParams kp)
     const int y = y0 + r - 1;
     const Site s = site_of(kp, x, y);
     const int64_t node = (int64_t)s.y * kp.nx + s.x;
-    const bool solid = GEOM && kp.solid != nullptr && kp.solid[node] != 0;
+    const bool solid = kp.solid != nullptr && kp.solid[node] != 0;
     const double psi_s = kp.cd.psi_s;
-    double f[9], psi;
+    double f[9], psi, mom[2] = {0.0, 0.0};
     if (!s.in) {
         psi = psi_s;
     } else if (solid) {
         psi = kp.wall_psi ? kp.wall_psi[node] : psi_s;
     } else {
-        pull_node_nb<double>(kp, around(kp, s.x, s.y), s.x, s.y, PlaneAt{kp}, f, (double *)nullptr);
+        pull_node_nb<double>(kp, around(kp, s.x, s.y), s.x, s.y, PlaneAt{kp}, f, MODE == TILE_DIAG ? mom : (double *)nullptr);
         psi = f64::psi_of(kp, f64::density(f));
     }
     sm[r][c] = psi;
     __syncthreads();
-    if (warp >= rows || x >= kp.nx || y >= kp.ny) return;
-    if (kp.psi_out != nullptr) static_cast<double *>(kp.psi_out)[node] = psi;
-    if (solid) return;
-    const double *q = &sm[r][c];
-    double fb[9], Sx, Sy, Fex, Fey, ux, uy;
-    f64::stencil_S([&](int i) { return q[ey_(i) * kTilePitch + ex_(i)]; }, Sx, Sy);
-    external_force<double>(kp, node, f64::density(f), Fex, Fey);
-    f64::collide(kp, f, psi, Sx, Sy, Fex, Fey, fb, ux, uy);
-    store_node<double>(kp, x, y, fb, 0.0);
+    const bool mine = warp < rows && x < kp.nx && y < kp.ny;
+    if constexpr (MODE != TILE_DIAG) {
+        if (!mine) return;
+        if (MODE == TILE_STEP && kp.psi_out != nullptr) static_cast<double *>(kp.psi_out)[node] = psi;
+        if (solid) {
+            if constexpr (MODE == TILE_MOMENTS) {
+                if (out.rho) out.rho[node] = kp.wall_rho ? kp.wall_rho[node] : kp.rho_s;
+                if (out.ux) out.ux[node] = 0.0;
+                if (out.uy) out.uy[node] = 0.0;
+            }
+            return;
+        }
+    }
+    double fb[9], Sx, Sy, Fex, Fey, ux = 0.0, uy = 0.0, rho = 0.0;
+    if (mine && !solid) {
+        const double *q = &sm[r][c];
+        f64::stencil_S([&](int i) { return q[ey_(i) * kTilePitch + ex_(i)]; }, Sx, Sy);
+        rho = f64::density(f);
+        external_force<double>(kp, node, rho, Fex, Fey);
+        f64::collide(kp, f, psi, Sx, Sy, Fex, Fey, fb, ux, uy);
+    }
+    if constexpr (MODE == TILE_STEP) {
+        store_node<double>(kp, x, y, fb, 0.0);
+    } else if constexpr (MODE == TILE_MOMENTS) {
+        if (out.rho) out.rho[node] = rho;
+        if (out.ux) out.ux[node] = ux;
+        if (out.uy) out.uy[node] = uy;
+    } else {
+        double um = 0.0;
+        int bad = 0;
+        if (warp < rows) {
+            const bool on = mine && !solid, liquid = on && rho > 0.5 * (kp.rho_l + kp.rho_g);
+            if (on) {
+                const double G = kp.cd.G;
+                const double t[kDiagSums] = {rho,
+                                             ((f[1] - f[3]) + (f[5] - f[6])) + (f[8] - f[7]),
+                                             ((f[2] - f[4]) + (f[5] + f[6])) - (f[7] + f[8]),
+                                             -G * psi * Sx + Fex,
+                                             -G * psi * Sy + Fey,
+                                             mom[0],
+                                             mom[1],
+                                             liquid ? rho * uy : 0.0,
+                                             liquid ? rho : 0.0};
+#pragma unroll
+                for (int k = 0; k < kDiagSums; ++k) sh.v[k][threadIdx.x] = t[k];
+                um = sqrt(ux * ux + uy * uy);
+                bad = !isfinite(rho) || !isfinite(um);
+                if (!(um > 0.0)) um = 0.0;  // (NaN counts as bad)
+            } else {
+#pragma unroll
+                for (int k = 0; k < kDiagSums; ++k) sh.v[k][threadIdx.x] = 0.0;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                um = fmax(um, __shfl_down_sync(0xffffffffu, um, o));
+                bad += __shfl_down_sync(0xffffffffu, bad, o);
+            }
+            if (lane == 0) sh.umax[warp] = um, sh.bad[warp] = bad;
+        }
+        __syncthreads();
+        double *row = out.part + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kDiagSlots;
+        block_add<double>(&sh.v[0][0], 32 * kTileRows, kDiagSums, 32 * kTileRows, kTileRows + 3, 0u,
+                          [&](int k, double t) { row[k] = t; });
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < kTileRows; ++w) um = fmax(um, sh.umax[w]), bad += sh.bad[w];
+            row[kDiagSums] = um;
+            row[kDiagSums + 1] = double(bad);
+        }
+    }
+}
+template <class S>
+__global__ void __launch_bounds__(32 * (kTileRows + 3), 2) k_tile1(KParams kp)
+{
+    __shared__ Tile1Shared sh;
+    grid_dependency_wait();
+    allow_dependent_launch();
+    tile1_block<TILE_STEP>(kp, TileOut{}, sh);
+}
+template <class S, int MODE>
+__global__ void __launch_bounds__(32 * (kTileRows + 3), 1) k_read1(KParams kp, TileOut out)
+{
+    __shared__ typename std::conditional<MODE == TILE_DIAG, Tile1SharedDiag, Tile1Shared>::type sh;
+    tile1_block<MODE>(kp, out, sh);
 }
 
 // Rows (units: pairs or rows) of a tile: of the heights from `most`/2 to `most`, the one whose fullest
@@ -439,6 +699,42 @@ inline int tile_height(const KParams &kp, int most, int rows_per_unit, int ring_
 
 template <class S>
 struct Tile {
+    static constexpr bool F64 = std::is_same<S, double>::value;
+    static constexpr int READ_ROWS = F64 ? kTileRows : 2 * kTilePairs;
+    static KParams with_pull(const KParams &kp)
+    {
+        KParams kq = kp;
+        for (int i = 0; i < 9; ++i) kq.pull[i] = (i * kp.plane - ey_(i) * kp.pitch) * (int64_t)sizeof(S);
+        return kq;
+    }
+    // rows between a tile and the one it prefetches: three blocks per SM further on, where the two
+    // population buffers exceed the 129 MB L2 (below that the lines are in L2 anyway)
+    static int ahead_of(const KParams &kp, dim3 grid, int rows)
+    {
+        const unsigned sms = kp.sm_count > 0 ? kp.sm_count : 148;
+        return 2.0 * 9.0 * kp.plane * sizeof(S) > 120e6 ? (int)(3u * sms / grid.x + 1) * rows : 0;
+    }
+    static dim3 read_grid(const KParams &kp) { return dim3((kp.nx + kTileX - 1) / kTileX, (kp.ny + READ_ROWS - 1) / READ_ROWS); }
+    template <int MODE>
+    static cudaError_t read(const KParams &kp, const TileOut &out, cudaStream_t st)
+    {
+        if constexpr (F64) k_read1<S, MODE><<<read_grid(kp), 32 * (kTileRows + 3), 0, st>>>(kp, out);
+        else k_read2<S, MODE><<<read_grid(kp), 32 * (kTilePairs + 2), 0, st>>>(with_pull(kp), ahead_of(kp, read_grid(kp), READ_ROWS), out);
+        return cudaGetLastError();
+    }
+    // rho and u = (j + F/2)/rho of the state kp.src, as the step computes them
+    static cudaError_t moments(const KParams &kp, double *rho, double *ux, double *uy, cudaStream_t st)
+    {
+        return read<TILE_MOMENTS>(kp, TileOut{rho, ux, uy, nullptr}, st);
+    }
+    static int64_t diag_rows(const KParams &kp) { return (int64_t)read_grid(kp).x * read_grid(kp).y; }
+    static cudaError_t diag(const KParams &kp, double *part, double *out, cudaStream_t st)
+    {
+        cudaError_t e = read<TILE_DIAG>(kp, TileOut{nullptr, nullptr, nullptr, part}, st);
+        if (e != cudaSuccess) return e;
+        k_diag_reduce<S><<<kDiagSlots, 256, 0, st>>>(part, diag_rows(kp), out);
+        return cudaGetLastError();
+    }
     static cudaError_t link_bits(const KParams &kp, uint16_t *out, cudaStream_t st)
     {
         k_link_bits<<<dim3((kp.nx + 127) / 128, kp.ny), 128, 0, st>>>(kp, out);
@@ -449,16 +745,12 @@ struct Tile {
         if constexpr (std::is_same<S, double>::value) {
             const int h = tile_height(kp, kTileRows, 1, 3);
             const dim3 grid((kp.nx + kTileX - 1) / kTileX, (kp.ny + h - 1) / h), block(32 * (h + 3));
-            return kp.solid ? launch_dependent(k_tile1<1>, grid, block, 0, st, kp) : launch_dependent(k_tile1<0>, grid, block, 0, st, kp);
+            return launch_dependent(k_tile1<S>, grid, block, 0, st, kp);
         } else {
             const int h = tile_height(kp, kTilePairs, 2, 2);
             const dim3 grid((kp.nx + kTileX - 1) / kTileX, (kp.ny + 2 * h - 1) / (2 * h)), block(32 * (h + 2));
-            // rows between a tile and the one it prefetches: three blocks per SM further on, where the
-            // two population buffers exceed the 129 MB L2 (below that the lines are in L2 anyway)
-            const int sms = kp.sm_count > 0 ? kp.sm_count : 148;
-            const int ahead = 2.0 * 9.0 * kp.plane * sizeof(S) > 120e6 ? (int)(3u * sms / grid.x + 1) * 2 * h : 0;
-            KParams kq = kp;
-            for (int i = 0; i < 9; ++i) kq.pull[i] = (i * kp.plane - ey_(i) * kp.pitch) * (int64_t)sizeof(S);
+            const int ahead = ahead_of(kp, grid, 2 * h);
+            const KParams kq = with_pull(kp);
             if (kp.q || kp.wall_u) return launch_dependent(k_tile2<S, 2, RuntimeOpts>, grid, block, 0, st, kq, ahead);
             if (kp.solid) return launch_dependent(k_tile2<S, 1, RuntimeOpts>, grid, block, 0, st, kq, ahead);
             return launch_dependent(k_tile2<S, 0, RuntimeOpts>, grid, block, 0, st, kq, ahead);

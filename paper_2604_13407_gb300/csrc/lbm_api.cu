@@ -35,7 +35,7 @@ struct lbm_ctx {
     double *wall_rho = nullptr, *wall_psi = nullptr;  // per solid node virtual density, its psi
     float2 *link = nullptr;             // wall-link records of the tile kernel (KParams::link)
     uint16_t *links = nullptr;          // wall bits of every node (KParams::links)
-    double *dacc = nullptr;             // diagnostics accumulators (9 doubles, 1 u64, 1 int)
+    double *dacc = nullptr;             // diagnostics: 9 sums, max |u|, count of non-finite nodes
     double *scratch = nullptr;          // host<->device staging for FP64 field copies
     size_t scratch_bytes = 0;
     int *derr = nullptr;
@@ -653,21 +653,13 @@ extern "C" lbm_status lbm_step(lbm_ctx *c, int64_t nsteps)
     return LBM_OK;
 }
 
-// psi field of the current state (needed by the moments and diagnostics kernels)
-static lbm_status psi_of_current(lbm_ctx *c)
-{
-    bind_buffers(c, c->cur);
-    CK(c->L.psi_pass(c->kp, c->stream), "psi kernel");
-    return LBM_OK;
-}
-
 extern "C" lbm_status lbm_get_moments(lbm_ctx *c, double *rho, double *ux, double *uy, int on_device)
 {
     if (!c) return LBM_EINVAL;
     if (!c->initialised) return fail(c, LBM_ESTATE, "fields not initialised");
     const size_t n = (size_t)c->p.nx * c->p.ny;
     lbm_status s;
-    if ((s = psi_of_current(c)) != LBM_OK) return s;
+    bind_buffers(c, c->cur);
     if (on_device) {
         CK(c->L.moments(c->kp, rho, ux, uy, c->stream), "moments kernel");
         return LBM_OK;
@@ -686,23 +678,14 @@ extern "C" lbm_status lbm_get_diagnostics(lbm_ctx *c, double out[LBM_NDIAG])
     if (!c || !out) return LBM_EINVAL;
     if (!c->initialised) return fail(c, LBM_ESTATE, "fields not initialised");
     lbm_status s;
-    if ((s = psi_of_current(c)) != LBM_OK) return s;
-    CK(cudaMemsetAsync(c->dacc, 0, 16 * sizeof(double), c->stream), "memset");
-    unsigned long long *umax = reinterpret_cast<unsigned long long *>(c->dacc + 9);
-    int *nanc = reinterpret_cast<int *>(c->dacc + 10);
-    CK(c->L.diag(c->kp, c->dacc, umax, nanc, c->stream), "diagnostics kernel");
-    double h[16];
+    bind_buffers(c, c->cur);
+    if ((s = need_scratch(c, (size_t)c->L.diag_rows(c->kp) * 11 * sizeof(double))) != LBM_OK) return s;
+    CK(c->L.diag(c->kp, c->scratch, c->dacc, c->stream), "diagnostics kernel");
+    double h[11];
     CK(cudaMemcpyAsync(h, c->dacc, sizeof h, cudaMemcpyDeviceToHost, c->stream), "D2H");
     if ((s = sync_and_check(c, "diagnostics")) != LBM_OK) return s;
-    for (int k = 0; k < 9; ++k) out[k] = h[k];
-    unsigned long long ub;
-    std::memcpy(&ub, &h[9], 8);
-    double um;
-    std::memcpy(&um, &ub, 8);
-    out[9] = um;
-    int nanc_h;
-    std::memcpy(&nanc_h, &h[10], sizeof(int));
-    if (nanc_h > 0 || !std::isfinite(out[0])) return fail(c, LBM_ENAN, "non-finite density or velocity");
+    for (int k = 0; k < 10; ++k) out[k] = h[k];
+    if (h[10] > 0 || !std::isfinite(out[0])) return fail(c, LBM_ENAN, "non-finite density or velocity");
     return LBM_OK;
 }
 

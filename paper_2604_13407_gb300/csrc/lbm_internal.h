@@ -146,8 +146,9 @@ struct Launchers {
     cudaError_t (*init)(const KParams &, const double *rho, const double *ux, const double *uy,
                         cudaStream_t);
     cudaError_t (*moments)(const KParams &, double *rho, double *ux, double *uy, cudaStream_t);
-    cudaError_t (*diag)(const KParams &, double *acc, unsigned long long *umax, int *nan_count,
-                        cudaStream_t);
+    int64_t (*diag_rows)(const KParams &);  // rows (of 11 doubles) of `part`
+    // out[11]: the nine sums of lbm_get_diagnostics, max |u|, number of nodes that are not finite
+    cudaError_t (*diag)(const KParams &, double *part, double *out, cudaStream_t);
     cudaError_t (*get_state)(const KParams &, double *out, cudaStream_t);
     cudaError_t (*set_state)(const KParams &, const double *in, cudaStream_t);
     // transposed step (FP64 arithmetic for FP64 storage, FP32 otherwise); AdjArgs in k_adjoint.cuh

@@ -78,3 +78,36 @@ def test_tile_step_with_solid_nodes(nx, ny, prec):
                 # 16-bit storage: a last-bit difference before rounding can move a stored deviation by one ulp of its type
                 ulp = 2.0 ** -23 if pid == lbm.F32 else 2.0 ** -10 if pid == lbm.F16DEV else 2.0 ** -7
                 assert np.abs(a - b).max() <= 4 * 8 * ulp * np.abs(a).max(), (px, py)
+
+
+@pytest.mark.parametrize("masked", [False, True])
+@pytest.mark.parametrize("prec", ["f64", "f32", "f16", "bf16"])
+@pytest.mark.parametrize("nx,ny", [(1, 5), (33, 17), (70, 37), (131, 40)])
+def test_readings_of_a_state(nx, ny, prec, masked):
+    """Moments and diagnostics of a stored state against the oracle's of the same (decoded) state: FP64 to
+    1e-12 of the mass (sums in another order) and bit for bit per node; FP32 arithmetic per node to
+    1e-6, some ten roundings (2^-24) of terms no larger than the density, and its sums to 1e-6 of the
+    mass."""
+    from oracle import oracle as O
+    pid, kw = PRECS[prec]
+    T, rg, rl = cs_case()
+    solid = (I.uniform(11, nx * ny).reshape(ny, nx) < 0.12).astype(np.uint8) if masked else None
+    for px, py in ((True, True), (True, False), (False, False)):
+        op = cs_params(nx=nx, ny=ny, periodic_x=px, periodic_y=py, scheme=1, force_mode=1, Fx=1e-5, Fy=-2e-5)
+        sim = lbm.Simulation(GC.gpu_params(op, pid, **kw))
+        if masked:
+            sim.set_geometry(solid)
+        u = I.uniform(7, 2 * nx * ny, -0.02, 0.02).reshape(2, ny, nx)
+        sim.init_fields(I.spinodal(nx, ny, 0.18, 0.3, 3), u[0], u[1])
+        sim.step(3)
+        ref = O.OracleSim(op, solid=solid)
+        ref.set_state(sim.get_state())
+        got, want = sim.moments(), ref.moments()
+        a, b = sim.diagnostics(), ref.diagnostics()
+        sim.close()
+        for g, w in zip(got, want):
+            assert np.array_equal(g, w) if prec == "f64" else np.abs(g - w).max() <= 1e-6
+        mass = b[0]
+        tol = 1e-12 if prec == "f64" else 1e-6
+        assert np.abs(a[:9] - b[:9]).max() <= tol * mass, (a, b)
+        assert abs(a[9] - b[9]) <= (1e-15 if prec == "f64" else 1e-6)
