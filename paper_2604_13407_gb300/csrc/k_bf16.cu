@@ -1,6 +1,7 @@
 // Kernel instantiations for __nv_bfloat16 population storage.
 #include "k_adjoint.cuh"
 #include "k_fused2.cuh"
+#include "k_small.cuh"
 #include "k_tile.cuh"
 #include "k_twopass.cuh"
 
@@ -22,6 +23,8 @@ Launchers launchers_bf16()
     L.fused_pass = &Fused2<__nv_bfloat16, LBM_FUSED2_NW, LBM_FUSED2_RING>::launch;
     L.fused_tile_x = FusedLayout2<__nv_bfloat16, LBM_FUSED2_NW, LBM_FUSED2_RING>::TX;
     L.tile_pass = &Tile<__nv_bfloat16>::step;
+    L.small_ctas = &Small<__nv_bfloat16>::ctas;
+    L.small_steps = &Small<__nv_bfloat16>::steps;
     L.link_bits = &Tile<__nv_bfloat16>::link_bits;
     L.init = &TwoPass<__nv_bfloat16>::init;
     L.moments = &Tile<__nv_bfloat16>::moments;

@@ -1,6 +1,7 @@
 // Kernel instantiations for __half population storage.
 #include "k_adjoint.cuh"
 #include "k_fused2.cuh"
+#include "k_small.cuh"
 #include "k_tile.cuh"
 #include "k_twopass.cuh"
 
@@ -22,6 +23,8 @@ Launchers launchers_f16()
     L.fused_pass = &Fused2<__half, LBM_FUSED2_NW, LBM_FUSED2_RING>::launch;
     L.fused_tile_x = FusedLayout2<__half, LBM_FUSED2_NW, LBM_FUSED2_RING>::TX;
     L.tile_pass = &Tile<__half>::step;
+    L.small_ctas = &Small<__half>::ctas;
+    L.small_steps = &Small<__half>::steps;
     L.link_bits = &Tile<__half>::link_bits;
     L.init = &TwoPass<__half>::init;
     L.moments = &Tile<__half>::moments;

@@ -1,6 +1,7 @@
 // Kernel instantiations for float population storage.
 #include "k_adjoint.cuh"
 #include "k_fused2.cuh"
+#include "k_small.cuh"
 #include "k_tile.cuh"
 #include "k_twopass.cuh"
 
@@ -22,6 +23,8 @@ Launchers launchers_f32()
     L.fused_pass = &Fused2<float, LBM_FUSED2_NW, LBM_FUSED2_RING>::launch;
     L.fused_tile_x = FusedLayout2<float, LBM_FUSED2_NW, LBM_FUSED2_RING>::TX;
     L.tile_pass = &Tile<float>::step;
+    L.small_ctas = &Small<float>::ctas;
+    L.small_steps = &Small<float>::steps;
     L.link_bits = &Tile<float>::link_bits;
     L.init = &TwoPass<float>::init;
     L.moments = &Tile<float>::moments;

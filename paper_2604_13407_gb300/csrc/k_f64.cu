@@ -1,5 +1,6 @@
 // Kernel instantiations for double population storage.
 #include "k_adjoint.cuh"
+#include "k_small.cuh"
 #include "k_tile.cuh"
 #include "k_twopass.cuh"
 
@@ -11,6 +12,8 @@ Launchers launchers_f64()
     L.psi_pass = &TwoPass<double>::psi_pass;
     L.collide_pass = &TwoPass<double>::collide_pass;
     L.tile_pass = &Tile<double>::step;
+    L.small_ctas = &Small<double>::ctas;
+    L.small_steps = &Small<double>::steps;
     L.link_bits = &Tile<double>::link_bits;
     L.init = &TwoPass<double>::init;
     L.moments = &Tile<double>::moments;

@@ -1,0 +1,455 @@
+// Many steps of a small lattice in one launch: the lattice lives in the shared memory of one thread-block
+// cluster, a strip of rows per CTA.
+//
+// What bounds a small lattice is neither bytes nor instructions but the launch and the two trips through
+// L2 that a step of its own kernel takes (2.9 us a step on 37 x 23 nodes, whatever is computed).  Here a step
+// is two phases between cluster barriers: pull, rho and psi; then the psi stencil, collision and the
+// write-back in place.  A thread owns one pair of nodes (FP64: one node) for the whole launch.  What a
+// neighbouring strip needs -- psi of the edge rows, and the populations that leave them -- is pushed into
+// its halo rows through distributed shared memory, so every load is a local one.
+//
+// Measured per step (us, one launch per step / here): 37 x 23 FP32 3.0 / 1.2, FP16 3.0 / 2.4; 64^2 FP32 3.0 / 1.2;
+// 128^2 3.0 / 2.2 (16 SMs are busy there: the last size that gains); FP64 4 x 128 column 18 / 7.5, 4 x 181
+// 18 / 11.5, 37 x 23 18 / 16.4.
+//
+// The functions, their order and the storage type's rounding are the tile kernel's (k_tile.cuh), so
+// the state after n steps is, bit for bit, what n of its launches leave.
+#pragma once
+
+#include "k_tile.cuh"
+
+namespace lbm {
+
+constexpr int kSmallThreads = 512;  // most threads of a CTA
+
+__device__ __forceinline__ void cluster_barrier()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Shared-memory address of this CTA as the same variable's address in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_to(const void *p, uint32_t rank)
+{
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void push(uint32_t a, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void push(uint32_t a, double v) { asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory"); }
+__device__ __forceinline__ void push(uint32_t a, __half v) { asm volatile("st.shared::cluster.b16 [%0], %1;" ::"r"(a), "h"(__half_as_ushort(v)) : "memory"); }
+__device__ __forceinline__ void push(uint32_t a, __nv_bfloat16 v) { asm volatile("st.shared::cluster.b16 [%0], %1;" ::"r"(a), "h"(__bfloat16_as_ushort(v)) : "memory"); }
+
+// Seed of the stochastic rounding of step t (the host's sr_seed_of).
+__device__ __forceinline__ uint32_t sr_seed_at(int64_t t)
+{
+    uint32_t h = (uint32_t)t * 0x9E3779B1u ^ (uint32_t)((uint64_t)t >> 32) * 0x85EBCA77u;
+    h ^= h >> 16;
+    h *= 0x85EBCA6Bu;
+    h ^= h >> 13;
+    h *= 0xC2B2AE35u;
+    h ^= h >> 16;
+    return h;
+}
+
+// Shared memory of a CTA: nine planes, the reference plane and psi, of `rows` own rows and a halo row
+// above and below; a psi row ends with one entry that always holds psi(rho_s), the neighbour beyond a
+// non-periodic x edge.
+template <class S>
+struct SmallLayout {
+    typedef typename Codec<S>::R R;
+    int nx, rows;
+    __host__ __device__ size_t plane() const { return (size_t)(rows + 2) * nx; }
+    __host__ __device__ size_t psi_at() const { return (9 * plane() * sizeof(S) + 15) / 16 * 16; }
+    __host__ __device__ size_t ref_at() const { return psi_at() + ((size_t)(rows + 2) * (nx + 1) * sizeof(R) + 15) / 16 * 16; }
+    __host__ __device__ size_t bytes(bool ref) const { return ref_at() + (ref ? plane() * sizeof(float) : 0); }
+};
+
+// A CTA's strip of the lattice in its shared memory.
+template <class S>
+struct Strip {
+    typedef typename Codec<S>::R R;
+    const KParams &kp;
+    S *pop;
+    R *psi;
+    float *ref;
+    int nx, C, rank, y0, m;  // own rows y0 .. y0 + m - 1: local rows 1 .. m
+    uint32_t PS;             // elements per plane
+    uint32_t up_pop, up_psi, up_ref, down_pop, down_psi, down_ref;  // halo rows of the strips above and below
+    bool has_ref;
+
+    __device__ __forceinline__ int first_row(int r) const { return (int)((int64_t)r * kp.ny / C); }
+    // Reads the strip and its halo rows; every thread of the cluster is past its end when it returns.
+    __device__ __forceinline__ void load(unsigned char *smem, int max_rows)
+    {
+        nx = kp.nx, C = (int)gridDim.x, rank = (int)cluster_rank();
+        const SmallLayout<S> L{nx, max_rows};
+        PS = (uint32_t)L.plane();
+        pop = reinterpret_cast<S *>(smem);
+        psi = reinterpret_cast<R *>(smem + L.psi_at());
+        ref = reinterpret_cast<float *>(smem + L.ref_at());
+        has_ref = IsDev<S>::value && kp.per_node_ref;
+        y0 = first_row(rank), m = first_row(rank + 1) - y0;
+        for (int lr = 0; lr < m + 2; ++lr) {
+            int gy = y0 + lr - 1;
+            const bool in = (gy >= 0 && gy < kp.ny) || kp.periodic_y;
+            gy = gy < 0 ? gy + kp.ny : gy >= kp.ny ? gy - kp.ny : gy;
+            for (int x = threadIdx.x; x < nx; x += blockDim.x) {
+                if (in) {
+                    const int64_t k = (int64_t)gy * kp.pitch + x;
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) pop[i * PS + lr * nx + x] = static_cast<const S *>(kp.src)[i * kp.plane + k];
+                    if (has_ref) ref[lr * nx + x] = kp.ref_src[k];
+                } else {
+                    psi[lr * (nx + 1) + x] = cst<R>(kp).psi_s;
+                }
+            }
+            if (threadIdx.x == 0) psi[lr * (nx + 1) + nx] = cst<R>(kp).psi_s;
+        }
+        const int up = rank == C - 1 ? 0 : rank + 1, down = rank == 0 ? C - 1 : rank - 1;
+        const uint32_t above_down = (uint32_t)(first_row(down + 1) - first_row(down) + 1);  // its halo row above its own
+        up_pop = map_to(pop, up), up_psi = map_to(psi, up), up_ref = map_to(ref, up);
+        down_pop = map_to(pop, down) + above_down * nx * (uint32_t)sizeof(S);
+        down_psi = map_to(psi, down) + above_down * (nx + 1) * (uint32_t)sizeof(R);
+        down_ref = map_to(ref, down) + above_down * nx * 4u;
+        cluster_barrier();
+    }
+    __device__ __forceinline__ void barrier() const
+    {
+        if (C == 1) __syncthreads();
+        else cluster_barrier();
+    }
+};
+
+// A node of a strip: its places in shared memory and in the lattice.
+template <class S>
+struct StripNode {
+    typedef typename Codec<S>::R R;
+    bool live, fluid, top, bottom;        // a node; a fluid one; in a row that the strip above / below reads
+    uint32_t row, cm, c0, cp, pm, pp;     // local row; columns x - 1, x, x + 1 of the populations, and of psi
+    uint32_t node, kg;                    // lattice and plane index
+    unsigned w;                           // wall bits
+    __device__ __forceinline__ StripNode(const Strip<S> &s, int idx)
+    {
+        const KParams &kp = s.kp;
+        live = idx < s.m * s.nx;
+        const int ly = live ? idx / s.nx : 0, x = live ? idx - ly * s.nx : 0, y = s.y0 + ly;
+        row = ly + 1;
+        const Around nb = around(kp, x, y);
+        cm = nb.xc[0], c0 = x, cp = nb.xc[2];
+        pm = x > 0 || kp.periodic_x ? cm : s.nx;
+        pp = x < s.nx - 1 || kp.periodic_x ? cp : s.nx;
+        node = (uint32_t)y * s.nx + x;
+        kg = (uint32_t)y * (uint32_t)kp.pitch + x;
+        w = kp.links != nullptr ? kp.links[node] : edge_walls(nb.inside);
+        fluid = live && !(w & 1u);
+        top = live && ly == s.m - 1 && (y < kp.ny - 1 || kp.periodic_y);
+        bottom = live && ly == 0 && (y > 0 || kp.periodic_y);
+    }
+    __device__ __forceinline__ uint32_t from(const Strip<S> &s, int i) const  // x - e_i
+    {
+        return (row - ey_(i)) * s.nx + (ex_(i) > 0 ? cm : ex_(i) < 0 ? cp : c0);
+    }
+    __device__ __forceinline__ uint32_t own(const Strip<S> &s) const { return row * s.nx + c0; }
+    __device__ __forceinline__ uint32_t psi_at(const Strip<S> &s, int i) const  // x + e_i
+    {
+        return (row + ey_(i)) * (s.nx + 1) + (ex_(i) > 0 ? pp : ex_(i) < 0 ? pm : c0);
+    }
+    __device__ __forceinline__ R read(const Strip<S> &s, int i, uint32_t o) const
+    {
+        if constexpr (IsDev<S>::value)
+            return Raw<S>::f(s.pop[i * s.PS + o], __fmul_rn(w_<float>(i), s.has_ref ? s.ref[o] : s.kp.cf.rho_ref), s.kp);
+        else return s.pop[i * s.PS + o];
+    }
+    // Pull, Eq. (lbe.str); on wall links the population that left the node toward the wall comes back.
+    __device__ __forceinline__ void pull(const Strip<S> &s, R (&f)[9]) const
+    {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = read(s, i, from(s, i));
+        if ((w & 0x1feu) && fluid) {
+#pragma unroll
+            for (int i = 1; i < 9; ++i)
+                if ((w >> i) & 1u) f[i] = read(s, opp_(i), own(s)) + R(0);
+        }
+    }
+    __device__ __forceinline__ void put_psi(const Strip<S> &s, R v) const
+    {
+        if (!live) return;
+        s.psi[row * (s.nx + 1) + c0] = v;
+        if (top) push(s.up_psi + c0 * (uint32_t)sizeof(R), v);
+        if (bottom) push(s.down_psi + c0 * (uint32_t)sizeof(R), v);
+    }
+    // Stores populations [first, first + count) of the node.
+    __device__ __forceinline__ void put(const Strip<S> &s, const S (&v)[9], int first = 0, int count = 9) const
+    {
+        if (!fluid) return;
+        S *p = s.pop + own(s);
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            if (i >= first && i < first + count) p[i * s.PS] = v[i];
+        if (top) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+                if (ey_(i) > 0 && i >= first && i < first + count) push(s.up_pop + (i * s.PS + c0) * (uint32_t)sizeof(S), v[i]);
+        }
+        if (bottom) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+                if (ey_(i) < 0 && i >= first && i < first + count) push(s.down_pop + (i * s.PS + c0) * (uint32_t)sizeof(S), v[i]);
+        }
+    }
+    // The state after an odd number of steps goes to the other buffer, as step by step.
+    __device__ __forceinline__ void write_back(const Strip<S> &s, bool odd, int first, int count) const
+    {
+        if (!fluid) return;
+        S *dst = static_cast<S *>(odd ? s.kp.dst : const_cast<void *>(s.kp.src));
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            if (i >= first && i < first + count) dst[i * s.kp.plane + kg] = s.pop[i * s.PS + own(s)];
+        if (s.has_ref) (odd ? s.kp.ref_dst : const_cast<float *>(s.kp.ref_src))[kg] = s.ref[own(s)];
+    }
+};
+
+// FP32 arithmetic: a thread owns two nodes of its strip, `pairs` apart, for the whole launch.
+template <class S>
+__global__ void __launch_bounds__(kSmallThreads) k_small2(KParams kp, int64_t nsteps, int64_t step0, int max_rows)
+{
+    constexpr bool DEV = IsDev<S>::value;
+    extern __shared__ __align__(128) unsigned char smem[];
+    Strip<S> s{kp};
+    s.load(smem, max_rows);
+    const int pairs = (s.m * s.nx + 1) / 2, t0 = (int)threadIdx.x;
+    // (threads past the last pair, and the second node of an odd strip's last thread: not live)
+    const StripNode<S> a(s, t0 < pairs ? t0 : s.m * s.nx), b(s, t0 < pairs ? t0 + pairs : s.m * s.nx);
+    // which half of its pair's random word each node takes: its column's parity
+    const unsigned pick = (a.c0 & 1u ? 0x32u : 0x10u) | (b.c0 & 1u ? 0x7600u : 0x5400u);
+    // psi of solid nodes (the FP64 field is converted once, not per step)
+    const float wall_a = (a.w & 1u) && kp.wall_psi ? float(kp.wall_psi[a.node]) : kp.cf.psi_s;
+    const float wall_b = (b.w & 1u) && kp.wall_psi ? float(kp.wall_psi[b.node]) : kp.cf.psi_s;
+
+    v2x fx = X2(0.f, 0.f), fy = fx;  // force field at the nodes
+    for (int64_t t = 0; t < nsteps; ++t) {
+        float fa[9], fb[9];
+        a.pull(s, fa);
+        b.pull(s, fb);
+        v2x d[9], rho, psi;
+        {
+            v2x f[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = X2(fa[i], fb[i]);
+            to_dev(f, d);
+        }
+        rho = density_dev(d);
+        psi = psi_v<v2x>(kp, rho);
+        if (a.w & 1u) psi.v.x = wall_a, rho.v.x = 1.f;
+        if (b.w & 1u) psi.v.y = wall_b, rho.v.y = 1.f;
+        a.put_psi(s, psi.v.x);
+        b.put_psi(s, psi.v.y);
+        s.barrier();
+
+        auto p = [&](int i) { return X2(s.psi[a.psi_at(s, i)], s.psi[b.psi_at(s, i)]); };
+        v2x Sx, Sy, Fex, Fey, o[9], ux, uy;
+        stencil_v<v2x>(p(1), p(2), p(3), p(4), p(5), p(6), p(7), p(8), Sx, Sy);
+        if (kp.force_mode == 0) {
+            Fex = v2x{kp.c2.Fx}, Fey = v2x{kp.c2.Fy};
+        } else if (kp.force_mode == 1) {
+            const v2x x = rho - v2x{kp.c2.rho_g};
+            Fex = x * v2x{kp.c2.Fx}, Fey = x * v2x{kp.c2.Fy};
+        } else if (kp.fext) {
+            const int64_t n = (int64_t)kp.nx * kp.ny;
+            if (t == 0) {
+                fx = X2(float(kp.fext[a.node]), float(kp.fext[b.node]));
+                fy = X2(float(kp.fext[n + a.node]), float(kp.fext[n + b.node]));
+            }
+            Fex = fx, Fey = fy;
+        } else {
+            Fex = Fey = X2(0.f, 0.f);
+        }
+        collide_v<v2x, RuntimeOpts>(kp, d, rho, psi, Sx, Sy, Fex, Fey, o, ux, uy);
+        S va[9], vb[9];
+        if constexpr (DEV) {
+            const uint32_t seed = sr_seed_at(step0 + t);
+            const uint32_t ha = sr_hash(a.kg >> 1, seed), hb = sr_hash(b.kg >> 1, seed);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const v2x wr = s.has_ref ? v2x{kp.c2.w[i]} * rho : v2x{kp.c2.dec[i]};
+                const v2x q = (o[i] - wr) * v2x{kp.c2.scale};
+                if (kp.sr) {
+                    const uint32_t h = SRound<S>::pack(q.v.x, q.v.y, __byte_perm(sr_bits(ha, i), sr_bits(hb, i), pick));
+                    va[i] = SRound<S>::from_bits((unsigned short)(h & 0xffffu)), vb[i] = SRound<S>::from_bits((unsigned short)(h >> 16));
+                } else {
+                    va[i] = Codec<S>::enc(q.v.x, 0.f, 1.f), vb[i] = Codec<S>::enc(q.v.y, 0.f, 1.f);
+                }
+            }
+            if (s.has_ref) {
+                auto put_ref = [&](const StripNode<S> &n, float v) {
+                    if (!n.fluid) return;
+                    s.ref[n.own(s)] = v;
+                    if (n.top) push(s.up_ref + n.c0 * 4u, v);
+                    if (n.bottom) push(s.down_ref + n.c0 * 4u, v);
+                };
+                put_ref(a, rho.v.x);
+                put_ref(b, rho.v.y);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) va[i] = o[i].v.x, vb[i] = o[i].v.y;
+        }
+        a.put(s, va);
+        b.put(s, vb);
+        s.barrier();
+    }
+    a.write_back(s, nsteps & 1, 0, 9);
+    b.write_back(s, nsteps & 1, 0, 9);
+}
+
+// FP64.  An FP64 instruction holds its scheduler's quarter of the SM for 64 cycles, whatever the
+// number of active lanes and however independent its neighbours are, so a node's 390 of them in one
+// warp take 12 us, and a small lattice leaves most schedulers idle.  Four warps therefore share a
+// group of 32 nodes, one per scheduler, and hand each other the few values they need through
+// shared memory: psi / moments / 1/rho; then the x and y force and velocity; then the relaxed moments;
+// then the populations.  The longest of the four takes about 120 FP64 instructions a step.  (4 x 128
+// column: 18 us a step with one launch per step, 13.2 with one warp per 32 nodes.)
+struct Small64Shared {
+    double r[kSmallThreads / 4];                                                   // 1/(G psi^2)
+    double Fix[kSmallThreads / 4], Fiy[kSmallThreads / 4], Fx[kSmallThreads / 4], Fy[kSmallThreads / 4];
+    double ux[kSmallThreads / 4], uy[kSmallThreads / 4];
+    double u[9][kSmallThreads / 4];                                                // m_bar_k without |M_k|^2's odd factor
+};
+template <class S>
+__global__ void __launch_bounds__(kSmallThreads) k_small1(KParams kp, int64_t nsteps, int64_t step0, int max_rows)
+{
+    using namespace f64;
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ Small64Shared x;
+    Strip<S> s{kp};
+    s.load(smem, max_rows);
+    const int role = (threadIdx.x >> 5) & 3, at = (threadIdx.x >> 7) * 32 + (threadIdx.x & 31);
+    const StripNode<S> a(s, at);
+
+    for (int64_t t = 0; t < nsteps; ++t) {
+        double f[9], sp = kp.sp, sq = kp.sq, m_a = 0.0, m_b = 0.0;
+        a.pull(s, f);
+        const double rho = density(f);
+        Divisor by_rho{};
+        if (role == 0) {
+            a.put_psi(s, a.w & 1u ? (kp.wall_psi ? kp.wall_psi[a.node] : kp.psi_s) : psi_of(kp, rho));
+        } else if (role == 1) {
+            moments_12(f, m_a, m_b);
+        } else if (role == 2) {
+            by_rho = divisor(rho);
+            m_a = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];                                  // j_x
+            m_b = fma_(2.0, f[3], -2.0 * f[1]) + f[5] - f[6] - f[7] + f[8];               // m_4
+        } else {
+            by_rho = divisor(rho);
+            m_a = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];                                  // j_y
+            m_b = fma_(2.0, f[4], -2.0 * f[2]) + f[5] + f[6] - f[7] - f[8];               // m_6
+        }
+        if (kp.var_tau && role != 0) relaxation(kp, rho, sp, sq);
+        s.barrier();
+
+        const double psi = s.psi[a.row * (s.nx + 1) + a.c0], Gpsi = kp.G * psi;
+        if (role >= 2) {
+            double S_ = 0.0, Fex, Fey;
+            auto ps = [&](int i) { return s.psi[a.psi_at(s, i)]; };
+            if (role == 2) S_ = stencil_x(ps);
+            else S_ = stencil_y(ps);
+            external_force<double>(kp, a.node, rho, Fex, Fey);
+            const double Fi = -Gpsi * S_, F = Fi + (role == 2 ? Fex : Fey), u = by_rho(fma_(0.5, F, m_a));
+            if (role == 2) x.Fix[at] = Fi, x.Fx[at] = F, x.ux[at] = u;
+            else x.Fiy[at] = Fi, x.Fy[at] = F, x.uy[at] = u;
+        } else if (role == 1) {
+            x.r[at] = __drcp_rn(Gpsi * psi);
+        } else {
+            m_a = f[1] - f[2] + f[3] - f[4], m_b = f[5] - f[6] + f[7] - f[8];               // m_7, m_8
+            x.u[0][at] = div_const<9>(rho);
+            if (kp.var_tau) relaxation(kp, rho, sp, sq);
+        }
+        __syncthreads();
+
+        const double Fix = x.Fix[at], Fiy = x.Fiy[at], Fx = x.Fx[at], Fy = x.Fy[at], ux = x.ux[at], uy = x.uy[at];
+        const double Gpsi2 = Gpsi * psi;
+        const Divisor by_Gpsi2{Gpsi2, x.r[at], in_range(Gpsi2) && is_nonzero(Gpsi2)};
+        if (role == 0) {
+            relaxed_78(kp, rho, m_a, m_b, Fx, Fy, ux, uy, Fix, Fiy, by_Gpsi2, sp, x.u[7][at], x.u[8][at]);
+        } else if (role == 1) {
+            double a1, a2;
+            relaxed_12(kp, rho, m_a, m_b, Fx, Fy, ux, uy, by_Gpsi2(Fix * Fix), by_Gpsi2(Fiy * Fiy), sp, a1, a2);
+            x.u[1][at] = div_const<9>(a1), x.u[2][at] = div_const<9>(a2);
+        } else {
+            double X = 0.0, Y = 0.0, aj, aq;
+            if (kp.improved) X = by_Gpsi2(Fix * Fix), Y = by_Gpsi2(Fiy * Fiy);
+            if (role == 2) relaxed_jq(kp, rho, m_a, m_b, Fx, ux, X, Y, sq, aj, aq);
+            else relaxed_jq(kp, rho, m_a, m_b, Fy, uy, Y, X, sq, aj, aq);
+            const int k = role == 2 ? 3 : 5;
+            x.u[k][at] = div_const<3>(aj), x.u[k + 1][at] = div_const<3>(aq);
+        }
+        __syncthreads();
+
+        double u[9], o[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) u[i] = x.u[i][at];
+        populations(u, o);  // (each warp evaluates the ones it stores)
+        if (role == 0) a.put(s, o, 0, 3);
+        else if (role == 1) a.put(s, o, 3, 2);
+        else if (role == 2) a.put(s, o, 5, 2);
+        else a.put(s, o, 7, 2);
+        s.barrier();
+    }
+    if (role == 0) a.write_back(s, nsteps & 1, 0, 9);
+}
+
+template <class S>
+struct Small {
+    typedef typename Codec<S>::R R;
+    static constexpr bool F64 = sizeof(R) == 8;
+    static int rows(const KParams &kp, int ctas) { return (kp.ny + ctas - 1) / ctas; }
+    // two nodes a thread; FP64: four warps per 32 nodes
+    static int threads(const KParams &kp, int ctas)
+    {
+        const int nodes = rows(kp, ctas) * kp.nx;
+        return F64 ? (nodes + 31) / 32 * 128 : (nodes + 63) / 64 * 32;
+    }
+    static void (*kernel())(KParams, int64_t, int64_t, int)
+    {
+        if constexpr (F64) return k_small1<S>;
+        else return k_small2<S>;
+    }
+    static size_t bytes(const KParams &kp, int ctas) { return SmallLayout<S>{kp.nx, rows(kp, ctas)}.bytes(IsDev<S>::value && kp.per_node_ref); }
+    static constexpr int SMEM = 190 * 1024;
+    static constexpr int64_t MAX_NODES = F64 ? 2048 : 16384;
+    // CTAs of the cluster that steps this lattice; 0: it is too large (or has interpolated or moving
+    // walls), or the device cannot hold the cluster.
+    static int ctas(const KParams &kp)
+    {
+        if (kp.q || kp.wall_u) return 0;
+        const int64_t n = (int64_t)kp.nx * kp.ny;
+        if (n > MAX_NODES) return 0;
+        int c = n > (F64 ? 128 : 1024) ? 16 : 8;
+        while (c > kp.ny) c /= 2;
+        if ((int64_t)rows(kp, c) * kp.nx > 2 * kSmallThreads || threads(kp, c) > kSmallThreads || bytes(kp, c) > SMEM) return 0;
+        return cluster_fits(reinterpret_cast<const void *>(kernel()), kp.device, c, kSmallThreads, SMEM) ? c : 0;
+    }
+    static cudaError_t steps(const KParams &kp, int ctas, int64_t nsteps, int64_t step0, cudaStream_t st)
+    {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(ctas);
+        cfg.blockDim = dim3(threads(kp, ctas));
+        cfg.dynamicSmemBytes = bytes(kp, ctas);
+        cfg.stream = st;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = ctas;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kernel(), kp, nsteps, step0, rows(kp, ctas));
+    }
+};
+
+}  // namespace lbm

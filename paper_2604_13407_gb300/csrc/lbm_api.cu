@@ -39,6 +39,7 @@ struct lbm_ctx {
     double *scratch = nullptr;          // host<->device staging for FP64 field copies
     size_t scratch_bytes = 0;
     int *derr = nullptr;
+    int small_ctas = 0;  // LBM_KERNEL_AUTO: CTAs of the cluster that steps a small lattice; 0: one launch per step
     bool initialised = false;
     bool fused_ok = false;
     cudaError_t (*one_pass)(const KParams &, cudaStream_t) = nullptr;  // the step's kernel; null: two-pass
@@ -184,7 +185,10 @@ static void fill_constants(lbm_ctx *c)
     k.q1c = 3.0 * (p.k1 + 2.0 * p.k2);
     k.q4a = (30.0 * eps - 15.0) / 16.0;
     k.q4b = 3.0 * eps / 8.0;
-    k.inv_G = 1.0 / p.G;
+    k.two_inv_G = 2.0 / p.G;
+    k.eos_b4 = p.b / 4.0;
+    k.unit_R = p.R == 1.0;
+    k.unit_K = p.K_eos == 1.0;
     int g_exp;
     k.G_pow2 = std::frexp(p.G, &g_exp) == -0.5 && std::abs(g_exp) < 500;
     k.kq1 = 3.0 * (p.k1 + 2.0 * p.k2) * p.G;
@@ -192,6 +196,7 @@ static void fill_constants(lbm_ctx *c)
     k.c1G = (30.0 * eps - 15.0) / 16.0 * p.G;
     k.c2G = 3.0 * eps / 8.0 * p.G;
     k.q2fac = (p.scheme == LBM_SCHEME_ORIGINAL || p.q2_original) ? -1.0 : -0.5;
+    k.q2_full = k.q2fac == -1.0;
     const double tau = p.tau_l;
     k.sp = 1.0 / tau;
     k.sq = 1.0 / (0.5 + p.Lambda / (tau - 0.5));
@@ -306,6 +311,7 @@ static void choose_kernel(lbm_ctx *c)
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
     const bool large = n >= (c->p.precision == LBM_F32 ? (int64_t)1 << 25 : (int64_t)3 << 20);
     c->one_pass = nullptr;
+    c->small_ctas = want == LBM_KERNEL_AUTO ? c->L.small_ctas(c->kp) : 0;
     if (want == LBM_KERNEL_TWO_PASS || (want == LBM_KERNEL_FUSED && !possible)) return;
     if (staged && (want == LBM_KERNEL_FUSED || large || !tile)) c->one_pass = c->L.fused_pass;
     else if (tile) c->one_pass = c->L.tile_pass;
@@ -604,6 +610,17 @@ static uint32_t sr_seed_of(int64_t t)
 
 static lbm_status run_steps(lbm_ctx *c, int64_t nsteps)
 {
+    // a small lattice: many steps in one launch (no more than 4096, so that no launch takes long; fewer
+    // than four are as fast one by one)
+    while (c->small_ctas > 0 && nsteps >= 4) {
+        const int64_t n = std::min<int64_t>(nsteps, 4096);
+        bind_buffers(c, c->cur);
+        CK(c->L.small_steps(c->kp, c->small_ctas, n, c->steps, c->stream), "small-lattice kernel");
+        c->cur ^= (int)(n & 1);
+        c->steps += n;
+        c->kp.sr_seed = sr_seed_of(c->steps - 1);
+        nsteps -= n;
+    }
     for (int64_t t = 0; t < nsteps; ++t) {
         bind_buffers(c, c->cur);
         c->kp.sr_seed = sr_seed_of(c->steps);
@@ -898,6 +915,39 @@ cudaError_t ensure_smem_attribute_ptr(const void *kernel, int device, int bytes)
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) done.emplace_back(kernel, device);
     return e;
+}
+
+bool cluster_fits(const void *kernel, int device, int ctas, int threads, int smem_bytes)
+{
+    struct Asked {
+        const void *kernel;
+        int device, ctas;
+        bool fits;
+    };
+    static std::mutex mu;
+    static std::vector<Asked> done;
+    std::lock_guard<std::mutex> lock(mu);
+    for (const Asked &d : done)
+        if (d.kernel == kernel && d.device == device && d.ctas == ctas) return d.fits;
+    int n = 0;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(ctas);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem_bytes;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = ctas;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+    }
+    if (e != cudaSuccess) cudaGetLastError();  // (not an error of the caller's: the lattice is stepped launch by launch)
+    done.push_back({kernel, device, ctas, e == cudaSuccess && n > 0});
+    return done.back().fits;
 }
 
 // psi of the EOS of *p at rho (the host evaluation create uses), for lbm_lbana.cu.

@@ -58,7 +58,8 @@ struct Divisor {
         return ok && in_range(a) ? q : a / b;
     }
 };
-__device__ __forceinline__ Divisor divisor(double b) { return Divisor{b, __drcp_rn(b), in_range(b) && b != 0.0}; }
+__device__ __forceinline__ bool is_nonzero(double b) { return (((unsigned)__double2hiint(b) & 0x7fffffffu) | (unsigned)__double2loint(b)) != 0u; }
+__device__ __forceinline__ Divisor divisor(double b) { return Divisor{b, __drcp_rn(b), in_range(b) && is_nonzero(b)}; }
 
 __device__ __forceinline__ double density(const double (&f)[9])
 {
@@ -70,53 +71,69 @@ __device__ __forceinline__ double density(const double (&f)[9])
 
 __device__ __forceinline__ double p_eos(const KParams &kp, double rho)
 {
-    if (kp.eos == 0) return kp.eos_K * (rho * kp.eos_R * kp.eos_T / (1.0 - kp.eos_b * rho) - kp.eos_a * rho * rho);
-    const double eta = kp.eos_b * rho * 0.25;
+    // products by a gas constant or a K of 1 (the usual ones) change nothing and are left out
+    const double rRT = (kp.unit_R ? rho : rho * kp.eos_R) * kp.eos_T;
+    if (kp.eos == 0) {
+        const double p = rRT / (1.0 - kp.eos_b * rho) - kp.eos_a * rho * rho;
+        return kp.unit_K ? p : kp.eos_K * p;
+    }
+    const double eta = kp.eos_b4 * rho;
     const double e2 = eta * eta, om = 1.0 - eta;
     const double num = 1.0 + eta + e2 - e2 * eta;
     const double den = om * om * om;
-    return kp.eos_K * (rho * kp.eos_R * kp.eos_T * num / den - kp.eos_a * rho * rho);
+    const double p = rRT * num / den - kp.eos_a * rho * rho;
+    return kp.unit_K ? p : kp.eos_K * p;
 }
 
 // sqrt(2 (p_EOS - rho/3)/G); a G that is a power of two (the usual -1) divides exactly
 __device__ __forceinline__ double psi_of(const KParams &kp, double rho)
 {
-    const double d = 2.0 * (p_eos(kp, rho) - div_const<3>(rho));
-    return sqrt(kp.G_pow2 ? d * kp.inv_G : d / kp.G);
+    const double d = p_eos(kp, rho) - div_const<3>(rho);
+    return sqrt(kp.G_pow2 ? d * kp.two_inv_G : 2.0 * d / kp.G);
 }
 
+// S of Eq. (fint), the terms in the order i = 1..8
+template <class Ps>
+__device__ __forceinline__ double stencil_x(const Ps &ps)
+{
+    const double w1 = 1.0 / 3.0, w5 = 1.0 / 12.0;
+    return w1 * ps(1) - w1 * ps(3) + w5 * ps(5) - w5 * ps(6) - w5 * ps(7) + w5 * ps(8);
+}
+template <class Ps>
+__device__ __forceinline__ double stencil_y(const Ps &ps)
+{
+    const double w1 = 1.0 / 3.0, w5 = 1.0 / 12.0;
+    return w1 * ps(2) - w1 * ps(4) + w5 * ps(5) + w5 * ps(6) - w5 * ps(7) - w5 * ps(8);
+}
 template <class Ps>
 __device__ __forceinline__ void stencil_S(const Ps &ps, double &Sx, double &Sy)
 {
-    double sx = 0.0, sy = 0.0;
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        const double p = ((i <= 4) ? 1.0 / 3.0 : 1.0 / 12.0) * ps(i);
-        if (ex_(i)) sx = i == 1 ? p : (ex_(i) > 0 ? sx + p : sx - p);
-        if (ey_(i)) sy = i == 2 ? p : (ey_(i) > 0 ? sy + p : sy - p);
-    }
-    Sx = sx;
-    Sy = sy;
+    Sx = stencil_x(ps);
+    Sy = stencil_y(ps);
 }
 
-// f = M^T (m_k/|M_k|^2), the terms in the order k = 0..8.  u_k is m_k/|M_k|^2 without its power of
+// f = M^T (m_k/|M_k|^2), the terms in the order k = 0..8, from u_k = m_k/|M_k|^2 without its power of
 // two (|M_k|^2 = 9, 36, 36, 6, 12, 6, 12, 4, 4), which the multiply-adds carry exactly.
+__device__ __forceinline__ void populations(const double (&u)[9], double (&f)[9])
+{
+    f[0] = (u[0] - u[1]) + u[2];
+    const double a = fma_(-0.5, u[2], fma_(-0.25, u[1], u[0]));  // axes
+    f[1] = fma_(0.25, u[7], fma_(-0.5, u[4], fma_(0.5, u[3], a)));
+    f[2] = fma_(-0.25, u[7], fma_(-0.5, u[6], fma_(0.5, u[5], a)));
+    f[3] = fma_(0.25, u[7], fma_(0.5, u[4], fma_(-0.5, u[3], a)));
+    f[4] = fma_(-0.25, u[7], fma_(0.5, u[6], fma_(-0.5, u[5], a)));
+    const double d = fma_(0.25, u[2], fma_(0.5, u[1], u[0]));    // diagonals
+    const double p = fma_(0.25, u[4], fma_(0.5, u[3], d)), q = fma_(-0.25, u[4], fma_(-0.5, u[3], d));
+    f[5] = fma_(0.25, u[8], fma_(0.25, u[6], fma_(0.5, u[5], p)));
+    f[6] = fma_(-0.25, u[8], fma_(0.25, u[6], fma_(0.5, u[5], q)));
+    f[7] = fma_(0.25, u[8], fma_(-0.25, u[6], fma_(-0.5, u[5], q)));
+    f[8] = fma_(-0.25, u[8], fma_(-0.25, u[6], fma_(-0.5, u[5], p)));
+}
 __device__ __forceinline__ void from_moments(const double (&m)[9], double (&f)[9])
 {
-    const double u0 = div_const<9>(m[0]), u1 = div_const<9>(m[1]), u2 = div_const<9>(m[2]);
-    const double u3 = div_const<3>(m[3]), u4 = div_const<3>(m[4]), u5 = div_const<3>(m[5]), u6 = div_const<3>(m[6]);
-    f[0] = (u0 - u1) + u2;
-    const double a = fma_(-0.5, u2, fma_(-0.25, u1, u0));  // axes
-    f[1] = fma_(0.25, m[7], fma_(-0.5, u4, fma_(0.5, u3, a)));
-    f[2] = fma_(-0.25, m[7], fma_(-0.5, u6, fma_(0.5, u5, a)));
-    f[3] = fma_(0.25, m[7], fma_(0.5, u4, fma_(-0.5, u3, a)));
-    f[4] = fma_(-0.25, m[7], fma_(0.5, u6, fma_(-0.5, u5, a)));
-    const double d = fma_(0.25, u2, fma_(0.5, u1, u0));    // diagonals
-    const double p = fma_(0.25, u4, fma_(0.5, u3, d)), q = fma_(-0.25, u4, fma_(-0.5, u3, d));
-    f[5] = fma_(0.25, m[8], fma_(0.25, u6, fma_(0.5, u5, p)));
-    f[6] = fma_(-0.25, m[8], fma_(0.25, u6, fma_(0.5, u5, q)));
-    f[7] = fma_(0.25, m[8], fma_(-0.25, u6, fma_(-0.5, u5, q)));
-    f[8] = fma_(-0.25, m[8], fma_(-0.25, u6, fma_(-0.5, u5, p)));
+    const double u[9] = {div_const<9>(m[0]), div_const<9>(m[1]), div_const<9>(m[2]), div_const<3>(m[3]), div_const<3>(m[4]),
+                         div_const<3>(m[5]), div_const<3>(m[6]), m[7], m[8]};
+    populations(u, f);
 }
 
 __device__ __forceinline__ void equilibrium_moments(double rho, double ux, double uy, double (&meq)[9])
@@ -141,15 +158,11 @@ __device__ __forceinline__ void equilibrium(double rho, double ux, double uy, do
     from_moments(meq, fb);
 }
 
-__device__ __forceinline__ void collide(const KParams &kp, const double (&f)[9], double psi, double Sx, double Sy,
-                                        double Fex, double Fey, double (&fb)[9], double &uxo, double &uyo)
+// ---- the collision, in the pieces that k_small1 spreads over four warps.
+// m_1 and m_2 of M f, the terms in the order i = 0..8
+__device__ __forceinline__ void moments_12(const double (&f)[9], double &m1, double &m2)
 {
-    const double rho = density(f);
-    const Divisor by_rho = divisor(rho);
-    // m = M f, the terms in the order i = 0..8 (m_0 = rho, m_3 = j_x, m_5 = j_y)
-    const double jx = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];
-    const double jy = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];
-    double m1 = -4.0 * f[0], m2 = 4.0 * f[0];
+    m1 = -4.0 * f[0], m2 = 4.0 * f[0];
 #pragma unroll
     for (int i = 1; i < 5; ++i) {
         m1 -= f[i];
@@ -160,6 +173,63 @@ __device__ __forceinline__ void collide(const KParams &kp, const double (&f)[9],
         m1 = fma_(2.0, f[i], m1);
         m2 += f[i];
     }
+}
+// s_p and s_q of two relaxation times
+__device__ __forceinline__ void relaxation(const KParams &kp, double rho, double &sp, double &sq)
+{
+    double w = (rho - kp.rho_g) / (kp.rho_l - kp.rho_g);
+    w = w < 0.0 ? 0.0 : (w > 1.0 ? 1.0 : w);
+    const double nu = kp.nu_g + w * (kp.nu_l - kp.nu_g);
+    const double tau = 3.0 * nu + 0.5;
+    sp = 1.0 / tau;
+    sq = 1.0 / (0.5 + kp.Lambda / (tau - 0.5));
+}
+// m_bar_k = m + F_m - s (m - m_eq + F_m/2) + s Q (Eq. lbe.col), Q_m with |F_int|^2 / (G psi^2) as written
+// in the paper (X = F_int,x^2 / (G psi^2), Y likewise)
+__device__ __forceinline__ void relaxed_12(const KParams &kp, double rho, double m1, double m2, double Fx, double Fy, double ux,
+                                           double uy, double X, double Y, double sp, double &a1, double &a2)
+{
+    const double u2 = ux * ux + uy * uy, r3u2 = 3.0 * rho * u2;
+    const double meq1 = fma_(-2.0, rho, r3u2), meq2 = rho - r3u2;
+    const double Fm1 = 6.0 * (Fx * ux + Fy * uy);  // F_m2 = -F_m1
+    const double sQ1 = sp * (kp.q1c * (X + Y));
+    a1 = (m1 + Fm1) - sp * fma_(0.5, Fm1, m1 - meq1) + sQ1;
+    const double c2 = (m2 - Fm1) - sp * fma_(-0.5, Fm1, m2 - meq2);
+    a2 = kp.q2_full ? c2 - sQ1 : fma_(-0.5, sQ1, c2);  // Q_2 = -Q_1 or -Q_1/2
+}
+// one direction's momentum (s_j = 1) and energy flux; X along it, Y across
+__device__ __forceinline__ void relaxed_jq(const KParams &kp, double rho, double j, double q, double F, double u, double X,
+                                           double Y, double sq, double &aj, double &aq)
+{
+    const double ru = rho * u;
+    aj = (j + F) - fma_(0.5, F, j - ru);
+    aq = (q - F) - sq * fma_(-0.5, F, q + ru);
+    if (kp.improved) aq += sq * ((kp.q4a * X - kp.q4b * Y) * u);
+}
+__device__ __forceinline__ void relaxed_78(const KParams &kp, double rho, double m7, double m8, double Fx, double Fy, double ux,
+                                           double uy, double Fix, double Fiy, const Divisor &by_Gpsi2, double sp, double &a7,
+                                           double &a8)
+{
+    const double rux = rho * ux, ruy = rho * uy;
+    const double meq7 = rux * ux - ruy * uy, meq8 = rux * uy;
+    const double h7 = Fx * ux - Fy * uy;  // F_m7/2
+    const double Fm8 = Fx * uy + Fy * ux;
+    const double Q7 = by_Gpsi2(kp.k1 * (Fix * Fix - Fiy * Fiy));
+    const double Q8 = by_Gpsi2(kp.k1 * Fix * Fiy);
+    a7 = fma_(2.0, h7, m7) - sp * ((m7 - meq7) + h7) + sp * Q7;
+    a8 = (m8 + Fm8) - sp * fma_(0.5, Fm8, m8 - meq8) + sp * Q8;
+}
+
+__device__ __forceinline__ void collide(const KParams &kp, const double (&f)[9], double psi, double Sx, double Sy,
+                                        double Fex, double Fey, double (&fb)[9], double &ux, double &uy)
+{
+    const double rho = density(f);
+    const Divisor by_rho = divisor(rho);
+    // m = M f, the terms in the order i = 0..8 (m_0 = rho, m_3 = j_x, m_5 = j_y)
+    const double jx = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];
+    const double jy = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];
+    double m1, m2;
+    moments_12(f, m1, m2);
     const double m4 = fma_(2.0, f[3], -2.0 * f[1]) + f[5] - f[6] - f[7] + f[8];
     const double m6 = fma_(2.0, f[4], -2.0 * f[2]) + f[5] + f[6] - f[7] - f[8];
     const double m7 = f[1] - f[2] + f[3] - f[4], m8 = f[5] - f[6] + f[7] - f[8];
@@ -167,48 +237,18 @@ __device__ __forceinline__ void collide(const KParams &kp, const double (&f)[9],
     const double Gpsi = kp.G * psi;
     const double Fix = -Gpsi * Sx, Fiy = -Gpsi * Sy;
     const double Fx = Fix + Fex, Fy = Fiy + Fey;
-    const double ux = by_rho(fma_(0.5, Fx, jx)), uy = by_rho(fma_(0.5, Fy, jy));
-    double meq[9];
-    equilibrium_moments(rho, ux, uy, meq);
-    const double Fxu = Fx * ux, Fyv = Fy * uy;
-    const double Fm1 = 6.0 * (Fxu + Fyv), h7 = Fxu - Fyv;  // h7 = F_m7/2
-    const double Fm8 = Fx * uy + Fy * ux;
-    // Q_m with |F_int|^2 / (G psi^2) as written in the paper
+    ux = by_rho(fma_(0.5, Fx, jx)), uy = by_rho(fma_(0.5, Fy, jy));
     const Divisor by_Gpsi2 = divisor(Gpsi * psi);
-    const double Fix2 = Fix * Fix, Fiy2 = Fiy * Fiy;
-    const double X = by_Gpsi2(Fix2), Y = by_Gpsi2(Fiy2);
-    const double Q1 = kp.q1c * (X + Y);
-    const double Q7 = by_Gpsi2(kp.k1 * (Fix2 - Fiy2));
-    const double Q8 = by_Gpsi2(kp.k1 * Fix * Fiy);
+    const double X = by_Gpsi2(Fix * Fix), Y = by_Gpsi2(Fiy * Fiy);
     double sp = kp.sp, sq = kp.sq;
-    if (kp.var_tau) {
-        double w = (rho - kp.rho_g) / (kp.rho_l - kp.rho_g);
-        w = w < 0.0 ? 0.0 : (w > 1.0 ? 1.0 : w);
-        const double nu = kp.nu_g + w * (kp.nu_l - kp.nu_g);
-        const double tau = 3.0 * nu + 0.5;
-        sp = 1.0 / tau;
-        sq = 1.0 / (0.5 + kp.Lambda / (tau - 0.5));
-    }
-    // m_bar_k = m + F_m - s (m - m_eq + F_m/2) + s Q (Eq. lbe.col); s_0 = s_j = 1
-    const double sQ1 = sp * Q1;
+    if (kp.var_tau) relaxation(kp, rho, sp, sq);
     double mb[9];
     mb[0] = rho;
-    mb[1] = (m1 + Fm1) - sp * fma_(0.5, Fm1, m1 - meq[1]) + sQ1;
-    const double c2 = (m2 - Fm1) - sp * fma_(-0.5, Fm1, m2 - meq[2]);
-    mb[2] = kp.q2fac == -1.0 ? c2 - sQ1 : fma_(-0.5, sQ1, c2);
-    mb[3] = (jx + Fx) - fma_(0.5, Fx, jx - meq[3]);
-    mb[5] = (jy + Fy) - fma_(0.5, Fy, jy - meq[5]);
-    mb[4] = (m4 - Fx) - sq * fma_(-0.5, Fx, m4 - meq[4]);
-    mb[6] = (m6 - Fy) - sq * fma_(-0.5, Fy, m6 - meq[6]);
-    if (kp.improved) {
-        mb[4] += sq * ((kp.q4a * X - kp.q4b * Y) * ux);
-        mb[6] += sq * ((kp.q4a * Y - kp.q4b * X) * uy);
-    }
-    mb[7] = fma_(2.0, h7, m7) - sp * ((m7 - meq[7]) + h7) + sp * Q7;
-    mb[8] = (m8 + Fm8) - sp * fma_(0.5, Fm8, m8 - meq[8]) + sp * Q8;
+    relaxed_12(kp, rho, m1, m2, Fx, Fy, ux, uy, X, Y, sp, mb[1], mb[2]);
+    relaxed_jq(kp, rho, jx, m4, Fx, ux, X, Y, sq, mb[3], mb[4]);
+    relaxed_jq(kp, rho, jy, m6, Fy, uy, Y, X, sq, mb[5], mb[6]);
+    relaxed_78(kp, rho, m7, m8, Fx, Fy, ux, uy, Fix, Fiy, by_Gpsi2, sp, mb[7], mb[8]);
     from_moments(mb, fb);
-    uxo = ux;
-    uyo = uy;
 }
 
 }  // namespace f64

@@ -50,8 +50,11 @@ struct KParams {
     double G;
     double k1, k2;        // raw source coefficients (FP64 path)
     double q1c, q4a, q4b;  // 3 (k1 + 2 k2), (30 eps - 15)/16, 3 eps/8 (FP64 path, evaluated on the host)
-    double inv_G;          // 1/G
-    int G_pow2;            // 1: G is +- a power of two, so that x/G = x inv_G exactly
+    double two_inv_G;      // 2/G
+    int G_pow2;            // 1: G is +- a power of two, so that 2 x/G = x two_inv_G exactly
+    double eos_b4;         // b/4
+    int unit_R, unit_K;    // R = 1, K = 1
+    int q2_full;           // 1: Q_2 = -Q_1; 0: -Q_1/2
     // source term with G folded in (|F_int|^2/(G psi^2) = G |S|^2, S = F_int/(-G psi)):
     // Q1 = kq1 |S|^2, Q2 = q2fac Q1, Q7 = kq7 (Sx^2 - Sy^2), Q8 = kq7 Sx Sy,
     // Q4 = (c1G Sx^2 - c2G Sy^2) ux, Q6 = (c1G Sy^2 - c2G Sx^2) uy
@@ -135,6 +138,10 @@ inline cudaError_t ensure_smem_attribute(K kernel, int device, int bytes)
     return ensure_smem_attribute_ptr(reinterpret_cast<const void *>(kernel), device, bytes);
 }
 
+// Whether the device can hold a cluster of `ctas` blocks of the kernel with these limits (shared memory
+// and cluster size are then allowed for it), asked once per kernel, device and size; lbm_api.cu.
+bool cluster_fits(const void *kernel, int device, int ctas, int threads, int smem_bytes);
+
 // Launchers, defined in the per-precision translation units (k_f64.cu, k_f32.cu,
 // k_f16.cu).  All run on `st` and return the launch status.
 struct Launchers {
@@ -142,6 +149,9 @@ struct Launchers {
     cudaError_t (*collide_pass)(const KParams &, cudaStream_t);
     cudaError_t (*fused_pass)(const KParams &, cudaStream_t);  // staged one-pass step (periodic, FP32 arithmetic); null in FP64
     cudaError_t (*tile_pass)(const KParams &, cudaStream_t);   // one-pass step on tiles (k_tile.cuh)
+    // many steps of a small lattice in one launch (k_small.cuh); small_ctas: 0 where it does not fit
+    int (*small_ctas)(const KParams &);
+    cudaError_t (*small_steps)(const KParams &, int ctas, int64_t nsteps, int64_t step0, cudaStream_t);
     cudaError_t (*link_bits)(const KParams &, uint16_t *out, cudaStream_t);  // KParams::links
     cudaError_t (*init)(const KParams &, const double *rho, const double *ux, const double *uy,
                         cudaStream_t);
