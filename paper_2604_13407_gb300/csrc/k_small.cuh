@@ -228,11 +228,9 @@ __global__ void __launch_bounds__(kSmallThreads) k_small2(KParams kp, int64_t ns
     const StripNode<S> a(s, t0 < pairs ? t0 : s.m * s.nx), b(s, t0 < pairs ? t0 + pairs : s.m * s.nx);
     // which half of its pair's random word each node takes: its column's parity
     const unsigned pick = (a.c0 & 1u ? 0x32u : 0x10u) | (b.c0 & 1u ? 0x7600u : 0x5400u);
-    // psi of solid nodes (the FP64 field is converted once, not per step)
-    const float wall_a = (a.w & 1u) && kp.wall_psi ? float(kp.wall_psi[a.node]) : kp.cf.psi_s;
-    const float wall_b = (b.w & 1u) && kp.wall_psi ? float(kp.wall_psi[b.node]) : kp.cf.psi_s;
+    const float wall_a = (a.w & 1u) && kp.wall_psi_f ? kp.wall_psi_f[a.node] : kp.cf.psi_s;  // psi of solid nodes
+    const float wall_b = (b.w & 1u) && kp.wall_psi_f ? kp.wall_psi_f[b.node] : kp.cf.psi_s;
 
-    v2x fx = X2(0.f, 0.f), fy = fx;  // force field at the nodes
     for (int64_t t = 0; t < nsteps; ++t) {
         float fa[9], fb[9];
         a.pull(s, fa);
@@ -260,13 +258,10 @@ __global__ void __launch_bounds__(kSmallThreads) k_small2(KParams kp, int64_t ns
         } else if (kp.force_mode == 1) {
             const v2x x = rho - v2x{kp.c2.rho_g};
             Fex = x * v2x{kp.c2.Fx}, Fey = x * v2x{kp.c2.Fy};
-        } else if (kp.fext) {
+        } else if (kp.fext_f) {
             const int64_t n = (int64_t)kp.nx * kp.ny;
-            if (t == 0) {
-                fx = X2(float(kp.fext[a.node]), float(kp.fext[b.node]));
-                fy = X2(float(kp.fext[n + a.node]), float(kp.fext[n + b.node]));
-            }
-            Fex = fx, Fey = fy;
+            Fex = X2(kp.fext_f[a.node], kp.fext_f[b.node]);
+            Fey = X2(kp.fext_f[n + a.node], kp.fext_f[n + b.node]);
         } else {
             Fex = Fey = X2(0.f, 0.f);
         }

@@ -246,14 +246,6 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
         ax = x0 - 1, bx = x0 + kTileX, ay = by = y0 + r - 1;
         ra = rb = r, ca = 0, cb = kTileX + 1;
     }
-    if (ahead > 0 && warp < np && lane < 18) {
-        // the lines of the tile that a block of the next wave will pull (row y, columns x0 .. x0 + 31)
-        const int i = lane < 9 ? lane : lane - 9, y = ay + (lane < 9 ? 0 : 1) + ahead;
-        if (y < kp.ny) {
-            const S *p = static_cast<const S *>(kp.src) + (i * kp.plane + (int64_t)y * kp.pitch + x0);
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-        }
-    }
     Site a{ax, ay, true}, b{bx, by, true};
     if constexpr (!INNER) a = site_of(kp, ax, ay), b = site_of(kp, bx, by);
     const uint32_t node_a = (uint32_t)a.y * (uint32_t)kp.nx + a.x, node_b = (uint32_t)b.y * (uint32_t)kp.nx + b.x;
@@ -262,113 +254,136 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
     const bool masked = GEOM == 3 ? kp.links != nullptr : GEOM != 0;
     if (masked) wa = kp.links[node_a], wb = kp.links[node_b];
 
-    // pull, Eq. (lbe.str)
-    const S *src = static_cast<const S *>(kp.src);
-    v2x f[9];
-    S va[9], vb[9];
-    float refa[9], refb[9];
-    if constexpr (INNER) {
-        const char *pa = reinterpret_cast<const char *>(src + ka), *pb = reinterpret_cast<const char *>(src + kb);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            va[i] = reinterpret_cast<const S *>(pa + kp.pull[i])[-ex_(i)];
-            vb[i] = reinterpret_cast<const S *>(pb + kp.pull[i])[-ex_(i)];
-        }
-        if (has_ref) {
-            const float *qa = kp.ref_src + ka, *qb = kp.ref_src + kb;
-            const int64_t P = kp.pitch;
-            if (warp < np) {  // rows y and y + 1: twelve references for both nodes
-#pragma unroll
-                for (int d = -1; d <= 1; ++d) {
-                    const int up = d < 0 ? 5 : d > 0 ? 6 : 2, in = d < 0 ? 1 : d > 0 ? 3 : 0, dn = d < 0 ? 8 : d > 0 ? 7 : 4;
-                    refa[up] = (qa - P)[d];
-                    refa[in] = refb[up] = qa[d];
-                    refa[dn] = refb[in] = qb[d];
-                    refb[dn] = (qb + P)[d];
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < 9; ++i) refa[i] = (qa - ey_(i) * P)[-ex_(i)], refb[i] = (qb - ey_(i) * P)[-ex_(i)];
-            }
-        }
-    } else {
-        unsigned ia, ib;
-        const Nine na = nine_of(kp, a, ia), nb = nine_of(kp, b, ib);
-        if (!masked) wa = edge_walls(ia), wb = edge_walls(ib);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const S *p = src + i * kp.plane;
-            va[i] = p[na.from(i)], vb[i] = p[nb.from(i)];
-            if (has_ref) refa[i] = kp.ref_src[na.from(i)], refb[i] = kp.ref_src[nb.from(i)];
+    // Up to here nothing that a step writes was read: the launch waits for the one before it now.
+    if constexpr (MODE == TILE_STEP) {
+        grid_dependency_wait();
+        allow_dependent_launch();
+    }
+    // A warp whose nodes are all solid has nothing to pull: psi is the walls'.  Only where solid nodes are
+    // many (KParams::skip_solid), since the others' pulls then wait for the wall bits: annulus 1024^2 (a
+    // third solid) 19.6 -> 17.0 us, FP16 23.8 -> 21.3; banded 2048^2 (0.1 %) 59.2 -> 63 with it.
+    const bool still = masked && kp.skip_solid && __all_sync(0xffffffffu, (wa & 1u) && (wb & 1u));
+    if (ahead > 0 && warp < np && lane < (masked ? 20 : 18)) {
+        // the lines of the tile that a block of the next wave will read (rows y and y + 1, columns x0 ..
+        // x0 + 31): the nine planes, and the wall bits
+        const int i = lane >> 1, y = ay + (lane & 1) + ahead;
+        if (y < kp.ny) {
+            const void *p = i < 9 ? (const void *)(static_cast<const S *>(kp.src) + (i * kp.plane + (int64_t)y * kp.pitch + x0))
+                                  : (const void *)(kp.links + ((int64_t)y * kp.nx + x0));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
         }
     }
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        v2x wr = X2(0.f, 0.f);
-        if (DEV) wr = has_ref ? v2x{kp.c2.w[i]} * X2(refa[i], refb[i]) : v2x{kp.c2.dec[i]};
-        f[i] = X2(Raw<S>::f(va[i], wr.v.x, kp), Raw<S>::f(vb[i], wr.v.y, kp));
-    }
+    v2x f[9], d[9], rho = X2(1.f, 1.f), psi = X2(0.f, 0.f);
     v2x momx = X2(0.f, 0.f), momy = momx;  // momentum handed to the walls (diagnostics)
-    if ((!INNER || GEOM) && ((wa | wb) & 0x1feu)) {
-        // wall links: the population that left the node toward the wall comes back
+    if (!still) {
+        // pull, Eq. (lbe.str)
+        const S *src = static_cast<const S *>(kp.src);
+        S va[9], vb[9];
+        float refa[9], refb[9];
+        if constexpr (INNER) {
+            const char *pa = reinterpret_cast<const char *>(src + ka), *pb = reinterpret_cast<const char *>(src + kb);
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const unsigned w = e ? wb : wa;
-            if (!(w & 0x1feu) || (w & 1u)) continue;
-            const uint32_t k = e ? kb : ka;
-            auto own = [&](int i) -> float {
-                float wr = 0.f;
-                if (DEV) wr = __fmul_rn(w_<float>(i), has_ref ? (e ? refb[0] : refa[0]) : kp.cf.rho_ref);
-                return Raw<S>::f((src + i * kp.plane)[k], wr, kp);
-            };
-            float rho_w = 0.f;
-            bool summed = false;
+            for (int i = 0; i < 9; ++i) {
+                va[i] = reinterpret_cast<const S *>(pa + kp.pull[i])[-ex_(i)];
+                vb[i] = reinterpret_cast<const S *>(pb + kp.pull[i])[-ex_(i)];
+            }
+            if (has_ref) {
+                const float *qa = kp.ref_src + ka, *qb = kp.ref_src + kb;
+                const int64_t P = kp.pitch;
+                if (warp < np) {  // rows y and y + 1: twelve references for both nodes
 #pragma unroll
-            for (int i = 1; i < 9; ++i) {
-                if (!((w >> i) & 1u)) continue;
-                const int o = opp_(i);
-                const float fo = own(o);
-                float g = fo + 0.f;
-                if constexpr (GEOM >= 2) if (GEOM == 2 || kp.link != nullptr) {
-                    // interpolated or moving wall: link fraction and moving-wall coefficient
-                    const float2 lk = kp.link[(int64_t)(i - 1) * kp.plane + k];
-                    float mw = 0.f;
-                    if (lk.y != 0.f) {
-                        if (!summed) {
-#pragma unroll
-                            for (int n = 0; n < 9; ++n) rho_w += own(n);
-                            summed = true;
-                        }
-                        mw = lk.y * rho_w;
+                    for (int d = -1; d <= 1; ++d) {
+                        const int up = d < 0 ? 5 : d > 0 ? 6 : 2, in = d < 0 ? 1 : d > 0 ? 3 : 0, dn = d < 0 ? 8 : d > 0 ? 7 : 4;
+                        refa[up] = (qa - P)[d];
+                        refa[in] = refb[up] = qa[d];
+                        refa[dn] = refb[in] = qb[d];
+                        refb[dn] = (qb + P)[d];
                     }
-                    const float q = lk.x;
-                    if (q < 0.5f) {
-                        // fbar_o of the second node x + e_i (fluid: the record's q is 1/2 otherwise), which
-                        // is what the pull of population o brought here
-                        const float f2 = e ? f[o].v.y : f[o].v.x;
-                        g = 2.f * q * fo + (1.f - 2.f * q) * f2 + mw;
-                    } else if (q == 0.5f) {
-                        g = fo + mw;
-                    } else {
-                        g = fo / (2.f * q) + (2.f * q - 1.f) / (2.f * q) * own(i) + mw / (2.f * q);
-                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) refa[i] = (qa - ey_(i) * P)[-ex_(i)], refb[i] = (qb - ey_(i) * P)[-ex_(i)];
                 }
-                if (e) f[i].v.y = g;
-                else f[i].v.x = g;
-                if constexpr (MODE == TILE_DIAG) {
-                    float &mx = e ? momx.v.y : momx.v.x, &my = e ? momy.v.y : momy.v.x;
-                    mx += -float(ex_(i)) * (fo + g), my += -float(ey_(i)) * (fo + g);
+            }
+        } else {
+            unsigned ia, ib;
+            const Nine na = nine_of(kp, a, ia), nb = nine_of(kp, b, ib);
+            if (!masked) wa = edge_walls(ia), wb = edge_walls(ib);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const S *p = src + i * kp.plane;
+                va[i] = p[na.from(i)], vb[i] = p[nb.from(i)];
+                if (has_ref) refa[i] = kp.ref_src[na.from(i)], refb[i] = kp.ref_src[nb.from(i)];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            v2x wr = X2(0.f, 0.f);
+            if (DEV) wr = has_ref ? v2x{kp.c2.w[i]} * X2(refa[i], refb[i]) : v2x{kp.c2.dec[i]};
+            f[i] = X2(Raw<S>::f(va[i], wr.v.x, kp), Raw<S>::f(vb[i], wr.v.y, kp));
+        }
+        if ((!INNER || GEOM) && ((wa | wb) & 0x1feu)) {
+            // wall links: the population that left the node toward the wall comes back
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const unsigned w = e ? wb : wa;
+                if (!(w & 0x1feu) || (w & 1u)) continue;
+                const uint32_t k = e ? kb : ka;
+                auto own = [&](int i) -> float {
+                    float wr = 0.f;
+                    if (DEV) wr = __fmul_rn(w_<float>(i), has_ref ? (e ? refb[0] : refa[0]) : kp.cf.rho_ref);
+                    return Raw<S>::f((src + i * kp.plane)[k], wr, kp);
+                };
+                float rho_w = 0.f;
+                bool summed = false;
+#pragma unroll
+                for (int i = 1; i < 9; ++i) {
+                    if (!((w >> i) & 1u)) continue;
+                    const int o = opp_(i);
+                    const float fo = own(o);
+                    float g = fo + 0.f;
+                    if constexpr (GEOM >= 2) if (GEOM == 2 || kp.link != nullptr) {
+                        // interpolated or moving wall: link fraction and moving-wall coefficient
+                        const float2 lk = kp.link[(int64_t)(i - 1) * kp.plane + k];
+                        float mw = 0.f;
+                        if (lk.y != 0.f) {
+                            if (!summed) {
+#pragma unroll
+                                for (int n = 0; n < 9; ++n) rho_w += own(n);
+                                summed = true;
+                            }
+                            mw = lk.y * rho_w;
+                        }
+                        const float q = lk.x;
+                        if (q < 0.5f) {
+                            // fbar_o of the second node x + e_i (fluid: the record's q is 1/2 otherwise), which
+                            // is what the pull of population o brought here
+                            const float f2 = e ? f[o].v.y : f[o].v.x;
+                            g = 2.f * q * fo + (1.f - 2.f * q) * f2 + mw;
+                        } else if (q == 0.5f) {
+                            g = fo + mw;
+                        } else {
+                            g = fo / (2.f * q) + (2.f * q - 1.f) / (2.f * q) * own(i) + mw / (2.f * q);
+                        }
+                    }
+                    if (e) f[i].v.y = g;
+                    else f[i].v.x = g;
+                    if constexpr (MODE == TILE_DIAG) {
+                        float &mx = e ? momx.v.y : momx.v.x, &my = e ? momy.v.y : momy.v.x;
+                        mx += -float(ex_(i)) * (fo + g), my += -float(ey_(i)) * (fo + g);
+                    }
                 }
             }
         }
+        to_dev(f, d);
+        rho = density_dev(d);
+        psi = psi_v<v2x>(kp, rho);
+    } else if constexpr (MODE == TILE_DIAG) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i] = X2(0.f, 0.f);
     }
-    v2x d[9];
-    to_dev(f, d);
-    v2x rho = density_dev(d);
-    v2x psi = psi_v<v2x>(kp, rho);
     if (GEOM) {
-        if (wa & 1u) psi.v.x = kp.wall_psi ? float(kp.wall_psi[node_a]) : kp.cf.psi_s, rho.v.x = 1.f;
-        if (wb & 1u) psi.v.y = kp.wall_psi ? float(kp.wall_psi[node_b]) : kp.cf.psi_s, rho.v.y = 1.f;
+        if (wa & 1u) psi.v.x = kp.wall_psi_f ? kp.wall_psi_f[node_a] : kp.cf.psi_s, rho.v.x = 1.f;
+        if (wb & 1u) psi.v.y = kp.wall_psi_f ? kp.wall_psi_f[node_b] : kp.cf.psi_s, rho.v.y = 1.f;
     }
     if (!INNER && !a.in) psi.v.x = kp.cf.psi_s;
     if (!INNER && !b.in) psi.v.y = kp.cf.psi_s;
@@ -405,10 +420,10 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
     } else if (mode == 1) {  // Sec. 3.3: (rho - rho_g) g
         const v2x e = rho - v2x{kp.c2.rho_g};
         Fex = e * v2x{kp.c2.Fx}, Fey = e * v2x{kp.c2.Fy};
-    } else if (kp.fext) {
+    } else if (kp.fext_f) {
         const int64_t n = (int64_t)kp.nx * kp.ny;
-        Fex = X2(float(kp.fext[node_a]), float(kp.fext[node_b]));
-        Fey = X2(float(kp.fext[n + node_a]), float(kp.fext[n + node_b]));
+        Fex = X2(kp.fext_f[node_a], kp.fext_f[node_b]);
+        Fey = X2(kp.fext_f[n + node_a], kp.fext_f[n + node_b]);
     } else {
         Fex = Fey = X2(0.f, 0.f);
     }
@@ -510,8 +525,6 @@ template <class S, int GEOM, class O>
 __global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, int ahead)
 {
     __shared__ Tile2Shared sh;
-    grid_dependency_wait();
-    allow_dependent_launch();
     const TileOut none{};
     if (tile_inner(kp, 2 * ((blockDim.x >> 5) - 2))) tile2_block<S, GEOM, O, TILE_STEP, true>(kp, ahead, none, sh);
     else tile2_block<S, GEOM, O, TILE_STEP, false>(kp, ahead, none, sh);

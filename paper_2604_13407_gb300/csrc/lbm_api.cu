@@ -33,6 +33,7 @@ struct lbm_ctx {
     uint8_t *solid = nullptr;
     double *wall_u = nullptr, *q = nullptr, *fext = nullptr;
     double *wall_rho = nullptr, *wall_psi = nullptr;  // per solid node virtual density, its psi
+    float *fext_f = nullptr, *wall_psi_f = nullptr;   // fext and wall_psi in FP32 (not for FP64 storage)
     float2 *link = nullptr;             // wall-link records of the tile kernel (KParams::link)
     uint16_t *links = nullptr;          // wall bits of every node (KParams::links)
     double *dacc = nullptr;             // diagnostics: 9 sums, max |u|, count of non-finite nodes
@@ -259,8 +260,11 @@ static void fill_constants(lbm_ctx *c)
     k.fext = c->fext;
     k.wall_rho = c->wall_rho;
     k.wall_psi = c->wall_psi;
+    k.fext_f = c->fext_f;
+    k.wall_psi_f = c->wall_psi_f;
     k.link = c->link;
     k.links = c->links;
+    k.skip_solid = c->n_fluid * 8 < (int64_t)p.nx * p.ny * 7;
     k.err = c->derr;
 }
 
@@ -325,7 +329,7 @@ static void free_all(lbm_ctx *c)
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
     void *bufs[] = {c->pops[0], c->pops[1], c->refp[0], c->refp[1], c->psi, c->solid,
-                    c->wall_u, c->q, c->fext, c->wall_rho, c->wall_psi, c->link, c->links, c->dacc, c->scratch, c->derr};
+                    c->wall_u, c->q, c->fext, c->wall_rho, c->wall_psi, c->fext_f, c->wall_psi_f, c->link, c->links, c->dacc, c->scratch, c->derr};
     for (void *b : bufs)
         if (b) cudaFree(b);
     adjoint_free(c->adj);
@@ -444,6 +448,27 @@ static lbm_status upload(lbm_ctx *c, T **dst, const T *src, size_t count, const 
     return LBM_OK;
 }
 
+static __global__ void k_narrow(const double *in, float *out, int64_t n)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n) out[k] = float(in[k]);
+}
+
+// *dst = src[count] in FP32 (null src: none), for the storage types whose arithmetic is FP32.
+static lbm_status narrow(lbm_ctx *c, float **dst, const double *src, size_t count, const char *what)
+{
+    if (*dst) {
+        cudaStreamSynchronize(c->stream);
+        cudaFree(*dst);
+        *dst = nullptr;
+    }
+    if (!src || c->p.precision == LBM_F64) return LBM_OK;
+    CK(cudaMalloc((void **)dst, count * sizeof(float)), what);
+    k_narrow<<<(unsigned)((count + 255) / 256), 256, 0, c->stream>>>(src, *dst, (int64_t)count);
+    CK(cudaGetLastError(), what);
+    return LBM_OK;
+}
+
 // Wall-link records of the tile kernel (KParams::link), built on the host from the
 // geometry as given: for each fluid node x and pulled population i whose source x - e_i is a
 // wall (a solid node or beyond a non-periodic edge), the link fraction q of the outgoing
@@ -516,6 +541,7 @@ extern "C" lbm_status lbm_set_geometry(lbm_ctx *c, const uint8_t *solid, const d
     if ((s = upload(c, &c->wall_u, wall_u, 2 * n, "wall_u")) != LBM_OK) return s;
     if ((s = upload(c, &c->q, q, 8 * n, "q")) != LBM_OK) return s;
     if ((s = upload(c, &c->fext, force_field, 2 * n, "force_field")) != LBM_OK) return s;
+    if ((s = narrow(c, &c->fext_f, c->fext, 2 * n, "force_field")) != LBM_OK) return s;
     if (c->p.precision != LBM_F64 && (s = build_link_records(c, solid, wall_u, q)) != LBM_OK) return s;
     if (c->links) {
         CK(cudaStreamSynchronize(c->stream), "set_geometry");
@@ -551,6 +577,7 @@ extern "C" lbm_status lbm_set_wall_density(lbm_ctx *c, const double *wall_rho)
     if ((s = upload(c, &c->wall_rho, wall_rho, n, "wall_rho")) != LBM_OK) return s;
     if ((s = upload(c, &c->wall_psi, wall_rho ? psi.data() : (const double *)nullptr, n, "wall_psi")) != LBM_OK)
         return s;
+    if ((s = narrow(c, &c->wall_psi_f, c->wall_psi, n, "wall_psi")) != LBM_OK) return s;
     CK(cudaStreamSynchronize(c->stream), "set_wall_density");
     fill_constants(c);
     choose_kernel(c);

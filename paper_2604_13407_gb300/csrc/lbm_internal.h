@@ -81,6 +81,7 @@ struct KParams {
     const double *fext;    // [2][ny*nx] or null
     const double *wall_rho;  // [ny*nx] virtual density of each solid node, or null (rho_s)
     const double *wall_psi;  // [ny*nx] psi of wall_rho, or null (psi_s)
+    const float *fext_f, *wall_psi_f;  // the same two in FP32 (kernels of FP32 arithmetic convert no FP64 value)
     // [8][ny][pitch] per fluid node and pulled population i = 1..8 whose source x - e_i is a
     // wall: (q, c) with q the link fraction after the fallback of a missing second node, and
     // c = 6 w_o (e_i . u_w) the moving-wall coefficient (mw = c rho_w); null without
@@ -89,6 +90,7 @@ struct KParams {
     // [ny*nx] per node: bit i (1..8) set when the source x - e_i is a wall, bit 0 when the node is
     // solid; null without solid nodes, link fractions and wall velocities.  Read by the tile kernel.
     const uint16_t *links;
+    int skip_solid;        // 1: more than an eighth of the nodes are solid
     int64_t pull[9];       // bytes from a node to population i of the row it is pulled from, (i plane - e_iy pitch)
     int *err;              // device error word (0 = fine)
     Consts<double> cd;     // constants for FP64 arithmetic
