@@ -275,73 +275,88 @@ __device__ __forceinline__ void adj_block(const KParams &kp, const AdjArgs &aa, 
                 if (aa.tail && own[e]) static_cast<R *>(aa.c_out)[(int64_t)at[e].y * kp.pitch + at[e].x] = Z::get(c, e);
         }
     }
+    // ---- the state: the pull of Eq. (lbe.str) with half-way walls (the only walls the adjoint
+    // accepts): f_i = A_o(x) + 0 when x - e_i is a wall, as the forward step evaluates it; what
+    // lambda_{t+1} takes of g; psi of A_t around the node.  With FP32 storage loaded before the barrier:
+    // nothing of the first part is live any more, and their latency passes while the ring's warps finish
+    // (2048^2: 244 -> 235 us a step of the call).  Behind it in the others: a 16-bit population's
+    // conversion would wait for the load (256 x 1024: 31.2 -> 32.1), and FP64 is bound by its pipe.
+    const bool update = any && !aa.tail;
+    constexpr bool DEV = IsDev<S>::value, EARLY = sizeof(S) == 4;
+    const R *g = static_cast<const R *>(aa.g_in), *psif = static_cast<const R *>(kp.psi);
+    T f[9], lam[9], ps[9];
+    R pa[N + 2][3];  // psi of the rows y - 1 .. y + N of the thread's column and the columns beside it
+    auto load_psi = [&] {
+        const R *p = psif + ((int64_t)(me.y[0] - 1) * kp.nx + me.x[0]);
+#pragma unroll
+        for (int r = 0; r < N + 2; ++r, p += kp.nx)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) pa[r][d] = p[d - 1];
+    };
+    auto load = [&](int e) {
+        const S *src = static_cast<const S *>(kp.src);
+        const int64_t k = (int64_t)at[e].y * kp.pitch + at[e].x;
+        if constexpr (INNER) {
+            const char *ps_ = reinterpret_cast<const char *>(src + k), *pg = reinterpret_cast<const char *>(g + k);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                R wref = R(0);
+                if constexpr (DEV) wref = __fmul_rn(w_<R>(i), kp.per_node_ref ? (kp.ref_src + (k - ey_(i) * kp.pitch))[-ex_(i)] : cc.rho_ref);
+                Z::set(f[i], e, Codec<S>::dec(reinterpret_cast<const S *>(ps_ + kp.pull[i])[-ex_(i)], wref, cc.inv_scale));
+                Z::set(lam[i], e, g != nullptr ? reinterpret_cast<const R *>(pg + aa.push[i])[ex_(i)] : R(0));
+                Z::set(ps[i], e, pa[e + 1 + ey_(i)][1 + ex_(i)]);
+            }
+        } else {
+            unsigned in;
+            const Nine nn = nine_of(kp, at[e], in);
+            const Around nb = around(kp, at[e].x, at[e].y);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                Z::set(f[i], e, load_pop_at<S>(kp, i, nn.from(i)));
+                Z::set(lam[i], e, g != nullptr ? g[i * P + nn.from(opp_(i))] : R(0));
+                Z::set(ps[i], e, nb.in(i) ? psif[nb.n(i)] : cc.psi_s);
+            }
+        }
+        if (!INNER && (w[e] & 0x1feu)) {
+#pragma unroll
+            for (int i = 1; i < 9; ++i) {
+                const int o = opp_(i);
+                if ((w[e] >> i) & 1u) Z::set(f[i], e, load_pop_at<S>(kp, o, k) + R(0));
+                if (((w[e] >> o) & 1u) && g != nullptr) Z::set(lam[i], e, g[o * P + k]);  // x + e_i is a wall
+            }
+        }
+    };
+    if (EARLY && update) {
+        if (INNER) load_psi();
+#pragma unroll
+        for (int e = 0; e < N; ++e) load(e);
+    }
     const bool walled = INNER ? (__syncthreads(), false) : __syncthreads_or(walls & 0x1feu) != 0;
 
     T gFx = zero, gFy = zero, gG = zero, gT = zero, Jt = zero;
-    if (any && !aa.tail) {
+    if (update) {
         const R wscale = sizeof(R) == 8 ? R(aa.w_scale) : R(aa.w_scale_f);
         const R inv_nf = sizeof(R) == 8 ? R(aa.inv_nfluid) : R(aa.inv_nfluid_f);
-        // ---- the state: the pull of Eq. (lbe.str) with half-way walls (the only walls the adjoint
-        // accepts): f_i = A_o(x) + 0 when x - e_i is a wall, as the forward step evaluates it;
-        // lambda_{t+1}; psi of A_t around the node
-        T f[9], lam[9], ps[9];
-        const R *g = static_cast<const R *>(aa.g_in), *psif = static_cast<const R *>(kp.psi);
-        const S *src = static_cast<const S *>(kp.src);
-        constexpr bool DEV = IsDev<S>::value;
-        // psi and c of the rows y - 1 .. y + N of the thread's column and the columns beside it
-        R ca[N + 2][3], pa[N + 2][3];
+        // ---- lambda_{t+1} = W + g + c
+        R ca[N + 2][3];  // c like pa
 #pragma unroll
         for (int r = 0; r < N + 2; ++r)
 #pragma unroll
             for (int d = 0; d < 3; ++d) ca[r][d] = g != nullptr ? cs[me.r[0] - 1 + r][me.c[0] - 1 + d] : R(0);
-        if constexpr (INNER) {
-            const R *p = psif + ((int64_t)(me.y[0] - 1) * kp.nx + me.x[0]);
-#pragma unroll
-            for (int r = 0; r < N + 2; ++r, p += kp.nx)
-#pragma unroll
-                for (int d = 0; d < 3; ++d) pa[r][d] = p[d - 1];
-        }
+        const R wi = aa.objective == 0 ? R(0) : wscale * inv_nf;  // objective 1: W_i = e_ix / N_fluid
+        if (!EARLY && INNER) load_psi();
 #pragma unroll
         for (int e = 0; e < N; ++e) {
-            const R wi = aa.objective == 0 ? R(0) : wscale * inv_nf;  // objective 1: W_i = e_ix / N_fluid
-            if constexpr (INNER) {
-                const int64_t k = (int64_t)me.y[e] * kp.pitch + me.x[e];
-                const char *ps_ = reinterpret_cast<const char *>(src + k), *pg = reinterpret_cast<const char *>(g + k);
+            if (!EARLY) load(e);
 #pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    R wref = R(0);
-                    if constexpr (DEV) wref = __fmul_rn(w_<R>(i), kp.per_node_ref ? (kp.ref_src + (k - ey_(i) * kp.pitch))[-ex_(i)] : cc.rho_ref);
-                    Z::set(f[i], e, Codec<S>::dec(reinterpret_cast<const S *>(ps_ + kp.pull[i])[-ex_(i)], wref, cc.inv_scale));
-                    R v = R(ex_(i)) * wi;
-                    if (g != nullptr) v += reinterpret_cast<const R *>(pg + aa.push[i])[ex_(i)] + ca[e + 1 + ey_(i)][1 + ex_(i)];
-                    Z::set(lam[i], e, v);
-                    Z::set(ps[i], e, pa[e + 1 + ey_(i)][1 + ex_(i)]);
+            for (int i = 0; i < 9; ++i) {
+                R v = R(ex_(i)) * wi, c = ca[e + 1 + ey_(i)][1 + ex_(i)];
+                if (!INNER && ((w[e] >> opp_(i)) & 1u) && i > 0) {  // x + e_i is a wall
+                    v = wscale * objective_weight<R>(aa.objective, i, true, inv_nf);
+                    c = ca[e + 1][1];
                 }
-            } else {
-                unsigned in;
-                const Nine nn = nine_of(kp, at[e], in);
-                const Around nb = around(kp, at[e].x, at[e].y);
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    Z::set(f[i], e, load_pop_at<S>(kp, i, nn.from(i)));
-                    R v = R(ex_(i)) * wi;
-                    if (g != nullptr) v += g[i * P + nn.from(opp_(i))] + ca[e + 1 + ey_(i)][1 + ex_(i)];
-                    Z::set(lam[i], e, v);
-                    Z::set(ps[i], e, nb.in(i) ? psif[nb.n(i)] : cc.psi_s);
-                }
-            }
-            if (!INNER && (w[e] & 0x1feu)) {
-                const int64_t k = (int64_t)at[e].y * kp.pitch + at[e].x;
-#pragma unroll
-                for (int i = 1; i < 9; ++i) {
-                    const int o = opp_(i);
-                    if ((w[e] >> i) & 1u) Z::set(f[i], e, load_pop_at<S>(kp, o, k) + R(0));
-                    if ((w[e] >> o) & 1u) {  // x + e_i is a wall
-                        R v = wscale * objective_weight<R>(aa.objective, i, true, inv_nf);
-                        if (g != nullptr) v += g[o * P + k] + ca[e + 1][1];
-                        Z::set(lam[i], e, v);
-                    }
-                }
+                if (g != nullptr) v += Z::get(lam[i], e) + c;
+                Z::set(lam[i], e, v);
             }
             // the pair's other node may be no fluid node (past the lattice, or solid): keep its arithmetic finite
             if (!INNER && !own[e]) {
@@ -620,8 +635,9 @@ __global__ void __launch_bounds__(256) k_adj_reduce(const double *part, int64_t 
 template <class S>
 struct Adjoint {
     // FP32 arithmetic: tall tiles and 128 registers on small lattices, where a block's ring is a large
-    // part of its work and there are few blocks to hide latency (256 x 1024: 27.5 us a step of the call
-    // against 30.9); short ones and five blocks per SM from 2^19 nodes (2048^2: 249 against 267).
+    // part of its work and there are few blocks to hide latency (256 x 1024: 27.0 us a step of the call
+    // against 28.8; between them, six units by three blocks, 29.2); short ones and five blocks per SM from
+    // 2^19 nodes (2048^2: 234 against 254; six by three 240).
     static constexpr bool F64 = sizeof(typename Codec<S>::R) == 8;
     static bool tall(const KParams &kp) { return F64 || (int64_t)kp.nx * kp.ny < (int64_t)1 << 19; }
     static int rows(const KParams &kp) { return F64 ? 8 : tall(kp) ? 16 : 8; }
