@@ -80,6 +80,25 @@ def test_tile_step_with_solid_nodes(nx, ny, prec):
                 assert np.abs(a - b).max() <= 4 * 8 * ulp * np.abs(a).max(), (px, py)
 
 
+@pytest.mark.parametrize("prec", ["f32", "f16", "f16_nearest", "bf16"])
+@pytest.mark.parametrize("force_mode", [0, 1, 2])
+@pytest.mark.parametrize("tau_g", [1.0, 0.7])
+def test_every_compiled_combination_of_options(prec, force_mode, tau_g):
+    """Force law, relaxation and reference plane are fixed at compile time in the tile kernel: bit for bit
+    the two-pass step in each, with and without solid nodes (three steps: none in the kernel of small
+    lattices), on a lattice with tiles at the edges and inside."""
+    pid, kw = PRECS[prec]
+    nx, ny = 131, 41
+    solid = (I.uniform(11, nx * ny).reshape(ny, nx) < 0.1).astype(np.uint8)
+    field = I.uniform(13, 2 * nx * ny, -1e-5, 1e-5).reshape(2, ny, nx) if force_mode == 2 else None
+    op = cs_params(nx=nx, ny=ny, periodic_x=True, periodic_y=False, scheme=1, force_mode=force_mode, Fx=1e-5, Fy=-2e-5, tau_l=1.0, tau_g=tau_g)
+    for mask in (None, solid):
+        a, b = (_state(op, nx, ny, pid, kw, kern, (mask, None, None, field), steps=3) for kern in (lbm.KERNEL_TWO_PASS, lbm.KERNEL_AUTO))
+        if mask is not None:
+            a, b = a[:, mask == 0], b[:, mask == 0]
+        assert np.all(np.isfinite(a)) and np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("masked", [False, True])
 @pytest.mark.parametrize("prec", ["f64", "f32", "f16", "bf16"])
 @pytest.mark.parametrize("nx,ny", [(1, 5), (33, 17), (70, 37), (131, 40)])
