@@ -4,12 +4,13 @@
 // What bounds a small lattice is neither bytes nor instructions but the launch and the two trips through
 // L2 that a step of its own kernel takes (2.9 us a step on 37 x 23 nodes, whatever is computed).  Here a step
 // is two phases between cluster barriers: pull, rho and psi; then the psi stencil, collision and the
-// write-back in place.  A thread owns one pair of nodes (FP64: one node) for the whole launch.  What a
+// write-back in place.  A thread owns one node for the whole launch (or, where a strip has more than 512,
+// two; in FP64 four threads share one).  What a
 // neighbouring strip needs -- psi of the edge rows, and the populations that leave them -- is pushed into
 // its halo rows through distributed shared memory, so every load is a local one.
 //
-// Measured per step (us, one launch per step / here): 37 x 23 FP32 3.0 / 1.2, FP16 3.0 / 2.4; 64^2 FP32 3.0 / 1.2;
-// 128^2 3.0 / 2.2 (16 SMs are busy there: the last size that gains); FP64 4 x 128 column 18 / 7.5, 4 x 181
+// Measured per step (us, one launch per step / here): 37 x 23 FP32 3.0 / 0.90, FP16 3.0 / 1.2; 64^2 FP32 3.0 / 1.06;
+// 128^2 3.0 / 2.1 (16 SMs are busy there: the last size that gains); FP64 4 x 128 column 18 / 7.5, 4 x 181
 // 18 / 11.5, 37 x 23 18 / 16.4.
 //
 // The functions, their order and the storage type's rounding are the tile kernel's (k_tile.cuh), so
@@ -134,6 +135,7 @@ struct StripNode {
     uint32_t row, cm, c0, cp, pm, pp;     // local row; columns x - 1, x, x + 1 of the populations, and of psi
     uint32_t node, kg;                    // lattice and plane index
     unsigned w;                           // wall bits
+    StripNode() = default;
     __device__ __forceinline__ StripNode(const Strip<S> &s, int idx)
     {
         const KParams &kp = s.kp;
@@ -215,92 +217,119 @@ struct StripNode {
     }
 };
 
-// FP32 arithmetic: a thread owns two nodes of its strip, `pairs` apart, for the whole launch.
-template <class S>
-__global__ void __launch_bounds__(kSmallThreads) k_small2(KParams kp, int64_t nsteps, int64_t step0, int max_rows)
+// FP32 arithmetic: a thread owns one node of its strip (v1) or two (v2x), `units` apart, for the whole launch.
+template <class T> struct Owned;
+template <> struct Owned<v1> {
+    static constexpr int N = 1;
+    static __device__ __forceinline__ v1 of(const float *v, int) { return v1{v[0]}; }
+    static __device__ __forceinline__ float get(v1 a, int) { return a.v; }
+    static __device__ __forceinline__ void set(v1 &a, int, float v) { a.v = v; }
+};
+template <> struct Owned<v2x> {
+    static constexpr int N = 2;
+    static __device__ __forceinline__ v2x of(const float *v, int pitch) { return X2(v[0], v[pitch]); }
+    static __device__ __forceinline__ float get(v2x a, int e) { return e ? a.v.y : a.v.x; }
+    static __device__ __forceinline__ void set(v2x &a, int e, float v) { (e ? a.v.y : a.v.x) = v; }
+};
+template <class S, class T, int THREADS>
+__global__ void __launch_bounds__(THREADS) k_small2(KParams kp, int64_t nsteps, int64_t step0, int max_rows)
 {
+    typedef Owned<T> Z;
     constexpr bool DEV = IsDev<S>::value;
+    constexpr int N = Z::N;
     extern __shared__ __align__(128) unsigned char smem[];
     Strip<S> s{kp};
     s.load(smem, max_rows);
-    const int pairs = (s.m * s.nx + 1) / 2, t0 = (int)threadIdx.x;
-    // (threads past the last pair, and the second node of an odd strip's last thread: not live)
-    const StripNode<S> a(s, t0 < pairs ? t0 : s.m * s.nx), b(s, t0 < pairs ? t0 + pairs : s.m * s.nx);
-    // which half of its pair's random word each node takes: its column's parity
-    const unsigned pick = (a.c0 & 1u ? 0x32u : 0x10u) | (b.c0 & 1u ? 0x7600u : 0x5400u);
-    const float wall_a = (a.w & 1u) && kp.wall_psi_f ? kp.wall_psi_f[a.node] : kp.cf.psi_s;  // psi of solid nodes
-    const float wall_b = (b.w & 1u) && kp.wall_psi_f ? kp.wall_psi_f[b.node] : kp.cf.psi_s;
+    const int nodes = s.m * s.nx, units = (nodes + N - 1) / N, t0 = (int)threadIdx.x;
+    StripNode<S> n[N];
+    float wall[N];       // psi of solid nodes
+    unsigned pick = 0x5400u;  // which half of its row pair's random word each node takes: its column's parity
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+        // (threads past the last unit, and the second node of an odd strip's last thread: not live)
+        n[e] = StripNode<S>(s, t0 < units ? t0 + e * units : nodes);
+        wall[e] = (n[e].w & 1u) && kp.wall_psi_f ? kp.wall_psi_f[n[e].node] : kp.cf.psi_s;
+        pick = e == 0 ? (pick & 0xff00u) | (n[e].c0 & 1u ? 0x32u : 0x10u) : (pick & 0xffu) | (n[e].c0 & 1u ? 0x7600u : 0x5400u);
+    }
 
     for (int64_t t = 0; t < nsteps; ++t) {
-        float fa[9], fb[9];
-        a.pull(s, fa);
-        b.pull(s, fb);
-        v2x d[9], rho, psi;
-        {
-            v2x f[9];
+        float f_[N][9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) f[i] = X2(fa[i], fb[i]);
+        for (int e = 0; e < N; ++e) n[e].pull(s, f_[e]);
+        T d[9], rho, psi;
+        {
+            T f[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = Z::of(&f_[0][i], 9);
             to_dev(f, d);
         }
         rho = density_dev(d);
-        psi = psi_v<v2x>(kp, rho);
-        if (a.w & 1u) psi.v.x = wall_a, rho.v.x = 1.f;
-        if (b.w & 1u) psi.v.y = wall_b, rho.v.y = 1.f;
-        a.put_psi(s, psi.v.x);
-        b.put_psi(s, psi.v.y);
+        psi = psi_v<T>(kp, rho);
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            if (n[e].w & 1u) Z::set(psi, e, wall[e]), Z::set(rho, e, 1.f);
+            n[e].put_psi(s, Z::get(psi, e));
+        }
         s.barrier();
 
-        auto p = [&](int i) { return X2(s.psi[a.psi_at(s, i)], s.psi[b.psi_at(s, i)]); };
-        v2x Sx, Sy, Fex, Fey, o[9], ux, uy;
-        stencil_v<v2x>(p(1), p(2), p(3), p(4), p(5), p(6), p(7), p(8), Sx, Sy);
+        auto p = [&](int i) {
+            float v[N];
+#pragma unroll
+            for (int e = 0; e < N; ++e) v[e] = s.psi[n[e].psi_at(s, i)];
+            return Z::of(v, 1);
+        };
+        T Sx, Sy, Fex = ks<T>(0.f), Fey = Fex, o[9], ux, uy;
+        stencil_v<T>(p(1), p(2), p(3), p(4), p(5), p(6), p(7), p(8), Sx, Sy);
         if (kp.force_mode == 0) {
-            Fex = v2x{kp.c2.Fx}, Fey = v2x{kp.c2.Fy};
+            Fex = kc<T>(kp.c2.Fx), Fey = kc<T>(kp.c2.Fy);
         } else if (kp.force_mode == 1) {
-            const v2x x = rho - v2x{kp.c2.rho_g};
-            Fex = x * v2x{kp.c2.Fx}, Fey = x * v2x{kp.c2.Fy};
+            const T x = rho - kc<T>(kp.c2.rho_g);
+            Fex = x * kc<T>(kp.c2.Fx), Fey = x * kc<T>(kp.c2.Fy);
         } else if (kp.fext_f) {
-            const int64_t n = (int64_t)kp.nx * kp.ny;
-            Fex = X2(kp.fext_f[a.node], kp.fext_f[b.node]);
-            Fey = X2(kp.fext_f[n + a.node], kp.fext_f[n + b.node]);
-        } else {
-            Fex = Fey = X2(0.f, 0.f);
+            const int64_t all = (int64_t)kp.nx * kp.ny;
+#pragma unroll
+            for (int e = 0; e < N; ++e) Z::set(Fex, e, kp.fext_f[n[e].node]), Z::set(Fey, e, kp.fext_f[all + n[e].node]);
         }
-        collide_v<v2x, RuntimeOpts>(kp, d, rho, psi, Sx, Sy, Fex, Fey, o, ux, uy);
-        S va[9], vb[9];
+        collide_v<T, RuntimeOpts>(kp, d, rho, psi, Sx, Sy, Fex, Fey, o, ux, uy);
+        S v[N][9];
         if constexpr (DEV) {
             const uint32_t seed = sr_seed_at(step0 + t);
-            const uint32_t ha = sr_hash(a.kg >> 1, seed), hb = sr_hash(b.kg >> 1, seed);
+            const uint32_t ha = sr_hash(n[0].kg >> 1, seed), hb = N == 2 ? sr_hash(n[N - 1].kg >> 1, seed) : 0u;
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-                const v2x wr = s.has_ref ? v2x{kp.c2.w[i]} * rho : v2x{kp.c2.dec[i]};
-                const v2x q = (o[i] - wr) * v2x{kp.c2.scale};
+                const T wr = s.has_ref ? kc<T>(kp.c2.w[i]) * rho : kc<T>(kp.c2.dec[i]);
+                const T q = (o[i] - wr) * kc<T>(kp.c2.scale);
+                const float qa = Z::get(q, 0), qb = N == 2 ? Z::get(q, N - 1) : 0.f;
                 if (kp.sr) {
-                    const uint32_t h = SRound<S>::pack(q.v.x, q.v.y, __byte_perm(sr_bits(ha, i), sr_bits(hb, i), pick));
-                    va[i] = SRound<S>::from_bits((unsigned short)(h & 0xffffu)), vb[i] = SRound<S>::from_bits((unsigned short)(h >> 16));
+                    const uint32_t h = SRound<S>::pack(qa, qb, __byte_perm(sr_bits(ha, i), N == 2 ? sr_bits(hb, i) : 0u, pick));
+                    v[0][i] = SRound<S>::from_bits((unsigned short)(h & 0xffffu));
+                    if (N == 2) v[N - 1][i] = SRound<S>::from_bits((unsigned short)(h >> 16));
                 } else {
-                    va[i] = Codec<S>::enc(q.v.x, 0.f, 1.f), vb[i] = Codec<S>::enc(q.v.y, 0.f, 1.f);
+                    v[0][i] = Codec<S>::enc(qa, 0.f, 1.f);
+                    if (N == 2) v[N - 1][i] = Codec<S>::enc(qb, 0.f, 1.f);
                 }
             }
             if (s.has_ref) {
-                auto put_ref = [&](const StripNode<S> &n, float v) {
-                    if (!n.fluid) return;
-                    s.ref[n.own(s)] = v;
-                    if (n.top) push(s.up_ref + n.c0 * 4u, v);
-                    if (n.bottom) push(s.down_ref + n.c0 * 4u, v);
-                };
-                put_ref(a, rho.v.x);
-                put_ref(b, rho.v.y);
+#pragma unroll
+                for (int e = 0; e < N; ++e) {
+                    if (!n[e].fluid) continue;
+                    s.ref[n[e].own(s)] = Z::get(rho, e);
+                    if (n[e].top) push(s.up_ref + n[e].c0 * 4u, Z::get(rho, e));
+                    if (n[e].bottom) push(s.down_ref + n[e].c0 * 4u, Z::get(rho, e));
+                }
             }
         } else {
 #pragma unroll
-            for (int i = 0; i < 9; ++i) va[i] = o[i].v.x, vb[i] = o[i].v.y;
+            for (int e = 0; e < N; ++e)
+#pragma unroll
+                for (int i = 0; i < 9; ++i) v[e][i] = Z::get(o[i], e);
         }
-        a.put(s, va);
-        b.put(s, vb);
+#pragma unroll
+        for (int e = 0; e < N; ++e) n[e].put(s, v[e]);
         s.barrier();
     }
-    a.write_back(s, nsteps & 1, 0, 9);
-    b.write_back(s, nsteps & 1, 0, 9);
+#pragma unroll
+    for (int e = 0; e < N; ++e) n[e].write_back(s, nsteps & 1, 0, 9);
 }
 
 // FP64.  An FP64 instruction holds its scheduler's quarter of the SM for 64 cycles, whatever the
@@ -404,16 +433,27 @@ struct Small {
     typedef typename Codec<S>::R R;
     static constexpr bool F64 = sizeof(R) == 8;
     static int rows(const KParams &kp, int ctas) { return (kp.ny + ctas - 1) / ctas; }
-    // two nodes a thread; FP64: four warps per 32 nodes
-    static int threads(const KParams &kp, int ctas)
+    typedef void (*Kernel)(KParams, int64_t, int64_t, int);
+    // The launch for a strip: its kernel, the most threads that is compiled for, and the threads.  FP64: four
+    // warps per 32 nodes.
+    struct Form {
+        Kernel kernel;
+        int most, threads;
+    };
+    static Form form(const KParams &kp, int ctas)
     {
         const int nodes = rows(kp, ctas) * kp.nx;
-        return F64 ? (nodes + 31) / 32 * 128 : (nodes + 63) / 64 * 32;
-    }
-    static void (*kernel())(KParams, int64_t, int64_t, int)
-    {
-        if constexpr (F64) return k_small1<S>;
-        else return k_small2<S>;
+        if constexpr (F64) {
+            return Form{k_small1<S>, kSmallThreads, (nodes + 31) / 32 * 128};
+        } else {
+            const int one = (nodes + 31) / 32 * 32, two = (nodes + 63) / 64 * 32;
+            // One node a thread as long as a strip's fit: a warp's instructions are a step's time, and a pair's
+            // loads and stores are twice a node's (100 x 40 FP32 1.44 -> 1.21 us a step).  Up to 128 threads the
+            // kernel may keep every address in registers (37 x 23 FP32 0.95 -> 0.89).
+            if (one <= 128) return Form{k_small2<S, v1, 128>, 128, one};
+            if (one <= kSmallThreads) return Form{k_small2<S, v1, kSmallThreads>, kSmallThreads, one};
+            return Form{k_small2<S, v2x, kSmallThreads>, kSmallThreads, two};
+        }
     }
     static size_t bytes(const KParams &kp, int ctas) { return SmallLayout<S>{kp.nx, rows(kp, ctas)}.bytes(IsDev<S>::value && kp.per_node_ref); }
     static constexpr int SMEM = 190 * 1024;
@@ -427,14 +467,16 @@ struct Small {
         if (n > MAX_NODES) return 0;
         int c = n > (F64 ? 128 : 1024) ? 16 : 8;
         while (c > kp.ny) c /= 2;
-        if ((int64_t)rows(kp, c) * kp.nx > 2 * kSmallThreads || threads(kp, c) > kSmallThreads || bytes(kp, c) > SMEM) return 0;
-        return cluster_fits(reinterpret_cast<const void *>(kernel()), kp.device, c, kSmallThreads, SMEM) ? c : 0;
+        if ((int64_t)rows(kp, c) * kp.nx > 2 * kSmallThreads || bytes(kp, c) > SMEM) return 0;
+        const Form f = form(kp, c);
+        return f.threads <= f.most && cluster_fits(reinterpret_cast<const void *>(f.kernel), kp.device, c, f.most, SMEM) ? c : 0;
     }
     static cudaError_t steps(const KParams &kp, int ctas, int64_t nsteps, int64_t step0, cudaStream_t st)
     {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(ctas);
-        cfg.blockDim = dim3(threads(kp, ctas));
+        const Form f = form(kp, ctas);
+        cfg.blockDim = dim3(f.threads);
         cfg.dynamicSmemBytes = bytes(kp, ctas);
         cfg.stream = st;
         cudaLaunchAttribute attr;
@@ -443,7 +485,7 @@ struct Small {
         attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, kernel(), kp, nsteps, step0, rows(kp, ctas));
+        return cudaLaunchKernelEx(&cfg, f.kernel, kp, nsteps, step0, rows(kp, ctas));
     }
 };
 

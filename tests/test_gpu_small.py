@@ -46,6 +46,17 @@ def test_one_launch_is_step_by_step(nx, ny, prec):
         assert np.array_equal(a, _run(op, prec, lbm.KERNEL_TWO_PASS, [13])), (px, py)
 
 
+@pytest.mark.parametrize("prec", ["f32", "f16", "f16_nearest", "bf16"])
+@pytest.mark.parametrize("nx,ny", [(32, 64), (43, 48), (128, 64), (171, 48)])
+def test_edges_of_one_and_two_nodes_a_thread(nx, ny, prec):
+    """Strips of 128, 129, 512 and 513 nodes: the last of the small blocks, the first of the large ones, the
+    last with one node a thread and the first (odd) with two."""
+    for px, force_mode in ((True, 0), (False, 1)):
+        op = cs_params(nx=nx, ny=ny, periodic_x=px, periodic_y=True, scheme=1, force_mode=force_mode, Fx=1e-5, Fy=-2e-5, tau_l=1.0, tau_g=0.8)
+        a = _run(op, prec, lbm.KERNEL_AUTO, [5, 4])
+        assert np.all(np.isfinite(a)) and np.array_equal(a, _run(op, prec, lbm.KERNEL_TWO_PASS, [9])), (px, force_mode)
+
+
 @pytest.mark.parametrize("prec", sorted(PRECS))
 @pytest.mark.parametrize("nx,ny", [(9, 9), (67, 37), (40, 18)])
 def test_solid_nodes_force_field_and_wall_densities(nx, ny, prec):
