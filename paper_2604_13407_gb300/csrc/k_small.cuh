@@ -10,8 +10,8 @@
 // its halo rows through distributed shared memory, so every load is a local one.
 //
 // Measured per step (us, one launch per step / here): 37 x 23 FP32 3.0 / 0.90, FP16 3.0 / 1.2; 64^2 FP32 3.0 / 1.06;
-// 128^2 3.0 / 2.1 (16 SMs are busy there: the last size that gains); FP64 4 x 128 column 18 / 7.5, 4 x 181
-// 18 / 11.5, 37 x 23 18 / 16.4.
+// 128^2 3.0 / 2.1 (16 SMs are busy there: the last size that gains); FP64 4 x 128 column 18 / 6.5, 4 x 181
+// 18 / 9.2, 37 x 23 18 / 13.1.
 //
 // The functions, their order and the storage type's rounding are the tile kernel's (k_tile.cuh), so
 // the state after n steps is, bit for bit, what n of its launches leave.
@@ -186,33 +186,33 @@ struct StripNode {
         if (top) push(s.up_psi + c0 * (uint32_t)sizeof(R), v);
         if (bottom) push(s.down_psi + c0 * (uint32_t)sizeof(R), v);
     }
-    // Stores populations [first, first + count) of the node.
-    __device__ __forceinline__ void put(const Strip<S> &s, const S (&v)[9], int first = 0, int count = 9) const
+    // Stores the populations of the node whose bits are set.
+    __device__ __forceinline__ void put(const Strip<S> &s, const S (&v)[9], unsigned which = 0x1ffu) const
     {
         if (!fluid) return;
         S *p = s.pop + own(s);
 #pragma unroll
         for (int i = 0; i < 9; ++i)
-            if (i >= first && i < first + count) p[i * s.PS] = v[i];
+            if ((which >> i) & 1u) p[i * s.PS] = v[i];
         if (top) {
 #pragma unroll
             for (int i = 0; i < 9; ++i)
-                if (ey_(i) > 0 && i >= first && i < first + count) push(s.up_pop + (i * s.PS + c0) * (uint32_t)sizeof(S), v[i]);
+                if (ey_(i) > 0 && ((which >> i) & 1u)) push(s.up_pop + (i * s.PS + c0) * (uint32_t)sizeof(S), v[i]);
         }
         if (bottom) {
 #pragma unroll
             for (int i = 0; i < 9; ++i)
-                if (ey_(i) < 0 && i >= first && i < first + count) push(s.down_pop + (i * s.PS + c0) * (uint32_t)sizeof(S), v[i]);
+                if (ey_(i) < 0 && ((which >> i) & 1u)) push(s.down_pop + (i * s.PS + c0) * (uint32_t)sizeof(S), v[i]);
         }
     }
     // The state after an odd number of steps goes to the other buffer, as step by step.
-    __device__ __forceinline__ void write_back(const Strip<S> &s, bool odd, int first, int count) const
+    __device__ __forceinline__ void write_back(const Strip<S> &s, bool odd) const
     {
         if (!fluid) return;
         S *dst = static_cast<S *>(odd ? s.kp.dst : const_cast<void *>(s.kp.src));
 #pragma unroll
         for (int i = 0; i < 9; ++i)
-            if (i >= first && i < first + count) dst[i * s.kp.plane + kg] = s.pop[i * s.PS + own(s)];
+            dst[i * s.kp.plane + kg] = s.pop[i * s.PS + own(s)];
         if (s.has_ref) (odd ? s.kp.ref_dst : const_cast<float *>(s.kp.ref_src))[kg] = s.ref[own(s)];
     }
 };
@@ -329,21 +329,24 @@ __global__ void __launch_bounds__(THREADS) k_small2(KParams kp, int64_t nsteps, 
         s.barrier();
     }
 #pragma unroll
-    for (int e = 0; e < N; ++e) n[e].write_back(s, nsteps & 1, 0, 9);
+    for (int e = 0; e < N; ++e) n[e].write_back(s, nsteps & 1);
 }
 
 // FP64.  An FP64 instruction holds its scheduler's quarter of the SM for 64 cycles, whatever the
 // number of active lanes and however independent its neighbours are, so a node's 390 of them in one
 // warp take 12 us, and a small lattice leaves most schedulers idle.  Four warps therefore share a
 // group of 32 nodes, one per scheduler, and hand each other the few values they need through
-// shared memory: psi / moments / 1/rho; then the x and y force and velocity; then the relaxed moments;
-// then the populations.  The longest of the four takes about 120 FP64 instructions a step.  (4 x 128
-// column: 18 us a step with one launch per step, 13.2 with one warp per 32 nodes.)
+// shared memory, in six parts between barriers (a barrier costs no more than one FP64 instruction):
+// density and the terms of p_EOS; psi, moments, 1/rho; the x and y force and velocity, 1/(G psi^2); the
+// quotients by G psi^2; the relaxed moments; the populations, each warp those it stores.  (4 x 128 column:
+// 18 us a step with one launch per step, 13.2 with one warp per 32 nodes, 7.5 in four parts, 6.5 in six.)
 struct Small64Shared {
-    double r[kSmallThreads / 4];                                                   // 1/(G psi^2)
-    double Fix[kSmallThreads / 4], Fiy[kSmallThreads / 4], Fx[kSmallThreads / 4], Fy[kSmallThreads / 4];
-    double ux[kSmallThreads / 4], uy[kSmallThreads / 4];
-    double u[9][kSmallThreads / 4];                                                // m_bar_k without |M_k|^2's odd factor
+    static constexpr int M = kSmallThreads / 4;
+    double num[M], attraction[M], third[M];                      // of psi: p_EOS = K (num/den - attraction), rho/3
+    double r[M];                                                 // 1/(G psi^2)
+    double Fix[M], Fiy[M], Fx[M], Fy[M], ux[M], uy[M];
+    double X[M], Y[M], Q7[M];
+    double u[9][M];                                              // m_bar_k without |M_k|^2's odd factor
 };
 template <class S>
 __global__ void __launch_bounds__(kSmallThreads) k_small1(KParams kp, int64_t nsteps, int64_t step0, int max_rows)
@@ -359,18 +362,27 @@ __global__ void __launch_bounds__(kSmallThreads) k_small1(KParams kp, int64_t ns
     for (int64_t t = 0; t < nsteps; ++t) {
         double f[9], sp = kp.sp, sq = kp.sq, m_a = 0.0, m_b = 0.0;
         a.pull(s, f);
-        const double rho = density(f);
-        Divisor by_rho{};
+        const double rho = density(f);  // (each warp its own: shorter than handing it over)
+        Divisor by{};
         if (role == 0) {
-            a.put_psi(s, a.w & 1u ? (kp.wall_psi ? kp.wall_psi[a.node] : kp.psi_s) : psi_of(kp, rho));
+            by = divisor(eos_den(kp, rho));
+        } else if (role == 2) {
+            x.attraction[at] = eos_attraction(kp, rho), x.third[at] = div_const<3>(rho);
+            m_a = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];                                  // j_x
+        } else if (role == 3) {
+            x.num[at] = eos_num(kp, rho);
+        }
+        __syncthreads();
+
+        if (role == 0) {
+            a.put_psi(s, a.w & 1u ? (kp.wall_psi ? kp.wall_psi[a.node] : kp.psi_s) : psi_of(kp, by(x.num[at]), x.attraction[at], x.third[at]));
         } else if (role == 1) {
             moments_12(f, m_a, m_b);
         } else if (role == 2) {
-            by_rho = divisor(rho);
-            m_a = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];                                  // j_x
+            by = divisor(rho);
             m_b = fma_(2.0, f[3], -2.0 * f[1]) + f[5] - f[6] - f[7] + f[8];               // m_4
         } else {
-            by_rho = divisor(rho);
+            by = divisor(rho);
             m_a = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];                                  // j_y
             m_b = fma_(2.0, f[4], -2.0 * f[2]) + f[5] + f[6] - f[7] - f[8];               // m_6
         }
@@ -384,7 +396,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_small1(KParams kp, int64_t ns
             if (role == 2) S_ = stencil_x(ps);
             else S_ = stencil_y(ps);
             external_force<double>(kp, a.node, rho, Fex, Fey);
-            const double Fi = -Gpsi * S_, F = Fi + (role == 2 ? Fex : Fey), u = by_rho(fma_(0.5, F, m_a));
+            const double Fi = -Gpsi * S_, F = Fi + (role == 2 ? Fex : Fey), u = by(fma_(0.5, F, m_a));
             if (role == 2) x.Fix[at] = Fi, x.Fx[at] = F, x.ux[at] = u;
             else x.Fiy[at] = Fi, x.Fy[at] = F, x.uy[at] = u;
         } else if (role == 1) {
@@ -399,33 +411,49 @@ __global__ void __launch_bounds__(kSmallThreads) k_small1(KParams kp, int64_t ns
         const double Fix = x.Fix[at], Fiy = x.Fiy[at], Fx = x.Fx[at], Fy = x.Fy[at], ux = x.ux[at], uy = x.uy[at];
         const double Gpsi2 = Gpsi * psi;
         const Divisor by_Gpsi2{Gpsi2, x.r[at], in_range(Gpsi2) && is_nonzero(Gpsi2)};
+        Stress12 st{};
+        double ru = 0.0;
         if (role == 0) {
-            relaxed_78(kp, rho, m_a, m_b, Fx, Fy, ux, uy, Fix, Fiy, by_Gpsi2, sp, x.u[7][at], x.u[8][at]);
+            ru = rho * ux;
+            x.u[8][at] = relaxed_8(ru, m_b, Fx, Fy, ux, uy, by_Gpsi2(kp.k1 * Fix * Fiy), sp);
+        } else if (role == 1) {
+            st = stress_12(rho, m_a, m_b, Fx, Fy, ux, uy);
+        } else if (role == 2) {
+            const double xx = Fix * Fix;
+            x.X[at] = by_Gpsi2(xx);
+            x.Q7[at] = by_Gpsi2(kp.k1 * (xx - Fiy * Fiy));
+        } else {
+            x.Y[at] = by_Gpsi2(Fiy * Fiy);
+            ru = rho * uy;
+            x.u[5][at] = div_const<3>(relaxed_j(m_a, Fy, ru));
+        }
+        __syncthreads();
+
+        if (role == 0) {
+            x.u[7][at] = relaxed_7(ru, rho * uy, m_a, Fx, Fy, ux, uy, x.Q7[at], sp);
         } else if (role == 1) {
             double a1, a2;
-            relaxed_12(kp, rho, m_a, m_b, Fx, Fy, ux, uy, by_Gpsi2(Fix * Fix), by_Gpsi2(Fiy * Fiy), sp, a1, a2);
+            relaxed_12(kp, st, m_a, m_b, x.X[at], x.Y[at], sp, a1, a2);
             x.u[1][at] = div_const<9>(a1), x.u[2][at] = div_const<9>(a2);
+        } else if (role == 2) {
+            ru = rho * ux;
+            x.u[3][at] = div_const<3>(relaxed_j(m_a, Fx, ru));
+            x.u[4][at] = div_const<3>(relaxed_q(kp, m_b, Fx, ru, ux, x.X[at], x.Y[at], sq));
         } else {
-            double X = 0.0, Y = 0.0, aj, aq;
-            if (kp.improved) X = by_Gpsi2(Fix * Fix), Y = by_Gpsi2(Fiy * Fiy);
-            if (role == 2) relaxed_jq(kp, rho, m_a, m_b, Fx, ux, X, Y, sq, aj, aq);
-            else relaxed_jq(kp, rho, m_a, m_b, Fy, uy, Y, X, sq, aj, aq);
-            const int k = role == 2 ? 3 : 5;
-            x.u[k][at] = div_const<3>(aj), x.u[k + 1][at] = div_const<3>(aq);
+            x.u[6][at] = div_const<3>(relaxed_q(kp, m_b, Fy, ru, uy, x.Y[at], x.X[at], sq));
         }
         __syncthreads();
 
         double u[9], o[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) u[i] = x.u[i][at];
-        populations(u, o);  // (each warp evaluates the ones it stores)
-        if (role == 0) a.put(s, o, 0, 3);
-        else if (role == 1) a.put(s, o, 3, 2);
-        else if (role == 2) a.put(s, o, 5, 2);
-        else a.put(s, o, 7, 2);
+        if (role == 0) populations_013(u, o), a.put(s, o, 0x00bu);
+        else if (role == 1) populations_24(u, o), a.put(s, o, 0x014u);
+        else if (role == 2) populations_58(u, o), a.put(s, o, 0x120u);
+        else populations_67(u, o), a.put(s, o, 0x0c0u);
         s.barrier();
     }
-    if (role == 0) a.write_back(s, nsteps & 1, 0, 9);
+    if (role == 0) a.write_back(s, nsteps & 1);
 }
 
 template <class S>

@@ -69,27 +69,32 @@ __device__ __forceinline__ double density(const double (&f)[9])
     return r;
 }
 
-__device__ __forceinline__ double p_eos(const KParams &kp, double rho)
+// p_EOS = K (num/den - a rho^2); psi = sqrt(2 (p_EOS - rho/3)/G).  In pieces, which k_small1 spreads over
+// four warps.  Products by a gas constant or a K of 1 (the usual ones) change nothing and are left out.
+__device__ __forceinline__ double eos_num(const KParams &kp, double rho)
 {
-    // products by a gas constant or a K of 1 (the usual ones) change nothing and are left out
     const double rRT = (kp.unit_R ? rho : rho * kp.eos_R) * kp.eos_T;
-    if (kp.eos == 0) {
-        const double p = rRT / (1.0 - kp.eos_b * rho) - kp.eos_a * rho * rho;
-        return kp.unit_K ? p : kp.eos_K * p;
-    }
-    const double eta = kp.eos_b4 * rho;
-    const double e2 = eta * eta, om = 1.0 - eta;
-    const double num = 1.0 + eta + e2 - e2 * eta;
-    const double den = om * om * om;
-    const double p = rRT * num / den - kp.eos_a * rho * rho;
-    return kp.unit_K ? p : kp.eos_K * p;
+    if (kp.eos == 0) return rRT;
+    const double eta = kp.eos_b4 * rho, e2 = eta * eta;
+    return rRT * (1.0 + eta + e2 - e2 * eta);
 }
-
-// sqrt(2 (p_EOS - rho/3)/G); a G that is a power of two (the usual -1) divides exactly
+__device__ __forceinline__ double eos_den(const KParams &kp, double rho)
+{
+    if (kp.eos == 0) return 1.0 - kp.eos_b * rho;
+    const double om = 1.0 - kp.eos_b4 * rho;
+    return om * om * om;
+}
+__device__ __forceinline__ double eos_attraction(const KParams &kp, double rho) { return kp.eos_a * rho * rho; }
+// a G that is a power of two (the usual -1) divides exactly
+__device__ __forceinline__ double psi_of(const KParams &kp, double ratio, double attraction, double third)
+{
+    const double p = ratio - attraction;
+    const double d = (kp.unit_K ? p : kp.eos_K * p) - third;
+    return sqrt(kp.G_pow2 ? d * kp.two_inv_G : 2.0 * d / kp.G);
+}
 __device__ __forceinline__ double psi_of(const KParams &kp, double rho)
 {
-    const double d = p_eos(kp, rho) - div_const<3>(rho);
-    return sqrt(kp.G_pow2 ? d * kp.two_inv_G : 2.0 * d / kp.G);
+    return psi_of(kp, eos_num(kp, rho) / eos_den(kp, rho), eos_attraction(kp, rho), div_const<3>(rho));
 }
 
 // S of Eq. (fint), the terms in the order i = 1..8
@@ -113,21 +118,41 @@ __device__ __forceinline__ void stencil_S(const Ps &ps, double &Sx, double &Sy)
 }
 
 // f = M^T (m_k/|M_k|^2), the terms in the order k = 0..8, from u_k = m_k/|M_k|^2 without its power of
-// two (|M_k|^2 = 9, 36, 36, 6, 12, 6, 12, 4, 4), which the multiply-adds carry exactly.
-__device__ __forceinline__ void populations(const double (&u)[9], double (&f)[9])
+// two (|M_k|^2 = 9, 36, 36, 6, 12, 6, 12, 4, 4), which the multiply-adds carry exactly.  In the pieces that
+// k_small1 spreads over four warps: f_0, f_1 and f_3; f_2 and f_4; f_5 and f_8; f_6 and f_7.
+__device__ __forceinline__ double axes(const double (&u)[9]) { return fma_(-0.5, u[2], fma_(-0.25, u[1], u[0])); }
+__device__ __forceinline__ double diagonals(const double (&u)[9]) { return fma_(0.25, u[2], fma_(0.5, u[1], u[0])); }
+__device__ __forceinline__ void populations_013(const double (&u)[9], double (&f)[9])
 {
     f[0] = (u[0] - u[1]) + u[2];
-    const double a = fma_(-0.5, u[2], fma_(-0.25, u[1], u[0]));  // axes
+    const double a = axes(u);
     f[1] = fma_(0.25, u[7], fma_(-0.5, u[4], fma_(0.5, u[3], a)));
-    f[2] = fma_(-0.25, u[7], fma_(-0.5, u[6], fma_(0.5, u[5], a)));
     f[3] = fma_(0.25, u[7], fma_(0.5, u[4], fma_(-0.5, u[3], a)));
+}
+__device__ __forceinline__ void populations_24(const double (&u)[9], double (&f)[9])
+{
+    const double a = axes(u);
+    f[2] = fma_(-0.25, u[7], fma_(-0.5, u[6], fma_(0.5, u[5], a)));
     f[4] = fma_(-0.25, u[7], fma_(0.5, u[6], fma_(-0.5, u[5], a)));
-    const double d = fma_(0.25, u[2], fma_(0.5, u[1], u[0]));    // diagonals
-    const double p = fma_(0.25, u[4], fma_(0.5, u[3], d)), q = fma_(-0.25, u[4], fma_(-0.5, u[3], d));
+}
+__device__ __forceinline__ void populations_58(const double (&u)[9], double (&f)[9])
+{
+    const double p = fma_(0.25, u[4], fma_(0.5, u[3], diagonals(u)));
     f[5] = fma_(0.25, u[8], fma_(0.25, u[6], fma_(0.5, u[5], p)));
+    f[8] = fma_(-0.25, u[8], fma_(-0.25, u[6], fma_(-0.5, u[5], p)));
+}
+__device__ __forceinline__ void populations_67(const double (&u)[9], double (&f)[9])
+{
+    const double q = fma_(-0.25, u[4], fma_(-0.5, u[3], diagonals(u)));
     f[6] = fma_(-0.25, u[8], fma_(0.25, u[6], fma_(0.5, u[5], q)));
     f[7] = fma_(0.25, u[8], fma_(-0.25, u[6], fma_(-0.5, u[5], q)));
-    f[8] = fma_(-0.25, u[8], fma_(-0.25, u[6], fma_(-0.5, u[5], p)));
+}
+__device__ __forceinline__ void populations(const double (&u)[9], double (&f)[9])
+{
+    populations_013(u, f);
+    populations_24(u, f);
+    populations_58(u, f);
+    populations_67(u, f);
 }
 __device__ __forceinline__ void from_moments(const double (&m)[9], double (&f)[9])
 {
@@ -186,38 +211,40 @@ __device__ __forceinline__ void relaxation(const KParams &kp, double rho, double
 }
 // m_bar_k = m + F_m - s (m - m_eq + F_m/2) + s Q (Eq. lbe.col), Q_m with |F_int|^2 / (G psi^2) as written
 // in the paper (X = F_int,x^2 / (G psi^2), Y likewise)
-__device__ __forceinline__ void relaxed_12(const KParams &kp, double rho, double m1, double m2, double Fx, double Fy, double ux,
-                                           double uy, double X, double Y, double sp, double &a1, double &a2)
+struct Stress12 {
+    double e1, e2, Fm1;  // m_k - m_eq_k, and F_m1 = -F_m2
+};
+__device__ __forceinline__ Stress12 stress_12(double rho, double m1, double m2, double Fx, double Fy, double ux, double uy)
 {
     const double u2 = ux * ux + uy * uy, r3u2 = 3.0 * rho * u2;
-    const double meq1 = fma_(-2.0, rho, r3u2), meq2 = rho - r3u2;
-    const double Fm1 = 6.0 * (Fx * ux + Fy * uy);  // F_m2 = -F_m1
+    return Stress12{m1 - fma_(-2.0, rho, r3u2), m2 - (rho - r3u2), 6.0 * (Fx * ux + Fy * uy)};
+}
+__device__ __forceinline__ void relaxed_12(const KParams &kp, const Stress12 &t, double m1, double m2, double X, double Y, double sp,
+                                           double &a1, double &a2)
+{
     const double sQ1 = sp * (kp.q1c * (X + Y));
-    a1 = (m1 + Fm1) - sp * fma_(0.5, Fm1, m1 - meq1) + sQ1;
-    const double c2 = (m2 - Fm1) - sp * fma_(-0.5, Fm1, m2 - meq2);
+    a1 = (m1 + t.Fm1) - sp * fma_(0.5, t.Fm1, t.e1) + sQ1;
+    const double c2 = (m2 - t.Fm1) - sp * fma_(-0.5, t.Fm1, t.e2);
     a2 = kp.q2_full ? c2 - sQ1 : fma_(-0.5, sQ1, c2);  // Q_2 = -Q_1 or -Q_1/2
 }
-// one direction's momentum (s_j = 1) and energy flux; X along it, Y across
-__device__ __forceinline__ void relaxed_jq(const KParams &kp, double rho, double j, double q, double F, double u, double X,
-                                           double Y, double sq, double &aj, double &aq)
+// one direction's momentum (s_j = 1) and energy flux, ru = rho u; X along it, Y across
+__device__ __forceinline__ double relaxed_j(double j, double F, double ru) { return (j + F) - fma_(0.5, F, j - ru); }
+__device__ __forceinline__ double relaxed_q(const KParams &kp, double q, double F, double ru, double u, double X, double Y, double sq)
 {
-    const double ru = rho * u;
-    aj = (j + F) - fma_(0.5, F, j - ru);
-    aq = (q - F) - sq * fma_(-0.5, F, q + ru);
-    if (kp.improved) aq += sq * ((kp.q4a * X - kp.q4b * Y) * u);
+    const double aq = (q - F) - sq * fma_(-0.5, F, q + ru);
+    return kp.improved ? aq + sq * ((kp.q4a * X - kp.q4b * Y) * u) : aq;
 }
-__device__ __forceinline__ void relaxed_78(const KParams &kp, double rho, double m7, double m8, double Fx, double Fy, double ux,
-                                           double uy, double Fix, double Fiy, const Divisor &by_Gpsi2, double sp, double &a7,
-                                           double &a8)
+__device__ __forceinline__ double relaxed_7(double rux, double ruy, double m7, double Fx, double Fy, double ux, double uy, double Q7, double sp)
 {
-    const double rux = rho * ux, ruy = rho * uy;
-    const double meq7 = rux * ux - ruy * uy, meq8 = rux * uy;
+    const double meq7 = rux * ux - ruy * uy;
     const double h7 = Fx * ux - Fy * uy;  // F_m7/2
+    return fma_(2.0, h7, m7) - sp * ((m7 - meq7) + h7) + sp * Q7;
+}
+__device__ __forceinline__ double relaxed_8(double rux, double m8, double Fx, double Fy, double ux, double uy, double Q8, double sp)
+{
+    const double meq8 = rux * uy;
     const double Fm8 = Fx * uy + Fy * ux;
-    const double Q7 = by_Gpsi2(kp.k1 * (Fix * Fix - Fiy * Fiy));
-    const double Q8 = by_Gpsi2(kp.k1 * Fix * Fiy);
-    a7 = fma_(2.0, h7, m7) - sp * ((m7 - meq7) + h7) + sp * Q7;
-    a8 = (m8 + Fm8) - sp * fma_(0.5, Fm8, m8 - meq8) + sp * Q8;
+    return (m8 + Fm8) - sp * fma_(0.5, Fm8, m8 - meq8) + sp * Q8;
 }
 
 __device__ __forceinline__ void collide(const KParams &kp, const double (&f)[9], double psi, double Sx, double Sy,
@@ -244,10 +271,12 @@ __device__ __forceinline__ void collide(const KParams &kp, const double (&f)[9],
     if (kp.var_tau) relaxation(kp, rho, sp, sq);
     double mb[9];
     mb[0] = rho;
-    relaxed_12(kp, rho, m1, m2, Fx, Fy, ux, uy, X, Y, sp, mb[1], mb[2]);
-    relaxed_jq(kp, rho, jx, m4, Fx, ux, X, Y, sq, mb[3], mb[4]);
-    relaxed_jq(kp, rho, jy, m6, Fy, uy, Y, X, sq, mb[5], mb[6]);
-    relaxed_78(kp, rho, m7, m8, Fx, Fy, ux, uy, Fix, Fiy, by_Gpsi2, sp, mb[7], mb[8]);
+    relaxed_12(kp, stress_12(rho, m1, m2, Fx, Fy, ux, uy), m1, m2, X, Y, sp, mb[1], mb[2]);
+    const double rux = rho * ux, ruy = rho * uy;
+    mb[3] = relaxed_j(jx, Fx, rux), mb[4] = relaxed_q(kp, m4, Fx, rux, ux, X, Y, sq);
+    mb[5] = relaxed_j(jy, Fy, ruy), mb[6] = relaxed_q(kp, m6, Fy, ruy, uy, Y, X, sq);
+    mb[7] = relaxed_7(rux, ruy, m7, Fx, Fy, ux, uy, by_Gpsi2(kp.k1 * (Fix * Fix - Fiy * Fiy)), sp);
+    mb[8] = relaxed_8(rux, m8, Fx, Fy, ux, uy, by_Gpsi2(kp.k1 * Fix * Fiy), sp);
     from_moments(mb, fb);
 }
 
