@@ -10,8 +10,8 @@
 // its halo rows through distributed shared memory, so every load is a local one.
 //
 // Measured per step (us, one launch per step / here): 37 x 23 FP32 3.0 / 0.90, FP16 3.0 / 1.2; 64^2 FP32 3.0 / 1.06;
-// 128^2 3.0 / 2.1 (16 SMs are busy there: the last size that gains); FP64 4 x 128 column 18 / 6.5, 4 x 181
-// 18 / 9.2, 37 x 23 18 / 13.1.
+// 128^2 3.0 / 2.1 (16 SMs are busy there: the last size that gains); FP64 4 x 128 column 18 / 5.4, 4 x 181
+// 18 / 7.9, 37 x 23 18 / 11.2.
 //
 // The functions, their order and the storage type's rounding are the tile kernel's (k_tile.cuh), so
 // the state after n steps is, bit for bit, what n of its launches leave.
@@ -333,13 +333,14 @@ __global__ void __launch_bounds__(THREADS) k_small2(KParams kp, int64_t nsteps, 
 }
 
 // FP64.  An FP64 instruction holds its scheduler's quarter of the SM for 64 cycles, whatever the
-// number of active lanes and however independent its neighbours are, so a node's 390 of them in one
-// warp take 12 us, and a small lattice leaves most schedulers idle.  Four warps therefore share a
+// number of active lanes and however independent its neighbours are, so a node's 328 of them in one
+// warp take 11 us, and a small lattice leaves most schedulers idle.  Four warps therefore share a
 // group of 32 nodes, one per scheduler, and hand each other the few values they need through
 // shared memory, in six parts between barriers (a barrier costs no more than one FP64 instruction):
 // density and the terms of p_EOS; psi, moments, 1/rho; the x and y force and velocity, 1/(G psi^2); the
 // quotients by G psi^2; the relaxed moments; the populations, each warp those it stores.  (4 x 128 column:
-// 18 us a step with one launch per step, 13.2 with one warp per 32 nodes, 7.5 in four parts, 6.5 in six.)
+// 18 us a step with one launch per step, 13.2 with one warp per 32 nodes, 7.5 in four parts, 6.5 in six, 5.4
+// with 328 FP64 instructions a node instead of 395.)
 struct Small64Shared {
     static constexpr int M = kSmallThreads / 4;
     double num[M], attraction[M], third[M];                      // of psi: p_EOS = K (num/den - attraction), rho/3

@@ -16,7 +16,9 @@
 //   * the coefficients of Q_m are formed once on the host, in the same order.
 // The dense evaluation with 17 general divisions issued 465 FP64 instructions a node in the collide
 // pass.  Against it, per step: 256 x 256 banded channel (two-pass) 100 -> 61 us, 1024 x 1024
-// periodic (one-pass) 1.58 -> 1.12 ms, 4 x 128 column (latency of one warp per SM) 24 -> 20 us.
+// periodic (one-pass) 1.58 -> 1.12 ms, 4 x 128 column (latency of one warp per SM) 24 -> 20 us; the
+// tile and small-lattice kernels and the general division out of line (below) take the rest of the way to
+// 47 us, 0.65 ms and 5.4 us.
 #pragma once
 
 namespace lbm {
@@ -34,6 +36,10 @@ __device__ __forceinline__ bool in_range(double a)
     const unsigned hi = (unsigned)__double2hiint(a) & 0x7fffffffu;
     return hi - (573u << 20) < (900u << 20) || (hi | (unsigned)__double2loint(a)) == 0u;
 }
+// The general division of those, a function of its own: inlined, its first instructions were executed at
+// every quotient, whether it was then needed or not (395 FP64 instructions a node instead of 328; 1024^2
+// periodic 0.77 -> 0.65 ms a step, 256^2 55.6 -> 47.3 us, 4 x 128 column 6.5 -> 5.4).
+static __device__ __noinline__ double div_general(double a, double b) { return a / b; }
 template <int D>
 __device__ __forceinline__ double div_const(double a)
 {
@@ -41,7 +47,7 @@ __device__ __forceinline__ double div_const(double a)
     constexpr double r = 1.0 / (double)D;
     const double q = a * r;
     const double t = fma_(fma_(-(double)D, q, a), r, q);
-    return in_range(a) ? t : a / (double)D;
+    return in_range(a) ? t : div_general(a, (double)D);
 }
 
 // Quotients by one divisor b, each correctly rounded: q = RN(a r) with r = RN(1/b) is within two
@@ -55,7 +61,7 @@ struct Divisor {
         double q = a * r;
         q = fma_(fma_(-b, q, a), r, q);
         q = fma_(fma_(-b, q, a), r, q);
-        return ok && in_range(a) ? q : a / b;
+        return ok && in_range(a) ? q : div_general(a, b);
     }
 };
 __device__ __forceinline__ bool is_nonzero(double b) { return (((unsigned)__double2hiint(b) & 0x7fffffffu) | (unsigned)__double2loint(b)) != 0u; }
