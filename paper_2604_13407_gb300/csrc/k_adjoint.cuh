@@ -540,7 +540,9 @@ __device__ __forceinline__ void adj_block(const KParams &kp, const AdjArgs &aa, 
         }
     }
     // ---- parameter sums, in the order of AdjSlot: one row of FP64 partial sums per block, accumulated over
-    // all steps of a call and reduced once at its end (no contended atomics, a fixed order)
+    // all steps of a call and reduced once at its end (no other block adds to it: a fixed order).  Added in L2:
+    // a load of the row's entry and an FP64 add were the last thing a block waited for (2048^2: 231 -> 226 us
+    // a step of the call).
     {
         const T v[7] = {gFx, gFy, gG, gT, Jt, gG2, gT2};
 #pragma unroll
@@ -552,7 +554,7 @@ __device__ __forceinline__ void adj_block(const KParams &kp, const AdjArgs &aa, 
     // away from walls the wall terms (and objective 0, the force on them) are zero
     const unsigned skip = walled ? 0u : (1u << SLOT_T1) | (aa.objective == 0 ? 1u << SLOT_J : 0u);
     block_add<R>(&red[0][0], N * 32 * UNITS, 7, N * 32 * UNITS, UNITS, skip,
-                 [&](int q, double t) { aa.part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kAdjSlots + q] += t; });
+                 [&](int q, double t) { atomicAdd(&aa.part[((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kAdjSlots + q], t); });
 }
 
 // One transposed step at A_t (kp.src) with the psi field of A_t (kp.psi).  U: units of a block, B: blocks
