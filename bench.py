@@ -32,7 +32,7 @@ RHO_G, RHO_L = 0.009291723294794338, 0.3581443962580134  # Maxwell densities of 
 T_07 = 0.7 * 0.3773 / 4.0
 TAU = 1.0
 BYTES = {"f64": 144, "f32": 72, "f16dev": 36, "bf16dev": 36}
-# DRAM bytes per lattice update of the packed fused kernel (k_fused2), from one ncu capture
+# DRAM bytes per lattice update of the staged kernel (k_fused2), from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum of one launch at 4096 x 4096; profiles/k_fused2_*;
 # f16dev: the per-node reference mode), scaled to a launch by the updates it makes.
 # Valid for the kernel as captured; an entry is removed when the kernel changes until it is captured
@@ -538,7 +538,7 @@ def main():
                 variants[name]["note"] = ("deviations from one reference density, stochastically rounded: about "
                                           "5e-2 of max |u| on the two-phase channel (16x the per-node mode)")
             if prec == "f64":
-                # FP64-ALU bound: ncu shows the FP64 pipe busy and DRAM nearly idle (k_fused_f64 profile)
+                # FP64-ALU bound: ncu shows the FP64 pipe busy and DRAM nearly idle (k_tile1)
                 variants[name]["bound"] = "fp64 alu"
             s2.close()
 

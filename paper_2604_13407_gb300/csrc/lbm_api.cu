@@ -300,10 +300,10 @@ static bool auto_prefers_fused(const lbm_ctx *c)
 // step's results.  The staged kernel reads each row once where the tile kernel re-reads its tiles'
 // rings from L2, but a CTA walks its rows in series, and it has no walls; the tile kernel has thousands
 // of short blocks.  Step times on a GB300 (us, tile / staged): FP32 periodic 512^2 5.4 / 10.3, 1024^2
-// 14.4 / 22.9, 2048^2 52 / 56.7, 4096^2 193 / 195, 8192^2 788 / 745; FP16, whose ring costs instructions
-// and not bytes, 1024^2 18.5 / 26.9, 1024 x 2048 35 / 43, 2048^2 67 / 59, 4096^2 249 / 194.  (Two-pass
+// 13.8 / 22.8, 2048^2 49.7 / 56.6, 4096^2 186 / 195, 8192^2 759 / 745; FP16, whose ring costs instructions
+// and not bytes, 1024^2 17.2 / 27.2, 1024 x 2048 33 / 44, 2048^2 64 / 59, 4096^2 238 / 194.  (Two-pass
 // kernels, FP32: 512^2 10.3, 1024^2 31, 2048^2 121; 256 x 2048 with walls 20.6 against the tile kernel's
-// 9.2; banded 512^2 17.6 / 5.9; annulus 1024^2 44 / 20.)
+// 8.9; banded 512^2 17.6 / 5.9; annulus 1024^2 44 / 16.)
 static void choose_kernel(lbm_ctx *c)
 {
     const int want = c->p.kernel;

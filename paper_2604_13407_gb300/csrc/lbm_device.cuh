@@ -1,7 +1,7 @@
 // Device building blocks of the D2Q9 pseudopotential MRT step: lattice constants,
 // storage codecs, EOS pseudopotential, pull streaming with wall links, collision.
-// Every kernel variant calls these same functions in the same order, so the two-pass
-// and the fused kernels produce bit-identical populations.
+// Every kernel variant evaluates the same expressions in the same order, so the two-pass, tile
+// and small-lattice kernels produce bit-identical populations.
 #pragma once
 
 #include <cuda_bf16.h>

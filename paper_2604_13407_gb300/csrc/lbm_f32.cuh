@@ -1,13 +1,14 @@
 // FP32 arithmetic of the step (FP32, FP16 and BF16 population storage): density, psi,
 // psi stencil and collision, written once for a lane type V that is either one node (v1,
 // scalar FP32 instructions) or two nodes (v2, packed FP32x2 instructions: FADD2, FMUL2,
-// FFMA2 of the sm_100 family).  The two-pass kernels use v1, the packed fused kernel v2;
-// both evaluate the same expressions in the same order.  The scalar _rn intrinsics round
+// FFMA2 of the sm_100 family).  The two-pass and small-lattice kernels use v1, the staged kernel and
+// the transposed step v2, the tile kernel a pair rounded like v1 (v2x, k_tile.cuh); all evaluate the
+// same expressions in the same order.  The scalar _rn intrinsics round
 // exactly as written (checked bit for bit against a numpy evaluation of the same
 // expressions).  The pair intrinsics do not always: measured on this toolchain, a packed
 // product that feeds a packed sum is sometimes fused into one multiply-add (a*b + c*d
 // with the halves of b and d swapped: 30% of random cases, every mismatch explained by
-// the fusion), so the fused kernel agrees with the two-pass kernel to rounding, and keeps
+// the fusion), so the staged kernel agrees with the others to rounding, and keeps
 // the x and y mirror symmetries exactly (the same instruction serves a node and its mirror
 // image) but the diagonal one only to rounding.
 //
