@@ -9,7 +9,11 @@
 // fuses a packed product into a following packed sum, which rounds once where the one-node
 // evaluation rounds twice; with them every node's result is the two-pass step's, bit for bit (the
 // links of interpolated and moving walls to rounding: their coefficients come from the link
-// records, formed in FP64).
+// records, formed in FP64).  16-bit storage on the lattices where LBM_KERNEL_FUSED is granted
+// (KParams::packed) takes plain packed products and the staged kernel's encode instead (v2): a
+// stored deviation is rounded from values that the staged kernel has too, so LBM_KERNEL_AUTO leaves the
+// same states there whichever of the two kernels a size gets, bit for bit.  (In FP32 storage the
+// two roundings differ by an ulp of a population and no more, and the exact products stay.)
 // FP64 (k_tile1): one node per thread, the two-pass step's own functions, the same bits.
 //
 // A tile of n pairs (rows) has n warps for them; one more warp pulls the rows above and below the
@@ -50,6 +54,8 @@ __device__ __forceinline__ v2x vsqrt(v2x a) { return X2(sqrt32(a.v.x), sqrt32(a.
 __device__ __forceinline__ v2x vclamp01(v2x a) { return X2(fminf(fmaxf(a.v.x, 0.f), 1.f), fminf(fmaxf(a.v.y, 0.f), 1.f)); }
 template <> __device__ __forceinline__ v2x ks<v2x>(float a) { return X2(a, a); }
 template <> __device__ __forceinline__ v2x kc<v2x>(const float2 &c) { return v2x{c}; }
+// two floats as a pair of either rounding (v2, v2x)
+template <class V> __device__ __forceinline__ V pair_of(float a, float b) { return V{make_float2(a, b)}; }
 
 // ------------------------------------------------------------- block sums --------
 __device__ __forceinline__ double warp_sum(double v)
@@ -224,11 +230,11 @@ struct Tile2SharedDiag : Tile2Shared {
     float umax[kTilePairs];
     int bad[kTilePairs];
 };
-template <class S, int GEOM, class O, int MODE, bool INNER, class Shared>
+template <class S, int GEOM, class O, int MODE, bool INNER, class V, class Shared>
 __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const TileOut &out, Shared &sh)
 {
     auto &sm = sh.psi;
-    constexpr bool DEV = IsDev<S>::value;
+    constexpr bool DEV = IsDev<S>::value, PACKED = std::is_same<V, v2>::value;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int np = (blockDim.x >> 5) - 2, rows = 2 * np;  // pairs and rows of this launch's tiles
     const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * rows;
@@ -273,8 +279,8 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
             asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
         }
     }
-    v2x f[9], d[9], rho = X2(1.f, 1.f), psi = X2(0.f, 0.f);
-    v2x momx = X2(0.f, 0.f), momy = momx;  // momentum handed to the walls (diagnostics)
+    V f[9], d[9], rho = pair_of<V>(1.f, 1.f), psi = pair_of<V>(0.f, 0.f);
+    V momx = pair_of<V>(0.f, 0.f), momy = momx;  // momentum handed to the walls (diagnostics)
     if (!still) {
         // pull, Eq. (lbe.str)
         const S *src = static_cast<const S *>(kp.src);
@@ -317,9 +323,9 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
         }
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-            v2x wr = X2(0.f, 0.f);
-            if (DEV) wr = has_ref ? v2x{kp.c2.w[i]} * X2(refa[i], refb[i]) : v2x{kp.c2.dec[i]};
-            f[i] = X2(Raw<S>::f(va[i], wr.v.x, kp), Raw<S>::f(vb[i], wr.v.y, kp));
+            V wr = pair_of<V>(0.f, 0.f);
+            if (DEV) wr = has_ref ? V{kp.c2.w[i]} * pair_of<V>(refa[i], refb[i]) : V{kp.c2.dec[i]};
+            f[i] = pair_of<V>(Raw<S>::f(va[i], wr.v.x, kp), Raw<S>::f(vb[i], wr.v.y, kp));
         }
         if ((!INNER || GEOM) && ((wa | wb) & 0x1feu)) {
             // wall links: the population that left the node toward the wall comes back
@@ -376,10 +382,10 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
         }
         to_dev(f, d);
         rho = density_dev(d);
-        psi = psi_v<v2x>(kp, rho);
+        psi = psi_v<V>(kp, rho);
     } else if constexpr (MODE == TILE_DIAG) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = X2(0.f, 0.f);
+        for (int i = 0; i < 9; ++i) f[i] = pair_of<V>(0.f, 0.f);
     }
     if (GEOM) {
         if (wa & 1u) psi.v.x = kp.wall_psi_f ? kp.wall_psi_f[node_a] : kp.cf.psi_s, rho.v.x = 1.f;
@@ -411,23 +417,23 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int k = 0; k < 3; ++k) c[r][k] = q[r * kTilePitch + k];
-    v2x Sx, Sy, Fex, Fey, fb[9], ux, uy;
-    stencil_v<v2x>(X2(c[1][2], c[2][2]), X2(c[2][1], c[3][1]), X2(c[1][0], c[2][0]), X2(c[0][1], c[1][1]),
-                   X2(c[2][2], c[3][2]), X2(c[2][0], c[3][0]), X2(c[0][0], c[1][0]), X2(c[0][2], c[1][2]), Sx, Sy);
+    V Sx, Sy, Fex, Fey, fb[9], ux, uy;
+    stencil_v<V>(pair_of<V>(c[1][2], c[2][2]), pair_of<V>(c[2][1], c[3][1]), pair_of<V>(c[1][0], c[2][0]), pair_of<V>(c[0][1], c[1][1]),
+                   pair_of<V>(c[2][2], c[3][2]), pair_of<V>(c[2][0], c[3][0]), pair_of<V>(c[0][0], c[1][0]), pair_of<V>(c[0][2], c[1][2]), Sx, Sy);
     const int mode = O::force_mode(kp);
     if (mode == 0) {
-        Fex = v2x{kp.c2.Fx}, Fey = v2x{kp.c2.Fy};
+        Fex = V{kp.c2.Fx}, Fey = V{kp.c2.Fy};
     } else if (mode == 1) {  // Sec. 3.3: (rho - rho_g) g
-        const v2x e = rho - v2x{kp.c2.rho_g};
-        Fex = e * v2x{kp.c2.Fx}, Fey = e * v2x{kp.c2.Fy};
+        const V e = rho - V{kp.c2.rho_g};
+        Fex = e * V{kp.c2.Fx}, Fey = e * V{kp.c2.Fy};
     } else if (kp.fext_f) {
         const int64_t n = (int64_t)kp.nx * kp.ny;
-        Fex = X2(kp.fext_f[node_a], kp.fext_f[node_b]);
-        Fey = X2(kp.fext_f[n + node_a], kp.fext_f[n + node_b]);
+        Fex = pair_of<V>(kp.fext_f[node_a], kp.fext_f[node_b]);
+        Fey = pair_of<V>(kp.fext_f[n + node_a], kp.fext_f[n + node_b]);
     } else {
-        Fex = Fey = X2(0.f, 0.f);
+        Fex = Fey = pair_of<V>(0.f, 0.f);
     }
-    collide_v<v2x, O>(kp, d, rho, psi, Sx, Sy, Fex, Fey, fb, ux, uy);
+    collide_v<V, O>(kp, d, rho, psi, Sx, Sy, Fex, Fey, fb, ux, uy);
 
     if constexpr (MODE == TILE_MOMENTS) {
         // solid nodes report their virtual density at rest
@@ -441,15 +447,15 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
         return;
     }
     if constexpr (MODE == TILE_DIAG) {
-        const v2x jx = ((f[1] - f[3]) + (f[5] - f[6])) + (f[8] - f[7]), jy = ((f[2] - f[4]) + (f[5] + f[6])) - (f[7] + f[8]);
-        const v2x nGpsi = v2x{kp.c2.m_G} * psi, Fx = vfma(nGpsi, Sx, Fex), Fy = vfma(nGpsi, Sy, Fey);
+        const V jx = ((f[1] - f[3]) + (f[5] - f[6])) + (f[8] - f[7]), jy = ((f[2] - f[4]) + (f[5] + f[6])) - (f[7] + f[8]);
+        const V nGpsi = V{kp.c2.m_G} * psi, Fx = vfma(nGpsi, Sx, Fex), Fy = vfma(nGpsi, Sy, Fey);
         const float half_lg = float(0.5 * (kp.rho_l + kp.rho_g));
         float um = 0.f;
         int bad = 0;
         if (warp < np) {
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                auto get = [&](v2x a) { return e ? a.v.y : a.v.x; };
+                auto get = [&](V a) { return e ? a.v.y : a.v.x; };
                 const bool on = e ? sb : sa;
                 const float r = get(rho), u = get(ux), v = get(uy);
                 const bool liquid = on && r > half_lg;
@@ -500,8 +506,10 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
         const unsigned pick = (ka & 1u) ? 0x7632u : 0x5410u;
 #pragma unroll
         for (int i = 0; i < 9; ++i, da += kp.plane, db += kp.plane) {
-            const v2x wr = has_ref ? v2x{kp.c2.w[i]} * rho : v2x{kp.c2.dec[i]};
-            const v2x s = (fb[i] - wr) * v2x{kp.c2.scale};
+            const V wr = has_ref ? V{kp.c2.w[i]} * rho : V{kp.c2.dec[i]};
+            V s;
+            if constexpr (PACKED) s = vfma(fb[i], V{kp.c2.scale}, has_ref ? V{kp.c2.m_scale} * wr : V{kp.c2.enc[i]});
+            else s = (fb[i] - wr) * V{kp.c2.scale};
             uint32_t h;
             if (kp.sr) {
                 h = SRound<S>::pack(s.v.x, s.v.y, __byte_perm(sr_bits(ha, i), sr_bits(hb, i), pick));
@@ -521,21 +529,21 @@ __device__ __forceinline__ bool tile_inner(const KParams &kp, int rows)
     const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * rows;
     return x0 >= 2 && x0 + kTileX + 2 <= kp.nx && y0 >= 2 && y0 + rows + 2 <= kp.ny;
 }
-template <class S, int GEOM, class O>
+template <class S, int GEOM, class O, class V>
 __global__ void __launch_bounds__(32 * (kTilePairs + 2), 5) k_tile2(KParams kp, int ahead)
 {
     __shared__ Tile2Shared sh;
     const TileOut none{};
-    if (tile_inner(kp, 2 * ((blockDim.x >> 5) - 2))) tile2_block<S, GEOM, O, TILE_STEP, true>(kp, ahead, none, sh);
-    else tile2_block<S, GEOM, O, TILE_STEP, false>(kp, ahead, none, sh);
+    if (tile_inner(kp, 2 * ((blockDim.x >> 5) - 2))) tile2_block<S, GEOM, O, TILE_STEP, true, V>(kp, ahead, none, sh);
+    else tile2_block<S, GEOM, O, TILE_STEP, false, V>(kp, ahead, none, sh);
 }
 // The readings of a state, on tiles of kTilePairs pairs (the whole block's sums want a full one).
 template <class S, int MODE>
 __global__ void __launch_bounds__(32 * (kTilePairs + 2), MODE == TILE_MOMENTS ? 5 : 4) k_read2(KParams kp, int ahead, TileOut out)
 {
     __shared__ typename std::conditional<MODE == TILE_DIAG, Tile2SharedDiag, Tile2Shared>::type sh;
-    if (tile_inner(kp, 2 * kTilePairs)) tile2_block<S, 3, RuntimeOpts, MODE, true>(kp, ahead, out, sh);
-    else tile2_block<S, 3, RuntimeOpts, MODE, false>(kp, ahead, out, sh);
+    if (tile_inner(kp, 2 * kTilePairs)) tile2_block<S, 3, RuntimeOpts, MODE, true, v2x>(kp, ahead, out, sh);
+    else tile2_block<S, 3, RuntimeOpts, MODE, false, v2x>(kp, ahead, out, sh);
 }
 
 // Column sums of the blocks' rows (kDiagSlots columns; the largest |u| by maximum), one block per column
@@ -710,6 +718,22 @@ inline cudaError_t with_options(const KParams &kp, const F &f)
     return kp.var_tau ? with_force<1, 0>(kp, f) : with_force<0, 0>(kp, f);
 }
 
+// The packed rounding fixes fewer of them: the assembler fuses a packed product into a sum where both stand in one
+// block of the code, so the relaxation and the scheme stay branches exactly where the staged kernel
+// (Fused2::launch) has them.  512 x 4096 with walls: 36.6 us with all at run time, 34.7 here, 35.4 with
+// exact products and the options above; bands 2048^2, two relaxation times, 72.6 / 70.6 / 80.3.
+template <class F>
+inline cudaError_t with_packed_options(const KParams &kp, bool plain, const F &f)
+{
+    const bool ref = kp.per_node_ref != 0;
+    if (plain && kp.force_mode == 0 && !kp.var_tau) {
+        if (ref) return kp.improved ? f(Opts<1, 0, 0, 1>()) : f(Opts<0, 0, 0, 1>());
+        return kp.improved ? f(Opts<1, 0, 0, 0>()) : f(Opts<0, 0, 0, 0>());
+    }
+    if (!ref) return f(Opts<-1, -1, -1, 0>());
+    return kp.force_mode == 0 ? f(Opts<-1, -1, 0, 1>()) : kp.force_mode == 1 ? f(Opts<-1, -1, 1, 1>()) : f(Opts<-1, -1, 2, 1>());
+}
+
 // Rows (units: pairs or rows) of a tile: of the heights from `most`/2 to `most`, the one whose fullest
 // SM has the least to do, a block counting its units and its ring warps.
 inline int tile_height(const KParams &kp, int most, int rows_per_unit, int ring_warps)
@@ -780,11 +804,19 @@ struct Tile {
             const dim3 grid((kp.nx + kTileX - 1) / kTileX, (kp.ny + 2 * h - 1) / (2 * h)), block(32 * (h + 2));
             const int ahead = ahead_of(kp, grid, 2 * h);
             const KParams kq = with_pull(kp);
+            auto go = [&](auto kernel) { return launch_dependent(kernel, grid, block, 0, st, kq, ahead); };
+            const bool links = kp.q || kp.wall_u, solid = kp.solid != nullptr;
+            if constexpr (IsDev<S>::value) {
+                if (kp.packed) {
+                    const bool open = kp.periodic_x && kp.periodic_y;
+                    if (links) return with_packed_options(kp, false, [&](auto o) { return go(k_tile2<S, 2, decltype(o), v2>); });
+                    if (solid) return with_packed_options(kp, false, [&](auto o) { return go(k_tile2<S, 1, decltype(o), v2>); });
+                    return with_packed_options(kp, open, [&](auto o) { return go(k_tile2<S, 0, decltype(o), v2>); });
+                }
+            }
             return with_options<IsDev<S>::value>(kp, [&](auto o) {
                 typedef decltype(o) O;
-                if (kp.q || kp.wall_u) return launch_dependent(k_tile2<S, 2, O>, grid, block, 0, st, kq, ahead);
-                if (kp.solid) return launch_dependent(k_tile2<S, 1, O>, grid, block, 0, st, kq, ahead);
-                return launch_dependent(k_tile2<S, 0, O>, grid, block, 0, st, kq, ahead);
+                return links ? go(k_tile2<S, 2, O, v2x>) : solid ? go(k_tile2<S, 1, O, v2x>) : go(k_tile2<S, 0, O, v2x>);
             });
         }
     }

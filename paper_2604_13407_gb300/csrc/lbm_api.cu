@@ -314,6 +314,7 @@ static void choose_kernel(lbm_ctx *c)
     const bool tile = c->L.tile_pass != nullptr;
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
     const bool large = n >= (c->p.precision == LBM_F32 ? (int64_t)1 << 25 : (int64_t)3 << 20);
+    c->kp.packed = c->fused_ok && c->p.precision >= LBM_F16DEV;
     c->one_pass = nullptr;
     c->small_ctas = want == LBM_KERNEL_AUTO ? c->L.small_ctas(c->kp) : 0;
     if (want == LBM_KERNEL_TWO_PASS || (want == LBM_KERNEL_FUSED && !possible)) return;
