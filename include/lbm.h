@@ -185,7 +185,8 @@ LBM_API lbm_status lbm_destroy(lbm_ctx *ctx);
  *                         conserving; against a dense liquid the fluid mass drifts, while
  *                         half-way links conserve it to round-off)
  *   force_field[2*ny*nx]  force density of LBM_FORCE_FIELD
- * Passing NULL clears the corresponding array.  Call before stepping. */
+ * Passing NULL clears the corresponding array.  A call that fails for want of memory (or for a
+ * CUDA error) leaves the context without any of them.  Call before stepping. */
 LBM_API lbm_status lbm_set_geometry(lbm_ctx *ctx, const uint8_t *solid, const double *wall_u,
                             const double *q, const double *force_field);
 
@@ -194,7 +195,7 @@ LBM_API lbm_status lbm_set_geometry(lbm_ctx *ctx, const uint8_t *solid, const do
  * rho_s node by node, e.g. a gas-wetted inner and a liquid-wetted outer cylinder).  Every
  * entry must be positive with psi(entry) real (LBM_EINVAL otherwise; the previous field
  * is kept).  Walls beyond a non-periodic edge keep rho_s.  NULL restores rho_s at every
- * wall.  lbm_get_moments reports the field at solid nodes.  lbm_adjoint_step rejects a
+ * wall, and so does a call that fails for want of memory.  lbm_get_moments reports the field at solid nodes.  lbm_adjoint_step rejects a
  * context with a field set (LBM_ENOTSUP).  Call before stepping. */
 LBM_API lbm_status lbm_set_wall_density(lbm_ctx *ctx, const double *wall_rho);
 

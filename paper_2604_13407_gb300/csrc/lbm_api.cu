@@ -436,13 +436,18 @@ static lbm_status need_scratch(lbm_ctx *c, size_t bytes)
 }
 
 template <class T>
+static void release(lbm_ctx *c, T **p)
+{
+    if (!*p) return;
+    cudaStreamSynchronize(c->stream);
+    cudaFree(*p);
+    *p = nullptr;
+}
+
+template <class T>
 static lbm_status upload(lbm_ctx *c, T **dst, const T *src, size_t count, const char *what)
 {
-    if (*dst) {
-        cudaStreamSynchronize(c->stream);
-        cudaFree(*dst);
-        *dst = nullptr;
-    }
+    release(c, dst);
     if (!src) return LBM_OK;
     CK(cudaMalloc((void **)dst, count * sizeof(T)), what);
     CK(cudaMemcpyAsync(*dst, src, count * sizeof(T), cudaMemcpyHostToDevice, c->stream), what);
@@ -458,11 +463,7 @@ static __global__ void k_narrow(const double *in, float *out, int64_t n)
 // *dst = src[count] in FP32 (null src: none), for the storage types whose arithmetic is FP32.
 static lbm_status narrow(lbm_ctx *c, float **dst, const double *src, size_t count, const char *what)
 {
-    if (*dst) {
-        cudaStreamSynchronize(c->stream);
-        cudaFree(*dst);
-        *dst = nullptr;
-    }
+    release(c, dst);
     if (!src || c->p.precision == LBM_F64) return LBM_OK;
     CK(cudaMalloc((void **)dst, count * sizeof(float)), what);
     k_narrow<<<(unsigned)((count + 255) / 256), 256, 0, c->stream>>>(src, *dst, (int64_t)count);
@@ -481,11 +482,7 @@ static lbm_status build_link_records(lbm_ctx *c, const uint8_t *solid, const dou
     static const int EX[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, EY[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
     static const int OPP[9] = {0, 3, 4, 1, 2, 7, 8, 5, 6};
     static const double W[9] = {4.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 36, 1.0 / 36, 1.0 / 36, 1.0 / 36};
-    if (c->link) {
-        cudaStreamSynchronize(c->stream);
-        cudaFree(c->link);
-        c->link = nullptr;
-    }
+    release(c, &c->link);
     if (!q && !wall_u) return LBM_OK;
     const int nx = c->p.nx, ny = c->p.ny;
     const int64_t n = (int64_t)nx * ny, pitch = c->pitch, plane = c->plane;
@@ -525,15 +522,10 @@ static lbm_status build_link_records(lbm_ctx *c, const uint8_t *solid, const dou
     return LBM_OK;
 }
 
-extern "C" lbm_status lbm_set_geometry(lbm_ctx *c, const uint8_t *solid, const double *wall_u, const double *q,
-                                       const double *force_field)
-{
-    if (!c) return LBM_EINVAL;
+static lbm_status build_geometry(lbm_ctx *c, const uint8_t *solid, const double *wall_u, const double *q,
+                                 const double *force_field)
+try {
     const size_t n = (size_t)c->p.nx * c->p.ny;
-    if (q) {
-        for (size_t k = 0; k < 8 * n; ++k)
-            if (!(q[k] > 0.0 && q[k] <= 1.0)) return fail(c, LBM_EINVAL, "q must lie in (0, 1]");
-    }
     lbm_status s;
     if ((s = upload(c, &c->solid, solid, n, "solid")) != LBM_OK) return s;
     c->n_fluid = (int64_t)n;
@@ -544,24 +536,52 @@ extern "C" lbm_status lbm_set_geometry(lbm_ctx *c, const uint8_t *solid, const d
     if ((s = upload(c, &c->fext, force_field, 2 * n, "force_field")) != LBM_OK) return s;
     if ((s = narrow(c, &c->fext_f, c->fext, 2 * n, "force_field")) != LBM_OK) return s;
     if (c->p.precision != LBM_F64 && (s = build_link_records(c, solid, wall_u, q)) != LBM_OK) return s;
-    if (c->links) {
-        CK(cudaStreamSynchronize(c->stream), "set_geometry");
-        cudaFree(c->links);
-        c->links = nullptr;
-    }
+    release(c, &c->links);
     if (solid || wall_u || q) {
         CK(cudaMalloc((void **)&c->links, n * sizeof(uint16_t)), "wall bits");
         fill_constants(c);
         CK(c->L.link_bits(c->kp, c->links, c->stream), "wall bits kernel");
     }
     CK(cudaStreamSynchronize(c->stream), "set_geometry");
+    return LBM_OK;
+} catch (const std::bad_alloc &) {
+    return fail(c, LBM_ENOMEM, "host allocation failed");
+}
+
+extern "C" lbm_status lbm_set_geometry(lbm_ctx *c, const uint8_t *solid, const double *wall_u, const double *q,
+                                       const double *force_field)
+{
+    if (!c) return LBM_EINVAL;
+    const size_t n = (size_t)c->p.nx * c->p.ny;
+    if (q) {
+        for (size_t k = 0; k < 8 * n; ++k)
+            if (!(q[k] > 0.0 && q[k] <= 1.0)) return fail(c, LBM_EINVAL, "q must lie in (0, 1]");
+    }
+    const lbm_status s = build_geometry(c, solid, wall_u, q, force_field);
+    if (s != LBM_OK) {
+        // the old arrays gave way to the new ones, of which some are missing: none at all
+        release(c, &c->solid), release(c, &c->wall_u), release(c, &c->q), release(c, &c->fext);
+        release(c, &c->fext_f), release(c, &c->link), release(c, &c->links);
+        c->n_fluid = (int64_t)n;
+    }
     fill_constants(c);
     choose_kernel(c);
+    return s;
+}
+
+static lbm_status build_wall_density(lbm_ctx *c, const double *wall_rho, const double *psi)
+{
+    const size_t n = (size_t)c->p.nx * c->p.ny;
+    lbm_status s;
+    if ((s = upload(c, &c->wall_rho, wall_rho, n, "wall_rho")) != LBM_OK) return s;
+    if ((s = upload(c, &c->wall_psi, psi, n, "wall_psi")) != LBM_OK) return s;
+    if ((s = narrow(c, &c->wall_psi_f, c->wall_psi, n, "wall_psi")) != LBM_OK) return s;
+    CK(cudaStreamSynchronize(c->stream), "set_wall_density");
     return LBM_OK;
 }
 
 extern "C" lbm_status lbm_set_wall_density(lbm_ctx *c, const double *wall_rho)
-{
+try {
     if (!c) return LBM_EINVAL;
     const size_t n = (size_t)c->p.nx * c->p.ny;
     std::vector<double> psi;
@@ -574,15 +594,13 @@ extern "C" lbm_status lbm_set_wall_density(lbm_ctx *c, const double *wall_rho)
                 return fail(c, LBM_EINVAL, "psi of a wall density is not real and positive");
         }
     }
-    lbm_status s;
-    if ((s = upload(c, &c->wall_rho, wall_rho, n, "wall_rho")) != LBM_OK) return s;
-    if ((s = upload(c, &c->wall_psi, wall_rho ? psi.data() : (const double *)nullptr, n, "wall_psi")) != LBM_OK)
-        return s;
-    if ((s = narrow(c, &c->wall_psi_f, c->wall_psi, n, "wall_psi")) != LBM_OK) return s;
-    CK(cudaStreamSynchronize(c->stream), "set_wall_density");
+    const lbm_status s = build_wall_density(c, wall_rho, wall_rho ? psi.data() : nullptr);
+    if (s != LBM_OK) release(c, &c->wall_rho), release(c, &c->wall_psi), release(c, &c->wall_psi_f);
     fill_constants(c);
     choose_kernel(c);
-    return LBM_OK;
+    return s;
+} catch (const std::bad_alloc &) {
+    return fail(c, LBM_ENOMEM, "host allocation failed");
 }
 
 // Bring `count` doubles from host or device into a device pointer (scratch slot `slot`).
