@@ -580,20 +580,25 @@ static lbm_status build_wall_density(lbm_ctx *c, const double *wall_rho, const d
     return LBM_OK;
 }
 
+// psi of n wall densities under the parameters p: the same host evaluation as psi(rho_s), so a uniform field
+// equals the scalar.  False where one is not real and positive.
+static bool wall_psi_of(const lbm_params &p, const double *wall_rho, size_t n, std::vector<double> &psi)
+{
+    psi.resize(n);
+    for (size_t k = 0; k < n; ++k) {
+        psi[k] = host_psi(p, wall_rho[k]);
+        if (!(wall_rho[k] > 0.0) || !(psi[k] > 0.0) || !std::isfinite(psi[k])) return false;
+    }
+    return true;
+}
+
 extern "C" lbm_status lbm_set_wall_density(lbm_ctx *c, const double *wall_rho)
 try {
     if (!c) return LBM_EINVAL;
     const size_t n = (size_t)c->p.nx * c->p.ny;
     std::vector<double> psi;
-    if (wall_rho) {
-        psi.resize(n);
-        for (size_t k = 0; k < n; ++k) {
-            // the same host evaluation as psi(rho_s), so a uniform field equals the scalar
-            psi[k] = host_psi(c->p, wall_rho[k]);
-            if (!(wall_rho[k] > 0.0) || !(psi[k] > 0.0) || !std::isfinite(psi[k]))
-                return fail(c, LBM_EINVAL, "psi of a wall density is not real and positive");
-        }
-    }
+    if (wall_rho && !wall_psi_of(c->p, wall_rho, n, psi))
+        return fail(c, LBM_EINVAL, "psi of a wall density is not real and positive");
     const lbm_status s = build_wall_density(c, wall_rho, wall_rho ? psi.data() : nullptr);
     if (s != LBM_OK) release(c, &c->wall_rho), release(c, &c->wall_psi), release(c, &c->wall_psi_f);
     fill_constants(c);
@@ -847,8 +852,23 @@ extern "C" lbm_status lbm_load_state(lbm_ctx *c, const void *host_buf, size_t nb
     return LBM_OK;
 }
 
-extern "C" lbm_status lbm_set_param(lbm_ctx *c, int32_t which, double value)
+// psi of the wall densities under the parameters p, into the arrays that hold it.
+static lbm_status refresh_wall_psi(lbm_ctx *c, const lbm_params &p)
 {
+    const size_t n = (size_t)c->p.nx * c->p.ny;
+    std::vector<double> rho(n), psi;
+    CK(cudaMemcpyAsync(rho.data(), c->wall_rho, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "wall_rho");
+    CK(cudaStreamSynchronize(c->stream), "wall_rho");
+    if (!wall_psi_of(p, rho.data(), n, psi)) return fail(c, LBM_EINVAL, "psi of a wall density is not real and positive");
+    CK(cudaMemcpyAsync(c->wall_psi, psi.data(), n * sizeof(double), cudaMemcpyHostToDevice, c->stream), "wall_psi");
+    if (c->wall_psi_f) k_narrow<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(c->wall_psi, c->wall_psi_f, (int64_t)n);
+    CK(cudaGetLastError(), "wall_psi");
+    CK(cudaStreamSynchronize(c->stream), "wall_psi");
+    return LBM_OK;
+}
+
+extern "C" lbm_status lbm_set_param(lbm_ctx *c, int32_t which, double value)
+try {
     if (!c) return LBM_EINVAL;
     lbm_params np = c->p;
     switch (which) {
@@ -860,9 +880,12 @@ extern "C" lbm_status lbm_set_param(lbm_ctx *c, int32_t which, double value)
     }
     lbm_status s = validate(c, np);
     if (s != LBM_OK) return s;
+    if (c->wall_rho && (which == LBM_PARAM_G || which == LBM_PARAM_T) && (s = refresh_wall_psi(c, np)) != LBM_OK) return s;
     c->p = np;
     fill_constants(c);
     return LBM_OK;
+} catch (const std::bad_alloc &) {
+    return fail(c, LBM_ENOMEM, "host allocation failed");
 }
 
 extern "C" lbm_status lbm_adjoint_step(lbm_ctx *c, int64_t nsteps, int32_t checkpoint_every, int32_t objective,

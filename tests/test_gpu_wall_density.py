@@ -126,3 +126,44 @@ def test_invalid_wall_density_is_rejected_and_adjoint_refuses_the_field():
     sim.init_fields(rho)
     J = sim.objective(2)
     assert np.isfinite(J)
+
+
+@pytest.mark.parametrize("precision", [lbm.F64, lbm.F32, lbm.F16DEV])
+@pytest.mark.parametrize("which,factor", [(lbm.PARAM_T, 0.96), (lbm.PARAM_G, 1.25)])
+def test_wall_psi_follows_a_changed_parameter(precision, which, factor):
+    """After lbm_set_param of T or G a uniform wall density is still the scalar rho_s, bit for bit; a value that
+    makes the pseudopotential of a wall density imaginary is refused and changes nothing."""
+    p, solid, _, _, rho, _ = channel_case()
+    states = []
+    for field in (False, True):
+        sim = lbm.Simulation(GC.gpu_params(p, precision, per_node_ref=1))
+        sim.set_geometry(solid)
+        if field:
+            sim.set_wall_density(np.full(solid.shape, sim.params.rho_s))
+        sim.init_fields(rho)
+        sim.step(3)
+        sim.set_param(which, factor * (p.T if which == lbm.PARAM_T else p.G))
+        sim.step(3)
+        states.append(sim.get_state())
+        sim.close()
+    assert np.all(np.isfinite(states[0])) and np.array_equal(states[0], states[1])
+
+
+def test_a_parameter_that_a_wall_density_forbids_is_refused():
+    p, solid, _, _, rho, _ = channel_case()
+    gp = GC.gpu_params(p, lbm.F64)
+    gp.rho_max = 0.37
+    sims = []
+    for refused in (False, True):
+        sim = lbm.Simulation(gp)
+        sim.set_geometry(solid)
+        sim.set_wall_density(np.where(solid == 1, 0.45, 0.1))
+        sim.init_fields(rho)
+        if refused:
+            with pytest.raises(lbm.LbmError) as e:
+                sim.set_param(lbm.PARAM_T, 1.3 * p.T)
+            assert e.value.status == 1
+        sim.step(3)
+        sims.append(sim.get_state().tobytes())  # (bits: so dense a wall overdrives the fluid beside it within three steps)
+        sim.close()
+    assert sims[0] == sims[1]
