@@ -1,7 +1,9 @@
 // Host side of the C ABI declared in include/lbm.h: parameter validation, device
 // buffers, kernel dispatch, checkpoint/resume and the adjoint driver.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -974,15 +976,49 @@ lbm_status kparams_for(const lbm_params *p, int64_t pitch, KParams *out)
     return LBM_OK;
 }
 
+// The driver's entry points are fetched through the runtime, so the library needs no link to the driver library.
+unsigned long long current_context()
+{
+    struct Driver {
+        CUresult (*get_current)(CUcontext *) = nullptr;
+        CUresult (*get_id)(CUcontext, unsigned long long *) = nullptr;
+        Driver()
+        {
+            void *a = nullptr, *b = nullptr;
+            cudaDriverEntryPointQueryResult qa, qb;
+            cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &qa);
+            if (e == cudaSuccess) e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &qb);
+            if (e != cudaSuccess || qa != cudaDriverEntryPointSuccess || qb != cudaDriverEntryPointSuccess) return;
+            get_current = reinterpret_cast<CUresult (*)(CUcontext *)>(a);
+            get_id = reinterpret_cast<CUresult (*)(CUcontext, unsigned long long *)>(b);
+        }
+    };
+    static const Driver d;
+    CUcontext ctx = nullptr;
+    unsigned long long id = 0;
+    if (!d.get_current || !d.get_id || d.get_current(&ctx) != CUDA_SUCCESS || !ctx || d.get_id(ctx, &id) != CUDA_SUCCESS) return 0;
+    return id;
+}
+
+// A kernel's attributes belong to a context: what was set in one is not there after a reset of the device, nor in
+// another context.  So what was set, and what the device answered, is kept with the context's ID.
 cudaError_t ensure_smem_attribute_ptr(const void *kernel, int device, int bytes)
 {
+    struct Done {
+        const void *kernel;
+        int device;
+        unsigned long long context;
+    };
     static std::mutex mu;
-    static std::vector<std::pair<const void *, int>> done;
+    static std::vector<Done> done;
+    const unsigned long long context = current_context();
     std::lock_guard<std::mutex> lock(mu);
-    for (const auto &d : done)
-        if (d.first == kernel && d.second == device) return cudaSuccess;
+    auto d = std::find_if(done.begin(), done.end(), [&](const Done &x) { return x.kernel == kernel && x.device == device; });
+    if (d != done.end() && context != 0 && d->context == context) return cudaSuccess;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) done.emplace_back(kernel, device);
+    if (e != cudaSuccess) return e;
+    if (d == done.end()) done.push_back({kernel, device, context});
+    else d->context = context;
     return e;
 }
 
@@ -991,13 +1027,15 @@ bool cluster_fits(const void *kernel, int device, int ctas, int threads, int sme
     struct Asked {
         const void *kernel;
         int device, ctas;
+        unsigned long long context;
         bool fits;
     };
     static std::mutex mu;
     static std::vector<Asked> done;
+    const unsigned long long context = current_context();
     std::lock_guard<std::mutex> lock(mu);
-    for (const Asked &d : done)
-        if (d.kernel == kernel && d.device == device && d.ctas == ctas) return d.fits;
+    auto d = std::find_if(done.begin(), done.end(), [&](const Asked &x) { return x.kernel == kernel && x.device == device && x.ctas == ctas; });
+    if (d != done.end() && context != 0 && d->context == context) return d->fits;
     int n = 0;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1015,8 +1053,10 @@ bool cluster_fits(const void *kernel, int device, int ctas, int threads, int sme
         e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
     }
     if (e != cudaSuccess) cudaGetLastError();  // (not an error of the caller's: the lattice is stepped launch by launch)
-    done.push_back({kernel, device, ctas, e == cudaSuccess && n > 0});
-    return done.back().fits;
+    if (d == done.end()) d = done.insert(done.end(), Asked{kernel, device, ctas, context, false});
+    d->context = context;
+    d->fits = e == cudaSuccess && n > 0;
+    return d->fits;
 }
 
 // psi of the EOS of *p at rho (the host evaluation create uses), for lbm_lbana.cu.

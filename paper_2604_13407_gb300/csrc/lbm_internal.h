@@ -132,8 +132,12 @@ enum Prec { P_F64 = 0, P_F32 = 1, P_F16 = 2, P_BF16 = 3 };
 // Device error word bits
 enum DevErr { DERR_TIMEOUT = 1, DERR_BOUNDS = 2 };
 
-// One-time set-up of a kernel's dynamic shared-memory limit, per kernel and device (an
-// attribute set with one device current does not apply to another); lbm_api.cu.
+// ID of the calling thread's current context (0: none is current, or it cannot be had).  A device that is
+// reset and another context made current get new ones; lbm_api.cu.
+unsigned long long current_context();
+
+// One-time set-up of a kernel's dynamic shared-memory limit, per kernel, device and context (an
+// attribute set in one context does not apply to another); lbm_api.cu.
 cudaError_t ensure_smem_attribute_ptr(const void *kernel, int device, int bytes);
 template <class K>
 inline cudaError_t ensure_smem_attribute(K kernel, int device, int bytes)
@@ -142,7 +146,7 @@ inline cudaError_t ensure_smem_attribute(K kernel, int device, int bytes)
 }
 
 // Whether the device can hold a cluster of `ctas` blocks of the kernel with these limits (shared memory
-// and cluster size are then allowed for it), asked once per kernel, device and size; lbm_api.cu.
+// and cluster size are then allowed for it), asked once per kernel, device, context and size; lbm_api.cu.
 bool cluster_fits(const void *kernel, int device, int ctas, int threads, int smem_bytes);
 
 // Launchers, defined in the per-precision translation units (k_f64.cu, k_f32.cu,

@@ -7,7 +7,6 @@
 // memory and keeps its only scratch buffer -- the pseudopotential field read by the
 // collide pass -- in a file-scope device array of fixed size.  Every device that loads the
 // library holds that array (LBM_NOALLOC_MAX_NODES floats) until the process exits.
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -37,32 +36,6 @@ struct NoallocSlot {
 static std::mutex g_noalloc_mutex;
 static NoallocSlot g_noalloc_slot[256];
 
-typedef CUresult (*PfnCtxGetCurrent)(CUcontext *);
-typedef CUresult (*PfnCtxGetId)(CUcontext, unsigned long long *);
-
-// ID of the calling thread's current context (0: none is current); driver entry points are
-// fetched through the runtime, so the library needs no link to the driver library.
-static lbm_status current_context_id(unsigned long long *id)
-{
-    static PfnCtxGetCurrent get_current = nullptr;
-    static PfnCtxGetId get_id = nullptr;
-    if (!get_current || !get_id) {
-        void *a = nullptr, *b = nullptr;
-        cudaDriverEntryPointQueryResult qa, qb;
-        cudaError_t e = cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &qa);
-        if (e == cudaSuccess) e = cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &qb);
-        if (e != cudaSuccess || !a || !b || qa != cudaDriverEntryPointSuccess || qb != cudaDriverEntryPointSuccess)
-            return set_global_error(LBM_ECUDA, "driver entry points cuCtxGetCurrent / cuCtxGetId not available");
-        get_current = reinterpret_cast<PfnCtxGetCurrent>(a);
-        get_id = reinterpret_cast<PfnCtxGetId>(b);
-    }
-    CUcontext ctx = nullptr;
-    if (get_current(&ctx) != CUDA_SUCCESS) return set_global_error(LBM_ECUDA, "cuCtxGetCurrent failed");
-    *id = 0;
-    if (ctx && get_id(ctx, id) != CUDA_SUCCESS) return set_global_error(LBM_ECUDA, "cuCtxGetId failed");
-    return LBM_OK;
-}
-
 static lbm_status noalloc_scratch(float **out)
 {
     int dev = 0;
@@ -70,9 +43,7 @@ static lbm_status noalloc_scratch(float **out)
     if (e != cudaSuccess) return set_global_error(LBM_ECUDA, std::string("cudaGetDevice: ") + cudaGetErrorString(e));
     if (dev < 0 || dev >= 256) return set_global_error(LBM_ENOTSUP, "device ordinal out of range");
     std::lock_guard<std::mutex> lock(g_noalloc_mutex);
-    unsigned long long ctx = 0;
-    lbm_status s = current_context_id(&ctx);
-    if (s != LBM_OK) return s;
+    unsigned long long ctx = current_context();
     NoallocSlot &slot = g_noalloc_slot[dev];
     if (ctx == 0 || ctx != slot.ctx_id || !slot.addr) {
         void *ptr = nullptr;
@@ -80,7 +51,7 @@ static lbm_status noalloc_scratch(float **out)
         if (e != cudaSuccess)
             return set_global_error(LBM_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
         // the look-up made the device's primary context current if none was
-        if ((s = current_context_id(&ctx)) != LBM_OK) return s;
+        ctx = current_context();
         slot.ctx_id = ctx;
         slot.addr = static_cast<float *>(ptr);
     }

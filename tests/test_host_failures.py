@@ -91,3 +91,16 @@ def test_set_wall_density_that_runs_out_of_memory(fakelib, prec, before):
         fake.sound(fakelib)
         k += 1
     assert k >= (2 if prec == lbm.F64 else 3)
+
+
+def test_a_reset_device_is_asked_again(fakelib):
+    """What a kernel was allowed (shared memory, cluster size) is gone after a reset of the device: it is set
+    again for the new context, and only once for each."""
+    fakelib.fake_reset(0)
+    for _ in range(3):
+        assert fakelib.fake_cluster_fits(16) == 1
+    assert fakelib.fake_attributes() == 2
+    fakelib.fake_device_reset()
+    for _ in range(3):
+        assert fakelib.fake_cluster_fits(16) == 1
+    assert fakelib.fake_attributes() == 4
