@@ -311,7 +311,7 @@ def geometry_throughput(hbm, steps=2000, warmup=20, only=None, kernel=0, precs=(
             out["%s_%s" % (name, prec)] = {
                 "GLUPS": g, "us_per_step": 1e6 * t / steps, "bytes_per_update": b, "achieved_GBs": b * g,
                 "frac_of_hbm": b * g / hbm, "state_MB": state_mb, "steps": steps,
-                "kernel": "fused" if s.kernel_in_use == lbm.KERNEL_FUSED else "two_pass"}
+                "kernel": s.step_launches(steps)[1]}
             s.close()
     return out
 
@@ -497,7 +497,7 @@ def main():
 
     sim = make_sim(n, prec_id[args.precision], per_node_ref=args.node_ref)
     sim.init_fields(rho)
-    kernels_per_step = 1 if sim.kernel_in_use == lbm.KERNEL_FUSED else 2
+    launches, step_kernel = sim.step_launches(args.steps)
     with ClockSampler(dev_uuid) as clk:
         t = timed_steps(sim, args.steps, args.warmup, dist_on)
     clocks = clk.summary()
@@ -506,9 +506,8 @@ def main():
     updates = job_updates(n, args.steps, world)
     value = updates / t / 1e9
     bpu = BYTES[args.precision] + (8 if args.precision in ("f16dev", "bf16dev") and args.node_ref else 0)
-    # one kernel launch per step on the fused path: the average launch duration is the timed
-    # region divided by the steps (CUDA events on the launching stream)
-    t_launch = t / args.steps / kernels_per_step
+    # the average launch duration is the timed region divided by its launches (CUDA events on the launching stream)
+    t_launch = t / launches
     achieved = bpu * n * n / (t / args.steps) / 1e9
 
     variants = {}
@@ -531,7 +530,7 @@ def main():
             b = BYTES[prec] + (8 if extra.get("per_node_ref") else 0)
             g = n * n * k / t2 / 1e9
             variants[name] = {"GLUPS": g, "bytes_per_update": b, "achieved_GBs": b * g, "frac": b * g / hbm,
-                              "kernel": "fused" if s2.kernel_in_use == lbm.KERNEL_FUSED else "two_pass"}
+                              "kernel": s2.step_launches(k)[1]}
             if name == "f16dev_node_ref_nearest":
                 variants[name]["note"] = "stored deviations rounded to nearest (storage_rounding = 0)"
             if name == "f16dev_global_ref":
@@ -579,12 +578,14 @@ def main():
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "peak_kind": peak_kind,
                          "traffic": (TRAFFIC_PER_UPDATE[args.precision] * n * n
-                                     if kernels_per_step == 1 and TRAFFIC_PER_UPDATE.get(args.precision)
+                                     if step_kernel == "staged" and TRAFFIC_PER_UPDATE.get(args.precision)
                                      and (args.precision == "f32" or args.node_ref) else None),
                          "traffic_unit": "DRAM bytes per launch (ncu, scaled to this lattice)",
                          "bytes_per_update": bpu, "launch_ms": 1e3 * t_launch,
-                         "kernel": "k_fused2" if kernels_per_step == 1 else "two_pass (step)"},
-            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": args.steps * kernels_per_step,
+                         "kernel": {"staged": "k_fused2", "tile": "k_tile1" if args.precision == "f64" else "k_tile2",
+                                    "small": "k_small1" if args.precision == "f64" else "k_small2",
+                                    "two_pass": "k_psi, k_collide"}[step_kernel]},
+            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches,
             "clocks": clocks, "variants": variants, "geometry": geometry, "adjoint": adjoint,
             "mass": d[0],
         }

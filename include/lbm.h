@@ -277,9 +277,24 @@ LBM_API lbm_status lbm_sync(lbm_ctx *ctx);
 /* Number of steps since the last lbm_init_fields / lbm_set_state. */
 LBM_API int64_t lbm_step_count(const lbm_ctx *ctx);
 
-/* Kind of step lbm_step runs: LBM_KERNEL_FUSED, or LBM_KERNEL_TWO_PASS for the two-pass step's results
- * (from the two-pass kernels, or in one pass from the tile kernel of LBM_KERNEL_AUTO). */
+/* Which of the two requestable steps the context takes: that of LBM_KERNEL_TWO_PASS or LBM_KERNEL_FUSED (for
+ * LBM_KERNEL_AUTO by size and geometry).  An AUTO context leaves the states that the kernel named here
+ * leaves on request: bit for bit in FP64 and 16-bit storage, and in FP32 storage for
+ * LBM_KERNEL_TWO_PASS; to rounding in FP32 storage for LBM_KERNEL_FUSED, and with interpolated or moving
+ * walls in FP32 arithmetic for LBM_KERNEL_TWO_PASS.  Which kernel it launches for that: lbm_step_launches. */
 LBM_API int32_t lbm_kernel_in_use(const lbm_ctx *ctx);
+
+typedef enum {
+    LBM_STEP_TWO_PASS = 0, /* psi pass and collide pass */
+    LBM_STEP_STAGED = 1,   /* one pass on staged rows */
+    LBM_STEP_TILE = 2,     /* one pass on tiles */
+    LBM_STEP_SMALL = 3     /* many steps of a small lattice in one launch (calls of four steps and more) */
+} lbm_step_kernel;
+
+/* Number of step kernels that lbm_step(ctx, nsteps) launches from here, and in *kernel (may be NULL) the
+ * lbm_step_kernel that takes the steps (LBM_STEP_SMALL also where the last few are taken one by one).
+ * -1 for an invalid argument. */
+LBM_API int64_t lbm_step_launches(const lbm_ctx *ctx, int64_t nsteps, int32_t *kernel);
 
 /* "LB-ana" (Sec. 3.1, Figs. 3-4): the steady velocity profile of two-phase Poiseuille flow that
  * the step itself predicts for a given density profile across the channel, from the

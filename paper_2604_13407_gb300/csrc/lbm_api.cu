@@ -288,7 +288,8 @@ static bool fused_possible(const lbm_ctx *c)
     return true;
 }
 
-// What lbm_kernel_in_use calls an LBM_KERNEL_AUTO context: LBM_KERNEL_FUSED from these sizes on.
+// Which of the two requestable steps an LBM_KERNEL_AUTO context takes (lbm_kernel_in_use): LBM_KERNEL_FUSED's from
+// these sizes on.  16-bit storage rounds accordingly (KParams::packed).
 static bool auto_prefers_fused(const lbm_ctx *c)
 {
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
@@ -661,12 +662,16 @@ static uint32_t sr_seed_of(int64_t t)
     return h;
 }
 
+// How many of the next nsteps steps the small-lattice kernel takes in one launch (no more than 4096, so that no
+// launch takes long); 0: none (fewer than four are as fast one by one).
+static int64_t at_once(const lbm_ctx *c, int64_t nsteps)
+{
+    return c->small_ctas > 0 && nsteps >= 4 ? std::min<int64_t>(nsteps, 4096) : 0;
+}
+
 static lbm_status run_steps(lbm_ctx *c, int64_t nsteps)
 {
-    // a small lattice: many steps in one launch (no more than 4096, so that no launch takes long; fewer
-    // than four are as fast one by one)
-    while (c->small_ctas > 0 && nsteps >= 4) {
-        const int64_t n = std::min<int64_t>(nsteps, 4096);
+    while (const int64_t n = at_once(c, nsteps)) {
         bind_buffers(c, c->cur);
         CK(c->L.small_steps(c->kp, c->small_ctas, n, c->steps, c->stream), "small-lattice kernel");
         c->cur ^= (int)(n & 1);
@@ -913,6 +918,25 @@ extern "C" int32_t lbm_kernel_in_use(const lbm_ctx *c)
 {
     if (!c) return -1;
     return c->fused_ok ? LBM_KERNEL_FUSED : LBM_KERNEL_TWO_PASS;
+}
+
+extern "C" int64_t lbm_step_launches(const lbm_ctx *c, int64_t nsteps, int32_t *kernel)
+{
+    if (!c || nsteps < 0) return -1;
+    const int64_t D = c->p.diag_every;
+    const int64_t first = D > 0 ? std::min<int64_t>(nsteps, D - c->steps % D) : nsteps, rest = nsteps - first;
+    auto launches = [&](int64_t n) {
+        const int64_t most = at_once(c, n);
+        if (most == 0) return c->one_pass ? n : 2 * n;
+        const int64_t left = n % most;
+        return n / most + (at_once(c, left) ? 1 : c->one_pass ? left : 2 * left);
+    };
+    if (kernel)
+        *kernel = at_once(c, rest > 0 ? std::max(first, std::min(rest, D)) : first) ? LBM_STEP_SMALL
+                  : !c->one_pass                                                    ? LBM_STEP_TWO_PASS
+                  : c->one_pass == c->L.fused_pass                                  ? LBM_STEP_STAGED
+                                                                                    : LBM_STEP_TILE;
+    return launches(first) + (rest > 0 ? rest / D * launches(D) + launches(rest % D) : 0);
 }
 
 extern "C" const char *lbm_last_error(const lbm_ctx *c)

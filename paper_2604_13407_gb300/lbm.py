@@ -17,6 +17,7 @@ EOS_VDW, EOS_CS = 0, 1
 FORCE_CONST, FORCE_BUOYANT, FORCE_FIELD = 0, 1, 2
 KERNEL_AUTO, KERNEL_TWO_PASS, KERNEL_FUSED = 0, 1, 2
 PARAM_FX, PARAM_FY, PARAM_G, PARAM_T = 0, 1, 2, 3
+STEP_KERNELS = ("two_pass", "staged", "tile", "small")  # lbm_step_kernel
 OBJ_WALL_FORCE_Y, OBJ_MEAN_JX = 0, 1
 NDIAG = 10
 
@@ -83,6 +84,7 @@ def load_library(path=None):
         "lbm_sync": (st, [_vp]),
         "lbm_step_count": (ctypes.c_int64, [_vp]),
         "lbm_kernel_in_use": (ctypes.c_int32, [_vp]),
+        "lbm_step_launches": (ctypes.c_int64, [_vp, ctypes.c_int64, _P(ctypes.c_int32)]),
         "lbm_last_error": (ctypes.c_char_p, [_vp]),
         "lbm_step_noalloc_f32": (st, [_P(LbmParams), _vp, _vp, ctypes.c_int64, _vp]),
         "lbm_lb_ana": (st, [_P(LbmParams), ctypes.c_int32, ctypes.c_int32, _dp, _dp, ctypes.c_double, _dp]),
@@ -231,6 +233,14 @@ class Simulation:
     @property
     def kernel_in_use(self):
         return self.lib.lbm_kernel_in_use(self._h)
+
+    def step_launches(self, nsteps=1):
+        """(number of step kernels that step(nsteps) launches, which: one of STEP_KERNELS)."""
+        k = ctypes.c_int32(0)
+        n = self.lib.lbm_step_launches(self._h, int(nsteps), ctypes.byref(k))
+        if n < 0:
+            raise ValueError("nsteps < 0")
+        return n, STEP_KERNELS[k.value]
 
     def set_param(self, which, value):
         self._check(self.lib.lbm_set_param(self._h, int(which), float(value)))

@@ -201,6 +201,7 @@ LBM_API void fake_reset(int small_ctas)
 LBM_API long fake_faults() { return g_faults; }
 LBM_API const char *fake_what() { return g_what.c_str(); }
 LBM_API const char *fake_last_step() { return g_last.c_str(); }
+LBM_API long fake_launches() { return g_launches; }
 LBM_API long fake_mallocs() { return g_mallocs; }
 LBM_API long fake_attributes() { return g_attributes; }
 LBM_API void fake_device_reset() { ++g_context; }
@@ -220,6 +221,7 @@ cudaError_t cudaMalloc(void **p, size_t n)
     if (g_mallocs_left > 0) --g_mallocs_left;
     if (g_bytes_left != (size_t)-1) g_bytes_left -= n;
     *p = std::calloc(n + 64, 1);
+    if (!*p) return cudaErrorMemoryAllocation;
     g_live[static_cast<char *>(*p)] = n + 64;
     ++g_mallocs;
     return cudaSuccess;
@@ -230,7 +232,8 @@ cudaError_t cudaFree(void *p)
     if (it == g_live.end()) fault("freed twice");
     else {
         if (g_bytes_left != (size_t)-1) g_bytes_left += it->second - 64;
-        g_live.erase(it);  // (the block itself stays, so that no later one takes its address)
+        if (it->second > (64u << 20)) std::free(p);  // (smaller blocks stay, so that no later one takes their address)
+        g_live.erase(it);
     }
     return cudaSuccess;
 }
@@ -243,7 +246,7 @@ cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind kin
 }
 cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t)
 {
-    std::memset(d, v, n);
+    std::memset(d, v, n < 4096 ? n : 4096);  // (blocks are zeroed when they are allocated; the largest are never touched)
     return cudaSuccess;
 }
 cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
