@@ -31,7 +31,7 @@ struct lbm_ctx {
     void *pops[2] = {nullptr, nullptr};
     float *refp[2] = {nullptr, nullptr};
     int cur = 0;
-    void *psi = nullptr;
+    void *psi = nullptr;    // psi field of the two-pass step; rows of sums of the diagnostics
     uint8_t *solid = nullptr;
     double *wall_u = nullptr, *q = nullptr, *fext = nullptr;
     double *wall_rho = nullptr, *wall_psi = nullptr;  // per solid node virtual density, its psi
@@ -389,8 +389,11 @@ extern "C" lbm_status lbm_create(const lbm_params *p, void *cuda_stream, lbm_ctx
         }
         return true;
     };
+    // the psi field, and between steps the diagnostics' rows of sums
+    c->kp.nx = p->nx, c->kp.ny = p->ny;
+    const size_t psi_bytes = std::max((size_t)n * c->real, (size_t)c->L.diag_rows(c->kp) * 11 * sizeof(double));
     bool ok = alloc(&c->pops[0], pop_bytes) && alloc(&c->pops[1], pop_bytes) &&
-              alloc(&c->psi, (size_t)n * c->real) && alloc((void **)&c->dacc, 16 * sizeof(double)) &&
+              alloc(&c->psi, psi_bytes) && alloc((void **)&c->dacc, 16 * sizeof(double)) &&
               alloc((void **)&c->derr, sizeof(int));
     if (ok && p->precision >= LBM_F16DEV && p->per_node_ref)
         ok = alloc((void **)&c->refp[0], (size_t)c->plane * 4) && alloc((void **)&c->refp[1], (size_t)c->plane * 4);
@@ -754,8 +757,7 @@ extern "C" lbm_status lbm_get_diagnostics(lbm_ctx *c, double out[LBM_NDIAG])
     if (!c->initialised) return fail(c, LBM_ESTATE, "fields not initialised");
     lbm_status s;
     bind_buffers(c, c->cur);
-    if ((s = need_scratch(c, (size_t)c->L.diag_rows(c->kp) * 11 * sizeof(double))) != LBM_OK) return s;
-    CK(c->L.diag(c->kp, c->scratch, c->dacc, c->stream), "diagnostics kernel");
+    CK(c->L.diag(c->kp, static_cast<double *>(c->psi), c->dacc, c->stream), "diagnostics kernel");
     double h[11];
     CK(cudaMemcpyAsync(h, c->dacc, sizeof h, cudaMemcpyDeviceToHost, c->stream), "D2H");
     if ((s = sync_and_check(c, "diagnostics")) != LBM_OK) return s;

@@ -104,3 +104,16 @@ def test_a_reset_device_is_asked_again(fakelib):
     for _ in range(3):
         assert fakelib.fake_cluster_fits(16) == 1
     assert fakelib.fake_attributes() == 4
+
+
+@pytest.mark.parametrize("prec", [lbm.F64, lbm.F32, lbm.F16DEV])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (1, 3000), (40, 24), (700, 1)])
+def test_diagnostics_allocate_nothing(fakelib, prec, nx, ny):
+    fakelib.fake_reset(0)
+    sim = lbm.Simulation(lbm.default_params(nx=nx, ny=ny, precision=prec, diag_every=2))
+    sim.init_fields(np.full((ny, nx), 0.2))
+    fake.limit(fakelib, mallocs=0)
+    sim.diagnostics()
+    sim.step(5)
+    sim.close()
+    fake.sound(fakelib)
