@@ -261,12 +261,12 @@ LBM_API lbm_status lbm_set_param(lbm_ctx *ctx, int32_t which, double value);
  * FP32 on the decoded states, taking the storage's rounding as the identity (the gradient
  * of the unrounded step along the 16-bit run's trajectory).  Device memory (allocated on
  * the first call, kept until lbm_destroy or a larger call): ceil(nsteps/K) + 2 (K - 1)
- * population states (with their reference-density plane), 2 K psi fields and 27 planes (FP64: 29) of
- * the arithmetic type (FP64 for FP64 storage, FP32 otherwise), K = min(checkpoint_every,
- * nsteps) (the
- * recompute of a segment overlaps, on a second stream, the transposed steps of the segment
- * after it); LBM_ENOMEM when it does not fit (lower checkpoint_every).  LBM_EINVAL: nsteps or
- * checkpoint_every < 1, unknown objective. */
+ * population states (with their reference-density plane), 2 K psi fields and 26 planes (FP64:
+ * 28) of the arithmetic type (FP64 for FP64 storage, FP32 otherwise), K = min(checkpoint_every,
+ * nsteps) (the recompute of a segment overlaps, on a second stream, the transposed steps of the
+ * segment after it; without the overlap, K - 1 states and K psi fields, where there is one segment or
+ * no memory for more; one state less for an odd nsteps); LBM_ENOMEM when that does not fit (lower
+ * checkpoint_every).  LBM_EINVAL: nsteps or checkpoint_every < 1, unknown objective. */
 LBM_API lbm_status lbm_adjoint_step(lbm_ctx *ctx, int64_t nsteps, int32_t checkpoint_every,
                             int32_t objective, double *J, double grad[4], double *lambda0);
 

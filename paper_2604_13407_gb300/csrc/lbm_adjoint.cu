@@ -6,19 +6,22 @@
 //   lambda_n = W/n,  lambda_t = W/n + Step'(A_t)^T lambda_{t+1}  (t = n-1 .. 1),
 //   lambda_0 = Step'(A_0)^T lambda_1,  dJ/dtheta = sum_t (dStep(A_t)/dtheta)^T lambda_{t+1}.
 //
-// Forward sweep: n steps, each from one buffer straight into another: the states at t = K, 2K, ... are written into their checkpoints, the others into scratch (the
-// segment states, not yet in use), A_n into the context's buffer that n steps would leave it in (where
-// that is A_0's own, A_0 is copied to its checkpoint first).  The steps of the last segment
-// write the segment's states and psi fields on the way, so that segment is never recomputed.
-// <W, A_n> is summed in FP64 there, <W, A_t> of the other states by the transposed steps (objective
-// alone: every state in the forward sweep).  Backward sweep, one segment of K steps at a time from the
-// last: the states of the segment are recomputed from its checkpoint with the step kernels the context
-// uses, each leaving the psi field of the state it reads in a buffer of its own (the two-pass step's
-// psi pass writes it anyway; the one-pass steps write it on request), then the transposed step runs
-// from the last state of the segment to the first.  The recompute of a segment runs on a second
-// stream, overlapping the transposed steps of the segment after it, so segment states and psi fields
-// come in two sets.  Device memory: ceil(n/K) checkpoints, 2 (K - 1) segment states, 2 K psi
-// fields and the adjoint planes; it is kept for the next call with the same sizes.
+// Forward sweep: n steps, each from one buffer straight into another: the states at t = K, 2K, ... are
+// written into their checkpoints, the others into scratch (the segment states, not yet in use), A_n
+// into the context's buffer that n steps would leave it in (where that is A_0's own, n even, A_0 is
+// copied to its checkpoint first).  The steps of the last segment write the segment's states and psi
+// fields on the way, so that segment is never recomputed.  <W, A_n> is summed in FP64 there, <W, A_t>
+// of the other states by the transposed steps (objective alone: every state in the forward sweep).
+// Backward sweep, one segment of K steps at a time from the last: the states of the segment are
+// recomputed from its checkpoint with the step kernels the context uses, each leaving the psi field of
+// the state it reads in a buffer of its own (the two-pass step's psi pass writes it anyway; the
+// one-pass steps write it on request), then the transposed step runs from the last state of the
+// segment to the first.  The recompute of a segment runs on a second stream, overlapping the
+// transposed steps of the segment after it, so segment states and psi fields come in two sets.  Device
+// memory: ceil(n/K) checkpoints, 2 (K - 1) segment states, 2 K psi fields and the adjoint planes; it is
+// kept for the next call with the same sizes.  Where two sets cannot be had the call takes one, and
+// recomputes a segment after those transposed steps: less than the layout whose transposed step ran
+// in two passes over single planes, so what fitted that still fits.
 //
 // 16-bit storage: a stored state is its nine planes of deviations plus, with a per-node
 // reference density, that plane; the recompute repeats the forward steps' stochastic
@@ -28,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdint>
 #include <string>
 #include <vector>
 
@@ -38,6 +42,7 @@ namespace lbm {
 struct AdjointState {
     void *base = nullptr;
     size_t bytes = 0;
+    size_t refused = SIZE_MAX;  // the smallest layout with two buffer sets that did not fit
     cudaStream_t side = nullptr;  // recomputes the next segment while the transposed steps run
     cudaEvent_t fork = nullptr, recomputed[2] = {nullptr, nullptr}, reversed[2] = {nullptr, nullptr};
 };
@@ -68,33 +73,39 @@ struct Carver {
 };
 
 struct Layout {
-    std::vector<void *> ckpt, seg[2], psi[2];  // two sets of segment states and psi fields
-    void *g[2], *dS[2], *dpsi[2], *rho[2], *psi_r[2], *c;  // psi_r: FP64 only
+    std::vector<void *> ckpt, seg[2], psi[2];  // one or two sets of segment states and psi fields
+    void *g[2], *dS[2], *dpsi[2], *rho[2], *psi_r[2];  // psi_r: FP64 only
     double *part;  // per-block partial sums of the transposed steps [blocks][kAdjSlots]
     double *red;   // their column sums (kAdjSlots)
     double *acc;
 };
 
-size_t carve(Carver &cv, Layout &L, int64_t nseg, int64_t K, size_t state_bytes, size_t plane_r, bool psi_planes,
-             size_t psi_bytes, size_t part_bytes)
+// Sizes of what a call keeps on the device.
+struct Sizes {
+    int64_t nseg = 0, K = 0;
+    bool keep_first = false;  // A_0 needs a checkpoint of its own
+    bool psi_planes = false;
+    size_t state = 0, plane_r = 0, psi = 0, part = 0;
+};
+
+size_t carve(Carver &cv, Layout &L, const Sizes &z, int sets)
 {
-    L.ckpt.resize(nseg);
-    for (auto &b : L.ckpt) b = cv.take(state_bytes);
-    for (int q = 0; q < 2; ++q) {
-        L.seg[q].resize(std::max<int64_t>(K - 1, 1));
-        L.psi[q].resize(K);
-        for (auto &b : L.seg[q]) b = cv.take(state_bytes);
-        for (auto &b : L.psi[q]) b = cv.take(psi_bytes);
+    L.ckpt.assign(z.nseg, nullptr);
+    for (int64_t s = z.keep_first ? 0 : 1; s < z.nseg; ++s) L.ckpt[s] = cv.take(z.state);
+    for (int q = 0; q < sets; ++q) {
+        L.seg[q].resize(z.K > 0 ? z.K - 1 : 0);
+        L.psi[q].resize(z.K);
+        for (auto &b : L.seg[q]) b = cv.take(z.state);
+        for (auto &b : L.psi[q]) b = cv.take(z.psi);
     }
     for (int s = 0; s < 2; ++s) {
-        L.g[s] = cv.take(9 * plane_r);
-        L.dS[s] = cv.take(2 * plane_r);
-        L.dpsi[s] = cv.take(plane_r);
-        L.rho[s] = cv.take(plane_r);
-        L.psi_r[s] = psi_planes ? cv.take(plane_r) : nullptr;
+        L.g[s] = cv.take(9 * z.plane_r);
+        L.dS[s] = cv.take(2 * z.plane_r);
+        L.dpsi[s] = cv.take(z.plane_r);
+        L.rho[s] = cv.take(z.plane_r);
+        L.psi_r[s] = z.psi_planes ? cv.take(z.plane_r) : nullptr;
     }
-    L.c = cv.take(plane_r);
-    L.part = static_cast<double *>(cv.take(part_bytes));
+    L.part = static_cast<double *>(cv.take(z.part));
     L.red = static_cast<double *>(cv.take(kAdjSlots * sizeof(double)));
     L.acc = static_cast<double *>(cv.take(8 * sizeof(double)));
     return cv.used;
@@ -156,33 +167,50 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
     // grad == NULL and lambda0 == NULL: the objective alone (forward sweep only)
     const bool backward = grad != nullptr || lambda0 != nullptr;
 
-    // device memory, kept across calls
+    // Device memory, kept across calls: two buffer sets, so that a segment is recomputed beside the transposed
+    // steps of the one after it; one where there is a single segment or the memory for two cannot be had.
+    Sizes z;
+    if (backward) {
+        z.nseg = nseg, z.K = Kseg;
+        z.keep_first = nsteps % 2 == 0;
+        z.psi_planes = real == 8;
+        z.state = state_bytes, z.plane_r = plane_r, z.psi = psi_bytes, z.part = part_bytes;
+    }
     Layout L;
-    Carver probe{nullptr};
-    const size_t need = backward ? carve(probe, L, nseg, Kseg, state_bytes, plane_r, real == 8, psi_bytes, part_bytes)
-                                 : carve(probe, L, 0, 1, 0, 0, false, 0, 0);
+    int sets = nseg > 1 && backward ? 2 : 1;
+    auto need = [&](int q) {
+        Carver probe{nullptr};
+        return carve(probe, L, z, q);
+    };
     AdjointState *&as = *v.adj;
     if (!as) as = new AdjointState();
-    if (as->bytes < need) {
+    if (sets == 2 && need(2) >= as->refused) sets = 1;
+    while (as->bytes < need(sets)) {
         if (as->base) {
             cudaStreamSynchronize(st);
             cudaFree(as->base);
             as->base = nullptr;
             as->bytes = 0;
         }
-        cudaError_t e = cudaMalloc(&as->base, need);
-        if (e != cudaSuccess) {
+        const size_t bytes = need(sets);
+        cudaError_t e = cudaMalloc(&as->base, bytes);
+        if (e == cudaSuccess) {
+            as->bytes = bytes;
+        } else {
             cudaGetLastError();
-            msg = "adjoint: cudaMalloc of " + std::to_string(need >> 20) +
-                  " MiB for checkpoints and segment states failed (lower checkpoint_every)";
-            return LBM_ENOMEM;
+            as->base = nullptr;
+            if (sets == 1) {
+                msg = "adjoint: cudaMalloc of " + std::to_string(bytes >> 20) +
+                      " MiB for checkpoints and segment states failed (lower checkpoint_every)";
+                return LBM_ENOMEM;
+            }
+            as->refused = bytes;
+            sets = 1;
         }
-        as->bytes = need;
     }
     Carver cv{static_cast<char *>(as->base)};
-    if (backward) carve(cv, L, nseg, Kseg, state_bytes, plane_r, real == 8, psi_bytes, part_bytes);
-    else carve(cv, L, 0, 1, 0, 0, false, 0, 0);
-    if (backward && !as->side) {
+    carve(cv, L, z, sets);
+    if (sets == 2 && !as->side) {
         ACK(cudaStreamCreateWithFlags(&as->side, cudaStreamNonBlocking), "cudaStreamCreate");
         cudaEvent_t *evs[] = {&as->fork, &as->recomputed[0], &as->recomputed[1], &as->reversed[0], &as->reversed[1]};
         for (cudaEvent_t *e : evs) ACK(cudaEventCreateWithFlags(e, cudaEventDisableTiming), "cudaEventCreate");
@@ -196,7 +224,8 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
     // ---- forward sweep: checkpoints and the objective
     KParams kq = *v.kp;
     const int64_t step0 = *v.steps;  // the forward sweep's step t runs as the context's step step0 + t
-    const int last_q = (int)((nseg - 1) & 1);  // buffer set of the last segment
+    auto set_of = [&](int64_t s) { return sets == 2 ? (int)(s & 1) : 0; };  // buffer set of a segment
+    const int last_q = set_of(nseg - 1);
     // One step of the context's kernel from one state buffer to another, leaving psi of the state it
     // reads in `psi` (null: where the context keeps it).
     auto step_to = [&](const void *src, const float *ref, void *dst, float *ref_dst, void *psi, int64_t t,
@@ -278,7 +307,6 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
     aa.inv_nfluid = inv_nfluid;
     aa.inv_nfluid_f = float(inv_nfluid);
     aa.part = L.part;
-    aa.c_out = L.c;
     int gi = 0;  // set of planes the last transposed step left; none before the first
     bool have_next = false;
     auto bind_in = [&]() {
@@ -294,37 +322,41 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
         *ref = ref_of(p);
         return p;
     };
-    // Segment s is recomputed on the side stream into buffer set s & 1 while the transposed
-    // steps of segment s + 1 run on the context stream from set (s + 1) & 1; events order a
-    // set's reuse after the transposed steps that read it.
+    // With two buffer sets segment s is recomputed on the side stream into set s & 1 while the
+    // transposed steps of segment s + 1 run on the context stream from set (s + 1) & 1; events order a
+    // set's reuse after the transposed steps that read it.  With one it is recomputed after them, on the
+    // context stream.
+    const cudaStream_t on = sets == 2 ? as->side : st;
     auto recompute = [&](int64_t s) -> lbm_status {
-        const int q = (int)(s & 1);
+        const int q = set_of(s);
         const int64_t t0 = s * K, t1 = std::min<int64_t>((s + 1) * K, nsteps);
-        if (s + 2 < nseg) ACK(cudaStreamWaitEvent(as->side, as->reversed[q], 0), "event wait");
+        if (sets == 2 && s + 2 < nseg) ACK(cudaStreamWaitEvent(as->side, as->reversed[q], 0), "event wait");
         for (int64_t t = t0; t < t1; ++t) {
             const float *ref;
             const void *src = state_at(s, q, t, &ref);
             if (t + 1 < t1) {
                 void *dst = L.seg[q][t - t0];
-                const lbm_status r = step_to(src, ref, dst, ref_of(dst), L.psi[q][t - t0], t, as->side);
+                const lbm_status r = step_to(src, ref, dst, ref_of(dst), L.psi[q][t - t0], t, on);
                 if (r != LBM_OK) return r;
             } else {
                 KParams kp = *v.kp;
                 kp.src = src, kp.ref_src = ref, kp.psi = L.psi[q][t - t0];
-                ACK(v.psi_pass(kp, as->side), "psi kernel");
+                ACK(v.psi_pass(kp, on), "psi kernel");
             }
         }
-        ACK(cudaEventRecord(as->recomputed[q], as->side), "event record");
+        if (sets == 2) ACK(cudaEventRecord(as->recomputed[q], on), "event record");
         return LBM_OK;
     };
-    ACK(cudaEventRecord(as->fork, st), "event record");
-    ACK(cudaStreamWaitEvent(as->side, as->fork, 0), "event wait");
+    if (sets == 2) {
+        ACK(cudaEventRecord(as->fork, st), "event record");
+        ACK(cudaStreamWaitEvent(as->side, as->fork, 0), "event wait");
+    }
     lbm_status rs;
     for (int64_t s = nseg - 1; s >= 0; --s) {
-        const int q = (int)(s & 1);
+        const int q = set_of(s);
         const int64_t t0 = s * K, t1 = std::min<int64_t>((s + 1) * K, nsteps);
-        if (s > 0 && (rs = recompute(s - 1)) != LBM_OK) return rs;
-        if (s < nseg - 1) ACK(cudaStreamWaitEvent(st, as->recomputed[q], 0), "event wait");
+        if (sets == 2 && s > 0 && (rs = recompute(s - 1)) != LBM_OK) return rs;
+        if (sets == 2 && s < nseg - 1) ACK(cudaStreamWaitEvent(st, as->recomputed[q], 0), "event wait");
         KParams kp = *v.kp;
         for (int64_t t = t1 - 1; t >= t0; --t) {
             kp.src = state_at(s, q, t, &kp.ref_src);
@@ -337,17 +369,19 @@ lbm_status adjoint_run(lbm_ctx *ctx, int64_t nsteps, int32_t K, int32_t objectiv
             gi = go;
             have_next = true;
         }
-        ACK(cudaEventRecord(as->reversed[q], st), "event record");
+        if (sets == 2) ACK(cudaEventRecord(as->reversed[q], st), "event record");
+        if (sets == 1 && s > 0 && (rs = recompute(s - 1)) != LBM_OK) return rs;
     }
 
     bind_in();
     aa.tail = 1;
+    void *const c = aa.c_out = L.g[gi ^ 1];  // (its own planes are the last ones read)
     ACK(v.L->adj_step(*v.kp, aa, st), "transposed step's tail");
     if (lambda0) {
         const size_t n = (size_t)p.nx * p.ny;
         double *dl = nullptr;
         ACK(cudaMalloc((void **)&dl, 9 * n * sizeof(double)), "cudaMalloc(lambda0)");
-        cudaError_t e = v.L->adj_lambda(*v.kp, L.g[gi], L.c, dl, st);
+        cudaError_t e = v.L->adj_lambda(*v.kp, L.g[gi], c, dl, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(lambda0, dl, 9 * n * sizeof(double), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         cudaFree(dl);

@@ -117,3 +117,45 @@ def test_diagnostics_allocate_nothing(fakelib, prec, nx, ny):
     sim.step(5)
     sim.close()
     fake.sound(fakelib)
+
+
+def _two_pass_adjoint_bytes(nx, ny, prec, n, K):
+    """What an adjoint call took while its transposed step ran in two passes: every checkpoint, two sets of
+    segment states (one state at least) and psi fields, 24 planes, and a row of 64 bytes for each 128 nodes of a lattice row."""
+    elem, real = {lbm.F64: (8, 8), lbm.F32: (4, 4), lbm.F16DEV: (2, 4)}[prec]
+    per_line = 128 // elem
+    plane = (nx + per_line - 1) // per_line * per_line * ny
+    up = lambda b: (b + 255) // 256 * 256  # noqa: E731
+    state = 9 * plane * elem if prec != lbm.F16DEV else up(9 * plane * elem) + 4 * plane
+    K = min(K, n)
+    parts = up((nx + 127) // 128 * ny * 64)
+    return ((n + K - 1) // K * up(state) + 2 * max(K - 1, 1) * up(state) + 2 * K * up(nx * ny * real) +
+            2 * up(9 * plane * real) + up(2 * plane * real) + 4 * up(plane * real) + parts + 512)
+
+
+@pytest.mark.parametrize("tight", [False, True])
+@pytest.mark.parametrize("prec", [lbm.F64, lbm.F32, lbm.F16DEV])
+@pytest.mark.parametrize("kernel", [lbm.KERNEL_AUTO, lbm.KERNEL_TWO_PASS])
+def test_adjoint_in_the_memory_it_used_to_take(fakelib, prec, kernel, tight):
+    """Every number of steps and checkpoint interval, with all the memory there is and with what the two-pass
+    transposed step took: each kernel reads the state, psi field and planes of its step, whichever buffers hold them."""
+    nx, ny = 33, 18
+    for n in range(1, 10):
+        for K in range(1, n + 2):
+            fakelib.fake_reset(0)
+            sim = lbm.Simulation(lbm.default_params(nx=nx, ny=ny, precision=prec, kernel=kernel, per_node_ref=1))
+            sim.init_fields(np.full((ny, nx), 0.2))
+            if tight:
+                fake.limit(fakelib, nbytes=_two_pass_adjoint_bytes(nx, ny, prec, n, K))
+            for call in range(2):  # (the second keeps the first one's memory)
+                J, g, _ = sim.adjoint(n, K, lbm.OBJ_MEAN_JX)
+                assert J == 1.0 and sim.step_count == n  # (the fake objective is the number of the state)
+                fake.sound(fakelib)
+                fake.limit(fakelib, mallocs=0)
+                sim.init_fields(np.full((ny, nx), 0.2))
+            fake.limit(fakelib)
+            sim.init_fields(np.full((ny, nx), 0.2))
+            sim.adjoint(n, K, lbm.OBJ_MEAN_JX, want_lambda0=True)
+            sim.step(1)
+            fake.sound(fakelib)
+            sim.close()
