@@ -6,7 +6,9 @@
 //
 // What bounds it: GB300's FP64 pipe takes one warp instruction per SM every 16 cycles, so an FP64
 // kernel's time is its FP64 instruction count and everything else hides behind it.  Operations
-// whose result needs no rounding are therefore left out or folded, which changes no bit:
+// whose result needs no rounding are therefore left out or folded, which changes no bit (but one that
+// nothing sees: a quotient of -0 by a positive divisor comes out as +0, and no such dividend of a step is
+// -0, since a sum that cancels is +0 and the forces are sums):
 //   * entries 0 and +-1 of M cost nothing or one add; entries +-2, +-4 scale by a power of two, so
 //     their product is exact and one multiply-add rounds as the separate product and sum do;
 //   * a product by 1/2, 2 or 6/2 of a term is folded the same way (0.5 F_m, Q_2 = -Q_1/2, F_m7);
@@ -26,7 +28,7 @@ namespace f64 {
 
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// a / D for D = 3 or 9, correctly rounded.  With r = RN(1/D) (relative error 2^-54 for both) the
+// a / D for D = 3 or 9, correctly rounded (-0 gives +0).  With r = RN(1/D) (relative error 2^-54 for both) the
 // product q = RN(a r) is within one ulp of a/D, and one correction by the exact remainder then
 // rounds correctly (Markstein, IBM J. Res. Dev. 34(1), 1990, on division by a correctly rounded
 // reciprocal).  Magnitudes outside 2^+-450 (0 excepted), infinities and NaN take the general

@@ -35,3 +35,27 @@ def test_fp64_step_is_the_oracles_at_any_magnitude(params, scheme, log2):
     sim.step(1)
     assert np.array_equal(sim.get_state(), want)
     sim.close()
+
+
+@pytest.mark.parametrize("params", [cs_params, lambda **k: vdw_params(1.895, 0.54, **k)], ids=["cs", "vdw"])
+@pytest.mark.parametrize("signs", [1.0, -1.0, 0.0])
+def test_signs_of_zero_are_the_oracles(params, signs):
+    """Populations at rest of +0, -0 or either sign beside the rest population (the sum of the forces and momenta is then
+    an exact zero): the bits of the moments and of the state after one step, signs of zero included."""
+    op = params(nx=33, ny=11, periodic_x=True, periodic_y=False, scheme=1, tau_l=0.9, tau_g=0.9)
+    A = np.zeros((9, 11, 33))
+    A[1:] *= signs if signs else np.where(np.random.default_rng(3).random((8, 11, 33)) < 0.5, -1.0, 1.0)
+    A[0] = 0.2
+    ref = O.OracleSim(op)
+    ref.set_state(A)
+    gp = GC.gpu_params(op, lbm.F64)
+    gp.rho_max = 0.3
+    sim = lbm.Simulation(gp)
+    sim.set_state(A)
+    bits = lambda a: np.ascontiguousarray(a).view(np.int64)  # noqa: E731
+    for g, w in zip(sim.moments(), ref.moments()):
+        assert np.array_equal(bits(g), bits(w))
+    sim.step(1)
+    ref.step(1)
+    assert np.array_equal(bits(sim.get_state()), bits(ref.get_state()))
+    sim.close()
