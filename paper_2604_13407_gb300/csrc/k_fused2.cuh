@@ -61,7 +61,6 @@ template <> struct Pair2<float> {
         if (OFF == 0) return v2{*reinterpret_cast<const float2 *>(p)};
         return V(p[OFF], p[OFF + 1]);
     }
-    static __device__ __forceinline__ float load1(const float *p) { return *p; }
     static __device__ __forceinline__ void store(float *p, v2 f) { *reinterpret_cast<float2 *>(p) = f.v; }
     static __device__ __forceinline__ void store_sr(float *p, v2 f, uint32_t) { store(p, f); }  // FP32: exact
 };
@@ -85,7 +84,6 @@ template <> struct Pair2<float> {
     }
 template <> struct Pair2<__half> {
     LBM_DEC_PAIR(__half, __half2, "f16")
-    static __device__ __forceinline__ float load1(const __half *p) { return __half2float(*p); }
     static __device__ __forceinline__ void store(__half *p, v2 f) { *reinterpret_cast<__half2 *>(p) = __float22half2_rn(f.v); }
     // stochastic rounding with the pair's random word r (element 0 from its low half)
     static __device__ __forceinline__ void store_sr(__half *p, v2 f, uint32_t r)
@@ -95,7 +93,6 @@ template <> struct Pair2<__half> {
 };
 template <> struct Pair2<__nv_bfloat16> {
     LBM_DEC_PAIR(__nv_bfloat16, __nv_bfloat162, "bf16")
-    static __device__ __forceinline__ float load1(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
     static __device__ __forceinline__ void store(__nv_bfloat16 *p, v2 f)
     {
         *reinterpret_cast<__nv_bfloat162 *>(p) = __float22bfloat162_rn(f.v);

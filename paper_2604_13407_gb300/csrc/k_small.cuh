@@ -46,18 +46,6 @@ __device__ __forceinline__ void push(uint32_t a, double v) { asm volatile("st.sh
 __device__ __forceinline__ void push(uint32_t a, __half v) { asm volatile("st.shared::cluster.b16 [%0], %1;" ::"r"(a), "h"(__half_as_ushort(v)) : "memory"); }
 __device__ __forceinline__ void push(uint32_t a, __nv_bfloat16 v) { asm volatile("st.shared::cluster.b16 [%0], %1;" ::"r"(a), "h"(__bfloat16_as_ushort(v)) : "memory"); }
 
-// Seed of the stochastic rounding of step t (the host's sr_seed_of).
-__device__ __forceinline__ uint32_t sr_seed_at(int64_t t)
-{
-    uint32_t h = (uint32_t)t * 0x9E3779B1u ^ (uint32_t)((uint64_t)t >> 32) * 0x85EBCA77u;
-    h ^= h >> 16;
-    h *= 0x85EBCA6Bu;
-    h ^= h >> 13;
-    h *= 0xC2B2AE35u;
-    h ^= h >> 16;
-    return h;
-}
-
 // Shared memory of a CTA: nine planes, the reference plane and psi, of `rows` own rows and a halo row
 // above and below; a psi row ends with one entry that always holds psi(rho_s), the neighbour beyond a
 // non-periodic x edge.
@@ -293,7 +281,7 @@ __global__ void __launch_bounds__(THREADS) k_small2(KParams kp, int64_t nsteps, 
         collide_v<T, RuntimeOpts>(kp, d, rho, psi, Sx, Sy, Fex, Fey, o, ux, uy);
         S v[N][9];
         if constexpr (DEV) {
-            const uint32_t seed = sr_seed_at(step0 + t);
+            const uint32_t seed = sr_seed_of(step0 + t);
             const uint32_t ha = sr_hash(n[0].kg >> 1, seed), hb = N == 2 ? sr_hash(n[N - 1].kg >> 1, seed) : 0u;
 #pragma unroll
             for (int i = 0; i < 9; ++i) {

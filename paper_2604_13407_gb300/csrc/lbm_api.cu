@@ -230,19 +230,14 @@ static void fill_constants(lbm_ctx *c)
         auto P = [](float v) { return make_float2(v, v); };
         PairConsts &q = k.c2;
         const Consts<float> &f = k.cf;
-        q.one = P(1.f), q.m_one = P(-1.f), q.half = P(0.5f), q.m_half = P(-0.5f), q.two = P(2.f), q.m_two = P(-2.f);
-        q.three = P(3.f), q.m_three = P(-3.f), q.four = P(4.f), q.m_four = P(-4.f), q.six = P(6.f), q.m_six = P(-6.f);
-        q.third = P(1.0f / 3.0f), q.m_third = P(-1.0f / 3.0f), q.twelfth = P(1.0f / 12.0f), q.ninth = P(1.0f / 9.0f);
-        q.w36 = P(1.0f / 36.0f), q.sixth = P(1.0f / 6.0f), q.quarter = P(0.25f);
         q.m_G = P(-f.G), q.kq1 = P(f.kq1), q.q2fac = P(f.q2fac), q.kq7 = P(f.kq7), q.c1G = P(f.c1G), q.m_c2G = P(-f.c2G);
-        q.sp = P(f.sp), q.sq = P(f.sq), q.hsp = P(f.hsp), q.hsq = P(f.hsq), q.six_hsp = P(6.f * f.hsp);
+        q.sp = P(f.sp), q.sq = P(f.sq), q.hsp = P(f.hsp), q.six_hsp = P(6.f * f.hsp);
         q.m_six_hsp = P(-6.f * f.hsp), q.m_hsq = P(-f.hsq);
         q.Fx = P(f.Fx), q.Fy = P(f.Fy), q.rho_g = P(f.rho_g), q.inv_drho = P(1.0f / (f.rho_l - f.rho_g));
         q.dnu = P(f.nu_l - f.nu_g), q.nu_g = P(f.nu_g), q.Lambda = P(f.Lambda);
         q.m_b = P(-f.eos_b), q.b4 = P(f.eos_b * 0.25f), q.K = P(f.eos_K), q.RT = P(f.eos_RT), q.a = P(f.eos_a);
         q.two_over_G = P(f.two_over_G);
-        q.inv_scale = P(f.inv_scale), q.scale = P(f.scale), q.m_scale = P(-f.scale), q.psi_s = P(f.psi_s);
-        q.rho_ref = P(f.rho_ref);
+        q.scale = P(f.scale), q.m_scale = P(-f.scale);
         // 2^-k as FP16 (normal for k <= 14, subnormal down to 2^-24) or BF16 bits
         const int kk = p.storage_scale_log2;
         if (p.precision == LBM_BF16DEV) k.inv_scale_bits = (unsigned short)((127 - kk) << 7);
@@ -314,16 +309,13 @@ static void choose_kernel(lbm_ctx *c)
     c->fused_ok = (want != LBM_KERNEL_TWO_PASS) && possible &&
                   (want == LBM_KERNEL_FUSED || c->p.precision == LBM_F64 || auto_prefers_fused(c));
     const bool staged = possible && c->L.fused_pass && c->p.periodic_x && c->p.periodic_y && !c->solid && !c->q && !c->wall_u;
-    const bool tile = c->L.tile_pass != nullptr;
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
     const bool large = n >= (c->p.precision == LBM_F32 ? (int64_t)1 << 25 : (int64_t)3 << 20);
     c->kp.packed = c->fused_ok && c->p.precision >= LBM_F16DEV;
     c->one_pass = nullptr;
     c->small_ctas = want == LBM_KERNEL_AUTO ? c->L.small_ctas(c->kp) : 0;
     if (want == LBM_KERNEL_TWO_PASS || (want == LBM_KERNEL_FUSED && !possible)) return;
-    if (staged && (want == LBM_KERNEL_FUSED || large || !tile)) c->one_pass = c->L.fused_pass;
-    else if (tile) c->one_pass = c->L.tile_pass;
-    else c->fused_ok = false;
+    c->one_pass = staged && (want == LBM_KERNEL_FUSED || large) ? c->L.fused_pass : c->L.tile_pass;
 }
 
 // ------------------------------------------------------------- lifetime ----
@@ -650,19 +642,6 @@ extern "C" lbm_status lbm_init_fields(lbm_ctx *c, const double *rho, const doubl
     c->steps = 0;
     c->initialised = true;
     return LBM_OK;
-}
-
-// Seed of the stochastic-rounding bits of step t (MurmurHash3's 32-bit finaliser of the
-// step count's two halves; any well-mixed function of t would do).
-static uint32_t sr_seed_of(int64_t t)
-{
-    uint32_t h = (uint32_t)t * 0x9E3779B1u ^ (uint32_t)((uint64_t)t >> 32) * 0x85EBCA77u;
-    h ^= h >> 16;
-    h *= 0x85EBCA6Bu;
-    h ^= h >> 13;
-    h *= 0xC2B2AE35u;
-    h ^= h >> 16;
-    return h;
 }
 
 // How many of the next nsteps steps the small-lattice kernel takes in one launch (no more than 4096, so that no

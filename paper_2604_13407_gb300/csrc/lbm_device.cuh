@@ -179,17 +179,6 @@ __device__ __forceinline__ S enc_pop(const KParams &kp, typename Codec<S>::R f, 
 // ------------------------------------------------------------- EOS ---------
 // Sec. 2: psi = sqrt(2 (p_EOS - rho c_s^2)/G); van der Waals (Sec. 3) or Carnahan-Starling.
 template <class R>
-__device__ __forceinline__ R p_eos(const KParams &kp, R rho)
-{
-    const R a = cst<R>(kp).eos_a, b = cst<R>(kp).eos_b, RT = cst<R>(kp).eos_RT, K = cst<R>(kp).eos_K;
-    if (kp.eos == 0) return K * (rho * RT / (R(1) - b * rho) - a * rho * rho);
-    const R eta = b * rho * R(0.25);
-    const R om = R(1) - eta;
-    const R num = R(1) + eta + eta * eta - eta * eta * eta;
-    return K * (rho * RT * num / (om * om * om) - a * rho * rho);
-}
-
-template <class R>
 __device__ __forceinline__ R psi_of(const KParams &kp, R rho)
 {
     if constexpr (is_f64<R>()) return f64::psi_of(kp, rho);
@@ -327,33 +316,8 @@ __device__ __forceinline__ R bounce(const KParams &kp, int x, int y, const At &a
     return f;
 }
 
-// Pull streaming, Eq. (lbe.str): f_i(x) = fbar_i(x - e_i), wall links bounced back.
-template <class R, int i, class At>
-__device__ __forceinline__ R pull_one(const KParams &kp, int x, int y, const At &at, R *mom)
-{
-    if (i == 0) return at(0, x, y);
-    int xs = x - ex_(i), ys = y - ey_(i);
-    const bool inside = wrap_xy(kp, xs, ys);
-    if (inside && (kp.solid == nullptr || kp.solid[(int64_t)ys * kp.nx + xs] == 0)) return at(i, xs, ys);
-    return bounce<R, i>(kp, x, y, at, mom);
-}
-
-template <class R, class At>
-__device__ __forceinline__ void pull_node(const KParams &kp, int x, int y, const At &at, R (&f)[9], R *mom)
-{
-    f[0] = pull_one<R, 0>(kp, x, y, at, mom);
-    f[1] = pull_one<R, 1>(kp, x, y, at, mom);
-    f[2] = pull_one<R, 2>(kp, x, y, at, mom);
-    f[3] = pull_one<R, 3>(kp, x, y, at, mom);
-    f[4] = pull_one<R, 4>(kp, x, y, at, mom);
-    f[5] = pull_one<R, 5>(kp, x, y, at, mom);
-    f[6] = pull_one<R, 6>(kp, x, y, at, mom);
-    f[7] = pull_one<R, 7>(kp, x, y, at, mom);
-    f[8] = pull_one<R, 8>(kp, x, y, at, mom);
-}
-
-// The same pull with the node's neighbourhood nb (x - e_i = x + e_opp(i)); `at.at_k(k, kk)`
-// reads population k at pitched index kk.
+// Pull streaming, Eq. (lbe.str): f_i(x) = fbar_i(x - e_i), wall links bounced back, with the node's
+// neighbourhood nb (x - e_i = x + e_opp(i)); `at.at_k(k, kk)` reads population k at pitched index kk.
 template <class R, int i, class At>
 __device__ __forceinline__ R pull_one_nb(const KParams &kp, const Around &nb, int x, int y, const At &at, R *mom)
 {

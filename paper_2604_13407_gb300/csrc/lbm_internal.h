@@ -14,15 +14,13 @@ struct Consts {
     R hsp, hsq;  // 1 - s_p/2 and 1 - s_q/2 of the constant relaxation rates
 };
 
-// Constant operands of the packed FP32x2 kernel (k_fused2.cuh), each splatted to a pair
+// Constant operands of the packed FP32x2 evaluation (lbm_f32.cuh), each splatted to a pair
 // (c, c) on the host, so that the kernel never assembles a constant pair at run time.
 struct PairConsts {
-    float2 one, m_one, half, m_half, two, m_two, three, m_three, four, m_four, six, m_six;
-    float2 third, m_third, twelfth, ninth, w36, sixth, quarter;
-    float2 m_G, kq1, q2fac, kq7, c1G, m_c2G, sp, sq, hsp, hsq, six_hsp, m_six_hsp, m_hsq;
+    float2 m_G, kq1, q2fac, kq7, c1G, m_c2G, sp, sq, hsp, six_hsp, m_six_hsp, m_hsq;
     float2 Fx, Fy, rho_g, inv_drho, dnu, nu_g, Lambda;
     float2 m_b, b4, K, RT, a, two_over_G;
-    float2 inv_scale, scale, m_scale, psi_s, rho_ref;
+    float2 scale, m_scale;
     float2 dec[9];  // w_i rho_ref (decode of deviations)
     float2 enc[9];  // -(w_i rho_ref) 2^k (encode of deviations)
     float2 w[9];    // w_i
@@ -96,7 +94,7 @@ struct KParams {
     int *err;              // device error word (0 = fine)
     Consts<double> cd;     // constants for FP64 arithmetic
     Consts<float> cf;      // constants for FP32 arithmetic
-    PairConsts c2;         // the same as pairs, for the packed kernel
+    PairConsts c2;         // the same as pairs, for the packed kernels
     unsigned short inv_scale_bits;  // 2^-k in the storage type (FP16 or BF16 bits)
 };
 
@@ -125,6 +123,22 @@ struct AdjArgs {
     float w_scale_f, inv_nfluid_f;  // the two scales rounded to FP32 on the host (FP32 arithmetic
                                     // converts no FP64 value per node)
 };
+
+// Seed of the stochastic-rounding bits of step t (MurmurHash3's 32-bit finaliser of the
+// step count's two halves; any well-mixed function of t would do).
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline uint32_t sr_seed_of(int64_t t)
+{
+    uint32_t h = (uint32_t)t * 0x9E3779B1u ^ (uint32_t)((uint64_t)t >> 32) * 0x85EBCA77u;
+    h ^= h >> 16;
+    h *= 0x85EBCA6Bu;
+    h ^= h >> 13;
+    h *= 0xC2B2AE35u;
+    h ^= h >> 16;
+    return h;
+}
 
 // Storage precisions (match lbm_precision)
 enum Prec { P_F64 = 0, P_F32 = 1, P_F16 = 2, P_BF16 = 3 };
