@@ -33,11 +33,11 @@ T_07 = 0.7 * 0.3773 / 4.0
 TAU = 1.0
 BYTES = {"f64": 144, "f32": 72, "f16dev": 36, "bf16dev": 36}
 # DRAM bytes per lattice update of the staged kernel (k_fused2), from one ncu capture
-# (dram__bytes_read.sum + dram__bytes_write.sum of one launch at 4096 x 4096; profiles/k_fused2_*;
-# f16dev: the per-node reference mode), scaled to a launch by the updates it makes.
+# (dram__bytes_read.sum + dram__bytes_write.sum of one launch, at 6144 x 6144 in FP32 and 4096 x 4096 in FP16
+# storage; profiles/k_fused2_*; f16dev: the per-node reference mode), scaled to a launch by the updates it makes.
 # Valid for the kernel as captured; an entry is removed when the kernel changes until it is captured
 # again (the line then reports traffic null).
-TRAFFIC_PER_UPDATE = {"f32": 73.86, "f16dev": 43.93}
+TRAFFIC_PER_UPDATE = {"f32": 73.00, "f16dev": 43.93}
 HBM_FALLBACK = 6800.0
 
 
@@ -277,12 +277,19 @@ def geometry_cases():
            I.droplet(nx, ny, RHO_L, RHO_G, 40.0, cx, cy, periodic_x=False, periodic_y=True), None, None, None)
 
 
+def wall_links(solid):
+    """Links from a fluid node into a solid one, on a lattice periodic in both directions."""
+    s = np.asarray(solid) != 0
+    return sum(int((~s & np.roll(s, (dy, dx), (0, 1))).sum())
+               for dy in (-1, 0, 1) for dx in (-1, 0, 1) if dy or dx)
+
+
 def geometry_throughput(hbm, steps=2000, warmup=20, only=None, kernel=0, precs=("f32", "f16dev")):
     """GLUPS of the step on the geometry_cases lattices (CUDA events on the launching
     stream), with the kernel the automatic choice takes ("kernel" names it) unless `kernel`
     asks for one.  Bytes per update (algorithmic): the population read and write of the
-    storage type, plus the node's solid flag where there is a mask; interpolated-link
-    distances and wall velocities are read only at wall links.  The two smaller lattices'
+    storage type, plus the node's two bytes of wall bits where there is a mask and, with interpolated or
+    moving walls, an eight-byte record for each wall link.  The two smaller lattices'
     state fits in L2 (and the step is bound by latency, not by HBM), so their fraction of the
     HBM copy bandwidth is reported for comparison only.  `only` restricts the run to one
     case (for profiling)."""
@@ -305,7 +312,9 @@ def geometry_throughput(hbm, steps=2000, warmup=20, only=None, kernel=0, precs=(
             nodes = over["nx"] * over["ny"]
             t = timed_steps(s, steps, warmup, False)
             g = nodes * steps / t / 1e9
-            b = BYTES[prec] + (8 if half else 0) + (1 if solid is not None else 0)
+            b = BYTES[prec] + (8 if half else 0) + (2 if solid is not None else 0)
+            if q is not None or wall_u is not None:
+                b += 8 * wall_links(solid) / nodes
             # two population buffers (and two reference planes for per-node 16-bit storage)
             state_mb = (BYTES[prec] + (8 if half else 0)) * nodes / 1e6
             out["%s_%s" % (name, prec)] = {
