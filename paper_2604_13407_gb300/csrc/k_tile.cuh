@@ -21,7 +21,7 @@
 // chosen per launch (tile_height) so that the last wave of blocks is nearly full.
 //
 // What bounds it (FP32): small lattices the latency of one block's chain, mid-size ones instruction
-// issue (558 a pair of rows and 32 columns, ring included; the two-pass kernels 1840), from 2048^2 on HBM:
+// issue (557 a pair of rows and 32 columns, ring included, FP16 787; the two-pass kernels 1840), from 2048^2 on HBM:
 // 4096^2 186 us, 97 % of the measured copy rate at 72 B a node. Four pairs and five blocks per SM (64
 // registers) against two blocks of eight pairs: 512 x 4096 46 -> 36 us; the L2 prefetch 70 -> 59 at 2048^2;
 // the instantiation without edge tests (INNER) 59 -> 52, FP16 81 -> 67.
@@ -266,8 +266,11 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
         allow_dependent_launch();
     }
     // A warp whose nodes are all solid has nothing to pull: psi is the walls'.  Only where solid nodes are
-    // many (KParams::skip_solid), since the others' pulls then wait for the wall bits: annulus 1024^2 (a
-    // third solid) 19.6 -> 17.0 us, FP16 23.8 -> 21.3; banded 2048^2 (0.1 %) 59.2 -> 63 with it.
+    // many (KParams::skip_solid, an eighth), since the others' pulls then wait for the wall bits.  Step without
+    // / with it at 1024^2 (us): a disc of 3, 9, 12.5 and 40 % of the nodes 15.8 / 15.6, 15.4 / 14.8, 15.2 /
+    // 14.3 and 13.8 / 11.9 (FP16 18.0 / 17.9, 17.8 / 17.4, 17.7 / 17.0, 16.5 / 14.3); grains of 24^2 nodes
+    // within 1 % either way at any share; solid bands (0.1 %) the same: the line is on the safe side, nothing
+    // was slower with it.
     const bool still = masked && kp.skip_solid && __all_sync(0xffffffffu, (wa & 1u) && (wb & 1u));
     if (ahead > 0 && warp < np && lane < (masked ? 20 : 18)) {
         // the lines of the tile that a block of the next wave will read (rows y and y + 1, columns x0 ..
@@ -705,7 +708,7 @@ __global__ void __launch_bounds__(32 * (kTileRows + 3), 1) k_read1(KParams kp, T
 // Options fixed at compile time: the force law, one or two relaxation times and, for 16-bit storage, the
 // reference plane.  Each costs a block a branch that the schedule does not cross and a value that is live
 // through it, in a kernel that is short of registers (64): 1024^2 14.4 -> 13.7 us, 512 x 4096 30.1 -> 29.3,
-// FP16 37.7 -> 35.4.  The EOS and the scheme stay run-time options (fixed as well: within 1 %).
+// FP16 (exact products) 37.7 -> 35.4.  The EOS and the scheme stay run-time options (fixed as well: within 1 %).
 template <int VT, int REF, class F>
 inline cudaError_t with_force(const KParams &kp, const F &f)
 {
