@@ -239,7 +239,7 @@ LBM_API lbm_status lbm_load_state(lbm_ctx *ctx, const void *host_buf, size_t nby
 
 /* Change one parameter (lbm_param_id) between steps.  psi(rho_s) and psi of the wall densities follow G
  * and T; a value that makes either imaginary, or psi somewhere on (0, rho_max], is refused
- * (LBM_EINVAL) and changes nothing. */
+ * (LBM_EINVAL) and changes nothing.  With wall densities set a change of G or T waits for the stream. */
 LBM_API lbm_status lbm_set_param(lbm_ctx *ctx, int32_t which, double value);
 
 /* Adjoint of nsteps forward steps from the current state for the time-averaged
