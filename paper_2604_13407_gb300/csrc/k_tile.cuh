@@ -7,13 +7,10 @@
 // needs no alignment of nx; the packed instructions halve the arithmetic instructions of the
 // one-node passes.  The packed products are written as multiply-adds with -0 (v2x): the assembler
 // fuses a packed product into a following packed sum, which rounds once where the one-node
-// evaluation rounds twice; with them every node's result is the two-pass step's, bit for bit (the
-// links of interpolated and moving walls to rounding: their coefficients come from the link
-// records, formed in FP64).  16-bit storage on the lattices where LBM_KERNEL_FUSED is granted
-// (KParams::packed) takes plain packed products and the staged kernel's encode instead (v2): a
-// stored deviation is rounded from values that the staged kernel has too, so LBM_KERNEL_AUTO leaves the
-// same states there whichever of the two kernels a size gets, bit for bit.  (In FP32 storage the
-// two roundings differ by an ulp of a population and no more, and the exact products stay.)
+// evaluation rounds twice; with them every node's result is the two-pass step's, bit for bit.  Where the
+// context takes the step of LBM_KERNEL_FUSED (KParams::packed) the products are plain packed ones and 16-bit
+// storage encodes as the staged kernel does (v2): the state is then the staged kernel's, bit for bit,
+// whichever of the two kernels a size gets.  (In FP32 storage the exact products stay.)
 // FP64 (k_tile1): one node per thread, the two-pass step's own functions, the same bits.
 //
 // A tile of n pairs (rows) has n warps for them; one more warp pulls the rows above and below the
@@ -353,6 +350,8 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
                     if constexpr (GEOM >= 2) if (GEOM == 2 || kp.link != nullptr) {
                         // interpolated or moving wall: link fraction and moving-wall coefficient
                         const float2 lk = kp.link[(int64_t)(i - 1) * kp.plane + k];
+                        // the coefficient's form: KParams::link
+                        const bool whole = MODE == TILE_STEP ? PACKED : kp.packed != 0;
                         float mw = 0.f;
                         if (lk.y != 0.f) {
                             if (!summed) {
@@ -360,14 +359,14 @@ __device__ __forceinline__ void tile2_block(const KParams &kp, int ahead, const 
                                 for (int n = 0; n < 9; ++n) rho_w += own(n);
                                 summed = true;
                             }
-                            mw = lk.y * rho_w;
+                            mw = whole ? lk.y * rho_w : 2.f * w_<float>(o) * rho_w * lk.y * 3.f;
                         }
                         const float q = lk.x;
                         if (q < 0.5f) {
                             // fbar_o of the second node x + e_i (fluid: the record's q is 1/2 otherwise), which
                             // is what the pull of population o brought here
                             const float f2 = e ? f[o].v.y : f[o].v.x;
-                            g = 2.f * q * fo + (1.f - 2.f * q) * f2 + mw;
+                            g = near_link<DEV>(q, fo, f2, mw);
                         } else if (q == 0.5f) {
                             g = fo + mw;
                         } else {
@@ -578,6 +577,7 @@ __global__ void __launch_bounds__(256) k_diag_reduce(const double *part, int64_t
 // FP64: one node per thread.  Warps 0 .. n-1 own the tile's rows, two more the rows above and below
 // it, one the columns beside it.
 struct PlaneAt {
+    static constexpr bool DEV = false;
     const KParams &kp;
     __device__ __forceinline__ double operator()(int k, int x, int y) const { return load_pop<double>(kp, k, x, y); }
     __device__ __forceinline__ double at_k(int k, int64_t kk) const { return load_pop_at<double>(kp, k, kk); }
@@ -723,18 +723,19 @@ inline cudaError_t with_options(const KParams &kp, const F &f)
 
 // The packed rounding fixes fewer of them: the assembler fuses a packed product into a sum where both stand in one
 // block of the code, so the relaxation and the scheme stay branches exactly where the staged kernel
-// (Fused2::launch) has them.  512 x 4096 with walls: 36.6 us with all at run time, 34.7 here, 35.4 with
-// exact products and the options above; bands 2048^2, two relaxation times, 72.6 / 70.6 / 80.3.
-template <class F>
+// (Fused2::launch) has them.  512 x 4096 with walls, FP16: 36.6 us with all at run time, 34.7 here, 35.4 with
+// exact products and the options above; bands 2048^2, two relaxation times, FP16 72.6 / 70.6 / 80.3.
+template <bool DEV, class F>
 inline cudaError_t with_packed_options(const KParams &kp, bool plain, const F &f)
 {
-    const bool ref = kp.per_node_ref != 0;
+    constexpr int ON = DEV ? 1 : 0;  // (the reference plane, where there can be one)
+    const bool ref = DEV && kp.per_node_ref;
     if (plain && kp.force_mode == 0 && !kp.var_tau) {
-        if (ref) return kp.improved ? f(Opts<1, 0, 0, 1>()) : f(Opts<0, 0, 0, 1>());
+        if (ref) return kp.improved ? f(Opts<1, 0, 0, ON>()) : f(Opts<0, 0, 0, ON>());
         return kp.improved ? f(Opts<1, 0, 0, 0>()) : f(Opts<0, 0, 0, 0>());
     }
-    if (!ref) return f(Opts<-1, -1, -1, 0>());
-    return kp.force_mode == 0 ? f(Opts<-1, -1, 0, 1>()) : kp.force_mode == 1 ? f(Opts<-1, -1, 1, 1>()) : f(Opts<-1, -1, 2, 1>());
+    if (DEV && !ref) return f(Opts<-1, -1, -1, 0>());
+    return kp.force_mode == 0 ? f(Opts<-1, -1, 0, ON>()) : kp.force_mode == 1 ? f(Opts<-1, -1, 1, ON>()) : f(Opts<-1, -1, 2, ON>());
 }
 
 // Rows (units: pairs or rows) of a tile: of the heights from `most`/2 to `most`, the one whose fullest
@@ -809,15 +810,15 @@ struct Tile {
             const KParams kq = with_pull(kp);
             auto go = [&](auto kernel) { return launch_dependent(kernel, grid, block, 0, st, kq, ahead); };
             const bool links = kp.q || kp.wall_u, solid = kp.solid != nullptr;
-            if constexpr (IsDev<S>::value) {
-                if (kp.packed) {
-                    const bool open = kp.periodic_x && kp.periodic_y;
-                    if (links) return with_packed_options(kp, false, [&](auto o) { return go(k_tile2<S, 2, decltype(o), v2>); });
-                    if (solid) return with_packed_options(kp, false, [&](auto o) { return go(k_tile2<S, 1, decltype(o), v2>); });
-                    return with_packed_options(kp, open, [&](auto o) { return go(k_tile2<S, 0, decltype(o), v2>); });
-                }
+            constexpr bool DEV = IsDev<S>::value;
+            if constexpr (DEV) if (kp.packed) {
+                const bool plain = !links && !solid && kp.periodic_x && kp.periodic_y;
+                return with_packed_options<DEV>(kp, plain, [&](auto o) {
+                    typedef decltype(o) O;
+                    return links ? go(k_tile2<S, 2, O, v2>) : solid ? go(k_tile2<S, 1, O, v2>) : go(k_tile2<S, 0, O, v2>);
+                });
             }
-            return with_options<IsDev<S>::value>(kp, [&](auto o) {
+            return with_options<DEV>(kp, [&](auto o) {
                 typedef decltype(o) O;
                 return links ? go(k_tile2<S, 2, O, v2x>) : solid ? go(k_tile2<S, 1, O, v2x>) : go(k_tile2<S, 0, O, v2x>);
             });

@@ -11,6 +11,7 @@ constexpr int kRowThreads = 128;
 // Reads population k of node (x, y) of kp.src from global memory.
 template <class S>
 struct GlobalAt {
+    static constexpr bool DEV = IsDev<S>::value;
     const KParams &kp;
     __device__ __forceinline__ typename Codec<S>::R operator()(int k, int x, int y) const { return load_pop<S>(kp, k, x, y); }
     __device__ __forceinline__ typename Codec<S>::R at_k(int k, int64_t kk) const { return load_pop_at<S>(kp, k, kk); }

@@ -283,14 +283,22 @@ static bool fused_possible(const lbm_ctx *c)
     return true;
 }
 
-// Which of the two requestable steps an LBM_KERNEL_AUTO context takes (lbm_kernel_in_use): LBM_KERNEL_FUSED's from
-// these sizes on.  16-bit storage rounds accordingly (KParams::packed).
+// Which of the two requestable steps an LBM_KERNEL_AUTO context takes: LBM_KERNEL_FUSED's from these sizes on.  16-bit
+// storage rounds accordingly (KParams::packed).
 static bool auto_prefers_fused(const lbm_ctx *c)
 {
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
     if (c->q || c->wall_u) return n >= (int64_t(1) << 22);
     if (c->solid) return n >= (int64_t(1) << (c->p.precision == LBM_F32 ? 19 : 18));
     return (n >= (int64_t(1) << 18) && c->p.nx >= 512) || n >= (int64_t(1) << 21);
+}
+
+// Whether the context takes the step of LBM_KERNEL_FUSED (lbm_kernel_in_use).
+static bool fused_step(const lbm_ctx *c)
+{
+    const int want = c->p.kernel;
+    return want != LBM_KERNEL_TWO_PASS && fused_possible(c) &&
+           (want == LBM_KERNEL_FUSED || c->p.precision == LBM_F64 || auto_prefers_fused(c));
 }
 
 // Which kernel steps the context: the two-pass kernels on request (LBM_KERNEL_TWO_PASS); else a
@@ -307,8 +315,7 @@ static void choose_kernel(lbm_ctx *c)
 {
     const int want = c->p.kernel;
     const bool possible = fused_possible(c);
-    c->fused_ok = (want != LBM_KERNEL_TWO_PASS) && possible &&
-                  (want == LBM_KERNEL_FUSED || c->p.precision == LBM_F64 || auto_prefers_fused(c));
+    c->fused_ok = fused_step(c);
     const bool staged = possible && c->L.fused_pass && c->p.periodic_x && c->p.periodic_y && !c->solid && !c->q && !c->wall_u;
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
     const bool large = n >= (c->p.precision == LBM_F32 ? (int64_t)1 << 25 : (int64_t)3 << 20);
@@ -475,7 +482,8 @@ static lbm_status narrow(lbm_ctx *c, float **dst, const double *src, size_t coun
 // wall (a solid node or beyond a non-periodic edge), the link fraction q of the outgoing
 // population o = opp(i) (1/2 without link fractions, and 1/2 where q < 1/2 but the second
 // node x + e_i is a wall too -- the same fallback as the two-pass step's bounce-back) and
-// the moving-wall coefficient 2 w_o (e_i . u_w) 3 of the wall node (0 beyond an edge).
+// the velocity of the wall node along e_i, or the whole moving-wall coefficient
+// 2 w_o (e_i . u_w) 3 for the packed step (0 beyond an edge).
 static lbm_status build_link_records(lbm_ctx *c, const uint8_t *solid, const double *wall_u, const double *q)
 {
     static const int EX[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, EY[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
@@ -483,6 +491,7 @@ static lbm_status build_link_records(lbm_ctx *c, const uint8_t *solid, const dou
     static const double W[9] = {4.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 36, 1.0 / 36, 1.0 / 36, 1.0 / 36};
     release(c, &c->link);
     if (!q && !wall_u) return LBM_OK;
+    const bool packed = fused_step(c) && c->p.precision >= LBM_F16DEV;
     const int nx = c->p.nx, ny = c->p.ny;
     const int64_t n = (int64_t)nx * ny, pitch = c->pitch, plane = c->plane;
     auto wall_at = [&](int x, int y, int64_t *node) -> bool {
@@ -509,9 +518,11 @@ static lbm_status build_link_records(lbm_ctx *c, const uint8_t *solid, const dou
                 double qq = q ? q[(int64_t)(o - 1) * n + node] : 0.5;
                 int64_t bn;
                 if (qq < 0.5 && wall_at(x + EX[i], y + EY[i], &bn)) qq = 0.5;
-                double cw = 0.0;
-                if (wall_u && wn >= 0) cw = 2.0 * W[o] * (EX[i] * wall_u[wn] + EY[i] * wall_u[n + wn]) * 3.0;
-                h[(size_t)((i - 1) * plane + k)] = make_float2((float)qq, (float)cw);
+                float cw = 0.f;
+                if (wall_u && wn >= 0)
+                    cw = packed ? (float)(2.0 * W[o] * (EX[i] * wall_u[wn] + EY[i] * wall_u[n + wn]) * 3.0)
+                                : (float)EX[i] * (float)wall_u[wn] + (float)EY[i] * (float)wall_u[n + wn];
+                h[(size_t)((i - 1) * plane + k)] = make_float2((float)qq, cw);
             }
         }
     CK(cudaMalloc((void **)&c->link, h.size() * sizeof(float2)), "link records");

@@ -268,6 +268,17 @@ __device__ __forceinline__ typename Codec<S>::R load_pop(const KParams &kp, int 
     return load_pop_at<S>(kp, i, (int64_t)y * kp.pitch + x);
 }
 
+// q < 1/2 of an interpolated link: 2q fbar_o(x) + (1 - 2q) fbar_o(x + e_i) + mw.  In FP32 arithmetic one of the two
+// products goes into the sum without a rounding of its own; written out, so that every kernel takes the
+// same one (16-bit storage the second, FP32 the first).
+template <bool DEV, class R>
+__device__ __forceinline__ R near_link(R q, R fo, R f2, R mw)
+{
+    if constexpr (is_f64<R>()) return R(2) * q * fo + (R(1) - R(2) * q) * f2 + mw;
+    else if constexpr (DEV) return __fadd_rn(__fmaf_rn(1.f - 2.f * q, f2, __fmul_rn(2.f * q, fo)), mw);
+    else return __fadd_rn(__fmaf_rn(2.f * q, fo, __fmul_rn(1.f - 2.f * q, f2)), mw);
+}
+
 // Link closed by a wall (x - e_i is a wall): the population that left (x, y) toward it
 // comes back.  `at(k, xx, yy)` reads population k of node (xx, yy) (xx, yy in domain).
 // half-way (q = 1/2): f_i = fbar_o(x) + mw
@@ -303,7 +314,7 @@ __device__ __forceinline__ R bounce(const KParams &kp, int x, int y, const At &a
     R f;
     if (q < R(0.5)) {
         wrap_xy(kp, xb, yb);
-        f = R(2) * q * fo + (R(1) - R(2) * q) * at(o, xb, yb) + mw;
+        f = near_link<At::DEV>(q, fo, at(o, xb, yb), mw);
     } else if (q == R(0.5)) {
         f = fo + mw;
     } else {

@@ -82,9 +82,10 @@ struct KParams {
     const double *wall_psi;  // [ny*nx] psi of wall_rho, or null (psi_s)
     const float *fext_f, *wall_psi_f;  // the same two in FP32 (kernels of FP32 arithmetic convert no FP64 value)
     // [8][ny][pitch] per fluid node and pulled population i = 1..8 whose source x - e_i is a
-    // wall: (q, c) with q the link fraction after the fallback of a missing second node, and
-    // c = 6 w_o (e_i . u_w) the moving-wall coefficient (mw = c rho_w); null without
-    // interpolated or moving walls, and in FP64.  Read by the tile kernel's wall links.
+    // wall: (q, c) with q the link fraction after the fallback of a missing second node, and c the wall's
+    // part of the moving-wall term: e_i . u_w as the two-pass step forms it (mw = 2 w_o rho_w c 3) or, in the
+    // packed step, 6 w_o (e_i . u_w) (mw = c rho_w).  Null without interpolated or moving walls, and in FP64.
+    // Read by the tile kernel's wall links.
     const float2 *link;
     // [ny*nx] per node: bit i (1..8) set when the source x - e_i is a wall, bit 0 when the node is
     // solid; null without solid nodes, link fractions and wall velocities.  Read by the tile kernel.
