@@ -279,8 +279,7 @@ LBM_API int64_t lbm_step_count(const lbm_ctx *ctx);
 
 /* Which of the two requestable steps the context takes: that of LBM_KERNEL_TWO_PASS or LBM_KERNEL_FUSED (for
  * LBM_KERNEL_AUTO by size and geometry).  An AUTO context leaves the states that the kernel named here
- * leaves on request, bit for bit, but for FP32 storage and LBM_KERNEL_FUSED, where it is to rounding.  Which
- * kernel it launches for that: lbm_step_launches. */
+ * leaves on request, bit for bit.  Which kernel it launches for that: lbm_step_launches. */
 LBM_API int32_t lbm_kernel_in_use(const lbm_ctx *ctx);
 
 typedef enum {

@@ -10,7 +10,7 @@
 // evaluation rounds twice; with them every node's result is the two-pass step's, bit for bit.  Where the
 // context takes the step of LBM_KERNEL_FUSED (KParams::packed) the products are plain packed ones and 16-bit
 // storage encodes as the staged kernel does (v2): the state is then the staged kernel's, bit for bit,
-// whichever of the two kernels a size gets.  (In FP32 storage the exact products stay.)
+// whichever of the two kernels a size gets.
 // FP64 (k_tile1): one node per thread, the two-pass step's own functions, the same bits.
 //
 // A tile of n pairs (rows) has n warps for them; one more warp pulls the rows above and below the
@@ -724,7 +724,8 @@ inline cudaError_t with_options(const KParams &kp, const F &f)
 // The packed rounding fixes fewer of them: the assembler fuses a packed product into a sum where both stand in one
 // block of the code, so the relaxation and the scheme stay branches exactly where the staged kernel
 // (Fused2::launch) has them.  512 x 4096 with walls, FP16: 36.6 us with all at run time, 34.7 here, 35.4 with
-// exact products and the options above; bands 2048^2, two relaxation times, FP16 72.6 / 70.6 / 80.3.
+// exact products and the options above (FP32 29.3 / 28.8 with exact products / here); bands 2048^2, two
+// relaxation times, FP16 72.6 / 70.6 / 80.3 (FP32 60.9 / 57.5); 4096^2 FP32 185.0 / 182.7.
 template <bool DEV, class F>
 inline cudaError_t with_packed_options(const KParams &kp, bool plain, const F &f)
 {
@@ -811,7 +812,7 @@ struct Tile {
             auto go = [&](auto kernel) { return launch_dependent(kernel, grid, block, 0, st, kq, ahead); };
             const bool links = kp.q || kp.wall_u, solid = kp.solid != nullptr;
             constexpr bool DEV = IsDev<S>::value;
-            if constexpr (DEV) if (kp.packed) {
+            if (kp.packed) {
                 const bool plain = !links && !solid && kp.periodic_x && kp.periodic_y;
                 return with_packed_options<DEV>(kp, plain, [&](auto o) {
                     typedef decltype(o) O;

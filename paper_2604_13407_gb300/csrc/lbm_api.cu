@@ -283,8 +283,8 @@ static bool fused_possible(const lbm_ctx *c)
     return true;
 }
 
-// Which of the two requestable steps an LBM_KERNEL_AUTO context takes: LBM_KERNEL_FUSED's from these sizes on.  16-bit
-// storage rounds accordingly (KParams::packed).
+// Which of the two requestable steps an LBM_KERNEL_AUTO context takes: LBM_KERNEL_FUSED's from these sizes on.  The
+// tile kernel rounds accordingly (KParams::packed).
 static bool auto_prefers_fused(const lbm_ctx *c)
 {
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
@@ -303,7 +303,7 @@ static bool fused_step(const lbm_ctx *c)
 
 // Which kernel steps the context: the two-pass kernels on request (LBM_KERNEL_TWO_PASS); else a
 // one-pass kernel, the staged one (k_fused2) or the tile kernel (k_tile), which gives the two-pass
-// step's results (16-bit storage where LBM_KERNEL_FUSED is granted: the staged one's).  The staged kernel
+// step's results (where the context takes the step of LBM_KERNEL_FUSED: the staged one's).  The staged kernel
 // reads each row once where the tile kernel re-reads its tiles' rings from L2, but a CTA walks its rows in
 // series, and it has no walls; the tile kernel has thousands of short blocks.  Step times on a GB300 (us, tile /
 // staged): FP32 periodic 512^2 5.4 / 10.3, 1024^2 13.8 / 22.8, 2048^2 49.7 / 56.6, 4096^2 186 / 195, 8192^2
@@ -319,7 +319,7 @@ static void choose_kernel(lbm_ctx *c)
     const bool staged = possible && c->L.fused_pass && c->p.periodic_x && c->p.periodic_y && !c->solid && !c->q && !c->wall_u;
     const int64_t n = (int64_t)c->p.nx * c->p.ny;
     const bool large = n >= (c->p.precision == LBM_F32 ? (int64_t)1 << 25 : (int64_t)3 << 20);
-    c->kp.packed = c->fused_ok && c->p.precision >= LBM_F16DEV;
+    c->kp.packed = c->fused_ok && c->p.precision != LBM_F64;
     c->one_pass = nullptr;
     c->small_ctas = want == LBM_KERNEL_AUTO ? c->L.small_ctas(c->kp) : 0;
     if (want == LBM_KERNEL_TWO_PASS || (want == LBM_KERNEL_FUSED && !possible)) return;
@@ -491,7 +491,7 @@ static lbm_status build_link_records(lbm_ctx *c, const uint8_t *solid, const dou
     static const double W[9] = {4.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 36, 1.0 / 36, 1.0 / 36, 1.0 / 36};
     release(c, &c->link);
     if (!q && !wall_u) return LBM_OK;
-    const bool packed = fused_step(c) && c->p.precision >= LBM_F16DEV;
+    const bool packed = fused_step(c);
     const int nx = c->p.nx, ny = c->p.ny;
     const int64_t n = (int64_t)nx * ny, pitch = c->pitch, plane = c->plane;
     auto wall_at = [&](int x, int y, int64_t *node) -> bool {

@@ -2,8 +2,8 @@
 // psi stencil and collision, written once for a lane type V that is either one node (v1,
 // scalar FP32 instructions) or two nodes (v2, packed FP32x2 instructions: FADD2, FMUL2,
 // FFMA2 of the sm_100 family).  The two-pass kernels use v1, the staged kernel and the
-// transposed step v2, the tile kernel a pair rounded like v1 (v2x, k_tile.cuh; v2 where 16-bit storage follows
-// the staged kernel), the small-lattice kernel v1 or, on strips of more than 512 nodes, v2x; all
+// transposed step v2, the tile kernel a pair rounded like v1 (v2x, k_tile.cuh; v2 where it follows the
+// staged kernel), the small-lattice kernel v1 or, on strips of more than 512 nodes, v2x; all
 // evaluate the same expressions in the same order.  The scalar _rn intrinsics round
 // exactly as written (checked bit for bit against a numpy evaluation of the same
 // expressions).  The pair intrinsics do not always: measured on this toolchain, a packed

@@ -41,7 +41,7 @@ struct KParams {
     int var_tau;     // 1: tau(rho) from the linear nu(rho) interpolation
     int per_node_ref;
     int sr;            // FP16/BF16 storage: 1 stochastic rounding, 0 to nearest
-    int packed;        // FP16/BF16 storage: 1 the tile kernel rounds as the staged kernel does (k_tile.cuh)
+    int packed;        // FP32 arithmetic: 1 the tile kernel rounds as the staged kernel does (k_tile.cuh)
     uint32_t sr_seed;  // random-bit seed of this step (a hash of the step count)
     // EOS: p = K (rho RT g(rho) - a rho^2); psi = sqrt(two_over_G (p - rho/3))
     double eos_a, eos_b, eos_RT, eos_K, two_over_G;

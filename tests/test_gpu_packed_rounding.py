@@ -1,5 +1,5 @@
 """FP32 arithmetic: LBM_KERNEL_AUTO leaves the states of the kernel that lbm_kernel_in_use names, bit for bit.  Where that
-is LBM_KERNEL_FUSED, in 16-bit storage, whether the size gets the staged kernel or the tile kernel; where it is LBM_KERNEL_TWO_PASS, with
+is LBM_KERNEL_FUSED, whether the size gets the staged kernel or the tile kernel; where it is LBM_KERNEL_TWO_PASS, with
 interpolated and moving walls too.  (A 16-bit deviation is rounded to the storage type, so a last-bit difference of
 the FP32 arithmetic before it would show as a whole ulp of that type.)"""
 import numpy as np
@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec,kw", [(p, kw) for p in (lbm.F16DEV, lbm.BF16DEV)
-                                     for kw in (dict(per_node_ref=1), dict(per_node_ref=1, storage_rounding=0), dict(per_node_ref=0))])
+                                     for kw in (dict(per_node_ref=1), dict(per_node_ref=1, storage_rounding=0), dict(per_node_ref=0))] +
+                         [(lbm.F32, {})])
 @pytest.mark.parametrize("scheme", [0, 1])
 @pytest.mark.parametrize("force_mode,tau_g", [(0, 1.0), (0, 0.7), (1, 1.0), (1, 0.7), (2, 1.0)])
 @pytest.mark.parametrize("nx,ny", [(512, 512), (520, 517)])

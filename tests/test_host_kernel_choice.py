@@ -49,7 +49,9 @@ F16, F32, F64 = lbm.F16DEV, lbm.F32, lbm.F64
 @pytest.mark.parametrize("nx,ny,prec,kw,kernel,ran,in_use", [
     # periodic: staged rows from 2^25 nodes in FP32, from 3 2^20 in 16 bits, never in FP64
     (4096, 8192, F32, {}, "staged", "staged", 2),
-    (4096, 8191, F32, {}, "tile", "tile", 2),
+    (4096, 8191, F32, {}, "tile", "tile packed", 2),
+    (512, 512, F32, {}, "tile", "tile packed", 2),
+    (512, 511, F32, {}, "tile", "tile", 1),
     (1024, 3072, F16, {}, "staged", "staged", 2),
     (1024, 3071, F16, {}, "tile", "tile packed", 2),
     (1024, 3071, lbm.BF16DEV, {}, "tile", "tile packed", 2),
@@ -57,18 +59,21 @@ F16, F32, F64 = lbm.F16DEV, lbm.F32, lbm.F64
     # a width that no staged row can have
     (4098, 8192, F32, {}, "tile", "tile", 1),
     (1028, 3072, F16, {}, "tile", "tile", 1),
-    # walls: tiles at every size; 16-bit storage rounds as the staged kernel from 2^18 nodes
-    (4096, 8192, F32, dict(periodic_x=0), "tile", "tile", 2),
+    # walls: tiles at every size, rounded as the staged kernel where the step is that of LBM_KERNEL_FUSED
+    (4096, 8192, F32, dict(periodic_x=0), "tile", "tile packed", 2),
+    (256, 2048, F32, dict(periodic_x=0), "tile", "tile", 1),
     (512, 512, F16, dict(periodic_y=0), "tile", "tile packed", 2),
     (512, 511, F16, dict(periodic_y=0), "tile", "tile", 1),
     (256, 2048, F16, dict(periodic_x=0), "tile", "tile", 1),
     (512, 512, F16, dict(geom="solid"), "tile", "tile packed", 2),
     (512, 511, F16, dict(geom="solid"), "tile", "tile", 1),
     (512, 512, F32, dict(geom="solid"), "tile", "tile", 1),
+    (1024, 512, F32, dict(geom="solid"), "tile", "tile packed", 2),
+    (512, 512, F64, dict(geom="solid"), "tile", "tile", 1),
     (1024, 1024, F16, dict(geom="q"), "tile", "tile", 1),
     # on request
     (256, 64, F32, dict(kernel=lbm.KERNEL_FUSED), "staged", "staged", 2),
-    (256, 64, F32, dict(kernel=lbm.KERNEL_FUSED, periodic_x=0), "tile", "tile", 2),
+    (256, 64, F32, dict(kernel=lbm.KERNEL_FUSED, periodic_x=0), "tile", "tile packed", 2),
     (256, 64, F16, dict(kernel=lbm.KERNEL_FUSED, geom="solid"), "tile", "tile packed", 2),
     (255, 64, F32, dict(kernel=lbm.KERNEL_FUSED), "two_pass", "two_pass", 1),
     (256, 64, F64, dict(kernel=lbm.KERNEL_FUSED, geom="solid"), "two_pass", "two_pass", 1),
