@@ -32,12 +32,15 @@ struct lbm_ctx {
     float *refp[2] = {nullptr, nullptr};
     int cur = 0;
     void *psi = nullptr;    // psi field of the two-pass step; rows of sums of the diagnostics
+    void *geometry = nullptr;  // one allocation, the arrays of lbm_set_geometry and what derives from them:
     uint8_t *solid = nullptr;
     double *wall_u = nullptr, *q = nullptr, *fext = nullptr;
-    double *wall_rho = nullptr, *wall_psi = nullptr;  // per solid node virtual density, its psi
-    float *fext_f = nullptr, *wall_psi_f = nullptr;   // fext and wall_psi in FP32 (not for FP64 storage)
+    float *fext_f = nullptr;            // fext in FP32 (not for FP64 storage)
     float2 *link = nullptr;             // wall-link records of the tile kernel (KParams::link)
     uint16_t *links = nullptr;          // wall bits of every node (KParams::links)
+    void *walls = nullptr;     // one allocation, the arrays of lbm_set_wall_density:
+    double *wall_rho = nullptr, *wall_psi = nullptr;  // per solid node virtual density, its psi
+    float *wall_psi_f = nullptr;        // wall_psi in FP32 (not for FP64 storage)
     double *dacc = nullptr;             // diagnostics: 9 sums, max |u|, count of non-finite nodes
     double *scratch = nullptr;          // host<->device staging for FP64 field copies
     size_t scratch_bytes = 0;
@@ -332,8 +335,7 @@ static void free_all(lbm_ctx *c)
 {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
-    void *bufs[] = {c->pops[0], c->pops[1], c->refp[0], c->refp[1], c->psi, c->solid,
-                    c->wall_u, c->q, c->fext, c->wall_rho, c->wall_psi, c->fext_f, c->wall_psi_f, c->link, c->links, c->dacc, c->scratch, c->derr};
+    void *bufs[] = {c->pops[0], c->pops[1], c->refp[0], c->refp[1], c->psi, c->geometry, c->walls, c->dacc, c->scratch, c->derr};
     for (void *b : bufs)
         if (b) cudaFree(b);
     adjoint_free(c->adj);
@@ -441,22 +443,27 @@ static lbm_status need_scratch(lbm_ctx *c, size_t bytes)
     return LBM_OK;
 }
 
+// Arrays one behind the other in an allocation: an array has its place before there is one.
+struct Places {
+    size_t used = 0;
+    size_t take(size_t bytes)
+    {
+        const size_t at = used;
+        used += (bytes + 255) / 256 * 256;
+        return at;
+    }
+};
+// An array at its place, or null where it is not wanted.
 template <class T>
-static void release(lbm_ctx *c, T **p)
+static void put_at(T **p, void *base, size_t at, bool wanted)
 {
-    if (!*p) return;
-    cudaStreamSynchronize(c->stream);
-    cudaFree(*p);
-    *p = nullptr;
+    *p = wanted ? reinterpret_cast<T *>(static_cast<char *>(base) + at) : nullptr;
 }
 
 template <class T>
-static lbm_status upload(lbm_ctx *c, T **dst, const T *src, size_t count, const char *what)
+static lbm_status upload(lbm_ctx *c, T *dst, const T *src, size_t count, const char *what)
 {
-    release(c, dst);
-    if (!src) return LBM_OK;
-    CK(cudaMalloc((void **)dst, count * sizeof(T)), what);
-    CK(cudaMemcpyAsync(*dst, src, count * sizeof(T), cudaMemcpyHostToDevice, c->stream), what);
+    if (src) CK(cudaMemcpyAsync(dst, src, count * sizeof(T), cudaMemcpyHostToDevice, c->stream), what);
     return LBM_OK;
 }
 
@@ -466,13 +473,11 @@ static __global__ void k_narrow(const double *in, float *out, int64_t n)
     if (k < n) out[k] = float(in[k]);
 }
 
-// *dst = src[count] in FP32 (null src: none), for the storage types whose arithmetic is FP32.
-static lbm_status narrow(lbm_ctx *c, float **dst, const double *src, size_t count, const char *what)
+// dst = src[count] in FP32, for the storage types whose arithmetic is FP32 (null dst: not wanted).
+static lbm_status narrow(lbm_ctx *c, float *dst, const double *src, size_t count, const char *what)
 {
-    release(c, dst);
-    if (!src || c->p.precision == LBM_F64) return LBM_OK;
-    CK(cudaMalloc((void **)dst, count * sizeof(float)), what);
-    k_narrow<<<(unsigned)((count + 255) / 256), 256, 0, c->stream>>>(src, *dst, (int64_t)count);
+    if (!dst) return LBM_OK;
+    k_narrow<<<(unsigned)((count + 255) / 256), 256, 0, c->stream>>>(src, dst, (int64_t)count);
     CK(cudaGetLastError(), what);
     return LBM_OK;
 }
@@ -484,13 +489,11 @@ static lbm_status narrow(lbm_ctx *c, float **dst, const double *src, size_t coun
 // node x + e_i is a wall too -- the same fallback as the two-pass step's bounce-back) and
 // the velocity of the wall node along e_i, or the whole moving-wall coefficient
 // 2 w_o (e_i . u_w) 3 for the packed step (0 beyond an edge).
-static lbm_status build_link_records(lbm_ctx *c, const uint8_t *solid, const double *wall_u, const double *q)
+static std::vector<float2> link_records(const lbm_ctx *c, const uint8_t *solid, const double *wall_u, const double *q)
 {
     static const int EX[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, EY[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
     static const int OPP[9] = {0, 3, 4, 1, 2, 7, 8, 5, 6};
     static const double W[9] = {4.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 36, 1.0 / 36, 1.0 / 36, 1.0 / 36};
-    release(c, &c->link);
-    if (!q && !wall_u) return LBM_OK;
     const bool packed = fused_step(c);
     const int nx = c->p.nx, ny = c->p.ny;
     const int64_t n = (int64_t)nx * ny, pitch = c->pitch, plane = c->plane;
@@ -525,30 +528,48 @@ static lbm_status build_link_records(lbm_ctx *c, const uint8_t *solid, const dou
                 h[(size_t)((i - 1) * plane + k)] = make_float2((float)qq, cw);
             }
         }
-    CK(cudaMalloc((void **)&c->link, h.size() * sizeof(float2)), "link records");
-    CK(cudaMemcpyAsync(c->link, h.data(), h.size() * sizeof(float2), cudaMemcpyHostToDevice, c->stream),
-       "link records");
-    CK(cudaStreamSynchronize(c->stream), "link records");
-    return LBM_OK;
+    return h;
+}
+
+static void drop_geometry(lbm_ctx *c)
+{
+    if (c->geometry) {
+        cudaStreamSynchronize(c->stream);
+        cudaFree(c->geometry);
+    }
+    c->geometry = nullptr;
+    c->solid = nullptr, c->wall_u = c->q = c->fext = nullptr, c->fext_f = nullptr, c->link = nullptr, c->links = nullptr;
+    c->n_fluid = (int64_t)c->p.nx * c->p.ny;
 }
 
 static lbm_status build_geometry(lbm_ctx *c, const uint8_t *solid, const double *wall_u, const double *q,
                                  const double *force_field)
 try {
     const size_t n = (size_t)c->p.nx * c->p.ny;
-    lbm_status s;
-    if ((s = upload(c, &c->solid, solid, n, "solid")) != LBM_OK) return s;
-    c->n_fluid = (int64_t)n;
+    const bool f32 = c->p.precision != LBM_F64, walls = solid || wall_u || q, records = f32 && (wall_u || q);
+    Places at;
+    const size_t at_solid = at.take(solid ? n : 0), at_wall_u = at.take(wall_u ? 2 * n * sizeof(double) : 0);
+    const size_t at_q = at.take(q ? 8 * n * sizeof(double) : 0), at_fext = at.take(force_field ? 2 * n * sizeof(double) : 0);
+    const size_t at_fext_f = at.take(force_field && f32 ? 2 * n * sizeof(float) : 0);
+    const size_t at_link = at.take(records ? 8 * c->plane * sizeof(float2) : 0), at_links = at.take(walls ? n * sizeof(uint16_t) : 0);
+    if (at.used == 0) return LBM_OK;
+    CK(cudaMalloc(&c->geometry, at.used), "geometry");
+    put_at(&c->solid, c->geometry, at_solid, solid != nullptr), put_at(&c->wall_u, c->geometry, at_wall_u, wall_u != nullptr);
+    put_at(&c->q, c->geometry, at_q, q != nullptr), put_at(&c->fext, c->geometry, at_fext, force_field != nullptr);
+    put_at(&c->fext_f, c->geometry, at_fext_f, force_field && f32), put_at(&c->link, c->geometry, at_link, records);
+    put_at(&c->links, c->geometry, at_links, walls);
     if (solid)
         for (size_t k = 0; k < n; ++k) c->n_fluid -= solid[k] != 0;
-    if ((s = upload(c, &c->wall_u, wall_u, 2 * n, "wall_u")) != LBM_OK) return s;
-    if ((s = upload(c, &c->q, q, 8 * n, "q")) != LBM_OK) return s;
-    if ((s = upload(c, &c->fext, force_field, 2 * n, "force_field")) != LBM_OK) return s;
-    if ((s = narrow(c, &c->fext_f, c->fext, 2 * n, "force_field")) != LBM_OK) return s;
-    if (c->p.precision != LBM_F64 && (s = build_link_records(c, solid, wall_u, q)) != LBM_OK) return s;
-    release(c, &c->links);
-    if (solid || wall_u || q) {
-        CK(cudaMalloc((void **)&c->links, n * sizeof(uint16_t)), "wall bits");
+    lbm_status s;
+    if ((s = upload(c, c->solid, solid, n, "solid")) != LBM_OK) return s;
+    if ((s = upload(c, c->wall_u, wall_u, 2 * n, "wall_u")) != LBM_OK) return s;
+    if ((s = upload(c, c->q, q, 8 * n, "q")) != LBM_OK) return s;
+    if ((s = upload(c, c->fext, force_field, 2 * n, "force_field")) != LBM_OK) return s;
+    if ((s = narrow(c, c->fext_f, c->fext, 2 * n, "force_field")) != LBM_OK) return s;
+    std::vector<float2> h;
+    if (records) h = link_records(c, solid, wall_u, q);
+    if (records && (s = upload(c, c->link, (const float2 *)h.data(), h.size(), "link records")) != LBM_OK) return s;
+    if (walls) {
         fill_constants(c);
         CK(c->L.link_bits(c->kp, c->links, c->stream), "wall bits kernel");
     }
@@ -567,25 +588,36 @@ extern "C" lbm_status lbm_set_geometry(lbm_ctx *c, const uint8_t *solid, const d
         for (size_t k = 0; k < 8 * n; ++k)
             if (!(q[k] > 0.0 && q[k] <= 1.0)) return fail(c, LBM_EINVAL, "q must lie in (0, 1]");
     }
+    drop_geometry(c);
     const lbm_status s = build_geometry(c, solid, wall_u, q, force_field);
-    if (s != LBM_OK) {
-        // the old arrays gave way to the new ones, of which some are missing: none at all
-        release(c, &c->solid), release(c, &c->wall_u), release(c, &c->q), release(c, &c->fext);
-        release(c, &c->fext_f), release(c, &c->link), release(c, &c->links);
-        c->n_fluid = (int64_t)n;
-    }
+    if (s != LBM_OK) drop_geometry(c);  // (the old arrays gave way to the new ones, which are not all there)
     fill_constants(c);
     choose_kernel(c);
     return s;
 }
 
+static void drop_wall_density(lbm_ctx *c)
+{
+    if (c->walls) {
+        cudaStreamSynchronize(c->stream);
+        cudaFree(c->walls);
+    }
+    c->walls = nullptr;
+    c->wall_rho = c->wall_psi = nullptr, c->wall_psi_f = nullptr;
+}
+
 static lbm_status build_wall_density(lbm_ctx *c, const double *wall_rho, const double *psi)
 {
     const size_t n = (size_t)c->p.nx * c->p.ny;
+    const bool f32 = c->p.precision != LBM_F64;
+    Places at;
+    const size_t at_rho = at.take(n * sizeof(double)), at_psi = at.take(n * sizeof(double)), at_psi_f = at.take(f32 ? n * sizeof(float) : 0);
+    CK(cudaMalloc(&c->walls, at.used), "wall densities");
+    put_at(&c->wall_rho, c->walls, at_rho, true), put_at(&c->wall_psi, c->walls, at_psi, true), put_at(&c->wall_psi_f, c->walls, at_psi_f, f32);
     lbm_status s;
-    if ((s = upload(c, &c->wall_rho, wall_rho, n, "wall_rho")) != LBM_OK) return s;
-    if ((s = upload(c, &c->wall_psi, psi, n, "wall_psi")) != LBM_OK) return s;
-    if ((s = narrow(c, &c->wall_psi_f, c->wall_psi, n, "wall_psi")) != LBM_OK) return s;
+    if ((s = upload(c, c->wall_rho, wall_rho, n, "wall_rho")) != LBM_OK) return s;
+    if ((s = upload(c, c->wall_psi, psi, n, "wall_psi")) != LBM_OK) return s;
+    if ((s = narrow(c, c->wall_psi_f, c->wall_psi, n, "wall_psi")) != LBM_OK) return s;
     CK(cudaStreamSynchronize(c->stream), "set_wall_density");
     return LBM_OK;
 }
@@ -609,8 +641,9 @@ try {
     std::vector<double> psi;
     if (wall_rho && !wall_psi_of(c->p, wall_rho, n, psi))
         return fail(c, LBM_EINVAL, "psi of a wall density is not real and positive");
-    const lbm_status s = build_wall_density(c, wall_rho, wall_rho ? psi.data() : nullptr);
-    if (s != LBM_OK) release(c, &c->wall_rho), release(c, &c->wall_psi), release(c, &c->wall_psi_f);
+    drop_wall_density(c);
+    const lbm_status s = wall_rho ? build_wall_density(c, wall_rho, psi.data()) : LBM_OK;
+    if (s != LBM_OK) drop_wall_density(c);
     fill_constants(c);
     choose_kernel(c);
     return s;
@@ -860,9 +893,9 @@ static lbm_status refresh_wall_psi(lbm_ctx *c, const lbm_params &p)
     CK(cudaMemcpyAsync(rho.data(), c->wall_rho, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "wall_rho");
     CK(cudaStreamSynchronize(c->stream), "wall_rho");
     if (!wall_psi_of(p, rho.data(), n, psi)) return fail(c, LBM_EINVAL, "psi of a wall density is not real and positive");
-    CK(cudaMemcpyAsync(c->wall_psi, psi.data(), n * sizeof(double), cudaMemcpyHostToDevice, c->stream), "wall_psi");
-    if (c->wall_psi_f) k_narrow<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(c->wall_psi, c->wall_psi_f, (int64_t)n);
-    CK(cudaGetLastError(), "wall_psi");
+    lbm_status s;
+    if ((s = upload(c, c->wall_psi, (const double *)psi.data(), n, "wall_psi")) != LBM_OK) return s;
+    if ((s = narrow(c, c->wall_psi_f, c->wall_psi, n, "wall_psi")) != LBM_OK) return s;
     CK(cudaStreamSynchronize(c->stream), "wall_psi");
     return LBM_OK;
 }
