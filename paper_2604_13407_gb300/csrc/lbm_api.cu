@@ -45,7 +45,6 @@ struct lbm_ctx {
     double *scratch = nullptr;          // host<->device staging for FP64 field copies
     size_t scratch_bytes = 0;
     int *derr = nullptr;
-    int small_ctas = 0;  // LBM_KERNEL_AUTO: CTAs of the cluster that steps a small lattice; 0: one launch per step
     bool initialised = false;
     bool fused_ok = false;
     cudaError_t (*one_pass)(const KParams &, cudaStream_t) = nullptr;  // the step's kernel; null: two-pass
@@ -324,7 +323,6 @@ static void choose_kernel(lbm_ctx *c)
     const bool large = n >= (c->p.precision == LBM_F32 ? (int64_t)1 << 25 : (int64_t)3 << 20);
     c->kp.packed = c->fused_ok && c->p.precision != LBM_F64;
     c->one_pass = nullptr;
-    c->small_ctas = want == LBM_KERNEL_AUTO ? c->L.small_ctas(c->kp) : 0;
     if (want == LBM_KERNEL_TWO_PASS || (want == LBM_KERNEL_FUSED && !possible)) return;
     c->one_pass = staged && (want == LBM_KERNEL_FUSED || large) ? c->L.fused_pass : c->L.tile_pass;
 }
@@ -689,18 +687,24 @@ extern "C" lbm_status lbm_init_fields(lbm_ctx *c, const double *rho, const doubl
     return LBM_OK;
 }
 
-// How many of the next nsteps steps the small-lattice kernel takes in one launch (no more than 4096, so that no
-// launch takes long); 0: none (fewer than four are as fast one by one).
-static int64_t at_once(const lbm_ctx *c, int64_t nsteps)
+// CTAs of the cluster that takes a call's steps in the small-lattice kernel; 0: one launch per step.  Asked when a
+// call could use it: the first question in a process loads the kernel (12 ms), which a program that takes its
+// steps one by one does not need.
+static int small_ctas(const lbm_ctx *c, int64_t nsteps)
 {
-    return c->small_ctas > 0 && nsteps >= 4 ? std::min<int64_t>(nsteps, 4096) : 0;
+    return c->p.kernel == LBM_KERNEL_AUTO && nsteps >= 4 ? c->L.small_ctas(c->kp) : 0;
 }
+
+// How many of the next nsteps steps it takes in one launch (no more than 4096, so that no launch takes long); 0:
+// none (fewer than four are as fast one by one).
+static int64_t at_once(int ctas, int64_t nsteps) { return ctas > 0 && nsteps >= 4 ? std::min<int64_t>(nsteps, 4096) : 0; }
 
 static lbm_status run_steps(lbm_ctx *c, int64_t nsteps)
 {
-    while (const int64_t n = at_once(c, nsteps)) {
+    const int ctas = small_ctas(c, nsteps);
+    while (const int64_t n = at_once(ctas, nsteps)) {
         bind_buffers(c, c->cur);
-        CK(c->L.small_steps(c->kp, c->small_ctas, n, c->steps, c->stream), "small-lattice kernel");
+        CK(c->L.small_steps(c->kp, ctas, n, c->steps, c->stream), "small-lattice kernel");
         c->cur ^= (int)(n & 1);
         c->steps += n;
         c->kp.sr_seed = sr_seed_of(c->steps - 1);
@@ -950,15 +954,16 @@ extern "C" int64_t lbm_step_launches(const lbm_ctx *c, int64_t nsteps, int32_t *
 {
     if (!c || nsteps < 0) return -1;
     const int64_t D = c->p.diag_every;
+    const int ctas = small_ctas(c, nsteps);
     const int64_t first = D > 0 ? std::min<int64_t>(nsteps, D - c->steps % D) : nsteps, rest = nsteps - first;
     auto launches = [&](int64_t n) {
-        const int64_t most = at_once(c, n);
+        const int64_t most = at_once(ctas, n);
         if (most == 0) return c->one_pass ? n : 2 * n;
         const int64_t left = n % most;
-        return n / most + (at_once(c, left) ? 1 : c->one_pass ? left : 2 * left);
+        return n / most + (at_once(ctas, left) ? 1 : c->one_pass ? left : 2 * left);
     };
     if (kernel)
-        *kernel = at_once(c, rest > 0 ? std::max(first, std::min(rest, D)) : first) ? LBM_STEP_SMALL
+        *kernel = at_once(ctas, rest > 0 ? std::max(first, std::min(rest, D)) : first) ? LBM_STEP_SMALL
                   : !c->one_pass                                                    ? LBM_STEP_TWO_PASS
                   : c->one_pass == c->L.fused_pass                                  ? LBM_STEP_STAGED
                                                                                     : LBM_STEP_TILE;

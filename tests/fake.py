@@ -21,7 +21,7 @@ def load(folder):
     lib = lbm.load_library(out)
     lib.fake_limit.argtypes = [ctypes.c_long, ctypes.c_size_t]
     lib.fake_reset.restype = lib.fake_limit.restype = None
-    lib.fake_faults.restype = lib.fake_launches.restype = lib.fake_mallocs.restype = lib.fake_attributes.restype = ctypes.c_long
+    lib.fake_faults.restype = lib.fake_launches.restype = lib.fake_small_asked.restype = lib.fake_mallocs.restype = lib.fake_attributes.restype = ctypes.c_long
     lib.fake_what.restype = lib.fake_last_step.restype = ctypes.c_char_p
     lib.fake_bytes.restype = ctypes.c_size_t
     return lib

@@ -21,7 +21,7 @@ namespace {
 std::map<const char *, size_t> g_live;
 long g_mallocs_left = -1;      // allocations that still succeed; -1: all
 size_t g_bytes_left = (size_t)-1;
-long g_faults = 0, g_launches = 0, g_attributes = 0, g_mallocs = 0;
+long g_faults = 0, g_launches = 0, g_attributes = 0, g_mallocs = 0, g_small_asked = 0;
 unsigned long long g_context = 1;
 int g_small_ctas = 0;
 std::string g_what, g_last;
@@ -88,7 +88,7 @@ struct Fake {
     }
     static cudaError_t fused_pass(const KParams &k, cudaStream_t) { return one(k, "staged"); }
     static cudaError_t tile_pass(const KParams &k, cudaStream_t) { return one(k, k.packed ? "tile packed" : "tile"); }
-    static int small_ctas(const KParams &k) { return k.q || k.wall_u ? 0 : g_small_ctas; }
+    static int small_ctas(const KParams &k) { return ++g_small_asked, k.q || k.wall_u ? 0 : g_small_ctas; }
     static cudaError_t small_steps(const KParams &k, int, int64_t n, int64_t, cudaStream_t)
     {
         check(k, F32);
@@ -195,13 +195,14 @@ LBM_API void fake_limit(long mallocs, size_t bytes) { g_mallocs_left = mallocs, 
 LBM_API void fake_reset(int small_ctas)
 {
     g_mallocs_left = -1, g_bytes_left = (size_t)-1, g_small_ctas = small_ctas;
-    g_faults = g_launches = g_attributes = g_mallocs = 0;
+    g_faults = g_launches = g_attributes = g_mallocs = g_small_asked = 0;
     g_what.clear(), g_last.clear();
 }
 LBM_API long fake_faults() { return g_faults; }
 LBM_API const char *fake_what() { return g_what.c_str(); }
 LBM_API const char *fake_last_step() { return g_last.c_str(); }
 LBM_API long fake_launches() { return g_launches; }
+LBM_API long fake_small_asked() { return g_small_asked; }
 LBM_API long fake_mallocs() { return g_mallocs; }
 LBM_API long fake_attributes() { return g_attributes; }
 LBM_API void fake_device_reset() { ++g_context; }

@@ -109,3 +109,18 @@ def test_small_lattices(fakelib, prec):
     sim = _sim(fakelib, 64, 64, prec, small=16, geom="q")  # link fractions: not in the small-lattice kernel
     _check(fakelib, sim, 9, "tile", "tile")
     sim.close()
+
+
+def test_the_small_lattice_kernel_is_asked_for_when_a_call_can_use_it(fakelib):
+    """Creating a context, geometry and single steps load nothing for it."""
+    sim = _sim(fakelib, 64, 64, F32, small=16, geom="solid")
+    for n in (1, 2, 3):
+        sim.step(n)
+    assert fakelib.fake_small_asked() == 0
+    sim.step(4)
+    assert fakelib.fake_small_asked() == 1 and fakelib.fake_last_step() == b"small"
+    sim.close()
+    sim = _sim(fakelib, 64, 64, F32, small=16, kernel=lbm.KERNEL_TWO_PASS)
+    sim.step(9)
+    assert fakelib.fake_small_asked() == 0
+    sim.close()
