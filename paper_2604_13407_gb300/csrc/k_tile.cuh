@@ -18,8 +18,8 @@
 // chosen per launch (tile_height) so that the last wave of blocks is nearly full.
 //
 // What bounds it (FP32): small lattices the latency of one block's chain, mid-size ones instruction
-// issue (557 a pair of rows and 32 columns, ring included, FP16 787; the two-pass kernels 1840), from 2048^2 on HBM:
-// 4096^2 186 us, 97 % of the measured copy rate at 72 B a node. Four pairs and five blocks per SM (64
+// issue (546 a pair of rows and 32 columns, ring included, 557 with exact products, FP16 787; the two-pass kernels
+// 1840), from 2048^2 on HBM: 4096^2 183 us, 99 % of the measured copy rate at 72 B a node. Four pairs and five blocks per SM (64
 // registers) against two blocks of eight pairs: 512 x 4096 46 -> 36 us; the L2 prefetch 70 -> 59 at 2048^2;
 // the instantiation without edge tests (INNER) 59 -> 52, FP16 81 -> 67.
 //

@@ -308,8 +308,8 @@ static bool fused_step(const lbm_ctx *c)
 // step's results (where the context takes the step of LBM_KERNEL_FUSED: the staged one's).  The staged kernel
 // reads each row once where the tile kernel re-reads its tiles' rings from L2, but a CTA walks its rows in
 // series, and it has no walls; the tile kernel has thousands of short blocks.  Step times on a GB300 (us, tile /
-// staged): FP32 periodic 512^2 5.4 / 10.3, 1024^2 13.8 / 22.8, 2048^2 49.7 / 56.6, 4096^2 186 / 195, 8192^2
-// 759 / 745; FP16, whose ring costs instructions and not bytes, constant (buoyant) force, 1024^2 16.6 / 27.0
+// staged): FP32 periodic 512^2 5.0 / 10.2, 1024^2 13.0 / 22.8, 2048^2 48.7 / 56.4, 4096^2 183 / 195, 8192^2
+// 744 / 746 (759 with exact products); FP16, whose ring costs instructions and not bytes, constant (buoyant) force, 1024^2 16.6 / 27.0
 // (16.8 / 28.6), 1536 x 2048 46.4 / 53.6 (47.2 / 58.2), 2048^2 60.6 / 58.8 (61.1 / 63.8), 4096^2 226 / 194
 // (226 / 213): the line at 3 2^20 is a little low.  (Two-pass kernels, FP32: 512^2 10.3, 1024^2 31, 2048^2
 // 121; 256 x 2048 with walls 20.6 against the tile kernel's 8.9; banded 512^2 17.6 / 5.9; annulus 1024^2 44 / 16.)
